@@ -16,10 +16,10 @@
 // reproduces the paper's global phase factors P_mu_nu by construction.
 //
 // Sigma (FP64).  The intermediate space is processed in chunks of whole categories
-// that fit the workspace: gather D[pq, K] = sum_J <K|E_pq|J> C_J for the chunk (J in
-// the target space, zero elsewhere: the categorical skip of empty blocks), E = G D on
-// the FP64 path, then every target determinant adds the terms <I|E_pq|K> E[pq, K]
-// whose K lies in the chunk.
+// that fit the workspace: D[pq, K] = sum_J <K|E_pq|J> C_J (J in the target space, zero
+// elsewhere: the categorical skip of empty blocks) and E = G D over the pairs that connect
+// K with the target space (fp64_active.cuh), then every target determinant adds the terms
+// <I|E_pq|K> E[pq, K] whose K lies in the chunk.
 #include <math.h>
 
 #include <stdlib.h>
@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "das_dev.cuh"
+#include "fp64_active.cuh"
 
 namespace {
 
@@ -39,36 +40,46 @@ using das_dev::das_strings;
 using das_dev::find_cat;
 using das_dev::make_dev;
 
-__global__ void __launch_bounds__(256) k_das_gather(DasDev d, int n_cat_int, int64_t a0, int64_t len,
-                                                    const int32_t *__restrict__ pairA,
-                                                    const int32_t *__restrict__ pairB,
-                                                    const double *__restrict__ C, double *__restrict__ D) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < len; k += (int64_t)gridDim.x * blockDim.x) {
+// The entries of the intermediate determinant a0 + k: the pairs whose alpha or beta move
+// stays in the target space (the source of D, and the reader of E).
+struct DasSource {
+    DasDev d;
+    int n_cat_int;
+    int64_t a0;
+    const int32_t *pairA, *pairB;
+    const double *C;
+    struct Ctx {
         int32_t A, B;
+    };
+    __device__ __forceinline__ Ctx ctx(int64_t k) const {
+        Ctx c;
         int pb;
-        das_strings(d, n_cat_int, a0 + k, A, B, pb);
-        for (int pp = 0; pp < d.npair; ++pp) {
-            double v = 0.0;
-            const int32_t ea = __ldg(pairA + (int64_t)pp * d.nsa + A);
-            if (ea >= 0) {
-                const int64_t j = das_addr(d, ea >> 1, B);
-                if (j >= 0 && j < d.n_det) {
-                    const double c = __ldg(C + j);
-                    v = (ea & 1) ? -c : c;
-                }
-            }
-            const int32_t eb = __ldg(pairB + (int64_t)pp * d.nsb + B);
-            if (eb >= 0) {
-                const int64_t j = das_addr(d, A, eb >> 1);
-                if (j >= 0 && j < d.n_det) {
-                    const double c = __ldg(C + j);
-                    v += (eb & 1) ? -c : c;
-                }
-            }
-            D[(int64_t)pp * len + k] = v;
-        }
+        das_strings(d, n_cat_int, a0 + k, c.A, c.B, pb);
+        return c;
     }
-}
+    __device__ __forceinline__ bool pair(const Ctx &c, int pp, double &v) const {
+        bool on = false;
+        const int32_t ea = __ldg(pairA + (int64_t)pp * d.nsa + c.A);
+        if (ea >= 0) {
+            const int64_t j = das_addr(d, ea >> 1, c.B);
+            if (j >= 0 && j < d.n_det) {
+                const double x = __ldg(C + j);
+                v = (ea & 1) ? -x : x;
+                on = true;
+            }
+        }
+        const int32_t eb = __ldg(pairB + (int64_t)pp * d.nsb + c.B);
+        if (eb >= 0) {
+            const int64_t j = das_addr(d, c.A, eb >> 1);
+            if (j >= 0 && j < d.n_det) {
+                const double x = __ldg(C + j);
+                v += (eb & 1) ? -x : x;
+                on = true;
+            }
+        }
+        return on;
+    }
+};
 
 __global__ void __launch_bounds__(256) k_das_scatter(DasDev d, int64_t a0, int64_t len,
                                                      const int32_t *__restrict__ pairA,
@@ -314,13 +325,14 @@ int das_build(fci_context *h, int S, const int *orbs, const int *ref_a, const in
     return FCI_OK;
 }
 
-// Chunk of the intermediate space processed per pass: whole categories, D and E both
-// resident; at most 16 GiB of workspace so very large spaces run in several passes.
+// Chunk of the intermediate space processed per pass: whole categories, E resident; at most
+// 8 GiB of workspace (a single larger category aside) so very large spaces run in several
+// passes.
 // FCI_DAS_FP64_CHUNK_DETS=n lowers the cap to n determinants (never below the largest
 // category), so that small problems can run the several-pass form too.
 static int64_t das_chunk_len(const fci_context *h) {
-    const int64_t cap_bytes = (int64_t)16 << 30;
-    const int64_t per_det = 2 * 8 * (int64_t)h->npair;
+    const int64_t cap_bytes = (int64_t)8 << 30;
+    const int64_t per_det = 8 * (int64_t)h->npair;
     const fci_das_layout &L = h->das;
     int64_t maxcat = 0;
     for (int c = 0; c < L.n_cat_int; ++c) maxcat = std::max(maxcat, L.cat_off[c + 1] - L.cat_off[c]);
@@ -335,7 +347,7 @@ static int64_t das_chunk_len(const fci_context *h) {
 size_t das_workspace_bytes(const fci_context *h, int precision, int n_slices) {
     if (precision == FCI_PREC_OZ_BF16) return dz_workspace_bytes(h, n_slices);
     const int64_t len = das_chunk_len(h);
-    return 2 * al((size_t)h->npair * len * 8);
+    return al((size_t)h->npair * len * 8);
 }
 
 int das_sigma_fp64(fci_context *h, const double *C, double *sigma, void *ws, size_t ws_bytes, cudaStream_t s) {
@@ -343,8 +355,7 @@ int das_sigma_fp64(fci_context *h, const double *C, double *sigma, void *ws, siz
     const fci_das_layout &L = h->das;
     const DasDev d = make_dev(h);
     const int64_t cap = das_chunk_len(h);
-    double *D = (double *)ws;
-    double *E = (double *)((char *)ws + al((size_t)h->npair * cap * 8));
+    double *E = (double *)ws;
     int c0 = 0;
     bool first = true;
     while (c0 < L.n_cat_int) {
@@ -352,13 +363,9 @@ int das_sigma_fp64(fci_context *h, const double *C, double *sigma, void *ws, siz
         while (c1 < L.n_cat_int && L.cat_off[c1 + 1] - L.cat_off[c0] <= cap) ++c1;
         const int64_t a0 = L.cat_off[c0], len = L.cat_off[c1] - a0;
         {
-            phase_scope ps(h, s, FCI_PHASE_GATHER, 1);
-            k_das_gather<<<grid_for(len), 256, 0, s>>>(d, L.n_cat_int, a0, len, h->d_pair_a, h->d_pair_b, C, D);
-            FCI_CUDA(h, cudaGetLastError());
-        }
-        {
             phase_scope ps(h, s, FCI_PHASE_CONTRACT, 1);
-            FCI_CUDA(h, launch_dgemm(h->npair, len, h->npair, h->d_G, D, len, E, len, s));
+            const DasSource src{d, L.n_cat_int, a0, h->d_pair_a, h->d_pair_b, C};
+            FCI_CUDA(h, fp64_active::launch_real(src, len, h->npair, h->d_GT, E, len, s));
         }
         {
             phase_scope ps(h, s, FCI_PHASE_SCATTER, 1);

@@ -164,7 +164,7 @@ static void free_strings(fci_context *h) {
     fci_dev_free(h->d_pair_a); fci_dev_free(h->d_pair_b);
     fci_dev_free(h->d_pair_a_t); fci_dev_free(h->d_pair_b_t);
     fci_dev_free(h->d_dstr);
-    fci_dev_free(h->d_G); fci_dev_free(h->d_hd); fci_dev_free(h->d_J); fci_dev_free(h->d_K);
+    fci_dev_free(h->d_G); fci_dev_free(h->d_GT); fci_dev_free(h->d_hd); fci_dev_free(h->d_J); fci_dev_free(h->d_K);
     fci_dev_free(h->d_Gs);
     fci_dev_free(h->d_Gt);
     h->d_str_a = h->d_str_b = nullptr;
@@ -172,7 +172,7 @@ static void free_strings(fci_context *h) {
     h->d_pair_a = h->d_pair_b = nullptr;
     h->d_pair_a_t = h->d_pair_b_t = nullptr;
     h->d_dstr = nullptr;
-    h->d_G = h->d_hd = h->d_J = h->d_K = nullptr;
+    h->d_G = h->d_GT = h->d_hd = h->d_J = h->d_K = nullptr;
     h->d_Gs = nullptr;
     h->Gs_slices = 0;
     h->d_Gt = nullptr;
@@ -362,7 +362,7 @@ int fci_setup_integrals(fci_handle h, int n, int dtype, const void *h1, const vo
 // G = 1/2 g', g'_pqrs = (pq|rs) + (h'_pq d_rs + d_pq h'_rs) / N_e, h' = h - 1/2 sum_r (pr|rq).
 // Real: packed over unordered pairs (p>=q, r>=s), row-major [npair][npair].
 // Complex: full [n^2][n^2], interleaved.
-static int prepare_operator(fci_context *h, int n_el) {
+static int prepare_operator(fci_context *h, int n_el, cudaStream_t s) {
     const int n = h->n_orb, w = h->dtype == FCI_C128 ? 2 : 1;
     const size_t n2 = (size_t)n * n;
     auto gidx = [&](int p, int q, int r, int s) { return (((size_t)p * n + q) * n + r) * n + s; };
@@ -411,6 +411,9 @@ static int prepare_operator(fci_context *h, int n_el) {
     int rc = fci_dev_alloc(h, (void **)&h->d_G, G.size() * 8);
     if (rc) return rc;
     FCI_CUDA(h, cudaMemcpy(h->d_G, G.data(), G.size() * 8, cudaMemcpyHostToDevice));
+    rc = fci_dev_alloc(h, (void **)&h->d_GT, G.size() * 8);
+    if (rc) return rc;
+    FCI_CUDA(h, launch_transpose_operator(h->npair, w, h->d_G, h->d_GT, s));
     // diagonal helpers (real parts; exact for Hermitian integrals)
     std::vector<double> hd(n), J(n2), K(n2);
     for (int p = 0; p < n; ++p) {
@@ -455,7 +458,7 @@ int fci_build_strings(fci_handle h, int n_alpha, int n_beta, fci_stream stream) 
     h->ndet = nsa * nsb;
     h->nent_a = n_alpha * (n - n_alpha + 1);
     h->nent_b = spinor ? 0 : n_beta * (n - n_beta + 1);
-    rc = prepare_operator(h, spinor ? n_alpha : n_alpha + n_beta);
+    rc = prepare_operator(h, spinor ? n_alpha : n_alpha + n_beta, s);
     if (rc) { free_strings(h); return rc; }
     rc = fci_dev_alloc(h, (void **)&h->d_str_a, nsa * 8);
     if (!rc && !spinor) rc = fci_dev_alloc(h, (void **)&h->d_str_b, nsb * 8);
@@ -1019,12 +1022,11 @@ size_t sigma_ws_bytes(const fci_context *h, int precision, int n_slices) {
     if (precision == FCI_PREC_OZ_BF16 && h->mode == FCI_MODE_SPINOR) return cz_workspace_bytes(h, n_slices);
     if (precision == FCI_PREC_OZ_BF16) return oz_workspace_bytes(h, n_slices);
     const size_t esz = h->dtype == FCI_C128 ? 16 : 8;
-    return 2 * al((size_t)h->npair * h->ndet * esz);
+    return al((size_t)h->npair * h->ndet * esz);
 }
 
 int sigma_dispatch(fci_context *h, const void *C, void *sigma, int precision, int n_slices, void *ws,
                    size_t ws_bytes, cudaStream_t s) {
-    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     if (h->das_active) {
         return precision == FCI_PREC_FP64 ? das_sigma_fp64(h, (const double *)C, (double *)sigma, ws, ws_bytes, s)
                                           : das_sigma_oz(h, (const double *)C, (double *)sigma, n_slices, ws, ws_bytes, s);
@@ -1032,19 +1034,12 @@ int sigma_dispatch(fci_context *h, const void *C, void *sigma, int precision, in
     if (precision == FCI_PREC_OZ_BF16 && h->mode == FCI_MODE_SPINOR)
         return cz_sigma(h, (const double *)C, (double *)sigma, n_slices, ws, ws_bytes, s);
     if (precision == FCI_PREC_OZ_BF16) return oz_sigma_fci(h, (const double *)C, (double *)sigma, n_slices, ws, ws_bytes, s);
-    const size_t esz = h->dtype == FCI_C128 ? 16 : 8;
-    double *D = (double *)ws;
-    double *E = (double *)((char *)ws + al((size_t)h->npair * h->ndet * esz));
+    double *E = (double *)ws;
     const bool real = h->mode == FCI_MODE_FCI;
     {
-        phase_scope ps(h, s, FCI_PHASE_GATHER, 1);
-        FCI_CUDA(h, real ? launch_gather_fci_r64(h, (const double *)C, D, s)
-                         : launch_gather_spinor(h, (const double *)C, D, s));
-    }
-    {
         phase_scope ps(h, s, FCI_PHASE_CONTRACT, 1);
-        FCI_CUDA(h, real ? launch_dgemm(h->npair, h->ndet, h->npair, h->d_G, D, h->ndet, E, h->ndet, s)
-                         : launch_zgemm(h->npair, h->ndet, h->npair, h->d_G, D, h->ndet, E, h->ndet, s));
+        FCI_CUDA(h, real ? launch_contract_fci_r64(h, (const double *)C, E, s)
+                         : launch_contract_spinor(h, (const double *)C, E, s));
     }
     {
         phase_scope ps(h, s, FCI_PHASE_SCATTER, 1);

@@ -114,6 +114,7 @@ struct fci_context {
 
     // contraction matrix G = 1/2 g' (packed real [npair x npair], or complex [n^2 x n^2])
     double *d_G = nullptr;
+    double *d_GT = nullptr;  // its transpose (the FP64 contraction reads rows of G^T)
     // diagonal helpers: h_pp, J_pq = (pp|qq), K_pq = (pq|qp) (real parts)
     double *d_hd = nullptr, *d_J = nullptr, *d_K = nullptr;
     // per alpha and beta string (alpha strings first, n_orb + 1 doubles each): the string's
@@ -197,21 +198,19 @@ cudaError_t launch_repl_table(int m, int ne, int64_t ns, const uint64_t *str, co
 cudaError_t launch_export_repl(int64_t ns, int n_ent, const uint64_t *rep, int32_t *dst, cudaStream_t s);
 
 // sigma_fp64.cu
-cudaError_t launch_gather_fci_r64(const fci_context *h, const double *C, double *D, cudaStream_t s);
+// E = G D on the entries that the scatter reads ([n_pair][n_det]; the others are not written).
+cudaError_t launch_contract_fci_r64(const fci_context *h, const double *C, double *E, cudaStream_t s);
 cudaError_t launch_scatter_fci_r64(const fci_context *h, const double *E, const double *C,
                                    double *sigma, cudaStream_t s);
-cudaError_t launch_dgemm(int M, int64_t N, int K, const double *A, const double *B, int64_t ldb,
-                         double *C, int64_t ldc, cudaStream_t s);
+cudaError_t launch_transpose_operator(int n, int w, const double *G, double *GT, cudaStream_t s);
 // Per-string diagonal tables (d_dstr) from the current integrals.
 cudaError_t launch_diag_strings(const fci_context *h, cudaStream_t s);
 cudaError_t launch_diag_fci(const fci_context *h, double *diag, cudaStream_t s);
 
 // spinor.cu
-cudaError_t launch_gather_spinor(const fci_context *h, const double *C, double *D, cudaStream_t s);
+cudaError_t launch_contract_spinor(const fci_context *h, const double *C, double *E, cudaStream_t s);
 cudaError_t launch_scatter_spinor(const fci_context *h, const double *E, const double *C,
                                   double *sigma, cudaStream_t s);
-cudaError_t launch_zgemm(int M, int64_t N, int K, const double *A, const double *B, int64_t ldb,
-                         double *C, int64_t ldc, cudaStream_t s);
 cudaError_t launch_diag_spinor(const fci_context *h, double *diag, cudaStream_t s);
 
 // das.cu

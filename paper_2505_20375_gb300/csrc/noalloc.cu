@@ -1,7 +1,8 @@
 // fci_sigma_noalloc: the FP64 sigma build with its scratch in a fixed device array.
 //
-// fci_sigma needs D and E intermediates (2 x n_pair x n_det elements) in a workspace
-// the caller allocates.  Some callers cannot allocate device memory when they need a
+// fci_sigma needs the E intermediate (n_pair x n_det elements) in a workspace the caller
+// allocates (the documented size limit still counts the D that an earlier form kept beside
+// it).  Some callers cannot allocate device memory when they need a
 // sigma vector: a process whose framework has already reserved the whole device
 // memory pool for its own caching allocator, code running where CUDA allocation calls
 // are not allowed (for example inside a host callback enqueued on a stream), or a
@@ -67,18 +68,15 @@ extern "C" int fci_sigma_noalloc(fci_handle h, const void *C, void *sigma, fci_s
         }
         scratch = g_noalloc_ptr[h->device];
     }
-    // D and E are written in full by the gather and the contraction before they are
-    // read, so the shared array needs no clearing between calls.
-    double *D = (double *)scratch;
-    double *E = (double *)((char *)scratch + half);
+    // The scatter reads only entries of E that the contraction of the same call has written,
+    // so the shared array needs no clearing between calls.
+    double *E = (double *)scratch;
     cudaStream_t s = (cudaStream_t)stream;
     if (h->mode == FCI_MODE_FCI) {
-        FCI_CUDA(h, launch_gather_fci_r64(h, (const double *)C, D, s));
-        FCI_CUDA(h, launch_dgemm(h->npair, h->ndet, h->npair, h->d_G, D, h->ndet, E, h->ndet, s));
+        FCI_CUDA(h, launch_contract_fci_r64(h, (const double *)C, E, s));
         FCI_CUDA(h, launch_scatter_fci_r64(h, E, (const double *)C, (double *)sigma, s));
     } else {
-        FCI_CUDA(h, launch_gather_spinor(h, (const double *)C, D, s));
-        FCI_CUDA(h, launch_zgemm(h->npair, h->ndet, h->npair, h->d_G, D, h->ndet, E, h->ndet, s));
+        FCI_CUDA(h, launch_contract_spinor(h, (const double *)C, E, s));
         FCI_CUDA(h, launch_scatter_spinor(h, E, (const double *)C, (double *)sigma, s));
     }
     return FCI_OK;

@@ -1,48 +1,48 @@
-// FP64 sigma build for alpha/beta strings (real spin-free orbitals), unfused form:
-//   gather  D[pq,K] = sum_J <K|E_pq|J> C_J                  (pair-packed pq)
-//   GEMM    E = G D, G = 1/2 g' packed                        (FP64)
-//   scatter sigma_I = e_core C_I + sum_{pq,K} <I|E_pq|K> E[pq,K]
+// FP64 sigma build for alpha/beta strings (real spin-free orbitals):
+//   gather + contraction  D[pq,K] = sum_J <K|E_pq|J> C_J (pair-packed pq), E = G D,
+//                         G = 1/2 g' packed, over the nonzero entries (fp64_active.cuh)
+//   scatter               sigma_I = e_core C_I + sum_{pq,K} <I|E_pq|K> E[pq,K]
 // (Methods, Eqs. sigmaL, sigmaL1e, sigmaL2e; the one-electron term is folded into g').
 //
-// Layouts: C and sigma are [N_alpha][N_beta] row-major; D and E are pair-major
-// [n_pair][N_det] so that consecutive threads (consecutive beta strings) touch
-// consecutive addresses.  The dense pair tables are [n_pair][N_str]: entry
-// (T << 1) | neg for the single replacement of the string that lands on pair pq, or -1.
-// Because a string's list never holds both (a,b) and (b,a) for a != b, each packed
-// pair has at most one entry per string and spin.
+// Layouts: C and sigma are [N_alpha][N_beta] row-major; E is pair-major [n_pair][N_det] so
+// that consecutive threads (consecutive beta strings) read consecutive addresses.  The
+// dense pair tables are [n_pair][N_str]: entry (T << 1) | neg for the single replacement
+// of the string that lands on pair pq, or -1.  Because a string's list never holds both
+// (a,b) and (b,a) for a != b, each packed pair has at most one entry per string and spin,
+// and the same pair leads back from T.
 #include <algorithm>
 
 #include "fci_internal.h"
+#include "fp64_active.cuh"
 
 namespace {
 
-__global__ void __launch_bounds__(256) k_gather_fci_r64(int64_t nsa, int64_t nsb, int npair,
-                                                        const int32_t *__restrict__ pairA,
-                                                        const int32_t *__restrict__ pairB,
-                                                        const double *__restrict__ C,
-                                                        double *__restrict__ D) {
-    const int64_t ndet = nsa * nsb;
-    const int64_t ib = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (ib >= nsb) return;
-    for (int64_t ia = blockIdx.y; ia < nsa; ia += gridDim.y) {
-        const int64_t det = ia * nsb + ib;
-        const double *Crow = C + ia * nsb;
-        for (int pp = 0; pp < npair; ++pp) {
-            double v = 0.0;
-            const int32_t ea = __ldg(pairA + (int64_t)pp * nsa + ia);
-            if (ea >= 0) {
-                const double c = __ldg(C + (int64_t)(ea >> 1) * nsb + ib);
-                v = (ea & 1) ? -c : c;
-            }
-            const int32_t eb = __ldg(pairB + (int64_t)pp * nsb + ib);
-            if (eb >= 0) {
-                const double c = __ldg(Crow + (eb >> 1));
-                v += (eb & 1) ? -c : c;
-            }
-            D[(int64_t)pp * ndet + det] = v;
-        }
+// The entries of K = (ia, ib): every pair on which the alpha or the beta string has a
+// replacement; D is the signed sum of the (at most two) sources.
+struct FciSource {
+    int64_t nsa, nsb;
+    const int32_t *pairA, *pairB;
+    const double *C;
+    struct Ctx {
+        int64_t ia, ib;
+    };
+    __device__ __forceinline__ Ctx ctx(int64_t K) const {
+        const int64_t ia = K / nsb;
+        return {ia, K - ia * nsb};
     }
-}
+    __device__ __forceinline__ bool pair(const Ctx &c, int pp, double &v) const {
+        const int32_t ea = __ldg(pairA + (int64_t)pp * nsa + c.ia), eb = __ldg(pairB + (int64_t)pp * nsb + c.ib);
+        if (ea >= 0) {
+            const double x = __ldg(C + (int64_t)(ea >> 1) * nsb + c.ib);
+            v = (ea & 1) ? -x : x;
+        }
+        if (eb >= 0) {
+            const double x = __ldg(C + c.ia * nsb + (eb >> 1));
+            v += (eb & 1) ? -x : x;
+        }
+        return ea >= 0 || eb >= 0;
+    }
+};
 
 __global__ void __launch_bounds__(256) k_scatter_fci_r64(int64_t nsa, int64_t nsb, int npair,
                                                          const int32_t *__restrict__ pairA,
@@ -73,55 +73,12 @@ __global__ void __launch_bounds__(256) k_scatter_fci_r64(int64_t nsa, int64_t ns
     }
 }
 
-// C[M x N] = A[M x K] * B[K x N], all row-major FP64, N large.  64 x 64 tiles,
-// 256 threads each owning a 4 x 4 block of outputs; K staged through shared memory in
-// chunks of 16.  The FP64 pipe bounds this kernel on GB300.
-constexpr int BM = 64, BN = 64, BK = 16;
-__global__ void __launch_bounds__(256) k_dgemm(int M, int64_t N, int K, const double *__restrict__ A,
-                                               const double *__restrict__ B, int64_t ldb,
-                                               double *__restrict__ Cm, int64_t ldc) {
-    __shared__ double sA[BK][BM + 1];
-    __shared__ double sB[BK][BN];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * BM;
-    const int64_t n0 = blockIdx.x * (int64_t)BN;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        for (int i = threadIdx.x; i < BK * BM; i += 256) {
-            int kk = i % BK, mm = i / BK;
-            int gm = m0 + mm, gk = k0 + kk;
-            sA[kk][mm] = (gm < M && gk < K) ? A[(int64_t)gm * K + gk] : 0.0;
-        }
-        for (int i = threadIdx.x; i < BK * BN; i += 256) {
-            int kk = i / BN, nn = i % BN;
-            int64_t gn = n0 + nn;
-            int gk = k0 + kk;
-            sB[kk][nn] = (gn < N && gk < K) ? B[(int64_t)gk * ldb + gn] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = sA[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = sB[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int gm = m0 + ty * 4 + i;
-        if (gm >= M) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int64_t gn = n0 + tx + 16 * j;
-            if (gn < N) Cm[(int64_t)gm * ldc + gn] = acc[i][j];
-        }
+// GT[c][r] = G[r][c] of the n x n operator (w = 1 real, 2 interleaved complex).
+__global__ void k_transpose_operator(int n, int w, const double *__restrict__ G, double *__restrict__ GT) {
+    const int64_t total = (int64_t)n * n;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t c = i / n, r = i - c * n;
+        for (int k = 0; k < w; ++k) GT[i * w + k] = G[(r * n + c) * w + k];
     }
 }
 
@@ -175,11 +132,9 @@ inline dim3 det_grid(int64_t nsa, int64_t nsb, int threads) {
 
 }  // namespace
 
-cudaError_t launch_gather_fci_r64(const fci_context *h, const double *C, double *D, cudaStream_t s) {
-    const int threads = 128;
-    k_gather_fci_r64<<<det_grid(h->nsa, h->nsb, threads), threads, 0, s>>>(
-        h->nsa, h->nsb, h->npair, h->d_pair_a, h->d_pair_b, C, D);
-    return cudaGetLastError();
+cudaError_t launch_contract_fci_r64(const fci_context *h, const double *C, double *E, cudaStream_t s) {
+    const FciSource src{h->nsa, h->nsb, h->d_pair_a, h->d_pair_b, C};
+    return fp64_active::launch_real(src, h->ndet, h->npair, h->d_GT, E, h->ndet, s);
 }
 
 cudaError_t launch_scatter_fci_r64(const fci_context *h, const double *E, const double *C,
@@ -190,11 +145,9 @@ cudaError_t launch_scatter_fci_r64(const fci_context *h, const double *E, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_dgemm(int M, int64_t N, int K, const double *A, const double *B, int64_t ldb,
-                         double *C, int64_t ldc, cudaStream_t s) {
-    if (M <= 0 || N <= 0) return cudaSuccess;
-    dim3 grid((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM));
-    k_dgemm<<<grid, 256, 0, s>>>(M, N, K, A, B, ldb, C, ldc);
+cudaError_t launch_transpose_operator(int n, int w, const double *G, double *GT, cudaStream_t s) {
+    const int64_t total = (int64_t)n * n;
+    k_transpose_operator<<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 152 * 8), 256, 0, s>>>(n, w, G, GT);
     return cudaGetLastError();
 }
 
