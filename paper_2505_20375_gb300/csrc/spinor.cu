@@ -145,7 +145,7 @@ cudaError_t launch_contract_spinor(const fci_context *h, const double *C, double
     if (m == 0) return cudaSuccess;  // no electron: the scatter reads nothing
     const int entry = (int)(sizeof(double2) + sizeof(int));
     const int T = fp64_active::batch_dets(m, h->nsa, entry);
-    const int64_t blocks = std::min<int64_t>(ceil_div(h->nsa, T), 152 * 6);
+    const int64_t blocks = std::min<int64_t>(ceil_div(h->nsa, T), 0x7FFFFFFF);
     k_contract_spinor<<<(unsigned)blocks, ZA_THREADS, (size_t)T * m * entry, s>>>(
         h->n_orb, h->na, h->nsa, T, h->d_str_a, h->d_binom, (const double2 *)C, (const double2 *)h->d_GT, (double2 *)E);
     return cudaGetLastError();
