@@ -41,6 +41,27 @@ __host__ __device__ constexpr int oz_gemm_L0(int s, int w) {
 // Pipeline stages that fit for s slices, kcc cores per chunk, and (resa_kc > 0) a resident
 // A image of resa_kc chunks (0: does not fit).
 int oz_gemm_ring(int s, int kcc, int resa_kc);
-// Launch over every (N-tile, M-tile) unit; w = digit bits.  Built forms: (w 7, kcc 4),
-// (w 8, kcc 4), (w 8, kcc 2, resident A, one M-tile).
+// Launch over every (N-tile, M-tile) unit; w = digit bits.  Built forms: (w 8, kcc 4),
+// (w 8, kcc 2, resident A, one M-tile).
 int oz_gemm_launch(fci_context *h, int s, int w, int kcc, bool resa, const oz_gemm_args &a, cudaStream_t st);
+
+// The block-sparse form (ozaki_blk.cu): the pair index is cut into n_blk blocks of 16, and
+// tile nt takes part in the blocks whose bit is set in masks[nt] only, as rows and as
+// columns of G.
+//   Gimg: [row block][K block][row group of 8][plane][K core][8 x 16 bytes]
+//   Dimg: [tile][K block][plane][row group of 8][K core][8 x 16 bytes] (inactive blocks unread)
+//   rowmap: [16 n_blk] row of E of each position, -1 for padding
+//   E: [tile][M_pad][64], written for the rows of active blocks
+// Digit widths w: 7 (s = 2 .. 8) and 8 (s = 4 .. 8).
+constexpr int OZG_MAX_BLK = 128;
+struct oz_blk_args {
+    int n_blk, M_pad;
+    int64_t n_nt;
+    const void *Gimg, *Dimg;
+    const ulonglong2 *masks;
+    const int32_t *rowmap;
+    int64_t *E;
+    int *status;
+};
+int oz_blk_ring(int s);  // pipeline stages that fit for s slices (0: none)
+int oz_blk_launch(fci_context *h, int s, int w, const oz_blk_args &a, cudaStream_t st);

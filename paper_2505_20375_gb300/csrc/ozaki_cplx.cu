@@ -5,10 +5,19 @@
 // real embedding (index 2x = real part, 2x + 1 = imaginary part of complex index x):
 //   [E_re; E_im] = [[G_re, -G_im]; [G_im, G_re]] [D_re; D_im],
 // M = K = 2 n^2 rows (1,152 at 24 spinors), N = the determinants.  Neither operand fits in
-// shared memory, so both are streamed: the G digit slices (prepared once) and the D digit
-// slices (split from the fixed-point C by k_cz_split each sigma) are stored in HBM in the
-// exact shared-memory layout of the MMA operands, tile by tile, and every K-chunk stage
-// of the pipeline is filled by two cp.async.bulk copies that complete on an mbarrier.
+// shared memory, so both are streamed from digit images in the shared-memory layout of the
+// MMA operands: the G digit slices (prepared once) and the D digit slices (split from the
+// fixed-point C by k_cz_split each sigma).
+//
+// A determinant has 156 of the 576 pairs at 24 spinors / 12 electrons, and 64 consecutive
+// strings (one tile) share most of them: the pair index is cut into blocks of 8 pairs (16
+// real rows or columns) by orbital ranges, L the 8 lowest spinors and U the others,
+//   (a in U, 8 b of U) and (a in U, b of L): active if some string of the tile has a;
+//   (8 a of L, b in U): active if some string of the tile lacks b;  (a in L, b of L): always,
+// for column pairs (a, b) = (r, s) of D[rs, K] and, with the roles of the indices exchanged,
+// (a, b) = (q, p) for the rows of E[pq, K], so one mask per tile serves both.  Inactive
+// blocks are neither written nor multiplied nor stored (ozaki_blk.cu): 45 of 72 blocks are
+// active on average at 24 / 12.
 //
 // Digits are balanced base-128 (7 bits, [-64, 63], exact in f16).  A D column has at
 // most 2 n_e (n - n_e + 1) nonzero entries (312 at 24 spinors / 12 electrons), so a level
@@ -18,9 +27,10 @@
 // away), and the scatter sums in int64:
 //   sigma_I = 2^{7 L0 - sh_G - sh_C} sum <I|E_x|K> E_int[x, K] + e_core C_I.
 //
-// The GEMM itself is the shared bulk-copy kernel (ozaki_gemm.cu) with 7-bit digits.
+// The GEMM itself is the block-sparse bulk-copy kernel (ozaki_blk.cu) with 7-bit digits.
 #include <math.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <algorithm>
 #include <complex>
@@ -34,12 +44,45 @@ namespace {
 
 using namespace tc;
 
-constexpr int CZ_M = OZG_M;
 constexpr int CZ_N = OZG_N;
-constexpr int CZ_KC = OZG_KC;
-constexpr int CZ_A_PLANE = OZG_A_PLANE;
-constexpr int CZ_B_PLANE = OZG_B_PLANE;
 constexpr int CZ_MAXS = OZG_MAXS;
+
+// The blocks of 8 pairs (a, b) of n spinors, in the order of the header comment.
+struct CzBlocks {
+    int n, L, U, ubk;        // spinors, low and upper ones, blocks of 8 over U
+    int ul, lu, ll, n_blk;   // first block of each later class, number of blocks
+};
+__host__ __device__ inline CzBlocks cz_blocks(int n) {
+    CzBlocks c;
+    c.n = n;
+    c.L = n < 8 ? n : 8;
+    c.U = n - c.L;
+    c.ubk = (c.U + 7) / 8;
+    c.ul = c.U * c.ubk;
+    c.lu = c.ul + c.U;
+    c.ll = c.lu + c.U;
+    c.n_blk = c.ll + c.L;
+    return c;
+}
+// Pair e (0 .. 7) of block k; false for a padding position.
+__host__ __device__ inline bool cz_pair(const CzBlocks &c, int k, int e, int &a, int &b) {
+    if (k < c.ul) {
+        a = c.L + k / c.ubk;
+        b = c.L + 8 * (k % c.ubk) + e;
+        return b < c.n;
+    }
+    if (k < c.lu) {
+        a = c.L + (k - c.ul);
+        b = e;
+    } else if (k < c.ll) {
+        a = e;
+        b = c.L + (k - c.lu);
+    } else {
+        a = k - c.ll;
+        b = e;
+    }
+    return e < c.L;
+}
 
 // ------------------------------------------------------------- helper kernels
 
@@ -93,33 +136,62 @@ __device__ __forceinline__ uint32_t digits7_f16x2(uint64_t x, uint64_t y, int j)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-// D digit image: block (N-tile nt, K-chunk kc) holds S planes of 64 determinants x 32
-// real-embedded K, each in canonical K-major core matrices (8 rows x 16 bytes; core
-// (row / 8, k / 8) at ((row / 8) * 4 + k / 8) * 128).  One CTA of 256 threads fills one
-// block: thread t covers determinant t % 64 and core t / 64 (4 complex pairs = 8 reals).
+// D digit image and block masks, one CTA of 256 threads per tile of 64 determinants: the
+// tile's union and intersection of occupations give the mask of active blocks; then the two
+// halves of the CTA take the active blocks in turn, thread (row, core) writing the 8 digits
+// of its 4 pairs (one core matrix row) per plane.
 template <int S>
-__global__ void __launch_bounds__(256) k_cz_split(int n, int64_t ndet, int n_kc, int64_t n_blocks,
-                                                  const uint64_t *__restrict__ str,
+__global__ void __launch_bounds__(256) k_cz_split(const CzBlocks bl, int64_t ndet, const uint64_t *__restrict__ str,
                                                   const uint64_t *__restrict__ binom,
-                                                  const int64_t *__restrict__ Cint, uint8_t *__restrict__ Dimg) {
+                                                  const int64_t *__restrict__ Cint, uint8_t *__restrict__ Dimg,
+                                                  ulonglong2 *__restrict__ masks) {
+    __shared__ uint32_t s_or[2], s_and[2], s_mask[4];
     uint64_t bias = 0;
 #pragma unroll
     for (int j = 0; j < S; ++j) bias |= (uint64_t)64 << (7 * j);
-    const int row = threadIdx.x & 63, cc = threadIdx.x >> 6;
-    const int n2 = n * n;
-    for (int64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
-        const int64_t nt = blk / n_kc;
-        const int kc = (int)(blk - nt * n_kc);
-        const int64_t K = nt * CZ_N + row;
-        uint64_t y[8];
-        const uint32_t Sm = K < ndet ? (uint32_t)__ldg(str + K) : 0u;
+    const int64_t nt = blockIdx.x;
+    const int row = threadIdx.x & 63, core = (threadIdx.x >> 6) & 1, half = threadIdx.x >> 7;
+    const int64_t K = nt * CZ_N + row;
+    const bool live = K < ndet;
+    const uint32_t Sm = live ? (uint32_t)__ldg(str + K) : 0u;
+    if (threadIdx.x < 64) {
+        const uint32_t o = __reduce_or_sync(0xFFFFFFFFu, Sm), a = __reduce_and_sync(0xFFFFFFFFu, live ? Sm : ~0u);
+        if ((threadIdx.x & 31) == 0) {
+            s_or[threadIdx.x >> 5] = o;
+            s_and[threadIdx.x >> 5] = a;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < OZG_MAX_BLK) {
+        const uint32_t occ = s_or[0] | s_or[1], full = s_and[0] & s_and[1];  // in some string; in every string
+        const int k = threadIdx.x;
+        bool on = k < bl.n_blk;
+        if (k < bl.ul) {
+            const int a = bl.L + k / bl.ubk, b0 = bl.L + 8 * (k % bl.ubk);
+            const uint32_t range = 0xFFu << b0;
+            on = ((occ >> a) & 1u) && ((~full | (1u << a)) & range) != 0;
+        } else if (k < bl.lu) {
+            on = (occ >> (bl.L + (k - bl.ul))) & 1u;
+        } else if (k < bl.ll) {
+            on = !((full >> (bl.L + (k - bl.lu))) & 1u);
+        }
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, on);
+        if ((threadIdx.x & 31) == 0) s_mask[threadIdx.x >> 5] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        masks[nt] = make_ulonglong2(s_mask[0] | ((uint64_t)s_mask[1] << 32), s_mask[2] | ((uint64_t)s_mask[3] << 32));
+    int turn = 0;
+    for (int w = 0; w < 4; ++w) {
+        for (uint32_t m = s_mask[w]; m; m &= m - 1, turn ^= 1) {
+            if (turn != half) continue;
+            const int k = 32 * w + __ffs(m) - 1;
+            uint64_t y[8];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int x = (kc * CZ_KC + cc * 8) / 2 + e;  // complex pair index
-            int64_t vr = 0, vi = 0;
-            if (K < ndet && x < n2) {
-                const int a = x / n, b = x - a * n;
-                if (((Sm >> a) & 1u) && (b == a || !((Sm >> b) & 1u))) {
+            for (int e = 0; e < 4; ++e) {
+                int64_t vr = 0, vi = 0;
+                int a, b;
+                if (cz_pair(bl, k, 4 * core + e, a, b) && ((Sm >> a) & 1u) && (b == a || !((Sm >> b) & 1u))) {
                     const uint32_t T = (Sm & ~(1u << a)) | (1u << b);
                     const int64_t t = cz_rank(T, binom);
                     const int64_t cr = __ldg(Cint + 2 * t), ci = __ldg(Cint + 2 * t + 1);
@@ -127,19 +199,19 @@ __global__ void __launch_bounds__(256) k_cz_split(int n, int64_t ndet, int n_kc,
                     vr = neg ? -cr : cr;
                     vi = neg ? -ci : ci;
                 }
+                y[2 * e] = (uint64_t)vr + bias;
+                y[2 * e + 1] = (uint64_t)vi + bias;
             }
-            y[2 * e] = (uint64_t)vr + bias;
-            y[2 * e + 1] = (uint64_t)vi + bias;
-        }
-        uint8_t *base = Dimg + (size_t)blk * S * CZ_B_PLANE + ((row >> 3) * 4 + cc) * 128 + (row & 7) * 16;
+            uint8_t *base = Dimg + ((size_t)nt * bl.n_blk + k) * S * 2048 + (row >> 3) * 256 + core * 128 + (row & 7) * 16;
 #pragma unroll
-        for (int j = 0; j < S; ++j) {
-            uint4 w;
-            w.x = digits7_f16x2(y[0], y[1], j);
-            w.y = digits7_f16x2(y[2], y[3], j);
-            w.z = digits7_f16x2(y[4], y[5], j);
-            w.w = digits7_f16x2(y[6], y[7], j);
-            __stcs((uint4 *)(base + j * CZ_B_PLANE), w);  // streaming: keep C_int in L2
+            for (int j = 0; j < S; ++j) {
+                uint4 d;
+                d.x = digits7_f16x2(y[0], y[1], j);
+                d.y = digits7_f16x2(y[2], y[3], j);
+                d.z = digits7_f16x2(y[4], y[5], j);
+                d.w = digits7_f16x2(y[6], y[7], j);
+                __stcs((uint4 *)(base + j * 2048), d);  // streaming: keep C_int in L2
+            }
         }
     }
 }
@@ -191,21 +263,6 @@ uint16_t half_bits_of_small_int(int d) {  // IEEE binary16 of an integer |d| <= 
     return (uint16_t)(sign | ((unsigned)(e + 15) << 10) | mant);
 }
 
-struct CzGeom {
-    int M_real, M_pad, K_pad, n_mt, n_kc;
-    int64_t n_nt;
-};
-
-void cz_geom(const fci_context *h, CzGeom &g) {
-    const int n2 = h->n_orb * h->n_orb;
-    g.M_real = 2 * n2;
-    g.M_pad = (g.M_real + CZ_M - 1) / CZ_M * CZ_M;
-    g.K_pad = (g.M_real + CZ_KC - 1) / CZ_KC * CZ_KC;
-    g.n_mt = g.M_pad / CZ_M;
-    g.n_kc = g.K_pad / CZ_KC;
-    g.n_nt = (h->ndet + CZ_N - 1) / CZ_N;
-}
-
 }  // namespace
 
 int cz_check(fci_context *h, int s) {
@@ -216,16 +273,16 @@ int cz_check(fci_context *h, int s) {
     if ((int64_t)s * nnz * 4096 >= ((int64_t)1 << 24))
         return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices x %lld nonzero terms could exceed 2^24 in a level sum", s,
                         (long long)nnz);
-    if (!oz_gemm_ring(s, 4, 0)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices do not fit two pipeline stages", s);
+    if (!oz_blk_ring(s)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices do not fit two pipeline stages", s);
     return FCI_OK;
 }
 
-// Real-embedded G digit image, tiles [M-tile][K-chunk][plane][128 x 32 core matrices].
+// Real-embedded G digit image in the A layout of the block-sparse GEMM, followed by the row
+// map (row of E of each position of a row block).
 static int cz_prepare_G(fci_context *h, int s) {
     if (h->Gs_slices == s && h->d_Gs) return FCI_OK;
-    CzGeom g;
-    cz_geom(h, g);
-    const int n2 = h->n_orb * h->n_orb;
+    const CzBlocks bl = cz_blocks(h->n_orb);
+    const int n = h->n_orb, n2 = n * n, np = bl.n_blk * 16;
     std::vector<double> G((size_t)n2 * n2 * 2);
     if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
         return fci_cuda_check(h, cudaGetLastError(), "G download");
@@ -236,26 +293,33 @@ static int cz_prepare_G(fci_context *h, int s) {
     const int shG = 7 * s - 2 - eG;
     uint64_t bias = 0;
     for (int j = 0; j < s; ++j) bias |= (uint64_t)64 << (7 * j);
-    const size_t stageA = (size_t)s * CZ_A_PLANE;
-    std::vector<uint16_t> img((size_t)g.n_mt * g.n_kc * stageA / 2, 0);
-    for (int m = 0; m < g.M_pad; ++m) {
-        const int mt = m / CZ_M, r = m % CZ_M;
-        for (int k = 0; k < g.K_pad; ++k) {
-            double v = 0.0;
-            if (m < g.M_real && k < g.M_real) {
-                const int x = m >> 1, u = m & 1, y = k >> 1, w = k & 1;  // complex row x, column y
-                const double gr = G[2 * ((size_t)x * n2 + y)], gi = G[2 * ((size_t)x * n2 + y) + 1];
-                v = (u == w) ? gr : (u == 0 ? -gi : gi);
+    // real-embedded index of each position as a column (r, s) = (a, b) and as a row (p, q) = (b, a)
+    std::vector<int32_t> col(np, -1), row(np, -1);
+    for (int k = 0; k < bl.n_blk; ++k)
+        for (int e = 0; e < 8; ++e) {
+            int a, b;
+            if (!cz_pair(bl, k, e, a, b)) continue;
+            for (int w = 0; w < 2; ++w) {
+                col[16 * k + 2 * e + w] = 2 * (a * n + b) + w;
+                row[16 * k + 2 * e + w] = 2 * (b * n + a) + w;
             }
-            const int64_t gi64 = llrint(ldexp(v, shG));
-            const uint64_t yb = (uint64_t)gi64 + bias;
-            const int kc = k / CZ_KC, kk = k % CZ_KC;
-            const size_t off = ((size_t)mt * g.n_kc + kc) * stageA + ((r >> 3) * 4 + (kk >> 3)) * 128 + (r & 7) * 16 +
-                               (kk & 7) * 2;
-            for (int j = 0; j < s; ++j)
-                img[(off + (size_t)j * CZ_A_PLANE) / 2] = half_bits_of_small_int((int)((yb >> (7 * j)) & 0x7F) - 64);
         }
-    }
+    const size_t map_off = (size_t)bl.n_blk * bl.n_blk * s * 512;
+    std::vector<uint16_t> img(map_off / 2 + (size_t)np * 2, 0);
+    for (int pr = 0; pr < np; ++pr)
+        for (int pc = 0; pc < np; ++pc) {
+            if (row[pr] < 0 || col[pc] < 0) continue;
+            const int x = row[pr] >> 1, u = row[pr] & 1, y = col[pc] >> 1, w = col[pc] & 1;  // complex row x, column y
+            const double gr = G[2 * ((size_t)x * n2 + y)], gi = G[2 * ((size_t)x * n2 + y) + 1];
+            const int64_t gi64 = llrint(ldexp(u == w ? gr : (u == 0 ? -gi : gi), shG));
+            const uint64_t yb = (uint64_t)gi64 + bias;
+            const int r = pr & 15, c = pc & 15;
+            const size_t off = ((size_t)(pr >> 4) * bl.n_blk + (pc >> 4)) * s * 512 + (size_t)(r >> 3) * s * 256 +
+                               (c >> 3) * 128 + (r & 7) * 16 + (c & 7) * 2;
+            for (int j = 0; j < s; ++j)
+                img[(off + (size_t)j * 256) / 2] = half_bits_of_small_int((int)((yb >> (7 * j)) & 0x7F) - 64);
+        }
+    memcpy(reinterpret_cast<char *>(img.data()) + map_off, row.data(), (size_t)np * 4);
     fci_dev_free(h->d_Gs);
     h->d_Gs = nullptr;
     h->Gs_slices = 0;
@@ -267,11 +331,11 @@ static int cz_prepare_G(fci_context *h, int s) {
     return FCI_OK;
 }
 
+// C_int, the D digit image, E_int, the block masks, 256 bytes of scalars.
 size_t cz_workspace_bytes(const fci_context *h, int s) {
-    CzGeom g;
-    cz_geom(h, g);
-    return al256((size_t)h->ndet * 16) + al256((size_t)g.n_nt * g.n_kc * s * CZ_B_PLANE) +
-           al256((size_t)g.n_nt * g.M_pad * CZ_N * 8) + 256;
+    const size_t n_nt = (size_t)ceil_div(h->ndet, CZ_N), n2 = (size_t)h->n_orb * h->n_orb;
+    return al256((size_t)h->ndet * 16) + al256(n_nt * cz_blocks(h->n_orb).n_blk * s * 2048) +
+           al256(n_nt * 2 * n2 * CZ_N * 8) + al256(n_nt * sizeof(ulonglong2)) + 256;
 }
 
 int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, size_t ws_bytes, cudaStream_t st) {
@@ -279,15 +343,18 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
     int rc = cz_check(h, s);
     if (!rc) rc = cz_prepare_G(h, s);
     if (rc) return rc;
-    CzGeom g;
-    cz_geom(h, g);
+    const CzBlocks bl = cz_blocks(h->n_orb);
+    const int64_t n_nt = ceil_div(h->ndet, CZ_N);
+    const int M_real = 2 * h->n_orb * h->n_orb;
     char *p = (char *)ws;
     int64_t *Cint = (int64_t *)p;
     p += al256((size_t)h->ndet * 16);
     uint8_t *Dimg = (uint8_t *)p;
-    p += al256((size_t)g.n_nt * g.n_kc * s * CZ_B_PLANE);
+    p += al256((size_t)n_nt * bl.n_blk * s * 2048);
     int64_t *E = (int64_t *)p;
-    p += al256((size_t)g.n_nt * g.M_pad * CZ_N * 8);
+    p += al256((size_t)n_nt * M_real * CZ_N * 8);
+    ulonglong2 *masks = (ulonglong2 *)p;
+    p += al256((size_t)n_nt * sizeof(ulonglong2));
     unsigned long long *maxbits = (unsigned long long *)p;
     int *shC = (int *)(p + 8), *status = (int *)(p + 16);
     {
@@ -296,32 +363,30 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
         const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(2 * h->ndet, 256), 152 * 8);
         k_cz_absmax<<<nb, 256, 0, st>>>(C, 2 * h->ndet, maxbits);
         k_cz_to_fixed<<<nb, 256, 0, st>>>(C, 2 * h->ndet, s, maxbits, Cint, shC);
-        const int64_t nblk = g.n_nt * g.n_kc;
-        const unsigned gb = (unsigned)std::min<int64_t>(nblk, 152 * 16);
         switch (s) {
-#define CZ_SPLIT(S_) case S_: k_cz_split<S_><<<gb, 256, 0, st>>>(h->n_orb, h->ndet, g.n_kc, nblk, h->d_str_a, h->d_binom, Cint, Dimg); break;
+#define CZ_SPLIT(S_) case S_: k_cz_split<S_><<<(unsigned)n_nt, 256, 0, st>>>(bl, h->ndet, h->d_str_a, h->d_binom, Cint, Dimg, masks); break;
             CZ_SPLIT(2) CZ_SPLIT(3) CZ_SPLIT(4) CZ_SPLIT(5) CZ_SPLIT(6) CZ_SPLIT(7) CZ_SPLIT(8)
 #undef CZ_SPLIT
         }
         FCI_CUDA(h, cudaGetLastError());
     }
     {
-        oz_gemm_args a;
-        a.n_mt = g.n_mt;
-        a.n_kc = g.n_kc;
-        a.M_pad = g.M_pad;
-        a.M_real = g.M_real;
-        a.n_nt = g.n_nt;
+        oz_blk_args a;
+        a.n_blk = bl.n_blk;
+        a.M_pad = M_real;
+        a.n_nt = n_nt;
         a.Gimg = h->d_Gs;
         a.Dimg = Dimg;
+        a.masks = masks;
+        a.rowmap = (const int32_t *)((const char *)h->d_Gs + (size_t)bl.n_blk * bl.n_blk * s * 512);
         a.E = E;
         a.status = status;
-        if ((rc = oz_gemm_launch(h, s, 7, 4, false, a, st))) return rc;
+        if ((rc = oz_blk_launch(h, s, 7, a, st))) return rc;
     }
     {
         phase_scope ps(h, st, FCI_PHASE_SCATTER, 1);
         const int L0 = oz_gemm_L0(s, 7);
-        k_cz_scatter<<<(unsigned)ceil_div(h->ndet, 128), 128, 0, st>>>(h->n_orb, h->ndet, g.M_pad, h->d_str_a,
+        k_cz_scatter<<<(unsigned)ceil_div(h->ndet, 128), 128, 0, st>>>(h->n_orb, h->ndet, M_real, h->d_str_a,
                                                                         h->d_binom, E, C, h->e_core,
                                                                         7 * L0 - h->G_exp, shC, status, h->d_status,
                                                                         sigma);

@@ -25,44 +25,16 @@
 #include <type_traits>
 
 #include "oz_gemm.cuh"
+#include "oz_pipe.cuh"
 #include "tc_ptx.cuh"
 
 namespace {
 
 using namespace tc;
+using namespace ozp;
 
-// Epilogue warps: 8 (two per TMEM lane quadrant, 32 columns each) when the level
-// accumulators are double-buffered, 16 (four per quadrant, 16 columns each) otherwise.
-__host__ __device__ constexpr int ozg_epi_warps(int s) { return 2 * s * OZG_N <= 512 ? 8 : 16; }
-constexpr int OZG_ISSUERS = 2;
-__host__ __device__ constexpr int ozg_threads(int s) { return 32 * (1 + OZG_ISSUERS + ozg_epi_warps(s)); }
-// The MMA issuer of level l of s (level l takes s - l products): levels in order of their
-// product counts, each to the issuer with the fewest products so far.
-__host__ __device__ constexpr int ozg_issuer(int s, int l) {
-    int load[OZG_ISSUERS] = {};
-    int who = 0;
-    for (int k = 0; k <= l; ++k) {
-        int m = 0;
-        for (int e = 1; e < OZG_ISSUERS; ++e)
-            if (load[e] < load[m]) m = e;
-        load[m] += s - k;
-        who = m;
-    }
-    return who;
-}
 constexpr int OZG_MAX_STAGES = 6;
 constexpr size_t OZG_SMEM_MAX = 232448 - 1024;
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(bar),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
 
 struct OzgParams {
     int n_mt, n_kc, M_pad, M_real, ring;
@@ -82,46 +54,6 @@ struct OzgShared {
     int abort;
 };
 
-template <bool FAST = false>
-__device__ __forceinline__ bool ozg_wait(uint32_t bar, uint32_t parity, volatile int *abort, int *status,
-                                        long long timeout) {
-    if (FAST && mbar_test_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    int spins = 0;
-    while (!mbar_try_wait_sleep(bar, parity)) {
-        if (((++spins) & 3) == 0) {
-            if (*abort) return false;
-            if (clock64() - t0 > timeout) {
-                *abort = 1;
-                atomicExch(status, FCI_ERR_TIMEOUT);
-                return false;
-            }
-        }
-    }
-    return true;
-}
-
-// Wait for a phase that must complete (copies or MMAs already issued) before the CTA may
-// leave: bounded like every other wait, but blind to the abort flag.
-__device__ __forceinline__ bool ozg_drain_wait(uint32_t bar, uint32_t parity, int *status, long long timeout) {
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (clock64() - t0 > timeout) {
-            atomicExch(status, FCI_ERR_TIMEOUT);
-            return false;
-        }
-    }
-    return true;
-}
-
-template <bool FAST = false>
-__device__ __forceinline__ bool ozg_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort, int *status,
-                                             long long timeout) {
-    int ok = 0;
-    if ((threadIdx.x & 31) == 0) ok = ozg_wait<FAST>(bar, parity, abort, status, timeout) ? 1 : 0;
-    return __shfl_sync(0xFFFFFFFFu, ok, 0) != 0;
-}
-
 // S slices, W-bit digits, KCC core matrices (8 K each) per pipeline stage, RESA: the whole
 // A image (one M-tile) is loaded into shared memory once and only B tiles stream.
 template <int S, int W, int KCC, bool RESA>
@@ -132,7 +64,6 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
     // group is free.
     constexpr int GH = 3;
     constexpr int NG = NBUF == 1 ? (S + GH - 1) / GH : 1;
-    constexpr int L0 = oz_gemm_L0(S, W);
     constexpr uint32_t A_PLANE = OZG_M * KCC * 16, B_PLANE = OZG_N * KCC * 16;
     constexpr uint32_t STAGE_A = S * A_PLANE, STAGE_B = S * B_PLANE;
     constexpr uint32_t STAGE_LOAD = RESA ? STAGE_B : STAGE_A + STAGE_B;
@@ -185,7 +116,7 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
                 bool ok = true;
                 for (int kc = 0; kc < p.n_kc; ++kc, ++q) {
                     if (q >= (uint32_t)R &&
-                        !ozg_wait<true>(smem_u32(&sh->empty[st]), ph ^ 1, abort, p.status, p.timeout_cycles)) {
+                        !wait_one<true>(smem_u32(&sh->empty[st]), ph ^ 1, abort, p.status, p.timeout_cycles)) {
                         ok = false;
                         break;
                     }
@@ -206,10 +137,10 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
             const uint32_t used = q < (uint32_t)R ? q : (uint32_t)R;
             for (uint32_t k = 1; k <= used; ++k) {
                 const uint32_t idx = q - k;
-                ozg_drain_wait(smem_u32(&sh->full[idx % (uint32_t)R]), (idx / (uint32_t)R) & 1u, p.status,
+                drain_wait(smem_u32(&sh->full[idx % (uint32_t)R]), (idx / (uint32_t)R) & 1u, p.status,
                                p.timeout_cycles);
             }
-            if (RESA) ozg_drain_wait(smem_u32(&sh->a_full), 0, p.status, p.timeout_cycles);
+            if (RESA) drain_wait(smem_u32(&sh->a_full), 0, p.status, p.timeout_cycles);
         }
     } else if (warp <= OZG_ISSUERS) {
         // ---------------------------------------------------------------- MMA issuers
@@ -220,7 +151,7 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
             // The ring slot and its parity advance with each stage (no division on the
             // issue path), and each wait first tests the barrier without blocking.
             auto wait = [&](uint32_t bar, uint32_t par) -> bool {
-                return ozg_wait<true>(bar, par, abort, p.status, p.timeout_cycles);
+                return wait_one<true>(bar, par, abort, p.status, p.timeout_cycles);
             };
             const uint32_t idesc = idesc_f16(OZG_M, OZG_N);
             const uint64_t a0 = smem_desc(smem_u32(sA), 128, KCC * 128);
@@ -295,8 +226,8 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
             // deallocation goes ahead
             if (issued) mma_commit(smem_u32(&sh->drain));
             else mbar_arrive(smem_u32(&sh->drain));
-            if (!ozg_drain_wait(smem_u32(&sh->drain), 0, p.status, p.timeout_cycles))
-                ozg_drain_wait(smem_u32(&sh->drain), 0, p.status, p.timeout_cycles);
+            if (!drain_wait(smem_u32(&sh->drain), 0, p.status, p.timeout_cycles))
+                drain_wait(smem_u32(&sh->drain), 0, p.status, p.timeout_cycles);
         };
         if (lane == 0) {
             if (warp == 1) issuer(std::integral_constant<int, 0>{});
@@ -305,98 +236,27 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
         }
     } else {
         // ---------------------------------------------------------------- epilogue
-        // Warp (quadrant qd, part) owns lanes 32 qd .. 32 qd + 31 and 16 CH columns from
-        // 16 CH part.  Single-buffered accumulators (s >= 5, CH = 1) are read GH levels at a
-        // time; each group is handed back to the MMA warp as soon as it is in registers, so
-        // the next unit's first K-chunk starts on it while the rest is read and combined.
-        // Double-buffered accumulators (s <= 4, CH = 2) are combined level by level and
-        // released at the end.
-        constexpr int CH = OZG_N / (4 * ozg_epi_warps(S));  // 16-column chunks per warp: 2 or 1
+        // Warp (quadrant qd, part) owns lanes 32 qd .. 32 qd + 31 and its share of the columns
+        // (oz_pipe.cuh).
         const int qd = warp & 3;
-        const int cw = 16 * CH * ((warp - 1 - OZG_ISSUERS) >> 2);
+        constexpr int NCOL = OZG_N / (ozg_epi_warps(S) / 4);  // columns per warp: 32 or 16
+        const int cw = NCOL * ((warp - 1 - OZG_ISSUERS) >> 2);
         const int row = 32 * qd + lane;
-        constexpr int lowshift = W * (L0 - (S - 1));
         uint32_t tau = 0;
         for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x, ++tau) {
             const int64_t nt = u / p.n_mt;
             const int mt = (int)(u - nt * p.n_mt);
             const int buf = NBUF == 2 ? (int)(tau & 1) : 0;
             const uint32_t par = NBUF == 2 ? (tau >> 1) & 1 : tau & 1;
-            if (!ozg_wait_warp(smem_u32(&sh->acc_full[buf]), par, abort, p.status, p.timeout_cycles)) break;
+            if (!wait_warp(smem_u32(&sh->acc_full[buf]), par, abort, p.status, p.timeout_cycles)) break;
             tc_fence_after();
-            const uint32_t tl0 = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * S * OZG_N + cw);
-            int64_t *dst0 = p.E + ((size_t)nt * p.M_pad + (size_t)mt * OZG_M + row) * OZG_N + cw;
+            const uint32_t tl = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * S * OZG_N);
+            int64_t *dst = p.E + ((size_t)nt * p.M_pad + (size_t)mt * OZG_M + row) * OZG_N;
             const bool keep = mt * OZG_M + row < p.M_real;  // rows past the operator's size are never read
-            if (NBUF == 1) {  // CH == 1: group by group, each released as soon as it is read
-                auto term = [](uint32_t x, int L) -> int64_t {
-                    const int64_t v = (int64_t)__float2int_rn(__uint_as_float(x));
-                    return L < L0 ? v * ((int64_t)1 << (W * (L - (S - 1)))) : v * ((int64_t)1 << (W * (L - L0)));
-                };
-                int64_t acc[16];
-#pragma unroll
-                for (int c = 0; c < 16; ++c) acc[c] = 0;
-#pragma unroll
-                for (int g = 0; g < NG; ++g) {
-                    uint32_t v[GH][16];
-#pragma unroll
-                    for (int l = g * GH; l < g * GH + GH && l < S; ++l) tmem_ld16(tl0 + (uint32_t)(l * OZG_N), v[l - g * GH]);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int l = g * GH; l < g * GH + GH && l < S; ++l) tmem_regs_ready(v[l - g * GH]);
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&sh->acc_empty[g]));
-#pragma unroll
-                    for (int l = g * GH; l < g * GH + GH && l < S; ++l) {
-                        const int L = S - 1 + l;
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            if (L == L0 && lowshift > 0)
-                                acc[c] = (acc[c] + ((int64_t)1 << (lowshift > 0 ? lowshift - 1 : 0))) >> lowshift;
-                            acc[c] += term(v[l - g * GH][c], L);
-                        }
-                    }
-                }
-                if (keep)
-#pragma unroll
-                    for (int c = 0; c < 16; c += 2) __stcs((longlong2 *)(dst0 + c), make_longlong2(acc[c], acc[c + 1]));
-            } else {
-                // double-buffered accumulators: combine level by level, release at the end
-#pragma unroll 1
-                for (int ch = 0; ch < CH; ++ch) {
-                    int64_t acc[16];
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) acc[c] = 0;
-#pragma unroll
-                    for (int L = S - 1; L <= 2 * S - 2; ++L) {
-                        uint32_t v[16];
-                        tmem_ld16(tl0 + (uint32_t)((L - (S - 1)) * OZG_N + 16 * ch), v);
-                        tmem_ld_wait();
-                        tmem_regs_ready(v);
-                        if (L < L0) {
-#pragma unroll
-                            for (int c = 0; c < 16; ++c)
-                                acc[c] += (int64_t)__float2int_rn(__uint_as_float(v[c])) * ((int64_t)1 << (W * (L - (S - 1))));
-                        } else {
-                            if (L == L0 && lowshift > 0) {
-#pragma unroll
-                                for (int c = 0; c < 16; ++c)
-                                    acc[c] = (acc[c] + ((int64_t)1 << (lowshift > 0 ? lowshift - 1 : 0))) >> lowshift;
-                            }
-#pragma unroll
-                            for (int c = 0; c < 16; ++c)
-                                acc[c] += (int64_t)__float2int_rn(__uint_as_float(v[c])) * ((int64_t)1 << (W * (L - L0)));
-                        }
-                    }
-                    if (keep)
-#pragma unroll
-                        for (int c = 0; c < 16; c += 2)
-                            __stcs((longlong2 *)(dst0 + 16 * ch + c), make_longlong2(acc[c], acc[c + 1]));
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sh->acc_empty[buf]));
-            }
+            if (NBUF == 1)
+                ozg_epilogue_grouped<S, W, GH>(tl, cw, dst, keep, [&](int g) { mbar_arrive(smem_u32(&sh->acc_empty[g])); });
+            else
+                ozg_epilogue_whole<S, W>(tl, cw, NCOL, dst, keep, [&]() { mbar_arrive(smem_u32(&sh->acc_empty[buf])); });
         }
     }
     tc_fence_before();
@@ -436,7 +296,6 @@ int oz_gemm_ring(int s, int kcc, int resa_kc) {
 
 int oz_gemm_launch(fci_context *h, int s, int w, int kcc, bool resa, const oz_gemm_args &a, cudaStream_t st) {
     void (*kern)(const OzgParams) = nullptr;
-    if (w == 7 && kcc == 4 && !resa) kern = oz_gemm_kernel<7, 4, false>(s);
     if (w == 8 && kcc == 2 && resa) kern = oz_gemm_kernel<8, 2, true>(s);
     if (w == 8 && kcc == 4 && !resa) kern = oz_gemm_kernel<8, 4, false>(s);
     if (resa && a.n_mt != 1) kern = nullptr;
