@@ -80,9 +80,13 @@ struct fci_das_layout {
     int32_t *d_dz_base = nullptr;  // [target | intermediate block offset per pattern pair (-1: none) | n_str_b]
     void *d_dz_G = nullptr;
     int dz_slices = 0, dz_shG = 0;
-    // the two-pass form (s >= 4): G digit slices in the A-tile layout of the bulk-copy GEMM
+    // the two-pass form (s >= 4): G digit slices in the A layout of the block-sparse GEMM, the
+    // pair of each position of its 16-wide blocks (-1: padding), and per category of the
+    // intermediate space the mask of blocks that connect it with the target space
     void *d_dg_G = nullptr;
     int dg_slices = 0, dg_shG = 0;
+    int32_t *d_dg_perm = nullptr;  // [16 n_blk]
+    ulonglong2 *d_dg_mask = nullptr;  // [n_cat_int]
     // kernel configuration chosen by the tuner for dz_tuned_slices (0: none)
     int dz_tuned_slices = 0, dz_tuned_kch = 0, dz_tuned_pw = 0;
 };

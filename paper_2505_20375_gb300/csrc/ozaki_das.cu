@@ -990,44 +990,133 @@ int dz_num_sms(fci_context *h, int *nsm) {
 //
 // For an FP64-class split (6 or 7 slices) the s level accumulators of the fused form do not
 // fit in TMEM, and neither do its G slices in shared memory, so the contraction turns back
-// to the orientation of the alpha/beta two-pass path: pair rows on M (ceil(n_pair / 128)
-// M-tiles of G digits), 64 determinants on N, and the operands streamed from HBM:
-//   k_dg_split   writes the digit image of D (int64 fixed point of C, gathered through the
-//                packed replacement tables and the target block offsets) for a piece of
-//                the intermediate space, in the B-tile layout of the bulk-copy GEMM;
-//   k_oz_gemm    (8-bit digits, K-chunks of 32) sums the top s levels exactly in TMEM and
-//                stores E_int (int64) [tile of 64][n_pair][64];
-//   k_dz_scatter (int64 form) sums E_int exactly per target determinant.
+// to the orientation of the alpha/beta two-pass path: pair rows on M, 64 determinants on N,
+// and the operands streamed from HBM:
+//   k_dg_split      writes the digit image of D (int64 fixed point of C, gathered through
+//                   the packed replacement tables and the target block offsets) for a piece
+//                   of the intermediate space, in the B layout of the block-sparse GEMM;
+//   k_oz_gemm_blk   (8-bit digits) sums the top s levels exactly in TMEM and stores E_int
+//                   (int64) [tile of 64][n_pair][64];
+//   k_dz_scatter    (int64 form) sums E_int exactly per target determinant.
 // Every level sum stays an integer below 2^24 when s n_pair <= 1023 (n_pair nonzero terms
 // of products below 2^14, s products per level), which the check enforces.  E covers up to
 // a cap of the intermediate space at a time (the scatter runs once per E chunk); the digit
 // image covers a smaller piece of that chunk at a time.
+//
+// Block sparsity.  A pair (r in space i, s in space j) moves an electron between spaces i and
+// j; from a category at the transfer limit only some of these moves end in the target space
+// (from an intermediate-only category no move inside a space does), so D and the rows of E
+// that are read are confined to the pairs of those space pairs.  The pairs are permuted into
+// blocks of 16 by space pair, each category has a mask of active blocks, and a tile of 64
+// determinants uses the union of its categories' masks (ozaki_blk.cu).
 namespace {
 
-constexpr int DG_KCC = 4;                      // core matrices (8 pairs) per K-chunk of the GEMM
-constexpr int DG_KW = 8 * DG_KCC;              // 32 pairs per K-chunk
-constexpr int DG_B_PLANE = OZG_N * DG_KW * 2;  // 4 KB: 64 determinants x 32 pairs, f16
-constexpr int DG_A_PLANE = OZG_M * DG_KW * 2;  // 8 KB: 128 pair rows x 32 pairs, f16
+constexpr int DG_BLK = 2048;  // bytes per slice of one (tile, block): 64 determinants x 16 pairs, f16
+
+// The pairs of the layout in blocks of 16: space pairs (classes) fill whole blocks first,
+// their remainders share blocks (largest first into the first block with room).
+struct DgBlocks {
+    std::vector<int32_t> perm;      // [16 n_blk]: pair, or -1
+    std::vector<uint64_t> classes;  // [n_blk]: bit c set if the block holds pairs of class c
+    int n_blk() const { return (int)classes.size(); }
+};
+int dg_class(int i, int j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; }
+
+DgBlocks dg_blocks(const fci_context *h) {
+    const fci_das_layout &L = h->das;
+    std::vector<int> space_of(h->n_orb);
+    for (int s = 0; s < L.n_spaces; ++s)
+        for (int k = 0; k < L.space_orbs[s]; ++k) space_of[L.space_off[s] + k] = s;
+    std::vector<std::vector<int32_t>> cls(dg_class(L.n_spaces - 1, L.n_spaces - 1) + 1);
+    for (int r = 0; r < h->n_orb; ++r)
+        for (int s = 0; s <= r; ++s) cls[dg_class(space_of[r], space_of[s])].push_back(pair_index(r, s));
+    DgBlocks b;
+    auto open_block = [&]() {
+        b.perm.insert(b.perm.end(), 16, -1);
+        b.classes.push_back(0);
+    };
+    std::vector<int> rest;
+    for (int c = 0; c < (int)cls.size(); ++c) {
+        size_t k = 0;
+        for (; k + 16 <= cls[c].size(); k += 16) {
+            open_block();
+            std::copy(cls[c].begin() + k, cls[c].begin() + k + 16, b.perm.end() - 16);
+            b.classes.back() = (uint64_t)1 << c;
+        }
+        cls[c].erase(cls[c].begin(), cls[c].begin() + k);
+        if (!cls[c].empty()) rest.push_back(c);
+    }
+    std::stable_sort(rest.begin(), rest.end(), [&](int x, int y) { return cls[x].size() > cls[y].size(); });
+    const int first = b.n_blk();
+    std::vector<int> used;  // positions taken of each shared block
+    for (int c : rest) {
+        size_t k = 0;
+        while (k < used.size() && used[k] + cls[c].size() > 16) ++k;
+        if (k == used.size()) {
+            open_block();
+            used.push_back(0);
+        }
+        std::copy(cls[c].begin(), cls[c].end(), b.perm.begin() + 16 * (first + k) + used[k]);
+        used[k] += (int)cls[c].size();
+        b.classes[first + k] |= (uint64_t)1 << c;
+    }
+    return b;
+}
+
+// Mask of active blocks per category: a space pair is active if a move of either direction
+// by the alpha or the beta string ends in a target category (total excess <= max_transfer).
+void dg_category_masks(const fci_context *h, const DgBlocks &b, std::vector<ulonglong2> &out) {
+    const fci_das_layout &L = h->das;
+    const int S = L.n_spaces, nc = dg_class(S - 1, S - 1) + 1, none = 1 << 20;
+    // smallest excess of a pattern after one move of each class
+    auto after = [&](const std::vector<int> &pats, const std::vector<int> &exc, const int *ref) {
+        const int n = (int)exc.size();
+        std::vector<int> best((size_t)n * nc, none);
+        for (int p = 0; p < n; ++p) {
+            const int *occ = &pats[(size_t)p * S];
+            for (int i = 0; i < S; ++i)
+                for (int j = 0; j < S; ++j) {  // one electron from space i to space j
+                    if (occ[i] == 0 || (i != j && occ[j] == L.space_orbs[j])) continue;
+                    int e = 0;
+                    for (int s = 0; s < S; ++s) e += std::max(0, occ[s] - (s == i) + (s == j) - ref[s]);
+                    int &v = best[(size_t)p * nc + dg_class(i, j)];
+                    v = std::min(v, e);
+                }
+        }
+        return best;
+    };
+    const std::vector<int> ba = after(L.pat_a, L.exc_a, L.ref_a), bb = after(L.pat_b, L.exc_b, L.ref_b);
+    out.assign(L.n_cat_int, make_ulonglong2(0, 0));
+    for (int c = 0; c < L.n_cat_int; ++c) {
+        const int pa = L.cat_pa[c], pb = L.cat_pb[c];
+        uint64_t on = 0;
+        for (int k = 0; k < nc; ++k)
+            if (ba[(size_t)pa * nc + k] + L.exc_b[pb] <= L.max_transfer ||
+                bb[(size_t)pb * nc + k] + L.exc_a[pa] <= L.max_transfer)
+                on |= (uint64_t)1 << k;
+        for (int k = 0; k < b.n_blk(); ++k)
+            if (b.classes[k] & on) (k < 64 ? out[c].x : out[c].y) |= (unsigned long long)1 << (k & 63);
+    }
+}
 
 struct DgGeom {
-    int n_mt, n_kc;        // M-tiles of 128 pair rows; K-chunks of 32 pairs
+    int n_blk;
     int64_t e_cap, d_cap;  // determinants per E chunk and per digit-image piece (multiples of 64)
     int n_echunks;
 };
 
 // FCI_DAS_CHUNK_DETS and FCI_DAS_IMAGE_DETS lower the two caps (in determinants) so that
 // tests can force several chunks and pieces on small problems.
-DgGeom dg_geom(const fci_context *h, int s) {
+DgGeom dg_geom(const fci_context *h, int s, int n_blk) {
     const fci_das_layout &L = h->das;
     DgGeom g;
-    g.n_mt = (h->npair + OZG_M - 1) / OZG_M;
-    g.n_kc = (h->npair_pad + DG_KW - 1) / DG_KW;
+    g.n_blk = n_blk;
     const int64_t all = ceil_div(std::max<int64_t>(L.n_det_int, 1), OZG_N) * OZG_N;
     int64_t e = (((int64_t)96 << 30) / (8 * (int64_t)h->npair)) / OZG_N * OZG_N;
     if (const char *env = getenv("FCI_DAS_CHUNK_DETS"))
         if (atoll(env) > 0) e = ceil_div(atoll(env), OZG_N) * OZG_N;
     g.e_cap = std::max<int64_t>(OZG_N, std::min(e, all));
-    int64_t d = (((int64_t)24 << 30) / ((int64_t)g.n_kc * s * DG_B_PLANE / OZG_N)) / OZG_N * OZG_N;
+    int64_t d = (((int64_t)24 << 30) / ((int64_t)n_blk * s * DG_BLK / OZG_N)) / OZG_N * OZG_N;
     if (const char *env = getenv("FCI_DAS_IMAGE_DETS"))
         if (atoll(env) > 0) d = ceil_div(atoll(env), OZG_N) * OZG_N;
     g.d_cap = std::max<int64_t>(OZG_N, std::min(d, g.e_cap));
@@ -1038,37 +1127,44 @@ DgGeom dg_geom(const fci_context *h, int s) {
 struct DgSplit {
     int64_t a0, len;   // intermediate addresses [a0, a0 + len) of this piece
     int64_t n_nt;      // tiles of 64
-    int n_kc, npair_pad, n_cat_int, n_pat_b;
+    int n_blk, n_cat_int, n_pat_b;
     int64_t nla, nlb;
     const int32_t *repA, *repB;
+    const int32_t *perm;        // [16 n_blk]: pair of each block position, -1: padding
+    const ulonglong2 *cmask;    // [n_cat_int]
     const int32_t *base_tgt;  // [n_pat_a * n_pat_b]: offset of a TARGET block, else -1 (C is zero)
     const int32_t *nstr_b32;
     const int64_t *cat_off, *locbase_a, *locbase_b;
     const int32_t *cat_pa, *cat_pb;
     const int64_t *Cint;
     uint8_t *Dimg;
+    ulonglong2 *masks;  // [n_nt]
 };
 
-// Digit image of D for one piece: tile nt (64 determinants) holds, per K-chunk of 32
-// pairs, S f16 planes of 64 x 32 in canonical K-major core matrices.  Thread t covers
-// determinant t % 64 of the tile (decoded once: category, patterns, local indices) and
-// pairs 8 (t / 64) .. 8 (t / 64) + 7 of every chunk; D_int of a pair is the alpha move's
-// and the beta move's signed C_int (zero where the move leaves the target space or does
-// not exist; replacement-table rows past n_pair_pad count as absent).  Capped at 64
-// registers for four resident blocks per SM (measured 4% faster than three at C3').
+// Digit image of D and the block masks of one piece: tile nt (64 determinants) holds, per
+// active block of 16 pairs, S f16 planes of 64 x 16 in K-major core matrices.  Thread
+// (row, core) decodes determinant `row` of the tile once (category, patterns, local
+// indices) and covers 8 pairs of a block; the two halves of the CTA take the active blocks
+// in turn.  D_int of a pair is the alpha move's and the beta move's signed C_int (zero
+// where the move leaves the target space or does not exist).  Capped at 64 registers for
+// four resident blocks per SM.
 template <int S>
-__global__ void __launch_bounds__(64 * DG_KCC, 4) k_dg_split(const __grid_constant__ DgSplit a) {
+__global__ void __launch_bounds__(256, 4) k_dg_split(const __grid_constant__ DgSplit a) {
     constexpr uint64_t bias = 0x8080808080808080ull >> (8 * (8 - S));
-    const int row = threadIdx.x & 63, cc = threadIdx.x >> 6;
+    __shared__ __align__(16) uint32_t s_mask[2][2][4];  // [tile parity][warp][word]
+    const int row = threadIdx.x & 63, core = (threadIdx.x >> 6) & 1, half = threadIdx.x >> 7;
     const int npb = a.n_pat_b;
-    for (int64_t nt = blockIdx.x; nt < a.n_nt; nt += gridDim.x) {
+    int par = 0;
+    for (int64_t nt = blockIdx.x; nt < a.n_nt; nt += gridDim.x, par ^= 1) {
         const int64_t off = nt * OZG_N + row;
         const bool live = off < a.len;
         int32_t pa = 0, pb = 0, la = 0, lb = 0, nb = 1;
         int64_t ida = 0, idb = 0;
+        uint4 cm = make_uint4(0, 0, 0, 0);
         if (live) {
             const int64_t addr = a.a0 + off;
             const int c = find_cat(a.cat_off, a.n_cat_int, addr);
+            cm = __ldg(reinterpret_cast<const uint4 *>(a.cmask + c));
             pa = __ldg(a.cat_pa + c);
             pb = __ldg(a.cat_pb + c);
             nb = __ldg(a.nstr_b32 + pb);
@@ -1078,55 +1174,87 @@ __global__ void __launch_bounds__(64 * DG_KCC, 4) k_dg_split(const __grid_consta
             ida = __ldg(a.locbase_a + pa) + la;
             idb = __ldg(a.locbase_b + pb) + lb;
         }
-        uint8_t *tile = a.Dimg + (size_t)nt * a.n_kc * S * DG_B_PLANE + ((row >> 3) * DG_KCC + cc) * 128 + (row & 7) * 16;
-#pragma unroll 1
-        for (int kc = 0; kc < a.n_kc; ++kc) {
-            const int rs0 = kc * DG_KW + cc * 8;
-            int32_t ea[8], eb[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const bool ok = live && rs0 + e < a.npair_pad;
-                ea[e] = ok ? __ldg(a.repA + (int64_t)(rs0 + e) * a.nla + ida) : -1;
-                eb[e] = ok ? __ldg(a.repB + (int64_t)(rs0 + e) * a.nlb + idb) : -1;
-            }
-            int32_t Ka[8], Kb[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int32_t ba = ea[e] >= 0 ? __ldg(a.base_tgt + (ea[e] >> 23) * npb + pb) : -1;
-                const int32_t bb = eb[e] >= 0 ? __ldg(a.base_tgt + pa * npb + (eb[e] >> 23)) : -1;
-                Ka[e] = ba >= 0 ? ba + ((ea[e] >> 1) & DZ_LOC_MASK) * nb + lb : -1;
-                Kb[e] = bb >= 0 ? bb + la * __ldg(a.nstr_b32 + (eb[e] >> 23)) + ((eb[e] >> 1) & DZ_LOC_MASK) : -1;
-            }
-            uint32_t ylo[8], yhi[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int64_t xa = Ka[e] >= 0 ? __ldg(a.Cint + Ka[e]) : 0;
-                const int64_t xb = Kb[e] >= 0 ? __ldg(a.Cint + Kb[e]) : 0;
-                const int64_t v = ((ea[e] & 1) ? -xa : xa) + ((eb[e] & 1) ? -xb : xb);
-                const uint64_t y = (uint64_t)v + bias;
-                ylo[e] = (uint32_t)y;
-                yhi[e] = (uint32_t)(y >> 32);
-            }
-            uint8_t *base = tile + (size_t)kc * S * DG_B_PLANE;
-#pragma unroll
-            for (int j = 0; j < S; ++j) {
-                const uint32_t bj = (uint32_t)(j & 3), sel = bj | ((4u + bj) << 8);
-                uint32_t w[4];
-#pragma unroll
-                for (int e = 0; e < 8; e += 2)
-                    w[e / 2] = j < 4 ? digits_f16x2(ylo[e], ylo[e + 1], sel) : digits_f16x2(yhi[e], yhi[e + 1], sel);
-                __stcs((uint4 *)(base + j * DG_B_PLANE), make_uint4(w[0], w[1], w[2], w[3]));
-            }
+        if (threadIdx.x < 64) {
+            cm.x = __reduce_or_sync(0xFFFFFFFFu, cm.x);
+            cm.y = __reduce_or_sync(0xFFFFFFFFu, cm.y);
+            cm.z = __reduce_or_sync(0xFFFFFFFFu, cm.z);
+            cm.w = __reduce_or_sync(0xFFFFFFFFu, cm.w);
+            if ((threadIdx.x & 31) == 0) *reinterpret_cast<uint4 *>(s_mask[par][threadIdx.x >> 5]) = cm;
         }
+        // one barrier per tile: the other parity's words are those of the previous tile
+        __syncthreads();
+        uint32_t word[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) word[w] = s_mask[par][0][w] | s_mask[par][1][w];
+        if (threadIdx.x == 0)
+            a.masks[nt] = make_ulonglong2(word[0] | ((uint64_t)word[1] << 32), word[2] | ((uint64_t)word[3] << 32));
+        int turn = 0;
+#pragma unroll 1
+        for (int w = 0; w < 4; ++w)
+#pragma unroll 1
+            for (uint32_t m = word[w]; m; m &= m - 1, turn ^= 1) {
+                if (turn != half) continue;
+                const int k = 32 * w + __ffs(m) - 1;
+                const int4 *pm = reinterpret_cast<const int4 *>(a.perm + 16 * k + 8 * core);
+                const int4 p0 = __ldg(pm), p1 = __ldg(pm + 1);
+                const int32_t pr[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+                int32_t ea[8], eb[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const bool ok = live && pr[e] >= 0;
+                    ea[e] = ok ? __ldg(a.repA + (int64_t)pr[e] * a.nla + ida) : -1;
+                    eb[e] = ok ? __ldg(a.repB + (int64_t)pr[e] * a.nlb + idb) : -1;
+                }
+                int32_t Ka[8], Kb[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int32_t ba = ea[e] >= 0 ? __ldg(a.base_tgt + (ea[e] >> 23) * npb + pb) : -1;
+                    const int32_t bb = eb[e] >= 0 ? __ldg(a.base_tgt + pa * npb + (eb[e] >> 23)) : -1;
+                    Ka[e] = ba >= 0 ? ba + ((ea[e] >> 1) & DZ_LOC_MASK) * nb + lb : -1;
+                    Kb[e] = bb >= 0 ? bb + la * __ldg(a.nstr_b32 + (eb[e] >> 23)) + ((eb[e] >> 1) & DZ_LOC_MASK) : -1;
+                }
+                uint32_t ylo[8], yhi[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int64_t xa = Ka[e] >= 0 ? __ldg(a.Cint + Ka[e]) : 0;
+                    const int64_t xb = Kb[e] >= 0 ? __ldg(a.Cint + Kb[e]) : 0;
+                    const int64_t v = ((ea[e] & 1) ? -xa : xa) + ((eb[e] & 1) ? -xb : xb);
+                    const uint64_t y = (uint64_t)v + bias;
+                    ylo[e] = (uint32_t)y;
+                    yhi[e] = (uint32_t)(y >> 32);
+                }
+                uint8_t *base = a.Dimg + ((size_t)nt * a.n_blk + k) * S * DG_BLK + (row >> 3) * 256 + core * 128 + (row & 7) * 16;
+#pragma unroll
+                for (int j = 0; j < S; ++j) {
+                    const uint32_t bj = (uint32_t)(j & 3), sel = bj | ((4u + bj) << 8);
+                    uint32_t w4[4];
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2)
+                        w4[e / 2] = j < 4 ? digits_f16x2(ylo[e], ylo[e + 1], sel) : digits_f16x2(yhi[e], yhi[e + 1], sel);
+                    __stcs((uint4 *)(base + j * DG_BLK), make_uint4(w4[0], w4[1], w4[2], w4[3]));
+                }
+            }
     }
 }
 
-// G digit slices in the A-tile layout of the bulk-copy GEMM: [M-tile][K-chunk][plane][128 x 32].
-int dg_prepare_G(fci_context *h, int s) {
+// The block plan's device tables and the G digit slices in the A layout of the block-sparse GEMM.
+int dg_prepare(fci_context *h, int s, const DgBlocks &b) {
     fci_das_layout &L = h->das;
+    int rc = FCI_OK;
+    if (!L.d_dg_mask) {
+        std::vector<ulonglong2> masks;
+        dg_category_masks(h, b, masks);
+        if (!L.d_dg_perm) {
+            if ((rc = fci_dev_alloc(h, (void **)&L.d_dg_perm, b.perm.size() * 4))) return rc;
+            FCI_CUDA(h, cudaMemcpy(L.d_dg_perm, b.perm.data(), b.perm.size() * 4, cudaMemcpyHostToDevice));
+        }
+        ulonglong2 *dm = nullptr;
+        if ((rc = fci_dev_alloc(h, (void **)&dm, masks.size() * sizeof(ulonglong2)))) return rc;
+        L.d_dg_mask = dm;
+        FCI_CUDA(h, cudaMemcpy(dm, masks.data(), masks.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
+    }
     if (L.dg_slices == s && L.d_dg_G) return FCI_OK;
-    const DgGeom g = dg_geom(h, s);
-    const int np = h->npair;
+    const int np = h->npair, nb = b.n_blk();
     std::vector<double> G((size_t)np * np);
     if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
         return fci_cuda_check(h, cudaGetLastError(), "G download");
@@ -1136,23 +1264,22 @@ int dg_prepare_G(fci_context *h, int s) {
     if (gmax > 0) frexp(gmax, &eG);  // gmax < 2^eG
     const int shG = 8 * s - 2 - eG;
     const uint64_t bias = 0x8080808080808080ull >> (8 * (8 - s));
-    const size_t stage = (size_t)s * DG_A_PLANE;
-    std::vector<uint16_t> img((size_t)g.n_mt * g.n_kc * stage / 2, 0);
-    for (int m = 0; m < g.n_mt * OZG_M; ++m)
-        for (int k = 0; k < g.n_kc * DG_KW; ++k) {
-            int64_t gi = 0;
-            if (m < np && k < np) gi = llrint(ldexp(G[(size_t)m * np + k], shG));
+    std::vector<uint16_t> img((size_t)nb * nb * s * 256, 0);
+    for (int pr = 0; pr < 16 * nb; ++pr)
+        for (int pc = 0; pc < 16 * nb; ++pc) {
+            if (b.perm[pr] < 0 || b.perm[pc] < 0) continue;
+            const int64_t gi = llrint(ldexp(G[(size_t)b.perm[pr] * np + b.perm[pc]], shG));
             const uint64_t y = (uint64_t)gi + bias;
-            const int mt = m / OZG_M, mm = m % OZG_M, kc = k / DG_KW, kk = k % DG_KW;
-            const size_t off = ((size_t)mt * g.n_kc + kc) * stage + ((mm >> 3) * DG_KCC + (kk >> 3)) * 128 + (mm & 7) * 16 +
-                               (kk & 7) * 2;
+            const int r = pr & 15, c = pc & 15;
+            const size_t off = ((size_t)(pr >> 4) * nb + (pc >> 4)) * s * 512 + (size_t)(r >> 3) * s * 256 + (c >> 3) * 128 +
+                               (r & 7) * 16 + (c & 7) * 2;
             for (int j = 0; j < s; ++j)
-                img[(off + (size_t)j * DG_A_PLANE) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
+                img[(off + (size_t)j * 256) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
         }
     fci_dev_free(L.d_dg_G);
     L.d_dg_G = nullptr;
     L.dg_slices = 0;
-    int rc = fci_dev_alloc(h, &L.d_dg_G, img.size() * 2);
+    rc = fci_dev_alloc(h, &L.d_dg_G, img.size() * 2);
     if (rc) return rc;
     FCI_CUDA(h, cudaMemcpy(L.d_dg_G, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
     L.dg_slices = s;
@@ -1175,32 +1302,38 @@ int dg_check(fci_context *h, int s) {
         if (v > DZ_LOC_MASK) return fci_fail(h, FCI_ERR_UNSUPPORTED, "a pattern has more than 2^22 strings");
     for (int64_t v : L.pat_nstr_b)
         if (v > DZ_LOC_MASK) return fci_fail(h, FCI_ERR_UNSUPPORTED, "a pattern has more than 2^22 strings");
-    if (!oz_gemm_ring(s, DG_KCC, 0)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices do not fit the GEMM pipeline", s);
+    if (!oz_blk_ring(s)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices do not fit the GEMM pipeline", s);
     return FCI_OK;
 }
 
 int das_split_check(fci_context *h, int s) { return s <= 3 ? dz_check(h, s) : dg_check(h, s); }
 
+// C_int, the D digit image and block masks of a piece, E_int of a chunk, the partial sums
+// kept across chunks, 256 bytes of scalars.
 size_t dg_workspace_bytes(const fci_context *h, int s) {
-    const DgGeom g = dg_geom(h, std::max(s, 4));
-    size_t b = al256((size_t)h->das.n_det * 8) + al256((size_t)(g.d_cap / OZG_N) * g.n_kc * std::max(s, 4) * DG_B_PLANE) +
-               al256((size_t)g.e_cap * h->npair * 8);
+    const DgGeom g = dg_geom(h, std::max(s, 4), dg_blocks(h).n_blk());
+    size_t b = al256((size_t)h->das.n_det * 8) + al256((size_t)(g.d_cap / OZG_N) * g.n_blk * std::max(s, 4) * DG_BLK) +
+               al256((size_t)(g.d_cap / OZG_N) * sizeof(ulonglong2)) + al256((size_t)g.e_cap * h->npair * 8);
     if (g.n_echunks > 1) b += al256((size_t)h->das.n_det * 8);
     return b + 256;
 }
 
 int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cudaStream_t st) {
     int rc = dg_check(h, s);
-    if (!rc) rc = dz_prepare_tables(h, st);
-    if (!rc) rc = dg_prepare_G(h, s);
+    if (rc) return rc;
+    const DgBlocks blk = dg_blocks(h);
+    rc = dz_prepare_tables(h, st);
+    if (!rc) rc = dg_prepare(h, s, blk);
     if (rc) return rc;
     const fci_das_layout &L = h->das;
-    const DgGeom g = dg_geom(h, s);
+    const DgGeom g = dg_geom(h, s, blk.n_blk());
     char *p = (char *)ws;
     int64_t *Cint = (int64_t *)p;
     p += al256((size_t)L.n_det * 8);
     uint8_t *Dimg = (uint8_t *)p;
-    p += al256((size_t)(g.d_cap / OZG_N) * g.n_kc * s * DG_B_PLANE);
+    p += al256((size_t)(g.d_cap / OZG_N) * g.n_blk * s * DG_BLK);
+    ulonglong2 *masks = (ulonglong2 *)p;
+    p += al256((size_t)(g.d_cap / OZG_N) * sizeof(ulonglong2));
     int64_t *E = (int64_t *)p;
     p += al256((size_t)g.e_cap * h->npair * 8);
     int64_t *acc = nullptr;
@@ -1217,14 +1350,15 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     }
     const size_t npab = (size_t)L.n_pat_a * L.n_pat_b;
     DgSplit sp;
-    sp.n_kc = g.n_kc;
-    sp.npair_pad = h->npair_pad;
+    sp.n_blk = g.n_blk;
     sp.n_cat_int = L.n_cat_int;
     sp.n_pat_b = L.n_pat_b;
     sp.nla = dz_nloc(L.pat_nstr_a);
     sp.nlb = dz_nloc(L.pat_nstr_b);
     sp.repA = L.d_dz_rep_a;
     sp.repB = L.d_dz_rep_b;
+    sp.perm = L.d_dg_perm;
+    sp.cmask = L.d_dg_mask;
     sp.base_tgt = L.d_dz_base;
     sp.nstr_b32 = L.d_dz_base + 2 * npab;
     sp.cat_off = L.d_cat_off;
@@ -1234,6 +1368,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     sp.cat_pb = L.d_cat_pb;
     sp.Cint = Cint;
     sp.Dimg = Dimg;
+    sp.masks = masks;
     for (int ec = 0; ec < g.n_echunks; ++ec) {
         const int64_t e0 = (int64_t)ec * g.e_cap, elen = std::min(g.e_cap, L.n_det_int - e0);
         for (int64_t d0 = 0; d0 < elen; d0 += g.d_cap) {
@@ -1244,25 +1379,25 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
                 phase_scope ps(h, st, FCI_PHASE_GATHER, 1);
                 const unsigned gb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(sp.n_nt, 152 * 16));
                 switch (s) {
-                    case 4: k_dg_split<4><<<gb, 64 * DG_KCC, 0, st>>>(sp); break;
-                    case 5: k_dg_split<5><<<gb, 64 * DG_KCC, 0, st>>>(sp); break;
-                    case 6: k_dg_split<6><<<gb, 64 * DG_KCC, 0, st>>>(sp); break;
-                    case 7: k_dg_split<7><<<gb, 64 * DG_KCC, 0, st>>>(sp); break;
-                    default: k_dg_split<8><<<gb, 64 * DG_KCC, 0, st>>>(sp); break;
+                    case 4: k_dg_split<4><<<gb, 256, 0, st>>>(sp); break;
+                    case 5: k_dg_split<5><<<gb, 256, 0, st>>>(sp); break;
+                    case 6: k_dg_split<6><<<gb, 256, 0, st>>>(sp); break;
+                    case 7: k_dg_split<7><<<gb, 256, 0, st>>>(sp); break;
+                    default: k_dg_split<8><<<gb, 256, 0, st>>>(sp); break;
                 }
                 FCI_CUDA(h, cudaGetLastError());
             }
-            oz_gemm_args a;
-            a.n_mt = g.n_mt;
-            a.n_kc = g.n_kc;
+            oz_blk_args a;
+            a.n_blk = g.n_blk;
             a.M_pad = h->npair;  // E row stride: the n_pair rows of each tile, no padding
-            a.M_real = h->npair;
             a.n_nt = sp.n_nt;
             a.Gimg = L.d_dg_G;
             a.Dimg = Dimg;
+            a.masks = masks;
+            a.rowmap = L.d_dg_perm;
             a.E = E + (size_t)(d0 / OZG_N) * h->npair * OZG_N;
             a.status = status;
-            if ((rc = oz_gemm_launch(h, s, 8, DG_KCC, false, a, st))) return rc;
+            if ((rc = oz_blk_launch(h, s, 8, a, st))) return rc;
         }
         DzScatter sc;
         sc.n_det = L.n_det;
@@ -1311,6 +1446,10 @@ void dz_free(fci_das_layout &L) {
     fci_dev_free(L.d_dz_base);
     fci_dev_free(L.d_dz_G);
     fci_dev_free(L.d_dg_G);
+    fci_dev_free(L.d_dg_perm);
+    fci_dev_free(L.d_dg_mask);
+    L.d_dg_perm = nullptr;
+    L.d_dg_mask = nullptr;
     L.d_dz_rep_a = L.d_dz_rep_b = nullptr;
     L.d_dz_base = nullptr;
     L.d_dz_G = nullptr;
