@@ -4,11 +4,16 @@
 // Every vector operation runs here in FP64 (complex vectors as interleaved pairs):
 // subspace projections V^H w, Ritz combinations, the residual, the preconditioner with
 // its 1e-12 guard and eps * ||s|| threshold, two rounds of classical Gram-Schmidt and
-// the projected eigenproblem (cyclic Jacobi in one thread block; complex Hermitian
-// matrices through their real symmetric embedding [[A, -B], [B, A]]).  The host reads
-// back a handful of scalars per iteration to decide convergence.
+// the projected eigenproblem (one thread block; complex Hermitian matrices through their
+// real symmetric embedding [[A, -B], [B, A]]).  The host reads back a handful of scalars per
+// iteration to decide convergence.  On small spaces the vector work is a chain of short
+// launches, so every reduction ends inside its own kernel: the last block to finish adds
+// the block partials in a fixed order and applies what follows (a sign, the new column of
+// the projected matrix, a norm).
 #include <math.h>
 #include <string.h>
+
+#include <cooperative_groups.h>
 
 #include <algorithm>
 #include <chrono>
@@ -16,128 +21,250 @@
 #include <vector>
 
 #include "fci_internal.h"
+#include "fp64_fast.cuh"
 
 namespace {
 
 constexpr int RED_BLOCKS = 608;  // 4 x 152 SMs
 constexpr int RED_THREADS = 256;
 constexpr int KMAX = 32;
-constexpr int JAC_THREADS = 256;  // the projected eigensolver's block
+constexpr int JAC_THREADS = 256;  // the projected eigensolver's blocks, and how many share it
+constexpr int JAC_CLUSTER = 8;
 
 struct dav_scalars {      // device-resident scalars, read back each iteration
     double lam;           // lowest Ritz value (sigma carries e_core C, so e_core is included)
     double rnorm2, snorm2, maxdc;
-    double ov_re, ov_im;  // <c_prev|c>
-    double tnorm2;
-    double pad;
 };
 
-// partial[b][i] (complex: 2 doubles) = sum over this block's slice of conj(V_i) x, for
-// i < k <= KB: KB (a power of two, at least k) sizes the accumulator arrays, so a call
-// with few vectors keeps few registers and many warps resident.
+// Butterfly over the lanes (exchange distances 16, 8, 4, 2, 1) that adds K per-lane values at
+// once: each of the first log2 K steps halves the values a lane carries, so K values cost
+// about K + 5 additions in place of 5 K (on small spaces the FP64 additions of the
+// reductions took longer than the multiply-adds of the dot products).  The sums are those
+// of K plain butterflies, bit for bit.  Lane l ends with value many_index<K>(l) in v[0];
+// lanes with many_writer<K>(l) cover every value once.  K: a power of two up to 32.
+template <int K>
+__device__ __forceinline__ void warp_sum_many(double (&v)[K]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int n = K; n > 1; n >>= 1, o >>= 1) {  // lanes that differ in bit o split the n values
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const double keep = (lane & o) ? v[2 * i + 1] : v[2 * i], give = (lane & o) ? v[2 * i] : v[2 * i + 1];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+        }
+    }
+#pragma unroll
+    for (; o; o >>= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
+}
+template <int K>
+__device__ __forceinline__ int many_index(int lane) { return (int)(__brev((unsigned)lane) >> 27) & (K - 1); }
+template <int K>
+__device__ __forceinline__ bool many_writer(int lane) { return (lane & (32 / K - 1)) == 0; }
+
+// True in every thread of the last block of the grid to arrive at *counter (which it leaves
+// at zero for the next kernel); that block then sees the partials every block has written.
+__device__ __forceinline__ bool last_block(unsigned *counter) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        if (last) *counter = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Sums over the nb block partials of a reduction in a fixed order (lane l adds blocks l,
+// l + 32, ..., then a butterfly over the lanes), so every result is reproducible: NI results
+// at p, p + step, ... side by side, eight loads of each in flight (one after another, the
+// loads of the last block took longer than the reduction itself).
+template <int NI>
+__device__ __forceinline__ void warp_sum_blocks(const double *p, int64_t stride, int nb, int step, double (&a)[NI]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < NI; ++q) a[q] = 0.0;
+    for (int b0 = lane; b0 < nb; b0 += 256) {
+        double v[NI][8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int q = 0; q < NI; ++q)
+                v[q][u] = b0 + 32 * u < nb ? __ldcg(p + (int64_t)(b0 + 32 * u) * stride + q * step) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (b0 + 32 * u < nb)
+#pragma unroll
+                for (int q = 0; q < NI; ++q) a[q] += v[q][u];
+    }
+    for (int o = 16; o; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < NI; ++q) a[q] += __shfl_xor_sync(0xFFFFFFFFu, a[q], o);
+}
+__device__ __forceinline__ double warp_sum_blocks(const double *p, int64_t stride, int nb) {
+    double a[1];
+    warp_sum_blocks<1>(p, stride, nb, 0, a);
+    return a[0];
+}
+
+// What the last block does with <V_i|x>, i = i0 .. i0 + k - 1.
+enum { DOT_PLAIN = 0,   // out[i] = the sum (complex)
+       DOT_NEGATE = 1,  // out[i] = minus the sum: the coefficients of a Gram-Schmidt update
+       DOT_COLUMN = 2   // the new column (and row) `col` of the projected matrix `out`
+};
+
+// <V_i|x> for i0 <= i < i0 + k (k <= KB): KB (a power of two) sizes the accumulator arrays, so
+// a call with few vectors keeps few registers and many warps resident.
 template <bool CPLX, int KB>
-__global__ void __launch_bounds__(RED_THREADS) k_multidot(const double *__restrict__ V, int64_t ldv, int k,
+__global__ void __launch_bounds__(RED_THREADS) k_multidot(const double *__restrict__ V, int64_t ldv, int i0, int k,
                                                           const double *__restrict__ x, int64_t n,
-                                                          double *__restrict__ partial) {
-    __shared__ double red[RED_THREADS / 32][2 * KB];
-    double acc_re[KB], acc_im[CPLX ? KB : 1];
+                                                          double *__restrict__ partial, unsigned *__restrict__ counter,
+                                                          int mode, int col, double *__restrict__ out) {
+    constexpr int NV = CPLX ? 2 * KB : KB;  // real values reduced: re, im interleaved if complex
+    __shared__ double red[RED_THREADS / 32][NV];
+    double acc[NV];
 #pragma unroll
-    for (int i = 0; i < KB; ++i) acc_re[i] = 0.0;
-#pragma unroll
-    for (int i = 0; i < (CPLX ? KB : 1); ++i) acc_im[i] = 0.0;
+    for (int i = 0; i < NV; ++i) acc[i] = 0.0;
+    const double *Vb = V + (int64_t)i0 * (CPLX ? 2 : 1) * ldv;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
         if (CPLX) {
             const double xr = x[2 * j], xi = x[2 * j + 1];
 #pragma unroll
             for (int i = 0; i < KB; ++i) {
                 if (i < k) {
-                    const double vr = V[i * 2 * ldv + 2 * j], vi = V[i * 2 * ldv + 2 * j + 1];
-                    acc_re[i] = fma(vr, xr, fma(vi, xi, acc_re[i]));
-                    acc_im[CPLX ? i : 0] = fma(vr, xi, fma(-vi, xr, acc_im[CPLX ? i : 0]));
+                    const double vr = Vb[i * 2 * ldv + 2 * j], vi = Vb[i * 2 * ldv + 2 * j + 1];
+                    acc[(2 * i) % NV] = fma(vr, xr, fma(vi, xi, acc[(2 * i) % NV]));
+                    acc[(2 * i + 1) % NV] = fma(vr, xi, fma(-vi, xr, acc[(2 * i + 1) % NV]));
                 }
             }
         } else {
             const double xr = x[j];
 #pragma unroll
             for (int i = 0; i < KB; ++i)
-                if (i < k) acc_re[i] = fma(V[i * ldv + j], xr, acc_re[i]);
+                if (i < k) acc[i] = fma(Vb[i * ldv + j], xr, acc[i]);
         }
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < KB; ++i) {
-        if (i >= k) break;
-        double a = acc_re[i], b = CPLX ? acc_im[CPLX ? i : 0] : 0.0;
-        for (int o = 16; o; o >>= 1) {
-            a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-            if (CPLX) b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
-        }
-        if (lane == 0) { red[wid][2 * i] = a; red[wid][2 * i + 1] = b; }
-    }
+    warp_sum_many<NV>(acc);
+    if (many_writer<NV>(lane)) red[wid][many_index<NV>(lane)] = acc[0];
     __syncthreads();
-    if (threadIdx.x < 2 * k) {
+    if (threadIdx.x < NV) {
         double s = 0.0;
         for (int w = 0; w < RED_THREADS / 32; ++w) s += red[w][threadIdx.x];
-        partial[(int64_t)blockIdx.x * 2 * KMAX + threadIdx.x] = s;
+        partial[(int64_t)blockIdx.x * NV + threadIdx.x] = s;
     }
-}
-
-// Sum over the nb block partials of a reduction in a fixed order (lane l adds blocks l,
-// l + 32, ..., then a butterfly over the lanes), so every result is reproducible.
-__device__ __forceinline__ double warp_sum_blocks(const double *__restrict__ p, int64_t stride, int nb) {
-    const int lane = threadIdx.x & 31;
-    double a = 0.0;
-    for (int b = lane; b < nb; b += 32) a += p[(int64_t)b * stride];
-    for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-    return a;
-}
-
-// out[i] (complex) = sum_b partial[b][i], one warp per entry.
-__global__ void k_reduce_partial(const double *__restrict__ partial, int nb, int k, double *__restrict__ out) {
-    for (int i = threadIdx.x >> 5; i < 2 * k; i += blockDim.x >> 5) {
-        const double a = warp_sum_blocks(partial + i, 2 * KMAX, nb);
-        if ((threadIdx.x & 31) == 0) out[i] = a;
+    if (!last_block(counter)) return;
+    // warp wid takes results wid, wid + 8, ...
+    constexpr int NW = RED_THREADS / 32, NI = (KB + NW - 1) / NW;
+    if (wid >= k) return;
+    double sum[CPLX ? 2 * NI : NI];  // complex: re, im of each
+    if (CPLX) {
+#pragma unroll
+        for (int q = 0; q < NI; ++q) {
+            double two[2];
+            warp_sum_blocks<2>(partial + 2 * min(wid + NW * q, KB - 1), NV, gridDim.x, 1, two);
+            sum[CPLX ? 2 * q : 0] = two[0];
+            sum[CPLX ? 2 * q + 1 : 0] = two[1];
+        }
+    } else {
+        double all[NI];
+        warp_sum_blocks<NI>(partial + wid, NV, gridDim.x, NW, all);
+#pragma unroll
+        for (int q = 0; q < NI; ++q) sum[q] = all[q];
     }
-}
-
-// out = sum_i y_i V_i  (+ beta * out when accumulate), y complex as 2 doubles per entry.
-template <bool CPLX>
-__global__ void k_lincomb(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ y,
-                          double scale, int64_t n, double *__restrict__ out, int accumulate) {
-    __shared__ double sy[2 * KMAX];
-    if (threadIdx.x < 2 * k) sy[threadIdx.x] = y[threadIdx.x] * scale;
-    __syncthreads();
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        if (CPLX) {
-            double re = accumulate ? out[2 * j] : 0.0, im = accumulate ? out[2 * j + 1] : 0.0;
-            for (int i = 0; i < k; ++i) {
-                const double vr = V[i * 2 * ldv + 2 * j], vi = V[i * 2 * ldv + 2 * j + 1];
-                re = fma(sy[2 * i], vr, fma(-sy[2 * i + 1], vi, re));
-                im = fma(sy[2 * i], vi, fma(sy[2 * i + 1], vr, im));
-            }
-            out[2 * j] = re;
-            out[2 * j + 1] = im;
+    if (lane) return;
+#pragma unroll
+    for (int q = 0; q < NI; ++q) {
+        const int i = wid + NW * q, g = i0 + i;
+        if (i >= k) break;
+        double re = sum[CPLX ? 2 * q : q], im = CPLX ? sum[CPLX ? 2 * q + 1 : 0] : 0.0;
+        if (mode == DOT_COLUMN) {
+            if (g == col) im = 0.0;
+            out[2 * (g * KMAX + col)] = re;
+            out[2 * (g * KMAX + col) + 1] = im;
+            out[2 * (col * KMAX + g)] = re;
+            out[2 * (col * KMAX + g) + 1] = g == col ? 0.0 : -im;
         } else {
-            double acc = accumulate ? out[j] : 0.0;
-            for (int i = 0; i < k; ++i) acc = fma(sy[2 * i], V[i * ldv + j], acc);
-            out[j] = acc;
+            if (mode == DOT_NEGATE) {
+                re = -re;
+                im = -im;
+            }
+            out[2 * g] = re;
+            out[2 * g + 1] = im;
+        }
+    }
+}
+
+// out_b = sum_i y_i V_b,i  (+ out_b when accumulate) for the vectors V0 (and V1 if out1), y
+// complex as 2 doubles per entry.  NORM (real vectors): also *n2 = ||out_0||^2,
+// added in the order of k_norm2.
+template <bool CPLX, bool NORM>
+__global__ void __launch_bounds__(RED_THREADS) k_lincomb(const double *__restrict__ V0, const double *__restrict__ V1,
+                                                         int64_t ldv, int k, const double *__restrict__ y, int64_t n,
+                                                         double *__restrict__ out0, double *__restrict__ out1,
+                                                         int accumulate, double *__restrict__ partial,
+                                                         unsigned *__restrict__ counter, double *__restrict__ n2) {
+    __shared__ double sy[2 * KMAX];
+    if (threadIdx.x < 2 * k) sy[threadIdx.x] = y[threadIdx.x];
+    __syncthreads();
+    double norm = 0.0;
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+        for (int b = 0; b < (out1 ? 2 : 1); ++b) {
+            const double *V = b ? V1 : V0;
+            double *out = b ? out1 : out0;
+            if (CPLX) {
+                double re = accumulate ? out[2 * j] : 0.0, im = accumulate ? out[2 * j + 1] : 0.0;
+#pragma unroll 4
+                for (int i = 0; i < k; ++i) {
+                    const double vr = V[i * 2 * ldv + 2 * j], vi = V[i * 2 * ldv + 2 * j + 1];
+                    re = fma(sy[2 * i], vr, fma(-sy[2 * i + 1], vi, re));
+                    im = fma(sy[2 * i], vi, fma(sy[2 * i + 1], vr, im));
+                }
+                out[2 * j] = re;
+                out[2 * j + 1] = im;
+                            } else {
+                double acc = accumulate ? out[j] : 0.0;
+#pragma unroll 4
+                for (int i = 0; i < k; ++i) acc = fma(sy[2 * i], V[i * ldv + j], acc);
+                out[j] = acc;
+                if (NORM && b == 0) norm = fma(acc, acc, norm);
+            }
+        }
+    }
+    if (NORM) {
+        __shared__ double red[RED_THREADS / 32];
+        for (int o = 16; o; o >>= 1) norm += __shfl_xor_sync(0xFFFFFFFFu, norm, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = norm;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0;
+            for (int w = 0; w < RED_THREADS / 32; ++w) s += red[w];
+            partial[blockIdx.x] = s;
+        }
+        if (!last_block(counter)) return;
+        if (threadIdx.x < 32) {
+            const double a = warp_sum_blocks(partial, 1, gridDim.x);
+            if (threadIdx.x == 0) *n2 = a;
         }
     }
 }
 
 // Phase-align (c, sc) to c_prev by the scalar ph = conj(ov)/|ov|, then
 //   r = sc - lam c;  s_i = r_i / (lam - H_ii) if |lam - H_ii| >= 1e-12 else 0;  t = s.
-// Partial sums: ||r||^2, ||s||^2; partial max |c - c_prev|.
+// ov = <c_prev|c>.  Into scal: ||r||^2, ||s||^2, max |c - c_prev|.
 template <bool CPLX>
 __global__ void __launch_bounds__(RED_THREADS) k_residual(double *__restrict__ c, double *__restrict__ sc,
                                                           const double *__restrict__ cprev, int have_prev,
                                                           const double *__restrict__ diag,
-                                                          const dav_scalars *__restrict__ sc_in, int64_t n,
-                                                          double *__restrict__ t, double *__restrict__ partial) {
-    const double lam = sc_in->lam;
+                                                          const double *__restrict__ ov, dav_scalars *__restrict__ scal,
+                                                          int64_t n, double *__restrict__ t,
+                                                          double *__restrict__ partial, unsigned *__restrict__ counter) {
+    const double lam = scal->lam;
     double pr = 1.0, pi = 0.0;
     if (have_prev) {
-        const double ore = sc_in->ov_re, oim = sc_in->ov_im, m = sqrt(ore * ore + oim * oim);
+        const double ore = ov[0], oim = ov[1], m = sqrt(ore * ore + oim * oim);
         if (m > 0) { pr = ore / m; pi = -oim / m; }
     }
     double r2 = 0.0, s2 = 0.0, mdc = 0.0;
@@ -187,21 +314,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual(double *__restrict__ c
         partial[blockIdx.x * 4 + 1] = b;
         partial[blockIdx.x * 4 + 2] = m;
     }
-}
-
-__global__ void k_reduce_residual(const double *__restrict__ partial, int nb, dav_scalars *__restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    double a = 0, b = 0, m = 0;
-    for (int i = lane; i < nb; i += 32) { a += partial[i * 4]; b += partial[i * 4 + 1]; m = fmax(m, partial[i * 4 + 2]); }
-    for (int o = 16; o; o >>= 1) {
-        a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-        b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
-        m = fmax(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    }
+    if (!last_block(counter) || wid != 0) return;
+    double ab[2];
+    warp_sum_blocks<2>(partial, 4, gridDim.x, 1, ab);
+    const double a = ab[0], b = ab[1];
+    double m = 0;
+    for (int i = lane; i < (int)gridDim.x; i += 32) m = fmax(m, __ldcg(partial + i * 4 + 2));
+    for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
     if (lane == 0) {
-        out->rnorm2 = a;
-        out->snorm2 = b;
-        out->maxdc = m;
+        scal->rnorm2 = a;
+        scal->snorm2 = b;
+        scal->maxdc = m;
     }
 }
 
@@ -219,9 +342,10 @@ __global__ void k_threshold(double *__restrict__ t, int64_t n, const dav_scalars
     }
 }
 
-// Squared norm partials of x (complex counted as 2n reals).
+// *n2 = ||x||^2 (complex counted as 2n reals).
 __global__ void __launch_bounds__(RED_THREADS) k_norm2(const double *__restrict__ x, int64_t nreal,
-                                                       double *__restrict__ partial) {
+                                                       double *__restrict__ partial, unsigned *__restrict__ counter,
+                                                       double *__restrict__ n2) {
     double a = 0.0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nreal; j += (int64_t)gridDim.x * blockDim.x)
         a = fma(x[j], x[j], a);
@@ -234,60 +358,89 @@ __global__ void __launch_bounds__(RED_THREADS) k_norm2(const double *__restrict_
         for (int w = 0; w < RED_THREADS / 32; ++w) s += red[w];
         partial[blockIdx.x] = s;
     }
+    if (!last_block(counter)) return;
+    if (threadIdx.x < 32) {
+        const double s = warp_sum_blocks(partial, 1, gridDim.x);
+        if (threadIdx.x == 0) *n2 = s;
+    }
 }
 
-__global__ void k_reduce_norm(const double *__restrict__ partial, int nb, double *__restrict__ out) {
-    const double a = warp_sum_blocks(partial, 1, nb);
-    if (threadIdx.x == 0) *out = a;
-}
-
-// x *= 1/sqrt(*n2) (or *scale directly when n2 == nullptr)
-__global__ void k_scale(double *__restrict__ x, int64_t nreal, const double *__restrict__ n2) {
+// out = x / sqrt(*n2) (out may be x)
+__global__ void k_scale(const double *x, double *out, int64_t nreal, const double *__restrict__ n2) {
     const double f = 1.0 / sqrt(*n2);
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nreal; j += (int64_t)gridDim.x * blockDim.x)
-        x[j] *= f;
+        out[j] = x[j] * f;
 }
 
-// Negate a complex coefficient vector (k entries).
-__global__ void k_negate(double *__restrict__ y, int k) {
-    if (threadIdx.x < 2 * k) y[threadIdx.x] = -y[threadIdx.x];
+// One rotation: (a, b) of a row (or column) pair becomes (c a - s b, s a + c b).
+__device__ __forceinline__ double rot_p(double c, double sn, double ap, double aq) { return fma(c, ap, -sn * aq); }
+__device__ __forceinline__ double rot_q(double c, double sn, double ap, double aq) { return fma(sn, ap, c * aq); }
+// Either of the two.
+__device__ __forceinline__ double rot_one(bool q, double c, double sn, double ap, double aq) {
+    return fma(q ? sn : c, ap, (q ? c : -sn) * aq);
 }
 
-// Hsub column/row update: Hsub[i][k] = dots[i] for i <= k, Hsub[k][i] = conj(dots[i]).
-__global__ void k_hsub_update(double *__restrict__ Hs, const double *__restrict__ dots, int k) {
-    const int i = threadIdx.x;
-    if (i > k) return;
-    Hs[2 * (i * KMAX + k)] = dots[2 * i];
-    Hs[2 * (i * KMAX + k) + 1] = dots[2 * i + 1];
-    Hs[2 * (k * KMAX + i)] = dots[2 * i];
-    Hs[2 * (k * KMAX + i) + 1] = -dots[2 * i + 1];
-    if (i == k) Hs[2 * (k * KMAX + k) + 1] = 0.0;
+// Pair t of round r (round-robin over M indices, M even): (M - 1, r), then (r + t, r - t) modulo
+// M - 1; and the pair of index x, with is_q telling which of the two x is.
+__device__ __forceinline__ void jac_pair(int M, int r, int t, int &p, int &q) {
+    if (t == 0) {
+        p = M - 1;
+        q = r;
+    } else {
+        p = r + t < M - 1 ? r + t : r + t - (M - 1);
+        q = r - t >= 0 ? r - t : r - t + (M - 1);
+    }
+}
+__device__ __forceinline__ int jac_find(int M, int r, int x, bool &is_q) {
+    if (x == M - 1 || x == r) {
+        is_q = x == r;
+        return 0;
+    }
+    const int d = x - r >= 0 ? x - r : x - r + (M - 1);
+    is_q = d > M / 2 - 1;
+    return is_q ? M - 1 - d : d;
 }
 
-// Lowest eigenpair of the k x k Hermitian Hs (leading dimension KMAX, complex entries)
-// by Jacobi on the real symmetric embedding of size m = k (real) or 2k (complex), with the
+// A low eigenpair of the k x k Hermitian Hs (leading dimension KMAX, complex entries) by
+// Jacobi on the real symmetric embedding of size m = k (real) or 2k (complex), with the
 // rotations of a sweep in round-robin order: each of the M - 1 rounds (M = m rounded up to
-// even) pairs every index with one other (index M - 1 with r, and (r + i) with (r - i)
-// modulo M - 1), so the M / 2 rotations of a round touch disjoint rows and columns and run
-// at once: angles from the current A (the classical formula, tan of the angle the smaller
-// root of t^2 + 2 theta t - 1 = 0, theta = (A_qq - A_pp) / (2 A_pq)), then the columns of A
-// and Q, then the rows of A.  Sweeps stop once the off-diagonal mass is below 1e-30 of the
-// total.  Writes y (complex, k entries) and lam.  One block of JAC_THREADS threads.
+// even) pairs every index with one other, so the M / 2 rotations of a round touch disjoint
+// rows and columns and run at once: angles from the current A (the classical formula, tan
+// of the angle the smaller root of t^2 + 2 theta t - 1 = 0, theta = (A_qq - A_pp) / (2 A_pq)),
+// then the columns of A and Q, then the rows of A.  Sweeps stop once the off-diagonal mass is
+// below 1e-30 of the total.  Writes y (complex, k entries) and lam.
+//
+// A 32 x 32 round is 6,144 FP64 operations, and one SM does two per clock: on one block the
+// projected eigenproblem took 360 us, half of a Davidson iteration on 63,504 determinants.
+// A cluster of JAC_CLUSTER blocks shares a round:
+//   - a 2 x 2 block (pair i, pair j) takes its column and its row rotation on its own, so a
+//     thread owns such a block, without a barrier between the two phases;
+//   - every block keeps a full copy of A (two buffers) and writes its results to all copies
+//     through distributed shared memory, one cluster barrier per round;
+//   - the rows of Q stay with one block each;
+//   - the angles of the next round are computed while the others rotate, by three warps of
+//     each block, from the old A: three elements of the new A per pair, then the angle (37
+//     FP64 instructions by fp64_fast.cuh, 64 cycles each: what bounds a round).
+// The operations on each element are those of the one-block form in the same order (the same
+// bits): 360 -> 228 us on average over a solve (10 electrons in 10 orbitals, up to 32 vectors).
 // root: 0 = lowest Ritz pair, 1 = second lowest (the real embedding of a complex Hermitian
 // matrix has every eigenvalue twice, so there the selected entry is the (2 root)-th).
-__global__ void __launch_bounds__(JAC_THREADS) k_jacobi(const double *__restrict__ Hs, int k, int cplx, int root,
-                                                        double *__restrict__ y, dav_scalars *__restrict__ out) {
-    extern __shared__ double jac_smem[];  // A and Q, each m x (m + 1)
-    __shared__ double cs[KMAX][2];
-    __shared__ int pr[KMAX][2];
+__global__ void __cluster_dims__(JAC_CLUSTER, 1, 1) __launch_bounds__(JAC_THREADS)
+    k_jacobi(const double *__restrict__ Hs, int k, int cplx, int root, double *__restrict__ y,
+             dav_scalars *__restrict__ out) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ double jac_smem[];  // A (two buffers, m x (m + 1)), own rows of Q
+    constexpr int QROWS = 2 * KMAX / JAC_CLUSTER;
+    __shared__ double cs[2][KMAX][2], el[2][KMAX];
     __shared__ double red[2][JAC_THREADS / 32];
-    __shared__ int stop;
+    __shared__ double ycol[2 * KMAX];
+    __shared__ int stop, best;
     const int m = cplx ? 2 * k : k;
     const int ld = m + 1;
     const int M = m + (m & 1), half = M / 2;
-    double *Ab = jac_smem, *Qb = jac_smem + m * ld;
-#define A(r, c) Ab[(r) * ld + (c)]
-#define Q(r, c) Qb[(r) * ld + (c)]
+    const int rank = (int)cluster.block_rank();
+    double *Ab = jac_smem, *Qb = jac_smem + 2 * m * ld;
     const int t = threadIdx.x, nt = blockDim.x;
     for (int i = t; i < m * m; i += nt) {
         const int r = i / m, c = i % m;
@@ -299,15 +452,45 @@ __global__ void __launch_bounds__(JAC_THREADS) k_jacobi(const double *__restrict
             const double re = Hs[2 * (rr * KMAX + cc)], im = Hs[2 * (rr * KMAX + cc) + 1];
             v = (rb == cb) ? re : (rb == 1 ? im : -im);
         }
-        A(r, c) = v;
-        Q(r, c) = (r == c) ? 1.0 : 0.0;
+        Ab[r * ld + c] = v;
+    }
+    for (int i = t; i < QROWS * m; i += nt) {  // row rank + JAC_CLUSTER * (i / m)
+        const int r = rank + JAC_CLUSTER * (i / m), c = i % m;
+        Qb[(i / m) * ld + c] = (r == c) ? 1.0 : 0.0;
     }
     __syncthreads();
+    // angle of the pair (p, q) from its three elements (comparisons on the bits: every FP64
+    // instruction of this chain costs 64 cycles)
+    auto angle = [&](double apq, double app, double aqq, double &c, double &sn) {
+        c = 1.0;
+        sn = 0.0;
+        const int ex = fp64_fast::exponent(apq);
+        if (ex > 30 ? ex < 2046 : fabs(apq) > 1e-300) {  // 2^-993 > 1e-300
+            const double theta = fp64_fast::divide(aqq - app, fp64_fast::twice(apq));
+            double y0, y1;
+            const double den = fabs(theta) + fp64_fast::root(theta * theta + 1.0, y0);
+            const double tt = fp64_fast::reciprocal(theta >= 0 ? 1.0 : -1.0, den);
+            const double s = fp64_fast::root(tt * tt + 1.0, y1);  // in [1, sqrt 2]
+            c = fp64_fast::reciprocal_near(s, y1);
+            sn = tt * c;
+        }
+    };
+    int buf = 0;  // current buffer of A and of the angles
+    if (t < half) {
+        int p, q;
+        jac_pair(M, 0, t, p, q);
+        double c = 1.0, sn = 0.0;
+        if (p < m && q < m) angle(Ab[p * ld + q], Ab[p * ld + p], Ab[q * ld + q], c, sn);
+        cs[0][t][0] = c;
+        cs[0][t][1] = sn;
+    }
+    cluster.sync();  // every copy of A is loaded before a neighbour writes to it
     for (int sweep = 0; sweep < 60 && m > 1; ++sweep) {
+        const double *A0 = Ab + buf * m * ld;
         double off = 0.0, tot = 0.0;
         for (int i = t; i < m * m; i += nt) {
             const int r = i / m, c = i % m;
-            const double a2 = A(r, c) * A(r, c);
+            const double a2 = A0[r * ld + c] * A0[r * ld + c];
             tot += a2;
             if (r != c) off += a2;
         }
@@ -329,77 +512,110 @@ __global__ void __launch_bounds__(JAC_THREADS) k_jacobi(const double *__restrict
             stop = (o <= 1e-30 * a) || o == 0.0;
         }
         __syncthreads();
-        if (stop) break;
-        for (int r = 0; r < M - 1; ++r) {
-            if (t < half) {
-                int p, q;
-                if (t == 0) {
-                    p = M - 1;
-                    q = r;
-                } else {
-                    p = (r + t) % (M - 1);
-                    q = (r - t + (M - 1)) % (M - 1);
+        if (stop) break;  // every block of the cluster has the same A and decides the same
+        for (int r = 0; r < M - 1; ++r, buf ^= 1) {
+            const double *A = Ab + buf * m * ld;
+            double *An = Ab + (buf ^ 1) * m * ld;
+            const double(*rot)[2] = cs[buf];
+            if (t < 96) {
+                // angles of the next round's pairs (round 0 after the last of a sweep), on one SM
+                // sub-partition per element: warp 0 takes A_pq, warp 1 A_pp, warp 2 A_qq of A after
+                // this round, then warp 0 the angle.  An identity rotation (1, 0) keeps its values,
+                // and the padding index of a pair reads as zero.
+                const int rn = r + 1 < M - 1 ? r + 1 : 0, warp = t >> 5, lane = t & 31;
+                int p = 0, q = 0;
+                bool on = lane < half;
+                if (on) jac_pair(M, rn, lane, p, q);
+                on = on && p < m && q < m;
+                double v = 0.0;
+                if (on) {
+                    const int row = warp == 2 ? q : p, col = warp == 1 ? p : q;
+                    bool row_q, col_q;
+                    const int i = jac_find(M, r, row, row_q), j = jac_find(M, r, col, col_q);
+                    int pi, qi, pj, qj;
+                    jac_pair(M, r, i, pi, qi);
+                    jac_pair(M, r, j, pj, qj);
+                    const double ci = rot[i][0], si = rot[i][1], cj = rot[j][0], sj = rot[j][1];
+                    const bool rp = pi < m, cp = pj < m;
+                    const double a00 = rp && cp ? A[pi * ld + pj] : 0.0, a01 = rp ? A[pi * ld + qj] : 0.0;
+                    const double a10 = cp ? A[qi * ld + pj] : 0.0, a11 = A[qi * ld + qj];
+                    v = rot_one(row_q, ci, si, rot_one(col_q, cj, sj, a00, a01), rot_one(col_q, cj, sj, a10, a11));
+                    if (warp) el[warp - 1][lane] = v;
                 }
-                double c = 1.0, sn = 0.0;
-                if (p < m && q < m) {
-                    const double apq = A(p, q);
-                    if (fabs(apq) > 1e-300) {
-                        const double theta = (A(q, q) - A(p, p)) / (2.0 * apq);
-                        const double tt = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                        c = 1.0 / sqrt(tt * tt + 1.0);
-                        sn = tt * c;
+                asm volatile("bar.sync 1, 96;" ::: "memory");
+                if (warp == 0 && lane < half) {
+                    double c = 1.0, sn = 0.0;
+                    if (on) angle(v, el[0][lane], el[1][lane], c, sn);
+                    cs[buf ^ 1][lane][0] = c;
+                    cs[buf ^ 1][lane][1] = sn;
+                }
+            } else {
+                const int w = t - 96, nw = nt - 96;
+                // own share of the 2 x 2 blocks
+                for (int b = rank + JAC_CLUSTER * w; b < half * half; b += JAC_CLUSTER * nw) {
+                    const int i = b / half, j = b - i * half;
+                    int pi, qi, pj, qj;
+                    jac_pair(M, r, i, pi, qi);
+                    jac_pair(M, r, j, pj, qj);
+                    const double ci = rot[i][0], si = rot[i][1], cj = rot[j][0], sj = rot[j][1];
+                    const bool rp = pi < m, cp = pj < m;  // only p can be the padding index
+                    double a00 = rp && cp ? A[pi * ld + pj] : 0.0, a01 = rp ? A[pi * ld + qj] : 0.0;
+                    double a10 = cp ? A[qi * ld + pj] : 0.0, a11 = A[qi * ld + qj];
+                    if (sj != 0.0) {
+                        const double b00 = rot_p(cj, sj, a00, a01), b01 = rot_q(cj, sj, a00, a01);
+                        const double b10 = rot_p(cj, sj, a10, a11), b11 = rot_q(cj, sj, a10, a11);
+                        a00 = b00; a01 = b01; a10 = b10; a11 = b11;
+                    }
+                    if (si != 0.0) {
+                        const double b00 = rot_p(ci, si, a00, a10), b10 = rot_q(ci, si, a00, a10);
+                        const double b01 = rot_p(ci, si, a01, a11), b11 = rot_q(ci, si, a01, a11);
+                        a00 = b00; a01 = b01; a10 = b10; a11 = b11;
+                    }
+#pragma unroll
+                    for (int g = 0; g < JAC_CLUSTER; ++g) {
+                        double *R = cluster.map_shared_rank(An, g);
+                        if (rp && cp) R[pi * ld + pj] = a00;
+                        if (rp) R[pi * ld + qj] = a01;
+                        if (cp) R[qi * ld + pj] = a10;
+                        R[qi * ld + qj] = a11;
                     }
                 }
-                pr[t][0] = p;
-                pr[t][1] = q;
-                cs[t][0] = c;
-                cs[t][1] = sn;
+                // own rows of Q
+                for (int b = w; b < QROWS * half; b += nw) {
+                    const int i = b / half, j = b - i * half;
+                    const double sj = rot[j][1], cj = rot[j][0];
+                    if (rank + JAC_CLUSTER * i >= m || sj == 0.0) continue;
+                    int pj, qj;
+                    jac_pair(M, r, j, pj, qj);
+                    const double qp = Qb[i * ld + pj], qq = Qb[i * ld + qj];
+                    Qb[i * ld + pj] = rot_p(cj, sj, qp, qq);
+                    Qb[i * ld + qj] = rot_q(cj, sj, qp, qq);
+                }
             }
-            __syncthreads();
-            for (int i = t; i < half * m; i += nt) {  // columns p, q of A and Q
-                const int j = i / m, row = i % m;
-                const double sn = cs[j][1];
-                if (sn == 0.0) continue;
-                const double c = cs[j][0];
-                const int p = pr[j][0], q = pr[j][1];
-                const double ap = A(row, p), aq = A(row, q);
-                A(row, p) = c * ap - sn * aq;
-                A(row, q) = sn * ap + c * aq;
-                const double qp = Q(row, p), qq = Q(row, q);
-                Q(row, p) = c * qp - sn * qq;
-                Q(row, q) = sn * qp + c * qq;
-            }
-            __syncthreads();
-            for (int i = t; i < half * m; i += nt) {  // rows p, q of A
-                const int j = i / m, col = i % m;
-                const double sn = cs[j][1];
-                if (sn == 0.0) continue;
-                const double c = cs[j][0];
-                const int p = pr[j][0], q = pr[j][1];
-                const double ap = A(p, col), aq = A(q, col);
-                A(p, col) = c * ap - sn * aq;
-                A(q, col) = sn * ap + c * aq;
-            }
-            __syncthreads();
+            cluster.sync();
         }
     }
-    if (t == 0) {
-        // the (root * (cplx ? 2 : 1))-th smallest diagonal entry (ties: lowest index)
-        const int want = root * (cplx ? 2 : 1);
-        int best = 0;
-        for (int r = 0; r <= want; ++r) {
-            best = -1;
-            for (int i = 0; i < m; ++i) {
-                int rank = 0;  // entries before i in the ascending order
-                for (int j = 0; j < m; ++j)
-                    if (A(j, j) < A(i, i) || (A(j, j) == A(i, i) && j < i)) ++rank;
-                if (rank == r) best = i;
-            }
-        }
-        out->lam = A(best, best);
+    // the (root * (cplx ? 2 : 1))-th smallest diagonal entry (ties: lowest index)
+    const double *A = Ab + buf * m * ld;
+    const int want = root * (cplx ? 2 : 1);
+    if (t < m) {
+        int before = 0;  // entries before t in the ascending order
+        for (int j = 0; j < m; ++j)
+            if (A[j * ld + j] < A[t * ld + t] || (A[j * ld + j] == A[t * ld + t] && j < t)) ++before;
+        if (before == want) best = t;
+    }
+    __syncthreads();
+    {
+        double *col = cluster.map_shared_rank(ycol, 0);
+        for (int i = t; i < QROWS; i += nt)
+            if (rank + JAC_CLUSTER * i < m) col[rank + JAC_CLUSTER * i] = Qb[i * ld + best];
+    }
+    cluster.sync();
+    if (rank == 0 && t == 0) {
+        out->lam = A[best * ld + best];
         double nrm = 0.0;
         for (int i = 0; i < k; ++i) {
-            const double re = Q(i, best), im = cplx ? Q(k + i, best) : 0.0;
+            const double re = ycol[i], im = cplx ? ycol[k + i] : 0.0;
             y[2 * i] = re;
             y[2 * i + 1] = im;
             nrm += re * re + im * im;
@@ -408,8 +624,6 @@ __global__ void __launch_bounds__(JAC_THREADS) k_jacobi(const double *__restrict
         for (int i = 0; i < 2 * k; ++i) y[i] *= nrm;
     }
 }
-#undef A
-#undef Q
 
 // argmin of diag (lowest index on ties) -> unit vector
 // Index of the smallest diagonal element (the lowest index among equal ones), in two
@@ -478,6 +692,9 @@ __global__ void k_set_start(double *__restrict__ x, int64_t nreal, int cplx, con
     }
 }
 
+// Shared memory of k_jacobi at size m: two buffers of A, this block's rows of Q.
+inline size_t jac_smem_bytes(int m) { return (size_t)(2 * m + 2 * KMAX / JAC_CLUSTER) * (m + 1) * sizeof(double); }
+
 inline size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -500,7 +717,9 @@ struct fci_davidson_state {
            *diag = nullptr;
     void *sig_ws = nullptr;
     size_t sig_bytes = 0;
-    double *partial = nullptr, *Hs = nullptr, *dots = nullptr, *y = nullptr, *nrm = nullptr;
+    double *partial = nullptr, *Hs = nullptr, *dots = nullptr, *y = nullptr, *nrm = nullptr, *ov = nullptr;
+    unsigned *counter = nullptr;  // blocks done in the running reduction (zero between kernels)
+    double *ritz = nullptr;       // the current Ritz vector (c, or c_prev after the exchange)
     dav_scalars *scal = nullptr;
     int64_t *argmin = nullptr;
     unsigned vb = 1;
@@ -523,42 +742,56 @@ struct fci_davidson_state {
     double *Vk(int i) { return (double *)((char *)V + (size_t)i * vec); }
     double *Sk(int i) { return (double *)((char *)S + (size_t)i * vec); }
 
-    // vectors i0 .. i0 + kk - 1 of Vb into entries i0 .. of each block's partial row
     template <int KB>
-    void multidot_kb(const double *Vb, int i0, int kk, const double *x) {
-        const double *v0 = Vb + (size_t)i0 * (cplx ? 2 : 1) * ldv;
-        if (cplx) k_multidot<true, KB><<<vb, RED_THREADS, 0, s>>>(v0, ldv, kk, x, n, partial + 2 * i0);
-        else k_multidot<false, KB><<<vb, RED_THREADS, 0, s>>>(v0, ldv, kk, x, n, partial + 2 * i0);
+    void multidot_kb(const double *Vb, int i0, int kk, const double *x, int mode, int col, double *out) {
+        if (cplx) k_multidot<true, (KB <= 16 ? KB : 16)><<<vb, RED_THREADS, 0, s>>>(Vb, ldv, i0, kk, x, n, partial, counter, mode, col, out);
+        else k_multidot<false, KB><<<vb, RED_THREADS, 0, s>>>(Vb, ldv, i0, kk, x, n, partial, counter, mode, col, out);
     }
-    // <V_i|x> for i < kk: up to 16 vectors per pass (more would cost occupancy)
-    cudaError_t multidot(const double *Vb, int kk, const double *x, double *out) {
-        if (kk <= 1) multidot_kb<1>(Vb, 0, kk, x);
-        else if (kk <= 4) multidot_kb<4>(Vb, 0, kk, x);
-        else if (kk <= 8) multidot_kb<8>(Vb, 0, kk, x);
-        else if (kk <= 16) multidot_kb<16>(Vb, 0, kk, x);
+    // <V_i|x> for i < kk: one pass (real, and complex up to 16 vectors), else 16 vectors per pass
+    cudaError_t multidot(const double *Vb, int kk, const double *x, double *out, int mode = DOT_PLAIN, int col = 0) {
+        if (kk <= 1) multidot_kb<1>(Vb, 0, kk, x, mode, col, out);
+        else if (kk <= 4) multidot_kb<4>(Vb, 0, kk, x, mode, col, out);
+        else if (kk <= 8) multidot_kb<8>(Vb, 0, kk, x, mode, col, out);
+        else if (kk <= 16) multidot_kb<16>(Vb, 0, kk, x, mode, col, out);
+        else if (!cplx) multidot_kb<32>(Vb, 0, kk, x, mode, col, out);
         else {
-            multidot_kb<16>(Vb, 0, 16, x);
-            multidot_kb<16>(Vb, 16, kk - 16, x);
+            multidot_kb<16>(Vb, 0, 16, x, mode, col, out);
+            multidot_kb<16>(Vb, 16, kk - 16, x, mode, col, out);
         }
-        k_reduce_partial<<<1, 256, 0, s>>>(partial, vb, kk, out);
         return cudaGetLastError();
     }
-    cudaError_t lincomb(const double *Vb, int kk, const double *yy, double scale, double *out, int acc) {
-        if (cplx) k_lincomb<true><<<vb, RED_THREADS, 0, s>>>(Vb, ldv, kk, yy, scale, n, out, acc);
-        else k_lincomb<false><<<vb, RED_THREADS, 0, s>>>(Vb, ldv, kk, yy, scale, n, out, acc);
+    // out0 (and out1) = sum_i yy_i V0_i (V1_i), added to what is there if acc; n2 = ||out0||^2 if given
+    cudaError_t lincomb(const double *V0, int kk, const double *yy, double *out0, int acc, double *n2 = nullptr,
+                        const double *V1 = nullptr, double *out1 = nullptr) {
+        if (cplx) {  // the norm of a complex vector adds its 2n reals in k_norm2's order
+            k_lincomb<true, false><<<vb, RED_THREADS, 0, s>>>(V0, V1, ldv, kk, yy, n, out0, out1, acc, partial, counter, n2);
+            if (n2) norm2(out0, n2);
+        } else if (n2) {
+            k_lincomb<false, true><<<vb, RED_THREADS, 0, s>>>(V0, V1, ldv, kk, yy, n, out0, out1, acc, partial, counter, n2);
+        } else {
+            k_lincomb<false, false><<<vb, RED_THREADS, 0, s>>>(V0, V1, ldv, kk, yy, n, out0, out1, acc, partial, counter, n2);
+        }
         return cudaGetLastError();
     }
+    void norm2(const double *x, double *n2) { k_norm2<<<vb, RED_THREADS, 0, s>>>(x, nreal, partial, counter, n2); }
+    void scale(const double *x, double *out, const double *n2) { k_scale<<<vb, RED_THREADS, 0, s>>>(x, out, nreal, n2); }
     cudaError_t normalize(double *x, double *n2out) {
-        k_norm2<<<vb, RED_THREADS, 0, s>>>(x, nreal, partial);
-        k_reduce_norm<<<1, 32, 0, s>>>(partial, vb, n2out);
-        k_scale<<<vb, RED_THREADS, 0, s>>>(x, nreal, n2out);
+        norm2(x, n2out);
+        scale(x, x, n2out);
         return cudaGetLastError();
+    }
+    // Ritz pair `root` of the projected matrix: y and scal->lam
+    void ritz_pair(int root) {
+        const int m = cplx ? 2 * k : k;
+        k_jacobi<<<JAC_CLUSTER, JAC_THREADS, jac_smem_bytes(m), s>>>(Hs, k, cplx ? 1 : 0, root, y, scal);
+    }
+    void residual(bool with_prev) {
+        if (cplx) k_residual<true><<<vb, RED_THREADS, 0, s>>>(c, sc, cp, with_prev, diag, ov, scal, n, t, partial, counter);
+        else k_residual<false><<<vb, RED_THREADS, 0, s>>>(c, sc, cp, with_prev, diag, ov, scal, n, t, partial, counter);
     }
     // New subspace column kk: Hs[:, kk] = V^H S_kk.
     int add_column(int kk) {
-        FCI_CUDA(h, multidot(V, kk + 1, Sk(kk), dots));
-        k_hsub_update<<<1, 64, 0, s>>>(Hs, dots, kk);
-        FCI_CUDA(h, cudaGetLastError());
+        FCI_CUDA(h, multidot(V, kk + 1, Sk(kk), Hs, DOT_COLUMN, kk));
         return FCI_OK;
     }
     int ask(int kind, double *x, double *yv) {
@@ -609,15 +842,19 @@ struct fci_davidson_state {
         dots = Hs + 2 * KMAX * KMAX;               // 2 * KMAX
         y = dots + 2 * KMAX;                       // 2 * KMAX
         nrm = y + 2 * KMAX;                        // 4
-        scal = (dav_scalars *)(nrm + 4);
+        ov = nrm + 4;                              // 2
+        scal = (dav_scalars *)(ov + 2);
         argmin = (int64_t *)(scal + 1);
+        counter = (unsigned *)(argmin + 1);
         vb = (unsigned)std::min<int64_t>(RED_BLOCKS, std::max<int64_t>(1, ceil_div(n, RED_THREADS)));
+        ritz = c;
+        FCI_CUDA(h, cudaMemsetAsync(counter, 0, sizeof(unsigned), s));
         prec = o.precision;
         slices = o.n_slices;
         if (o.eps < 0.0) o.eps = 10.0 / sqrt((double)n);  // the paper's eps <~ 10 / sqrt(N_dets) rule
         final_phase = o.precision == FCI_PREC_FP64 || (o.precision == o.final_precision && o.n_slices == o.final_slices);
         FCI_CUDA(h, cudaFuncSetAttribute(k_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         2 * (2 * KMAX) * (2 * KMAX + 1) * (int)sizeof(double)));
+                                         (int)jac_smem_bytes(2 * KMAX)));
         if (h->das_active) FCI_CUDA(h, launch_diag_das(h, diag, s));
         else if (h->mode == FCI_MODE_SPINOR) FCI_CUDA(h, launch_diag_spinor(h, diag, s));
         else FCI_CUDA(h, launch_diag_fci(h, diag, s));
@@ -674,20 +911,11 @@ struct fci_davidson_state {
             }
             if (!gap_phase) ++it;  // second-root passes have their own limit (max_iter of them)
             t_iter = std::chrono::steady_clock::now();
-            {
-                const int m = cplx ? 2 * k : k;
-                k_jacobi<<<1, JAC_THREADS, 2 * m * (m + 1) * sizeof(double), s>>>(Hs, k, cplx ? 1 : 0, gap_phase ? 1 : 0, y,
-                                                                          scal);
-            }
-            FCI_CUDA(h, lincomb(V, k, y, 1.0, c, 0));
-            FCI_CUDA(h, lincomb(S, k, y, 1.0, sc, 0));
-            if (have_prev) {
-                FCI_CUDA(h, multidot(cp, 1, c, dots));  // <c_prev|c>
-                FCI_CUDA(h, cudaMemcpyAsync(&scal->ov_re, dots, 16, cudaMemcpyDeviceToDevice, s));
-            }
-            if (cplx) k_residual<true><<<vb, RED_THREADS, 0, s>>>(c, sc, cp, have_prev, diag, scal, n, t, partial);
-            else k_residual<false><<<vb, RED_THREADS, 0, s>>>(c, sc, cp, have_prev, diag, scal, n, t, partial);
-            k_reduce_residual<<<1, 32, 0, s>>>(partial, vb, scal);
+            ritz_pair(gap_phase ? 1 : 0);
+            FCI_CUDA(h, lincomb(V, k, y, c, 0, nullptr, S, sc));
+            ritz = c;
+            if (have_prev) FCI_CUDA(h, multidot(cp, 1, c, ov));  // <c_prev|c>
+            residual(have_prev);
             FCI_CUDA(h, cudaGetLastError());
             FCI_CUDA(h, cudaMemcpyAsync(&hs, scal, sizeof hs, cudaMemcpyDeviceToHost, s));
             FCI_CUDA(h, cudaStreamSynchronize(s));
@@ -746,12 +974,9 @@ struct fci_davidson_state {
             if (k >= ms && !gap_phase) {
                 // collapse to the current and previous Ritz vectors (sigma by linearity)
                 // V_0 = c / ||c||, S_0 = sc / ||c||
-                FCI_CUDA(h, cudaMemcpyAsync(Vk(0), c, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
-                FCI_CUDA(h, cudaMemcpyAsync(Sk(0), sc, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
-                k_norm2<<<vb, RED_THREADS, 0, s>>>(Vk(0), nreal, partial);
-                k_reduce_norm<<<1, 32, 0, s>>>(partial, vb, nrm);
-                k_scale<<<vb, RED_THREADS, 0, s>>>(Vk(0), nreal, nrm);
-                k_scale<<<vb, RED_THREADS, 0, s>>>(Sk(0), nreal, nrm);
+                norm2(c, nrm);
+                scale(c, Vk(0), nrm);
+                scale(sc, Sk(0), nrm);
                 int knew = 1;
                 if (have_prev && ms > 2) {
                     // p = c_prev - <c|c_prev> c, S_p = sc_prev - <c|c_prev> sc, both / ||p||.
@@ -761,19 +986,16 @@ struct fci_davidson_state {
                     FCI_CUDA(h, cudaMemcpyAsync(Vk(1), cp, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
                     FCI_CUDA(h, cudaMemcpyAsync(Sk(1), scp, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
                     for (int pass = 0; pass < 2; ++pass) {
-                        FCI_CUDA(h, multidot(Vk(0), 1, Vk(1), dots));
-                        k_negate<<<1, 64, 0, s>>>(dots, 1);
-                        FCI_CUDA(h, lincomb(Vk(0), 1, dots, 1.0, Vk(1), 1));
-                        FCI_CUDA(h, lincomb(Sk(0), 1, dots, 1.0, Sk(1), 1));
+                        FCI_CUDA(h, multidot(Vk(0), 1, Vk(1), dots, DOT_NEGATE));
+                        FCI_CUDA(h, lincomb(Vk(0), 1, dots, Vk(1), 1, nullptr, Sk(0), Sk(1)));
                     }
-                    k_norm2<<<vb, RED_THREADS, 0, s>>>(Vk(1), nreal, partial);
-                    k_reduce_norm<<<1, 32, 0, s>>>(partial, vb, nrm);
+                    norm2(Vk(1), nrm);
                     double pn2 = 0.0;
                     FCI_CUDA(h, cudaMemcpyAsync(&pn2, nrm, 8, cudaMemcpyDeviceToHost, s));
                     FCI_CUDA(h, cudaStreamSynchronize(s));
                     if (sqrt(pn2) > 1e-10) {
-                        k_scale<<<vb, RED_THREADS, 0, s>>>(Vk(1), nreal, nrm);
-                        k_scale<<<vb, RED_THREADS, 0, s>>>(Sk(1), nreal, nrm);
+                        scale(Vk(1), Vk(1), nrm);
+                        scale(Sk(1), Sk(1), nrm);
                         knew = 2;
                     }
                 }
@@ -786,30 +1008,19 @@ struct fci_davidson_state {
                 // collapse to the ground-state Ritz vector (it must stay in the subspace for
                 // the final E_0) and the current second Ritz vector orthogonalised against it;
                 // c_prev / sc_prev are free in this phase and hold the ground state meanwhile
-                {
-                    const int m = cplx ? 2 * k : k;
-                    k_jacobi<<<1, JAC_THREADS, 2 * m * (m + 1) * sizeof(double), s>>>(Hs, k, cplx ? 1 : 0, 0, y, scal);
-                }
-                FCI_CUDA(h, lincomb(V, k, y, 1.0, cp, 0));
-                FCI_CUDA(h, lincomb(S, k, y, 1.0, scp, 0));
-                FCI_CUDA(h, cudaMemcpyAsync(Vk(0), cp, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
-                FCI_CUDA(h, cudaMemcpyAsync(Sk(0), scp, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
-                k_norm2<<<vb, RED_THREADS, 0, s>>>(Vk(0), nreal, partial);
-                k_reduce_norm<<<1, 32, 0, s>>>(partial, vb, nrm);
-                k_scale<<<vb, RED_THREADS, 0, s>>>(Vk(0), nreal, nrm);
-                k_scale<<<vb, RED_THREADS, 0, s>>>(Sk(0), nreal, nrm);
+                ritz_pair(0);
+                FCI_CUDA(h, lincomb(V, k, y, cp, 0, nrm, S, scp));
+                scale(cp, Vk(0), nrm);
+                scale(scp, Sk(0), nrm);
                 FCI_CUDA(h, cudaMemcpyAsync(Vk(1), c, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
                 FCI_CUDA(h, cudaMemcpyAsync(Sk(1), sc, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
                 for (int pass = 0; pass < 2; ++pass) {
-                    FCI_CUDA(h, multidot(Vk(0), 1, Vk(1), dots));
-                    k_negate<<<1, 64, 0, s>>>(dots, 1);
-                    FCI_CUDA(h, lincomb(Vk(0), 1, dots, 1.0, Vk(1), 1));
-                    FCI_CUDA(h, lincomb(Sk(0), 1, dots, 1.0, Sk(1), 1));
+                    FCI_CUDA(h, multidot(Vk(0), 1, Vk(1), dots, DOT_NEGATE));
+                    FCI_CUDA(h, lincomb(Vk(0), 1, dots, Vk(1), 1, nullptr, Sk(0), Sk(1)));
                 }
-                k_norm2<<<vb, RED_THREADS, 0, s>>>(Vk(1), nreal, partial);
-                k_reduce_norm<<<1, 32, 0, s>>>(partial, vb, nrm);
-                k_scale<<<vb, RED_THREADS, 0, s>>>(Vk(1), nreal, nrm);
-                k_scale<<<vb, RED_THREADS, 0, s>>>(Sk(1), nreal, nrm);
+                norm2(Vk(1), nrm);
+                scale(Vk(1), Vk(1), nrm);
+                scale(Sk(1), Sk(1), nrm);
                 FCI_CUDA(h, cudaGetLastError());
                 FCI_CUDA(h, cudaMemsetAsync(Hs, 0, 2 * KMAX * KMAX * 8, s));
                 for (int jj = 0; jj < 2; ++jj)
@@ -818,18 +1029,11 @@ struct fci_davidson_state {
             }
             // two rounds of classical Gram-Schmidt against V[0..k)
             for (int round = 0; round < 2; ++round) {
-                FCI_CUDA(h, multidot(V, k, t, dots));
-                k_negate<<<1, 64, 0, s>>>(dots, k);
-                FCI_CUDA(h, lincomb(V, k, dots, 1.0, t, 1));
+                FCI_CUDA(h, multidot(V, k, t, dots, DOT_NEGATE));
+                FCI_CUDA(h, lincomb(V, k, dots, t, 1, round ? nrm : nullptr));
             }
-            k_norm2<<<vb, RED_THREADS, 0, s>>>(t, nreal, partial);
-            k_reduce_norm<<<1, 32, 0, s>>>(partial, vb, nrm);
             double tn2 = 0.0;
             FCI_CUDA(h, cudaMemcpyAsync(&tn2, nrm, 8, cudaMemcpyDeviceToHost, s));
-            if (!gap_phase) {
-                FCI_CUDA(h, cudaMemcpyAsync(cp, c, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
-                FCI_CUDA(h, cudaMemcpyAsync(scp, sc, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
-            }
             FCI_CUDA(h, cudaStreamSynchronize(s));
             if (!gap_phase) {
                 have_prev = true;
@@ -840,8 +1044,12 @@ struct fci_davidson_state {
                 done = true;
                 break;
             }
-            k_scale<<<vb, RED_THREADS, 0, s>>>(t, nreal, nrm);
-            FCI_CUDA(h, cudaMemcpyAsync(Vk(k), t, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
+            if (!gap_phase) {  // this Ritz pair is the next step's previous one
+                std::swap(c, cp);
+                std::swap(sc, scp);
+            }
+            scale(t, Vk(k), nrm);
+            FCI_CUDA(h, cudaGetLastError());
             return ask(REQ_APPEND, Vk(k), Sk(k));
         }
         return FCI_OK;
@@ -851,13 +1059,10 @@ struct fci_davidson_state {
     // gamma_0^- = (E_1 - ||r_1||) - E_0 and |dE| <= ||r_0||^2 / gamma_0^- (gap theorem).
     int finish_gap() {
         dav_scalars hs{};
-        const int m = cplx ? 2 * k : k;
-        k_jacobi<<<1, JAC_THREADS, 2 * m * (m + 1) * sizeof(double), s>>>(Hs, k, cplx ? 1 : 0, 0, y, scal);
-        FCI_CUDA(h, lincomb(V, k, y, 1.0, c, 0));
-        FCI_CUDA(h, lincomb(S, k, y, 1.0, sc, 0));
-        if (cplx) k_residual<true><<<vb, RED_THREADS, 0, s>>>(c, sc, cp, false, diag, scal, n, t, partial);
-        else k_residual<false><<<vb, RED_THREADS, 0, s>>>(c, sc, cp, false, diag, scal, n, t, partial);
-        k_reduce_residual<<<1, 32, 0, s>>>(partial, vb, scal);
+        ritz_pair(0);
+        FCI_CUDA(h, lincomb(V, k, y, c, 0, nullptr, S, sc));
+        ritz = c;
+        residual(false);
         FCI_CUDA(h, cudaGetLastError());
         FCI_CUDA(h, cudaMemcpyAsync(&hs, scal, sizeof hs, cudaMemcpyDeviceToHost, s));
         FCI_CUDA(h, cudaStreamSynchronize(s));
@@ -869,7 +1074,7 @@ struct fci_davidson_state {
     }
 
     int finish(void *C_out, double *energy, fci_davidson_log *lg) {
-        if (C_out) FCI_CUDA(h, cudaMemcpyAsync(C_out, c, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
+        if (C_out) FCI_CUDA(h, cudaMemcpyAsync(C_out, ritz, (size_t)n * esz, cudaMemcpyDeviceToDevice, s));
         FCI_CUDA(h, cudaStreamSynchronize(s));
         if (energy) *energy = E_prev;
         if (lg) {
