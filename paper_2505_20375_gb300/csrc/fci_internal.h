@@ -249,9 +249,20 @@ int cz_check(fci_context *h, int n_slices);
 size_t cz_workspace_bytes(const fci_context *h, int n_slices);
 int cz_sigma(fci_context *h, const double *C, double *sigma, int n_slices, void *ws, size_t ws_bytes, cudaStream_t s);
 
+// fixed_point.cu: C in fixed point for the split paths.  The scalars of a split sigma (in its
+// workspace) are cleared by the launch: the largest |C| as bits, the shift of C, the status
+// of the contraction (FCI_ERR_TIMEOUT).
+struct fci_split_scalars {
+    unsigned long long maxbits;
+    int shC, pad;
+    int status, pad2;
+};
+cudaError_t launch_fixed_point(const double *C, int64_t n, int top, fci_split_scalars *sc, int64_t *Cint,
+                               cudaStream_t st);
+cudaError_t launch_fixed_point_pairs(const double *C, int64_t n, int top, fci_split_scalars *sc, int32_t *Cint,
+                                     cudaStream_t st);
+
 // ozaki.cu
-cudaError_t launch_to_fixed64(const double *C, int64_t n, int s, unsigned long long *maxbits, int64_t *Cint, int *shC,
-                              cudaStream_t st);
 int oz_prepare_G(fci_context *h, int n_slices);
 int oz_tune_candidates(const fci_context *h, int n_slices, int *nt, int *path, int max);  // configurations that fit
 void oz_set_config(fci_context *h, int n_slices, int nt, int path);                     // nt = 0: default

@@ -405,27 +405,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_contract(const __grid_cons
 
 // ------------------------------------------------------------- helper kernels
 
-__global__ void k_absmax_bits(const double *__restrict__ x, int64_t n, unsigned long long *__restrict__ out) {
-    unsigned long long m = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)__double_as_longlong(x[i]) & 0x7FFFFFFFFFFFFFFFull);
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
-// C_int = round(C 2^{sh_C}), sh_C = 8 s - 3 - e_C with max|C| < 2^{e_C}: |C_int| < 2^{8s-3}
-// and |D_int| < 2^{8s-2}, inside the range of s balanced digits.
-__global__ void k_to_fixed(const double *__restrict__ C, int64_t n, int s,
-                           const unsigned long long *__restrict__ maxbits, int64_t *__restrict__ Cint,
-                           int *__restrict__ shC) {
-    const unsigned long long mb = *maxbits;
-    const int e = mb ? (int)((mb >> 52) & 0x7FF) - 1022 : 0;  // max|C| < 2^e (normal numbers)
-    const int sh = 8 * s - 3 - e;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *shC = sh;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        Cint[i] = __double2ll_rn(scalbn(C[i], sh));
-}
-
 // sigma_I = scale * sum over the replacements of I of sign * E_int[pq, K] + e_core C_I, in
 // int64.  Thread = beta string ib (consecutive threads, consecutive determinants), looping
 // over alpha strings; pairs are taken 8 at a time, their 16 table entries loaded first,
@@ -650,13 +629,15 @@ int oz_ring(int s, int KC, int nt) {
 // environment (32 or 64), else 64.
 // Contraction path for s slices: 1 = two-pass (digit image of D in HBM, then the
 // bulk-copy GEMM), 0 = fused producer kernel.  The tuner's choice, else FCI_OZ_PATH
-// ("gemm" / "fused") from the environment, else two-pass from 2^20 determinants on (where
-// it was measured faster at every slice count) and fused below (small problems, which
-// also share grouped launches).
+// ("gemm" / "fused") from the environment, else two-pass from 2^13 determinants on (faster
+// there at every slice count: us per sigma, fused / two-pass, 4,900 determinants (8 orbitals)
+// s = 3 32 / 30, s = 6 35 / 32; 15,876 37 / 33, 45 / 38; 63,504 70 / 55, 94 / 71; 853,776
+// 731 / 494, 1028 / 669) and fused below, where both are a chain of launches and small
+// problems share one launch of a group.
 int oz_path(const fci_context *h, int s) {
     if (s >= 2 && s <= 8 && h->oz_tuned_nt[s]) return h->oz_tuned_path[s];
     if (const char *env = getenv("FCI_OZ_PATH")) return strcmp(env, "gemm") == 0 ? 1 : 0;
-    return (h->ndet >= ((int64_t)1 << 20) && s <= 7) ? 1 : 0;
+    return (h->ndet >= ((int64_t)1 << 13) && s <= 7) ? 1 : 0;
 }
 int oz_nt(const fci_context *h, int s) {
     if (s >= 2 && s <= 8 && h->oz_tuned_nt[s]) return h->oz_tuned_nt[s];
@@ -668,16 +649,6 @@ int oz_nt(const fci_context *h, int s) {
 }
 
 }  // namespace
-
-// Fixed point of C for the split paths with int64 digits: maxbits (zeroed by the caller)
-// receives the largest |C| bit pattern, shC the shift, Cint = round(C 2^{sh_C}).
-cudaError_t launch_to_fixed64(const double *C, int64_t n, int s, unsigned long long *maxbits, int64_t *Cint, int *shC,
-                              cudaStream_t st) {
-    const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 152 * 8));
-    k_absmax_bits<<<nb, 256, 0, st>>>(C, n, maxbits);
-    k_to_fixed<<<nb, 256, 0, st>>>(C, n, s, maxbits, Cint, shC);
-    return cudaGetLastError();
-}
 
 // IEEE binary16 encoding of an integer |d| <= 1024 (exact).
 static uint16_t half_bits_of_small_int(int d) {
@@ -814,16 +785,11 @@ static int oz_prepare_job(fci_context *h, const double *C, int s, void *ws, cuda
     p += al256((size_t)N * 8);
     int64_t *E = (int64_t *)p;
     p += al256((size_t)((N + OZ_TILE - 1) / OZ_TILE) * h->npair * OZ_TILE * 8);
-    unsigned long long *maxbits = (unsigned long long *)p;
-    int *shC = (int *)(p + 8);
-    int *status = (int *)(p + 16);
+    fci_split_scalars *sc = (fci_split_scalars *)p;
+    int *shC = &sc->shC, *status = &sc->status;
     {
         phase_scope ps(h, st, FCI_PHASE_OTHER, 2);
-        FCI_CUDA(h, cudaMemsetAsync(p, 0, 256, st));
-        const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(N, 256), 152 * 8);
-        k_absmax_bits<<<nb, 256, 0, st>>>(C, N, maxbits);
-        k_to_fixed<<<nb, 256, 0, st>>>(C, N, s, maxbits, Cint, shC);
-        FCI_CUDA(h, cudaGetLastError());
+        FCI_CUDA(h, launch_fixed_point(C, N, 8 * s - 3, sc, Cint, st));
     }
     prm.N = N;
     prm.nsa = h->nsa;
@@ -915,14 +881,11 @@ static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int
     p += al256((size_t)n_nt * OZG_M * OZG_N * 8);
     // the misc block sits at the end of the larger of the two layouts
     char *misc = (char *)ws + (oz_workspace_bytes(h, s) - 256);
-    unsigned long long *maxbits = (unsigned long long *)misc;
-    int *shC = (int *)(misc + 8), *status = (int *)(misc + 16);
+    fci_split_scalars *sc = (fci_split_scalars *)misc;
+    int *shC = &sc->shC, *status = &sc->status;
     {
         phase_scope ps(h, st, FCI_PHASE_GATHER, 3);
-        FCI_CUDA(h, cudaMemsetAsync(misc, 0, 256, st));
-        const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(N, 256), 152 * 8);
-        k_absmax_bits<<<nb, 256, 0, st>>>(C, N, maxbits);
-        k_to_fixed<<<nb, 256, 0, st>>>(C, N, s, maxbits, Cint, shC);
+        FCI_CUDA(h, launch_fixed_point(C, N, 8 * s - 3, sc, Cint, st));
         const size_t row_smem = (size_t)h->nsb * 8 + (size_t)h->npair_pad * 4;  // one C row + its alpha entries
         if (row_smem > OZ_SMEM_MAX) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split precision: %lld beta strings", (long long)h->nsb);
         const unsigned gr = (unsigned)h->nsa;  // one block per alpha string: no tail of unequal row counts

@@ -104,27 +104,6 @@ __device__ __forceinline__ int cz_sign(uint32_t S, int a, int b) {
     return __popc(S & between) & 1;
 }
 
-__global__ void k_cz_absmax(const double *__restrict__ x, int64_t n, unsigned long long *__restrict__ out) {
-    unsigned long long m = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)__double_as_longlong(x[i]) & 0x7FFFFFFFFFFFFFFFull);
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
-// C_int = round(C 2^{sh_C}) for real and imaginary parts, sh_C = 7 s - 3 - e_C with every
-// |part| < 2^{e_C}: |C_int| < 2^{7s-3}, inside the range of s balanced base-128 digits.
-__global__ void k_cz_to_fixed(const double *__restrict__ C, int64_t n2, int s,
-                              const unsigned long long *__restrict__ maxbits, int64_t *__restrict__ Cint,
-                              int *__restrict__ shC) {
-    const unsigned long long mb = *maxbits;
-    const int e = mb ? (int)((mb >> 52) & 0x7FF) - 1022 : 0;
-    const int sh = 7 * s - 3 - e;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *shC = sh;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x)
-        Cint[i] = __double2ll_rn(scalbn(C[i], sh));
-}
-
 // Two balanced base-128 digits (bits 7j .. 7j+6 of the biased values) as an f16x2 word:
 // 0x6400 | d encodes 1024 + d exactly, and one packed subtraction of 1024 + 64 leaves
 // d - 64 in [-64, 63].
@@ -355,14 +334,11 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
     p += al256((size_t)n_nt * M_real * CZ_N * 8);
     ulonglong2 *masks = (ulonglong2 *)p;
     p += al256((size_t)n_nt * sizeof(ulonglong2));
-    unsigned long long *maxbits = (unsigned long long *)p;
-    int *shC = (int *)(p + 8), *status = (int *)(p + 16);
+    fci_split_scalars *sc = (fci_split_scalars *)p;
+    int *shC = &sc->shC, *status = &sc->status;
     {
         phase_scope ps(h, st, FCI_PHASE_GATHER, 3);
-        FCI_CUDA(h, cudaMemsetAsync(p, 0, 256, st));
-        const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(2 * h->ndet, 256), 152 * 8);
-        k_cz_absmax<<<nb, 256, 0, st>>>(C, 2 * h->ndet, maxbits);
-        k_cz_to_fixed<<<nb, 256, 0, st>>>(C, 2 * h->ndet, s, maxbits, Cint, shC);
+        FCI_CUDA(h, launch_fixed_point(C, 2 * h->ndet, 7 * s - 3, sc, Cint, st));
         switch (s) {
 #define CZ_SPLIT(S_) case S_: k_cz_split<S_><<<(unsigned)n_nt, 256, 0, st>>>(bl, h->ndet, h->d_str_a, h->d_binom, Cint, Dimg, masks); break;
             CZ_SPLIT(2) CZ_SPLIT(3) CZ_SPLIT(4) CZ_SPLIT(5) CZ_SPLIT(6) CZ_SPLIT(7) CZ_SPLIT(8)

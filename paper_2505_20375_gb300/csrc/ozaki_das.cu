@@ -471,32 +471,6 @@ __global__ void k_dz_rep(const int32_t *__restrict__ pairtab, int64_t ns, int ro
     }
 }
 
-__global__ void k_dz_absmax(const double *__restrict__ x, int64_t n, unsigned long long *__restrict__ out) {
-    unsigned long long m = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)__double_as_longlong(x[i]) & 0x7FFFFFFFFFFFFFFFull);
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
-// C_int = round(C 2^{sh_C}), sh_C = 8 s - 3 - e_C with max|C| < 2^{e_C}: |C_int| < 2^{8s-3}
-// (< 2^21 for s <= 3, so int32 holds it), stored as signed pairs (C_int, -C_int) per
-// determinant followed by one zero pair at index n: the producers read the value of a
-// move with its sign, or zero for an absent move, with one load and no arithmetic.
-__global__ void k_dz_to_fixed(const double *__restrict__ C, int64_t n, int s,
-                              const unsigned long long *__restrict__ maxbits, int32_t *__restrict__ Cint,
-                              int *__restrict__ shC) {
-    const unsigned long long mb = *maxbits;
-    const int e = mb ? (int)((mb >> 52) & 0x7FF) - 1022 : 0;
-    const int sh = 8 * s - 3 - e;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *shC = sh;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *(int2 *)(Cint + 2 * n) = make_int2(0, 0);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = (int32_t)__double2ll_rn(scalbn(C[i], sh));
-        *(int2 *)(Cint + 2 * i) = make_int2(v, -v);
-    }
-}
-
 struct DzScatter {
     int64_t n_det, a0, len;
     int nla, nlb;
@@ -864,15 +838,11 @@ int dz_prepare_job(fci_context *h, const double *C, double *sigma, int s, void *
         j.acc = (int64_t *)p;
         p += al256((size_t)L.n_det * 8);
     }
-    unsigned long long *maxbits = (unsigned long long *)p;
-    j.shC = (int *)(p + 8);
-    j.status = (int *)(p + 16);
+    fci_split_scalars *sc = (fci_split_scalars *)p;
+    j.shC = &sc->shC;
+    j.status = &sc->status;
     phase_scope ps(h, st, FCI_PHASE_OTHER, 2);
-    FCI_CUDA(h, cudaMemsetAsync(p, 0, 256, st));
-    const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(L.n_det, 256), 152 * 8);
-    k_dz_absmax<<<nb, 256, 0, st>>>(C, L.n_det, maxbits);
-    k_dz_to_fixed<<<nb, 256, 0, st>>>(C, L.n_det, s, maxbits, j.Cint, j.shC);
-    FCI_CUDA(h, cudaGetLastError());
+    FCI_CUDA(h, launch_fixed_point_pairs(C, L.n_det, 8 * s - 3, sc, j.Cint, st));
     return FCI_OK;
 }
 
@@ -1341,12 +1311,11 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
         acc = (int64_t *)p;
         p += al256((size_t)L.n_det * 8);
     }
-    unsigned long long *maxbits = (unsigned long long *)p;
-    int *shC = (int *)(p + 8), *status = (int *)(p + 16);
+    fci_split_scalars *scal = (fci_split_scalars *)p;
+    int *shC = &scal->shC, *status = &scal->status;
     {
         phase_scope ps(h, st, FCI_PHASE_OTHER, 2);
-        FCI_CUDA(h, cudaMemsetAsync(p, 0, 256, st));
-        FCI_CUDA(h, launch_to_fixed64(C, L.n_det, s, maxbits, Cint, shC, st));
+        FCI_CUDA(h, launch_fixed_point(C, L.n_det, 8 * s - 3, scal, Cint, st));
     }
     const size_t npab = (size_t)L.n_pat_a * L.n_pat_b;
     DgSplit sp;
