@@ -21,11 +21,14 @@
 //   3. every column J emits its single replacements L inside the target space: the
 //      structural support of sigma, made distinct by a second hash table and sorted
 //      (radix sort on the address), which is the compressed output order;
-//   4. sigma_L = sum_pq <L|E_pq|J> E[pq, J] + e_core C_L for every L of the support,
-//      gathering over L's replacements in pair order (alpha then beta), looking each J up
-//      in the first table (absent J have E = 0): the arithmetic and its order are those of
-//      the dense FP64 DAS path, so the result equals the dense sigma on the support and
-//      the dense sigma is zero elsewhere.
+//   4. sigma_L = sum_pq <L|E_pq|J> E[pq, J] + e_core C_L for every L of the support, in pair
+//      order (alpha then beta; absent J have E = 0): the arithmetic and its order are those
+//      of the dense FP64 DAS path, so the result equals the dense sigma on the support and
+//      the dense sigma is zero elsewhere.  The columns J that L reaches share its beta
+//      string (an alpha move) or its alpha string (a beta move), so they are found on the
+//      lists of columns per string, a few entries long for nearly every L; only where a
+//      list is long or many columns match are L's replacements walked, each J looked up in
+//      the first table.
 // The pair tables are read string-major (one string's row contiguous; copies built on the
 // first call and kept by the handle).  Hash tables use open addressing with linear
 // probing over a power-of-two capacity of at least twice the largest number of keys, so no
@@ -97,6 +100,10 @@ struct CsArgs {
     uint64_t hj_mask;
     int64_t *j_addr;                 // [n1]: the J of each column
     uint32_t *bm_a, *bm_b;           // bit A (B) set: some column has alpha (beta) string A (B)
+    const uint64_t *str_a, *str_b;   // string masks
+    int32_t *head_a, *head_b;        // [n_str]: first column with this alpha (beta) string, -1: none
+    int2 *node_a, *node_b;           // [n1]: next column of the same alpha (beta) string, and the
+                                     // column's other string (mask)
     double *D, *E;                   // [n_pair][ldd]
     int64_t ldd;
     unsigned long long *hl;          // target determinants L of the support
@@ -171,21 +178,23 @@ __device__ __forceinline__ bool cs_coef(const CsArgs &a, int64_t K, double &v) {
 
 // D[pair, column] for every column J and pair: the alpha source and the beta source of J
 // under the pair, each looked up among the nonzero coefficients (Algorithm 1's
-// intersection of J's excitation list with the compressed vector).
+// intersection of J's excitation list with the compressed vector).  One warp per column, so
+// that J is decoded once.
 __global__ void __launch_bounds__(256) k_cs_gather(const __grid_constant__ CsArgs a, int64_t n1) {
-    const int64_t total = n1 * a.npair;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = t / a.npair;
-        const int pp = (int)(t - j * a.npair);
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < n1; j += nw) {
         int32_t A, B;
         int pb;
         das_strings(a.d, a.n_cat_int, a.j_addr[j], A, B, pb);
-        double d = 0.0, v;
-        const int32_t ea = __ldg(a.pair_a + (int64_t)A * a.ldp + pp);
-        if (ea >= 0 && cs_coef(a, das_addr(a.d, ea >> 1, B), v)) d += (ea & 1) ? -v : v;
-        const int32_t eb = __ldg(a.pair_b + (int64_t)B * a.ldp + pp);
-        if (eb >= 0 && cs_coef(a, das_addr(a.d, A, eb >> 1), v)) d += (eb & 1) ? -v : v;
-        a.D[(int64_t)pp * a.ldd + j] = d;
+        for (int pp = lane; pp < a.npair; pp += 32) {
+            double d = 0.0, v;
+            const int32_t ea = __ldg(a.pair_a + (int64_t)A * a.ldp + pp);
+            if (ea >= 0 && cs_coef(a, das_addr(a.d, ea >> 1, B), v)) d += (ea & 1) ? -v : v;
+            const int32_t eb = __ldg(a.pair_b + (int64_t)B * a.ldp + pp);
+            if (eb >= 0 && cs_coef(a, das_addr(a.d, A, eb >> 1), v)) d += (eb & 1) ? -v : v;
+            a.D[(int64_t)pp * a.ldd + j] = d;
+        }
     }
 }
 
@@ -244,8 +253,9 @@ __global__ void k_cs_transpose(const int32_t *__restrict__ src, int64_t R, int64
     }
 }
 
-// The alpha and beta strings of every column, as bitmaps (a sigma entry looks a candidate
-// column up only if both of its strings occur in some column).
+// The alpha and beta strings of every column, as bitmaps (a walk of the replacements looks a
+// candidate column up only if both of its strings occur in some column) and as lists of
+// columns per string (in any order: the terms found on them are sorted).
 __global__ void k_cs_mark(const __grid_constant__ CsArgs a, int64_t n1) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n1; j += (int64_t)gridDim.x * blockDim.x) {
         int32_t A, B;
@@ -253,20 +263,54 @@ __global__ void k_cs_mark(const __grid_constant__ CsArgs a, int64_t n1) {
         das_strings(a.d, a.n_cat_int, a.j_addr[j], A, B, pb);
         atomicOr(a.bm_a + (A >> 5), 1u << (A & 31));
         atomicOr(a.bm_b + (B >> 5), 1u << (B & 31));
+        a.node_a[j] = make_int2(atomicExch(a.head_a + A, (int32_t)j), (int)(uint32_t)a.str_b[B]);
+        a.node_b[j] = make_int2(atomicExch(a.head_b + B, (int32_t)j), (int)(uint32_t)a.str_a[A]);
     }
 }
 
 __device__ __forceinline__ bool bit(const uint32_t *__restrict__ bm, int32_t i) { return (__ldg(bm + (i >> 5)) >> (i & 31)) & 1u; }
 
-// Distinct keys of a table get consecutive columns.
-__global__ void k_cs_compact(unsigned long long *keys, int32_t *cols, uint64_t cap, int64_t *addr,
-                             unsigned long long *counter) {
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < cap; p += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned long long k = keys[p];
-        if (k == HT_EMPTY) continue;
-        const unsigned long long c = atomicAdd(counter, 1ull);
-        if (cols) cols[p] = (int32_t)c;
-        addr[c] = (int64_t)k;
+// Distinct keys of a table get consecutive columns.  A block takes 2,048 slots at a time
+// (8 per thread) and claims the columns of its keys with one addition to the counter (one
+// per key, all to the same word, took ten times as long as reading the table).
+__global__ void __launch_bounds__(256) k_cs_compact(const unsigned long long *__restrict__ keys, int32_t *__restrict__ cols,
+                                                    uint64_t cap, int64_t *__restrict__ addr,
+                                                    unsigned long long *__restrict__ counter) {
+    __shared__ unsigned wsum[8];
+    __shared__ unsigned long long base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint64_t p0 = blockIdx.x * (uint64_t)2048; p0 < cap; p0 += (uint64_t)gridDim.x * 2048) {
+        unsigned long long k[8];  // the capacity is a power of two of at least 1,024
+        unsigned n = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint64_t p = p0 + (uint64_t)i * 256 + threadIdx.x;
+            k[i] = p < cap ? keys[p] : HT_EMPTY;
+            n += k[i] != HT_EMPTY;
+        }
+        unsigned x = n;  // inclusive scan over the warp
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        unsigned before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) before += wsum[w];
+            all += wsum[w];
+        }
+        if (threadIdx.x == 0 && all) base = atomicAdd(counter, (unsigned long long)all);
+        __syncthreads();
+        unsigned long long c = base + before + x - n;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (k[i] == HT_EMPTY) continue;
+            if (cols) cols[p0 + (uint64_t)i * 256 + threadIdx.x] = (int32_t)c;
+            addr[c++] = (int64_t)k[i];
+        }
+        __syncthreads();  // wsum and base are rewritten by the next slots
     }
 }
 
@@ -289,6 +333,82 @@ __global__ void __launch_bounds__(256) k_cs_support(const __grid_constant__ CsAr
 }
 
 // Step 4: sigma on the sorted support, in the dense DAS path's order of terms.
+
+// The sum over L's replacements, each column looked up in the table of columns.
+__device__ __noinline__ double cs_walk(const CsArgs &a, int32_t A, int32_t B) {
+    double acc = 0.0;
+    const int4 *ra = reinterpret_cast<const int4 *>(a.pair_a + (int64_t)A * a.ldp);
+    const int4 *rb = reinterpret_cast<const int4 *>(a.pair_b + (int64_t)B * a.ldp);
+    // an alpha move keeps B and a beta move keeps A: no column has them, no lookup
+    const bool try_a = bit(a.bm_b, B), try_b = bit(a.bm_a, A);
+    const int4 none = make_int4(-1, -1, -1, -1);
+    for (int p4 = 0; p4 < a.npair && (try_a || try_b); p4 += 4) {  // four pairs per 16-byte load of a row
+        const int4 va = try_a ? __ldg(ra + p4 / 4) : none, vb = try_b ? __ldg(rb + p4 / 4) : none;
+        const int32_t ea4[4] = {va.x, va.y, va.z, va.w}, eb4[4] = {vb.x, vb.y, vb.z, vb.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double *Ep = a.E + (int64_t)(p4 + k) * a.ldd;  // rows past n_pair hold -1
+            const int32_t ea = ea4[k];
+            if (ea >= 0 && bit(a.bm_a, ea >> 1)) {
+                const int64_t J = das_addr(a.d, ea >> 1, B);
+                const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+                if (col >= 0) {
+                    const double e = Ep[col];
+                    acc += (ea & 1) ? -e : e;
+                }
+            }
+            const int32_t eb = eb4[k];
+            if (eb >= 0 && bit(a.bm_b, eb >> 1)) {
+                const int64_t J = das_addr(a.d, A, eb >> 1);
+                const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+                if (col >= 0) {
+                    const double e = Ep[col];
+                    acc += (eb & 1) ? -e : e;
+                }
+            }
+        }
+    }
+    return acc;
+}
+
+// Terms of L found on one list: the columns whose string `mask` on the list's other spin is
+// one move from S.  Each goes into the ascending keys (2 pair + spin, sign) with its column.
+// False if a term does not fit, the list is longer than a walk of the replacements, or L
+// itself is a column (its diagonal terms are many).
+constexpr int CS_TERMS = 8;      // terms kept per L
+constexpr int CS_MAX_HOPS = 320; // list entries visited per spin
+__device__ __forceinline__ bool cs_list(const int2 *__restrict__ node, int32_t c, uint32_t S, int spin,
+                                        uint32_t (&key)[CS_TERMS], int32_t (&col)[CS_TERMS], int &n) {
+    for (int hop = 0; c >= 0; ++hop) {
+        if (hop >= CS_MAX_HOPS) return false;
+        const int2 nd = __ldg(node + c);
+        const uint32_t x = S ^ (uint32_t)nd.y;
+        const int d = __popc(x);
+        if (d == 0) return false;
+        if (d == 2) {
+            if (n == CS_TERMS) return false;
+            const int hi = 31 - __clz(x), lo = __ffs(x) - 1;
+            const uint32_t between = ((1u << hi) - 1u) & ~((2u << lo) - 1u);
+            uint32_t k = ((uint32_t)(hi * (hi + 1) / 2 + lo) << 2) | (uint32_t)(spin << 1) | (__popc(S & between) & 1u);
+            int32_t v = c;
+#pragma unroll
+            for (int i = 0; i < CS_TERMS; ++i) {  // insertion, the entries past n being larger than any key
+                if (k < key[i]) {
+                    const uint32_t tk = key[i];
+                    const int32_t tv = col[i];
+                    key[i] = k;
+                    col[i] = v;
+                    k = tk;
+                    v = tv;
+                }
+            }
+            ++n;
+        }
+        c = nd.x;
+    }
+    return true;
+}
+
 __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
                                                   int64_t n2, double *__restrict__ out_val) {
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n2; o += (int64_t)gridDim.x * blockDim.x) {
@@ -297,36 +417,25 @@ __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs
         int pb;
         das_strings(a.d, a.d.n_cat, L, A, B, pb);
         double acc = 0.0;
-        const int4 *ra = reinterpret_cast<const int4 *>(a.pair_a + (int64_t)A * a.ldp);
-        const int4 *rb = reinterpret_cast<const int4 *>(a.pair_b + (int64_t)B * a.ldp);
-        // an alpha move keeps B and a beta move keeps A: no column has them, no lookup
-        const bool try_a = bit(a.bm_b, B), try_b = bit(a.bm_a, A);
-        const int4 none = make_int4(-1, -1, -1, -1);
-        for (int p4 = 0; p4 < a.npair && (try_a || try_b); p4 += 4) {  // four pairs per 16-byte load of a row
-            const int4 va = try_a ? __ldg(ra + p4 / 4) : none, vb = try_b ? __ldg(rb + p4 / 4) : none;
-            const int32_t ea4[4] = {va.x, va.y, va.z, va.w}, eb4[4] = {vb.x, vb.y, vb.z, vb.w};
+        uint32_t key[CS_TERMS];
+        int32_t col[CS_TERMS];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double *Ep = a.E + (int64_t)(p4 + k) * a.ldd;  // rows past n_pair hold -1
-                const int32_t ea = ea4[k];
-                if (ea >= 0 && bit(a.bm_a, ea >> 1)) {
-                    const int64_t J = das_addr(a.d, ea >> 1, B);
-                    const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
-                    if (col >= 0) {
-                        const double e = Ep[col];
-                        acc += (ea & 1) ? -e : e;
-                    }
-                }
-                const int32_t eb = eb4[k];
-                if (eb >= 0 && bit(a.bm_b, eb >> 1)) {
-                    const int64_t J = das_addr(a.d, A, eb >> 1);
-                    const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
-                    if (col >= 0) {
-                        const double e = Ep[col];
-                        acc += (eb & 1) ? -e : e;
-                    }
-                }
-            }
+        for (int i = 0; i < CS_TERMS; ++i) {
+            key[i] = ~0u;
+            col[i] = 0;
+        }
+        int n = 0;
+        if (cs_list(a.node_b, __ldg(a.head_b + B), (uint32_t)__ldg(a.str_a + A), 0, key, col, n) &&
+            cs_list(a.node_a, __ldg(a.head_a + A), (uint32_t)__ldg(a.str_b + B), 1, key, col, n)) {
+            double e[CS_TERMS];
+#pragma unroll
+            for (int i = 0; i < CS_TERMS; ++i)
+                e[i] = key[i] != ~0u ? __ldg(a.E + (int64_t)(key[i] >> 2) * a.ldd + col[i]) : 0.0;
+#pragma unroll
+            for (int i = 0; i < CS_TERMS; ++i)
+                if (key[i] != ~0u) acc += (key[i] & 1u) ? -e[i] : e[i];
+        } else {
+            acc = cs_walk(a, A, B);
         }
         // C_L from the sorted nonzero addresses (binary search)
         double cl = 0.0;
@@ -363,57 +472,59 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint64_t *__restri
     }
 }
 
-// Exclusive scan of m counts in one block of 1024 threads, 8192 counts at a time: each
-// thread loads 8 consecutive counts (issued together) and scans them, a scan of the 1024
-// thread totals (inside each warp, then over the 32 warp totals) gives each thread its
-// offset, plus the running total of the chunks before.
-__global__ void __launch_bounds__(1024) k_rs_scan(unsigned long long *__restrict__ c, int64_t m) {
-    constexpr int IPT = 8;
-    __shared__ unsigned long long wsum[32];
+// Exclusive scan of each digit's counts over the tiles, one block per digit, and the digit's
+// total; the scatter adds the totals of the smaller digits.
+__global__ void __launch_bounds__(RS_THREADS) k_rs_scan(unsigned long long *__restrict__ counts, int64_t ntiles,
+                                                        unsigned long long *__restrict__ totals) {
+    __shared__ unsigned long long wsum[RS_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long *c = counts + (int64_t)blockIdx.x * ntiles;
     unsigned long long carry = 0;  // the same in every thread
-    for (int64_t base = 0; base < m; base += 1024 * IPT) {
-        const int64_t i0 = base + (int64_t)threadIdx.x * IPT;
-        unsigned long long v[IPT], tot = 0;
-#pragma unroll
-        for (int k = 0; k < IPT; ++k) v[k] = i0 + k < m ? c[i0 + k] : 0ull;
-#pragma unroll
-        for (int k = 0; k < IPT; ++k) {
-            const unsigned long long t = v[k];
-            v[k] = tot;  // exclusive inside the thread
-            tot += t;
-        }
-        unsigned long long x = tot;  // inclusive scan of the thread totals inside the warp
+    for (int64_t b = 0; b < ntiles; b += RS_THREADS) {
+        const int64_t i = b + threadIdx.x;
+        const unsigned long long v = i < ntiles ? c[i] : 0ull;
+        unsigned long long x = v;  // inclusive scan inside the warp
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) wsum[warp] = x;
         __syncthreads();
-        if (warp == 0) {
-            unsigned long long t = wsum[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, t, o);
-                if (lane >= o) t += y;
-            }
-            wsum[lane] = t;  // inclusive over the warps
-        }
-        __syncthreads();
-        const unsigned long long off = carry + (warp ? wsum[warp - 1] : 0ull) + x - tot;
+        unsigned long long before = 0, all = 0;
 #pragma unroll
-        for (int k = 0; k < IPT; ++k)
-            if (i0 + k < m) c[i0 + k] = off + v[k];
-        carry += wsum[31];
-        __syncthreads();  // wsum is rewritten by the next chunk
+        for (int w = 0; w < RS_THREADS / 32; ++w) {
+            if (w < warp) before += wsum[w];
+            all += wsum[w];
+        }
+        if (i < ntiles) c[i] = carry + before + x - v;
+        carry += all;
+        __syncthreads();  // wsum is rewritten by the next tiles
     }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
 __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t *__restrict__ in, uint64_t *__restrict__ out,
                                                            int64_t n, int shift, int64_t ntiles,
-                                                           const unsigned long long *__restrict__ base) {
+                                                           const unsigned long long *__restrict__ base,
+                                                           const unsigned long long *__restrict__ totals) {
     __shared__ unsigned int run[256];
     __shared__ unsigned int wc[RS_THREADS / 32][256];
+    __shared__ unsigned long long dbase[256], dsum[RS_THREADS / 32];  // keys of smaller digits
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    {
+        const unsigned long long v = totals[threadIdx.x];
+        unsigned long long x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) dsum[warp] = x;
+        __syncthreads();
+        x -= v;
+        for (int w = 0; w < warp; ++w) x += dsum[w];
+        dbase[threadIdx.x] = x;
+        __syncthreads();
+    }
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         run[threadIdx.x] = 0;
         for (int r = 0; r < RS_ITEMS; ++r) {
@@ -430,7 +541,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t *__res
             if (valid) {
                 unsigned off = run[dg] + rank;
                 for (int w = 0; w < warp; ++w) off += wc[w][dg];
-                out[base[(int64_t)dg * ntiles + tile] + off] = key;
+                out[dbase[dg] + base[(int64_t)dg * ntiles + tile] + off] = key;
             }
             __syncthreads();
             unsigned add = 0;
@@ -456,8 +567,9 @@ struct CsSizes {
     uint64_t capj, capl;
     int64_t ntiles;
     size_t bytes;
-    size_t off_hj, off_hjc, off_jaddr, off_D, off_E, off_hl, off_laddr, off_tmp, off_cnt, off_hist, off_nzlo, off_bm;
-    size_t bm_bytes;
+    size_t off_hj, off_hjc, off_jaddr, off_D, off_E, off_hl, off_laddr, off_tmp, off_cnt, off_hist, off_nzlo, off_bm, off_head,
+        off_node;
+    size_t bm_bytes, head_bytes;
 };
 
 CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
@@ -477,10 +589,13 @@ CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
     z.off_hl = o; o += al(z.capl * 8);
     z.off_laddr = o; o += al((size_t)z.n2max * 8);
     z.off_tmp = o; o += al((size_t)z.n2max * 8);
-    z.off_hist = o; o += al((size_t)256 * z.ntiles * 8);
+    z.off_hist = o; o += al((size_t)256 * (z.ntiles + 1) * 8);  // counts, then the digits' totals
     z.off_nzlo = o; o += al((size_t)(h->das.n_cat + 1) * 8);
     z.bm_bytes = (size_t)((h->nsa + 31) / 32 + (h->nsb + 31) / 32) * 4;
     z.off_bm = o; o += al(z.bm_bytes);
+    z.head_bytes = (size_t)(h->nsa + h->nsb) * 4;
+    z.off_head = o; o += al(z.head_bytes);
+    z.off_node = o; o += al((size_t)z.n1max * 2 * sizeof(int2));
     z.off_cnt = o; o += 256;
     z.bytes = o;
     return z;
@@ -554,6 +669,12 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     a.nz_lo = (int64_t *)(w + z.off_nzlo);
     a.bm_a = (uint32_t *)(w + z.off_bm);
     a.bm_b = a.bm_a + (h->nsa + 31) / 32;
+    a.str_a = h->d_str_a;
+    a.str_b = h->d_str_b;
+    a.head_a = (int32_t *)(w + z.off_head);
+    a.head_b = a.head_a + h->nsa;
+    a.node_a = (int2 *)(w + z.off_node);
+    a.node_b = a.node_a + z.n1max;
     a.hj = (unsigned long long *)(w + z.off_hj);
     a.hj_col = (int32_t *)(w + z.off_hjc);
     a.hj_mask = z.capj - 1;
@@ -575,12 +696,13 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
         const int64_t moves = nnz_c * (a.nent_a + a.nent_b);
         k_cs_expand<<<grid_of(moves), 256, 0, s>>>(a);
         k_cs_cat_ranges<<<(unsigned)ceil_div(h->das.n_cat + 1, 256), 256, 0, s>>>(a);
-        k_cs_compact<<<grid_of((int64_t)z.capj), 256, 0, s>>>(a.hj, a.hj_col, z.capj, a.j_addr, a.counts);
+        k_cs_compact<<<grid_of((int64_t)z.capj / 8), 256, 0, s>>>(a.hj, a.hj_col, z.capj, a.j_addr, a.counts);
         FCI_CUDA(h, cudaMemcpyAsync(cnt, a.counts, sizeof cnt, cudaMemcpyDeviceToHost, s));
         FCI_CUDA(h, cudaStreamSynchronize(s));
         if (cnt[2]) return fci_fail(h, FCI_ERR_CUDA, "compressed sigma: hash table overflow");
-        k_cs_gather<<<grid_of((int64_t)cnt[0] * h->npair), 256, 0, s>>>(a, (int64_t)cnt[0]);
+        k_cs_gather<<<grid_of((int64_t)cnt[0] * 32), 256, 0, s>>>(a, (int64_t)cnt[0]);
         FCI_CUDA(h, cudaMemsetAsync(a.bm_a, 0, z.bm_bytes, s));
+        FCI_CUDA(h, cudaMemsetAsync(a.head_a, 0xFF, z.head_bytes, s));
         k_cs_mark<<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
         FCI_CUDA(h, cudaGetLastError());
     }
@@ -597,7 +719,7 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
         phase_scope ps(h, s, FCI_PHASE_OTHER, 3);
         FCI_CUDA(h, cudaMemsetAsync(a.hl, 0xFF, z.capl * 8, s));
         k_cs_support<<<grid_of(n1 * (a.nent_a + a.nent_b)), 256, 0, s>>>(a, n1);
-        k_cs_compact<<<grid_of((int64_t)z.capl), 256, 0, s>>>(a.hl, nullptr, z.capl, a.l_addr, a.counts + 1);
+        k_cs_compact<<<grid_of((int64_t)z.capl / 8), 256, 0, s>>>(a.hl, nullptr, z.capl, a.l_addr, a.counts + 1);
         FCI_CUDA(h, cudaMemcpyAsync(cnt, a.counts, sizeof cnt, cudaMemcpyDeviceToHost, s));
         FCI_CUDA(h, cudaStreamSynchronize(s));
         if (cnt[2]) return fci_fail(h, FCI_ERR_CUDA, "compressed sigma: hash table overflow");
@@ -616,8 +738,8 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
         const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nt, 152 * 8));
         for (int shift = 0; shift < bits; shift += 8) {
             k_rs_hist<<<g, RS_THREADS, 0, s>>>(src, n2, shift, nt, hist);
-            k_rs_scan<<<1, 1024, 0, s>>>(hist, 256 * nt);
-            k_rs_scatter<<<g, RS_THREADS, 0, s>>>(src, dst, n2, shift, nt, hist);
+            k_rs_scan<<<256, RS_THREADS, 0, s>>>(hist, nt, hist + 256 * nt);
+            k_rs_scatter<<<g, RS_THREADS, 0, s>>>(src, dst, n2, shift, nt, hist, hist + 256 * nt);
             std::swap(src, dst);
         }
         FCI_CUDA(h, cudaGetLastError());
