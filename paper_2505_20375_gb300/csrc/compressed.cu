@@ -26,9 +26,10 @@
 //      of the dense FP64 DAS path, so the result equals the dense sigma on the support and
 //      the dense sigma is zero elsewhere.  The columns J that L reaches share its beta
 //      string (an alpha move) or its alpha string (a beta move), so they are found on the
-//      lists of columns per string, a few entries long for nearly every L; only where a
-//      list is long or many columns match are L's replacements walked, each J looked up in
-//      the first table.
+//      lists of columns per string.  Entries with short lists (most: the alpha-beta doubles
+//      of a nonzero determinant) take one thread each, those with long lists (its same-spin
+//      doubles and singles) one warp each; only where the lists are longer than a walk of
+//      L's replacements is that walk made, each J looked up in the first table.
 // The pair tables are read string-major (one string's row contiguous; copies built on the
 // first call and kept by the handle).  Hash tables use open addressing with linear
 // probing over a power-of-two capacity of at least twice the largest number of keys, so no
@@ -36,6 +37,8 @@
 // the same and reports an overflow instead.
 #include <stdint.h>
 #include <string.h>
+
+#include <cooperative_groups.h>
 
 #include <algorithm>
 #include <vector>
@@ -101,15 +104,17 @@ struct CsArgs {
     int64_t *j_addr;                 // [n1]: the J of each column
     uint32_t *bm_a, *bm_b;           // bit A (B) set: some column has alpha (beta) string A (B)
     const uint64_t *str_a, *str_b;   // string masks
-    int32_t *head_a, *head_b;        // [n_str]: first column with this alpha (beta) string, -1: none
-    int2 *node_a, *node_b;           // [n1]: next column of the same alpha (beta) string, and the
-                                     // column's other string (mask)
+    // columns per string: entries off[S] .. off[S + 1] of list_a (list_b) hold the columns with
+    // alpha (beta) string S, as (column, mask of its other string)
+    uint32_t *off_a, *off_b;         // [n_str + 1]
+    int2 *list_a, *list_b;           // [n1]
+    int64_t *work;                   // support entries left to the warp form
     double *D, *E;                   // [n_pair][ldd]
     int64_t ldd;
     unsigned long long *hl;          // target determinants L of the support
     uint64_t hl_mask;
     int64_t *l_addr;                 // [n2]
-    unsigned long long *counts;      // [0]: columns n1, [1]: support n2, [2]: overflow flag
+    unsigned long long *counts;      // [0]: columns n1, [1]: support n2, [2]: overflow flag, [3]: entries in work
     double e_core;
 };
 
@@ -254,17 +259,75 @@ __global__ void k_cs_transpose(const int32_t *__restrict__ src, int64_t R, int64
 }
 
 // The alpha and beta strings of every column, as bitmaps (a walk of the replacements looks a
-// candidate column up only if both of its strings occur in some column) and as lists of
-// columns per string (in any order: the terms found on them are sorted).
+// candidate column up only if both of its strings occur in some column), and the lists of
+// columns per string: FILL = false counts them (into off[S]), FILL = true, after the scan,
+// writes them backwards from the end of each string's range, which leaves off[S] at its start
+// (the order inside a list is free: the terms found on it are sorted).
+template <bool FILL>
 __global__ void k_cs_mark(const __grid_constant__ CsArgs a, int64_t n1) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n1; j += (int64_t)gridDim.x * blockDim.x) {
         int32_t A, B;
         int pb;
         das_strings(a.d, a.n_cat_int, a.j_addr[j], A, B, pb);
-        atomicOr(a.bm_a + (A >> 5), 1u << (A & 31));
-        atomicOr(a.bm_b + (B >> 5), 1u << (B & 31));
-        a.node_a[j] = make_int2(atomicExch(a.head_a + A, (int32_t)j), (int)(uint32_t)a.str_b[B]);
-        a.node_b[j] = make_int2(atomicExch(a.head_b + B, (int32_t)j), (int)(uint32_t)a.str_a[A]);
+        if (FILL) {
+            a.list_a[atomicSub(a.off_a + A, 1u) - 1u] = make_int2((int)j, (int)(uint32_t)a.str_b[B]);
+            a.list_b[atomicSub(a.off_b + B, 1u) - 1u] = make_int2((int)j, (int)(uint32_t)a.str_a[A]);
+        } else {
+            atomicOr(a.bm_a + (A >> 5), 1u << (A & 31));
+            atomicOr(a.bm_b + (B >> 5), 1u << (B & 31));
+            atomicAdd(a.off_a + A, 1u);
+            atomicAdd(a.off_b + B, 1u);
+        }
+    }
+}
+
+// Inclusive scan of c[0 .. m) in place (then c[S] is the end of string S's range), in two
+// launches: block b adds up its 4,096 counts; then every block scans its own and adds the
+// sums of the blocks before it.
+constexpr int SCAN_TILE = 4096;
+__device__ __forceinline__ uint32_t block_sum_256(uint32_t v, uint32_t *sh) {
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    uint32_t s = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s += sh[w];
+    __syncthreads();
+    return s;
+}
+__global__ void __launch_bounds__(256) k_cs_scan_sums(const uint32_t *__restrict__ c, int64_t m, uint32_t *__restrict__ sums) {
+    __shared__ uint32_t sh[8];
+    uint32_t v = 0;
+    for (int64_t i = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x; i < m && i < (int64_t)(blockIdx.x + 1) * SCAN_TILE; i += 256)
+        v += c[i];
+    v = block_sum_256(v, sh);
+    if (threadIdx.x == 0) sums[blockIdx.x] = v;
+}
+__global__ void __launch_bounds__(256) k_cs_scan(uint32_t *__restrict__ c, int64_t m, const uint32_t *__restrict__ sums) {
+    __shared__ uint32_t sh[8];
+    uint32_t before = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += 256) before += sums[b];
+    uint32_t carry = block_sum_256(before, sh);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t b = (int64_t)blockIdx.x * SCAN_TILE; b < m && b < (int64_t)(blockIdx.x + 1) * SCAN_TILE; b += 256) {
+        const int64_t i = b + threadIdx.x;
+        const uint32_t v = i < m ? c[i] : 0u;
+        uint32_t x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) sh[warp] = x;
+        __syncthreads();
+        uint32_t ahead = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) ahead += sh[w];
+            all += sh[w];
+        }
+        if (i < m) c[i] = carry + ahead + x;
+        carry += all;
+        __syncthreads();
     }
 }
 
@@ -334,81 +397,32 @@ __global__ void __launch_bounds__(256) k_cs_support(const __grid_constant__ CsAr
 
 // Step 4: sigma on the sorted support, in the dense DAS path's order of terms.
 
-// The sum over L's replacements, each column looked up in the table of columns.
-__device__ __noinline__ double cs_walk(const CsArgs &a, int32_t A, int32_t B) {
-    double acc = 0.0;
-    const int4 *ra = reinterpret_cast<const int4 *>(a.pair_a + (int64_t)A * a.ldp);
-    const int4 *rb = reinterpret_cast<const int4 *>(a.pair_b + (int64_t)B * a.ldp);
-    // an alpha move keeps B and a beta move keeps A: no column has them, no lookup
-    const bool try_a = bit(a.bm_b, B), try_b = bit(a.bm_a, A);
-    const int4 none = make_int4(-1, -1, -1, -1);
-    for (int p4 = 0; p4 < a.npair && (try_a || try_b); p4 += 4) {  // four pairs per 16-byte load of a row
-        const int4 va = try_a ? __ldg(ra + p4 / 4) : none, vb = try_b ? __ldg(rb + p4 / 4) : none;
-        const int32_t ea4[4] = {va.x, va.y, va.z, va.w}, eb4[4] = {vb.x, vb.y, vb.z, vb.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const double *Ep = a.E + (int64_t)(p4 + k) * a.ldd;  // rows past n_pair hold -1
-            const int32_t ea = ea4[k];
-            if (ea >= 0 && bit(a.bm_a, ea >> 1)) {
-                const int64_t J = das_addr(a.d, ea >> 1, B);
-                const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
-                if (col >= 0) {
-                    const double e = Ep[col];
-                    acc += (ea & 1) ? -e : e;
-                }
-            }
-            const int32_t eb = eb4[k];
-            if (eb >= 0 && bit(a.bm_b, eb >> 1)) {
-                const int64_t J = das_addr(a.d, A, eb >> 1);
-                const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
-                if (col >= 0) {
-                    const double e = Ep[col];
-                    acc += (eb & 1) ? -e : e;
-                }
-            }
-        }
-    }
-    return acc;
+// The key of the move between strings S and T that differ in two orbitals: pair, spin (alpha
+// before beta), and the sign of <L|E|J> in the lowest bit.
+__device__ __forceinline__ uint32_t cs_key(uint32_t S, uint32_t x, int spin) {
+    const int hi = 31 - __clz(x), lo = __ffs(x) - 1;
+    const uint32_t between = ((1u << hi) - 1u) & ~((2u << lo) - 1u);
+    return ((uint32_t)(hi * (hi + 1) / 2 + lo) << 2) | (uint32_t)(spin << 1) | (__popc(S & between) & 1u);
 }
 
-// Terms of L found on one list: the columns whose string `mask` on the list's other spin is
-// one move from S.  Each goes into the ascending keys (2 pair + spin, sign) with its column.
-// False if a term does not fit, the list is longer than a walk of the replacements, or L
-// itself is a column (its diagonal terms are many).
-constexpr int CS_TERMS = 8;      // terms kept per L
-constexpr int CS_MAX_HOPS = 320; // list entries visited per spin
-__device__ __forceinline__ bool cs_list(const int2 *__restrict__ node, int32_t c, uint32_t S, int spin,
-                                        uint32_t (&key)[CS_TERMS], int32_t (&col)[CS_TERMS], int &n) {
-    for (int hop = 0; c >= 0; ++hop) {
-        if (hop >= CS_MAX_HOPS) return false;
-        const int2 nd = __ldg(node + c);
-        const uint32_t x = S ^ (uint32_t)nd.y;
-        const int d = __popc(x);
-        if (d == 0) return false;
-        if (d == 2) {
-            if (n == CS_TERMS) return false;
-            const int hi = 31 - __clz(x), lo = __ffs(x) - 1;
-            const uint32_t between = ((1u << hi) - 1u) & ~((2u << lo) - 1u);
-            uint32_t k = ((uint32_t)(hi * (hi + 1) / 2 + lo) << 2) | (uint32_t)(spin << 1) | (__popc(S & between) & 1u);
-            int32_t v = c;
-#pragma unroll
-            for (int i = 0; i < CS_TERMS; ++i) {  // insertion, the entries past n being larger than any key
-                if (k < key[i]) {
-                    const uint32_t tk = key[i];
-                    const int32_t tv = col[i];
-                    key[i] = k;
-                    col[i] = v;
-                    k = tk;
-                    v = tv;
-                }
-            }
-            ++n;
-        }
-        c = nd.x;
+// sigma_L from the sum of its terms: the coefficient C_L by binary search.  A nonzero
+// determinant with electrons is a column itself (its diagonal replacements), so an L that is
+// found not to be a column has C_L = 0 and no search.
+__device__ __forceinline__ double cs_value(const CsArgs &a, int64_t L, double acc) {
+    double cl = 0.0;
+    int64_t lo = 0, hi = a.nnz_c - 1;
+    while (lo <= hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        const int64_t v = a.c_addr[mid];
+        if (v == L) { cl = a.c_val[mid]; break; }
+        if (v < L) lo = mid + 1; else hi = mid - 1;
     }
-    return true;
+    return fma(a.e_core, cl, acc);  // as the dense FP64 scatter
 }
 
+// Thread form: entries whose two lists hold at most CS_SHORT columns, none of them L itself.
+// The (at most CS_SHORT) terms go into ascending keys.  The others are appended to `work`.
+constexpr int CS_SHORT = 8;
 __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
                                                   int64_t n2, double *__restrict__ out_val) {
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n2; o += (int64_t)gridDim.x * blockDim.x) {
@@ -416,37 +430,173 @@ __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs
         int32_t A, B;
         int pb;
         das_strings(a.d, a.d.n_cat, L, A, B, pb);
-        double acc = 0.0;
-        uint32_t key[CS_TERMS];
-        int32_t col[CS_TERMS];
+        const uint32_t b0 = __ldg(a.off_b + B), nb = __ldg(a.off_b + B + 1) - b0;
+        const uint32_t a0 = __ldg(a.off_a + A), na = __ldg(a.off_a + A + 1) - a0;
+        bool ok = na + nb <= CS_SHORT;
+        uint32_t key[CS_SHORT];
+        int32_t col[CS_SHORT];
 #pragma unroll
-        for (int i = 0; i < CS_TERMS; ++i) {
+        for (int i = 0; i < CS_SHORT; ++i) {
             key[i] = ~0u;
             col[i] = 0;
         }
-        int n = 0;
-        if (cs_list(a.node_b, __ldg(a.head_b + B), (uint32_t)__ldg(a.str_a + A), 0, key, col, n) &&
-            cs_list(a.node_a, __ldg(a.head_a + A), (uint32_t)__ldg(a.str_b + B), 1, key, col, n)) {
-            double e[CS_TERMS];
+        if (ok) {
+            const uint32_t SA = (uint32_t)__ldg(a.str_a + A), SB = (uint32_t)__ldg(a.str_b + B);
+            for (uint32_t c = 0; c < na + nb; ++c) {
+                const bool alpha = c < nb;  // the columns with L's beta string are its alpha moves
+                const int2 nd = __ldg(alpha ? a.list_b + b0 + c : a.list_a + a0 + (c - nb));
+                const uint32_t S = alpha ? SA : SB, x = S ^ (uint32_t)nd.y;
+                const int d = __popc(x);
+                if (d == 0) ok = false;
+                if (d != 2) continue;
+                uint32_t k = cs_key(S, x, alpha ? 0 : 1);
+                int32_t v = nd.x;
 #pragma unroll
-            for (int i = 0; i < CS_TERMS; ++i)
-                e[i] = key[i] != ~0u ? __ldg(a.E + (int64_t)(key[i] >> 2) * a.ldd + col[i]) : 0.0;
+                for (int i = 0; i < CS_SHORT; ++i) {  // insertion; free places hold the largest key
+                    if (k < key[i]) {
+                        const uint32_t tk = key[i];
+                        const int32_t tv = col[i];
+                        key[i] = k;
+                        col[i] = v;
+                        k = tk;
+                        v = tv;
+                    }
+                }
+            }
+        }
+        if (!ok) {
+            const cooperative_groups::coalesced_group g = cooperative_groups::coalesced_threads();
+            unsigned long long at = 0;
+            if (g.thread_rank() == 0) at = atomicAdd(a.counts + 3, (unsigned long long)g.size());
+            a.work[g.shfl(at, 0) + g.thread_rank()] = o;
+            continue;
+        }
+        double e[CS_SHORT], acc = 0.0;
 #pragma unroll
-            for (int i = 0; i < CS_TERMS; ++i)
-                if (key[i] != ~0u) acc += (key[i] & 1u) ? -e[i] : e[i];
-        } else {
-            acc = cs_walk(a, A, B);
+        for (int i = 0; i < CS_SHORT; ++i)
+            e[i] = key[i] != ~0u ? __ldg(a.E + (int64_t)(key[i] >> 2) * a.ldd + col[i]) : 0.0;
+#pragma unroll
+        for (int i = 0; i < CS_SHORT; ++i)
+            if (key[i] != ~0u) acc += (key[i] & 1u) ? -e[i] : e[i];
+        out_val[o] = fma(a.e_core, 0.0, acc);
+    }
+}
+
+// Warp form.  The lanes check 32 columns of a list at a time; the terms (at most CS_LONG,
+// the diagonal ones included if L itself is a column) are ranked by key in shared memory
+// and added in that order.  Entries with longer lists or more terms walk their
+// replacements, 32 pairs at a time, each lane looking up its pair's two columns; the terms
+// of the lanes are added in pair order.
+constexpr int CS_LONG = 128;
+__global__ void __launch_bounds__(256) k_cs_sigma_warp(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
+                                                       double *__restrict__ out_val) {
+    __shared__ uint32_t s_key[8][CS_LONG];
+    __shared__ double s_val[8][CS_LONG], s_ord[8][CS_LONG];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n = (int64_t)a.counts[3], nw = (int64_t)gridDim.x * 8;
+    for (int64_t it = (int64_t)blockIdx.x * 8 + warp; it < n; it += nw) {
+        const int64_t o = a.work[it], L = l_sorted[o];
+        int32_t A, B;
+        int pb;
+        das_strings(a.d, a.d.n_cat, L, A, B, pb);
+        const uint32_t b0 = __ldg(a.off_b + B), nb = __ldg(a.off_b + B + 1) - b0;
+        const uint32_t a0 = __ldg(a.off_a + A), na = __ldg(a.off_a + A + 1) - a0;
+        double acc = 0.0;
+        int terms = 0;
+        bool itself = false;
+        bool ok = na + nb <= (uint32_t)a.npair;
+        if (ok) {
+            const uint32_t SA = (uint32_t)__ldg(a.str_a + A), SB = (uint32_t)__ldg(a.str_b + B);
+            for (uint32_t c0 = 0; c0 < na + nb && ok; c0 += 32) {
+                const uint32_t c = c0 + lane;
+                const bool alpha = c < nb, live = c < na + nb;
+                const int2 nd = live ? __ldg(alpha ? a.list_b + b0 + c : a.list_a + a0 + (c - nb)) : make_int2(0, 0);
+                const uint32_t S = alpha ? SA : SB, x = live ? S ^ (uint32_t)nd.y : ~0u;
+                const bool hit = __popc(x) == 2;
+                const unsigned hits = __ballot_sync(0xFFFFFFFFu, hit);
+                if (terms + __popc(hits) > CS_LONG) {
+                    ok = false;
+                    break;
+                }
+                if (hit) {
+                    const uint32_t k = cs_key(S, x, alpha ? 0 : 1);
+                    const double e = __ldg(a.E + (int64_t)(k >> 2) * a.ldd + nd.x);
+                    const int at = terms + __popc(hits & ((1u << lane) - 1u));
+                    s_key[warp][at] = k;
+                    s_val[warp][at] = (k & 1u) ? -e : e;
+                }
+                terms += __popc(hits);
+                unsigned self = __ballot_sync(0xFFFFFFFFu, x == 0u);  // L itself: a term per electron
+                itself |= self != 0;
+                while (self) {
+                    const int src = __ffs(self) - 1;
+                    self &= self - 1;
+                    const uint32_t T = __shfl_sync(0xFFFFFFFFu, S, src);
+                    const int cl = __shfl_sync(0xFFFFFFFFu, nd.x, src), spin = __shfl_sync(0xFFFFFFFFu, alpha ? 0 : 1, src);
+                    if (terms + __popc(T) > CS_LONG) {
+                        ok = false;
+                        break;
+                    }
+                    if ((T >> lane) & 1u) {
+                        const uint32_t pp = (uint32_t)(lane * (lane + 1) / 2 + lane);
+                        const int at = terms + __popc(T & ((1u << lane) - 1u));
+                        s_key[warp][at] = (pp << 2) | (uint32_t)(spin << 1);
+                        s_val[warp][at] = __ldg(a.E + (int64_t)pp * a.ldd + cl);
+                    }
+                    terms += __popc(T);
+                }
+            }
+            __syncwarp();
+            if (ok) {
+                for (int i = lane; i < terms; i += 32) {  // keys differ: the rank is the place
+                    const uint32_t k = s_key[warp][i];
+                    int r = 0;
+                    for (int q = 0; q < terms; ++q) r += s_key[warp][q] < k;
+                    s_ord[warp][r] = s_val[warp][i];
+                }
+                __syncwarp();
+                for (int i = 0; i < terms; ++i) acc += s_ord[warp][i];
+                __syncwarp();
+            }
         }
-        // C_L from the sorted nonzero addresses (binary search)
-        double cl = 0.0;
-        int64_t lo = 0, hi = a.nnz_c - 1;
-        while (lo <= hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            const int64_t v = a.c_addr[mid];
-            if (v == L) { cl = a.c_val[mid]; break; }
-            if (v < L) lo = mid + 1; else hi = mid - 1;
+        if (!ok) {
+            acc = 0.0;
+            // an alpha move keeps B and a beta move keeps A: no column has them, no lookup
+            const bool try_a = bit(a.bm_b, B), try_b = bit(a.bm_a, A);
+            const int32_t *ra = a.pair_a + (int64_t)A * a.ldp, *rb = a.pair_b + (int64_t)B * a.ldp;
+            for (int p0 = 0; p0 < a.npair && (try_a || try_b); p0 += 32) {
+                const int pp = p0 + lane;
+                const int32_t ea = try_a && pp < a.npair ? __ldg(ra + pp) : -1, eb = try_b && pp < a.npair ? __ldg(rb + pp) : -1;
+                double va = 0.0, vb = 0.0;
+                bool fa = false, fb = false;
+                if (ea >= 0 && bit(a.bm_a, ea >> 1)) {
+                    const int64_t J = das_addr(a.d, ea >> 1, B);
+                    const int64_t c = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+                    if (c >= 0) {
+                        fa = true;
+                        va = a.E[(int64_t)pp * a.ldd + c];
+                        if (ea & 1) va = -va;
+                    }
+                }
+                if (eb >= 0 && bit(a.bm_b, eb >> 1)) {
+                    const int64_t J = das_addr(a.d, A, eb >> 1);
+                    const int64_t c = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+                    if (c >= 0) {
+                        fb = true;
+                        vb = a.E[(int64_t)pp * a.ldd + c];
+                        if (eb & 1) vb = -vb;
+                    }
+                }
+                const unsigned ma = __ballot_sync(0xFFFFFFFFu, fa), mb = __ballot_sync(0xFFFFFFFFu, fb);
+                for (unsigned m = ma | mb; m; m &= m - 1) {
+                    const int src = __ffs(m) - 1;
+                    const double ta = __shfl_sync(0xFFFFFFFFu, va, src), tb = __shfl_sync(0xFFFFFFFFu, vb, src);
+                    if ((ma >> src) & 1u) acc += ta;
+                    if ((mb >> src) & 1u) acc += tb;
+                }
+            }
         }
-        out_val[o] = fma(a.e_core, cl, acc);  // as the dense FP64 scatter
+        if (lane == 0) out_val[o] = !ok || itself ? cs_value(a, L, acc) : fma(a.e_core, 0.0, acc);
     }
 }
 
@@ -567,9 +717,10 @@ struct CsSizes {
     uint64_t capj, capl;
     int64_t ntiles;
     size_t bytes;
-    size_t off_hj, off_hjc, off_jaddr, off_D, off_E, off_hl, off_laddr, off_tmp, off_cnt, off_hist, off_nzlo, off_bm, off_head,
-        off_node;
-    size_t bm_bytes, head_bytes;
+    size_t off_hj, off_hjc, off_jaddr, off_D, off_E, off_hl, off_laddr, off_tmp, off_cnt, off_hist, off_nzlo, off_bm, off_str,
+        off_list, off_work;
+    size_t bm_bytes, str_bytes;
+    int64_t n_sums;  // scan blocks over the strings of both spins
 };
 
 CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
@@ -593,9 +744,11 @@ CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
     z.off_nzlo = o; o += al((size_t)(h->das.n_cat + 1) * 8);
     z.bm_bytes = (size_t)((h->nsa + 31) / 32 + (h->nsb + 31) / 32) * 4;
     z.off_bm = o; o += al(z.bm_bytes);
-    z.head_bytes = (size_t)(h->nsa + h->nsb) * 4;
-    z.off_head = o; o += al(z.head_bytes);
-    z.off_node = o; o += al((size_t)z.n1max * 2 * sizeof(int2));
+    z.str_bytes = (size_t)(h->nsa + 1 + h->nsb + 1) * 4;
+    z.n_sums = ceil_div(h->nsa + 1, SCAN_TILE) + ceil_div(h->nsb + 1, SCAN_TILE);
+    z.off_str = o; o += al(z.str_bytes + (size_t)z.n_sums * 4);
+    z.off_list = o; o += al((size_t)z.n1max * 2 * sizeof(int2));
+    z.off_work = z.off_hl;  // the support's hash table is done with by then (8 bytes per slot, two slots per entry)
     z.off_cnt = o; o += 256;
     z.bytes = o;
     return z;
@@ -671,10 +824,12 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     a.bm_b = a.bm_a + (h->nsa + 31) / 32;
     a.str_a = h->d_str_a;
     a.str_b = h->d_str_b;
-    a.head_a = (int32_t *)(w + z.off_head);
-    a.head_b = a.head_a + h->nsa;
-    a.node_a = (int2 *)(w + z.off_node);
-    a.node_b = a.node_a + z.n1max;
+    a.off_a = (uint32_t *)(w + z.off_str);
+    a.off_b = a.off_a + h->nsa + 1;
+    uint32_t *sums = a.off_b + h->nsb + 1;
+    a.list_a = (int2 *)(w + z.off_list);
+    a.list_b = a.list_a + z.n1max;
+    a.work = (int64_t *)(w + z.off_work);
     a.hj = (unsigned long long *)(w + z.off_hj);
     a.hj_col = (int32_t *)(w + z.off_hjc);
     a.hj_mask = z.capj - 1;
@@ -702,8 +857,16 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
         if (cnt[2]) return fci_fail(h, FCI_ERR_CUDA, "compressed sigma: hash table overflow");
         k_cs_gather<<<grid_of((int64_t)cnt[0] * 32), 256, 0, s>>>(a, (int64_t)cnt[0]);
         FCI_CUDA(h, cudaMemsetAsync(a.bm_a, 0, z.bm_bytes, s));
-        FCI_CUDA(h, cudaMemsetAsync(a.head_a, 0xFF, z.head_bytes, s));
-        k_cs_mark<<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
+        FCI_CUDA(h, cudaMemsetAsync(a.off_a, 0, z.str_bytes, s));
+        k_cs_mark<false><<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
+        auto scan = [&](uint32_t *c, int64_t m, uint32_t *block_sums) {
+            const unsigned nb = (unsigned)ceil_div(m, SCAN_TILE);
+            k_cs_scan_sums<<<nb, 256, 0, s>>>(c, m, block_sums);
+            k_cs_scan<<<nb, 256, 0, s>>>(c, m, block_sums);
+        };
+        scan(a.off_a, h->nsa + 1, sums);
+        scan(a.off_b, h->nsb + 1, sums + ceil_div(h->nsa + 1, SCAN_TILE));
+        k_cs_mark<true><<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
         FCI_CUDA(h, cudaGetLastError());
     }
     const int64_t n1 = (int64_t)cnt[0];
@@ -747,8 +910,9 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     }
     // 4. sigma on the support
     {
-        phase_scope ps(h, s, FCI_PHASE_SCATTER, 1);
+        phase_scope ps(h, s, FCI_PHASE_SCATTER, 2);
         k_cs_sigma<<<grid_of(n2), 256, 0, s>>>(a, out_addr, n2, out_val);
+        k_cs_sigma_warp<<<152 * 8, 256, 0, s>>>(a, out_addr, out_val);
         FCI_CUDA(h, cudaGetLastError());
     }
     FCI_CUDA(h, cudaStreamSynchronize(s));
