@@ -962,9 +962,10 @@ int dz_num_sms(fci_context *h, int *nsm) {
 // fit in TMEM, and neither do its G slices in shared memory, so the contraction turns back
 // to the orientation of the alpha/beta two-pass path: pair rows on M, 64 determinants on N,
 // and the operands streamed from HBM:
-//   k_dg_split      writes the digit image of D (int64 fixed point of C, gathered through
+//   k_dg_rows       writes the digit image of D (int64 fixed point of C, gathered through
 //                   the packed replacement tables and the target block offsets) for a piece
-//                   of the intermediate space, in the B layout of the block-sparse GEMM;
+//                   of the intermediate space, in the B layout of the block-sparse GEMM
+//                   (k_dg_split where an alpha string's row of C does not fit shared memory);
 //   k_oz_gemm_blk   (8-bit digits) sums the top s levels exactly in TMEM and stores E_int
 //                   (int64) [tile of 64][n_pair][64];
 //   k_dz_scatter    (int64 form) sums E_int exactly per target determinant.
@@ -1106,6 +1107,8 @@ struct DgSplit {
     const int32_t *nstr_b32;
     const int64_t *cat_off, *locbase_a, *locbase_b;
     const int32_t *cat_pa, *cat_pb;
+    const int32_t *base_int;  // the same for blocks of the intermediate space
+    int n_pat_a, row_max;     // longest row: target values that share an alpha string
     const int64_t *Cint;
     uint8_t *Dimg;
     ulonglong2 *masks;  // [n_nt]
@@ -1204,6 +1207,184 @@ __global__ void __launch_bounds__(256, 4) k_dg_split(const __grid_constant__ DgS
                     __stcs((uint4 *)(base + j * DG_BLK), make_uint4(w4[0], w4[1], w4[2], w4[3]));
                 }
             }
+    }
+}
+
+// Block masks of the piece's tiles: the union over the categories a tile meets.
+__global__ void k_dg_masks(const __grid_constant__ DgSplit a) {
+    for (int64_t nt = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; nt < a.n_nt; nt += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t lo = a.a0 + nt * OZG_N, hi = a.a0 + (nt * OZG_N + OZG_N < a.len ? nt * OZG_N + OZG_N : a.len);
+        ulonglong2 m = make_ulonglong2(0, 0);
+        for (int c = find_cat(a.cat_off, a.n_cat_int, lo); c < a.n_cat_int && __ldg(a.cat_off + c) < hi; ++c) {
+            const ulonglong2 x = a.cmask[c];
+            m.x |= x.x;
+            m.y |= x.y;
+        }
+        a.masks[nt] = m;
+    }
+}
+
+// The digit image by rows: one CTA per alpha string.  All beta moves of the determinants with
+// that string stay in the same row of C (the target values with this alpha string, category
+// by category), so the row is staged in shared memory and the scattered half of the gather
+// reads it there (one determinant at a time, the gather through L1 took 16 tag lookups per
+// warp load and bound the kernel).  Alpha moves lead from a category to runs of consecutive
+// values: their targets are resolved once per category.  Thread (determinant of 64, core,
+// quarter): the quarters take the active blocks in turn.  ROWS_TIME
+constexpr int DG_ROW_THREADS = 512;
+constexpr size_t DG_ROW_SMEM = 113 * 1024;
+template <int S>
+__global__ void __launch_bounds__(DG_ROW_THREADS, 2) k_dg_rows(const __grid_constant__ DgSplit a) {
+    constexpr uint64_t bias = 0x8080808080808080ull >> (8 * (8 - S));
+    extern __shared__ int64_t dg_row[];                      // [row_max]: C_int of the row
+    int32_t *sOff = reinterpret_cast<int32_t *>(dg_row + a.row_max);  // [n_pat_b]: place of a target block, -1: C is zero
+    int32_t *sPair = sOff + a.n_pat_b;                       // [16 n_blk]: pair of a position
+    int32_t *sEa = sPair + 16 * a.n_blk;                     // [16 n_blk]: the row's alpha entries
+    int32_t *sKa = sEa + 16 * a.n_blk;                       // [16 n_blk]: (target of lb = 0) << 1 | sign, -1: none
+    const int t = threadIdx.x, row = t & 63, core = (t >> 6) & 1, quarter = t >> 7;
+    const int npb = a.n_pat_b;
+    const int64_t ida = blockIdx.x;
+    int pa = 0;
+    for (int lo = 0, hi = a.n_pat_a - 1; lo <= hi;) {  // the pattern of the alpha string
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(a.locbase_a + mid) <= ida) {
+            pa = mid;
+            lo = mid + 1;
+        } else {
+            hi = mid - 1;
+        }
+    }
+    const int64_t la = ida - __ldg(a.locbase_a + pa);
+    int mine = 0;  // some block of the row lies in the piece
+    for (int pb = t; pb < npb; pb += DG_ROW_THREADS) {
+        const int32_t b = __ldg(a.base_int + pa * npb + pb);
+        const int64_t nb = __ldg(a.nstr_b32 + pb), x = b + la * nb;
+        if (b >= 0 && x < a.a0 + a.len && x + nb > a.a0) mine = 1;
+    }
+    if (!__syncthreads_or(mine)) return;
+    if (t == 0) {
+        int o = 0;
+        for (int pb = 0; pb < npb; ++pb) {
+            const bool on = __ldg(a.base_tgt + pa * npb + pb) >= 0;
+            sOff[pb] = on ? o : -1;
+            if (on) o += __ldg(a.nstr_b32 + pb);
+        }
+    }
+    for (int i = t; i < 16 * a.n_blk; i += DG_ROW_THREADS) {
+        const int32_t pr = __ldg(a.perm + i);
+        sPair[i] = pr;
+        sEa[i] = pr >= 0 ? __ldg(a.repA + (int64_t)pr * a.nla + ida) : -1;
+    }
+    __syncthreads();
+    for (int pb = t >> 5; pb < npb; pb += DG_ROW_THREADS / 32) {
+        if (sOff[pb] < 0) continue;
+        const int nb = __ldg(a.nstr_b32 + pb);
+        const int64_t *src = a.Cint + __ldg(a.base_tgt + pa * npb + pb) + la * nb;
+        for (int i = t & 31; i < nb; i += 32) dg_row[sOff[pb] + i] = __ldg(src + i);
+    }
+    for (int pb = 0; pb < npb; ++pb) {
+        const int32_t b0 = __ldg(a.base_int + pa * npb + pb);
+        if (b0 < 0) continue;
+        const int nb = __ldg(a.nstr_b32 + pb);
+        const int64_t x0 = b0 + la * nb, lo = max(x0, a.a0), hi = min(x0 + nb, a.a0 + a.len);
+        if (lo >= hi) continue;
+        __syncthreads();  // the previous category is done with sKa; the row is staged
+        for (int i = t; i < 16 * a.n_blk; i += DG_ROW_THREADS) {
+            const int32_t ea = sEa[i];
+            const int32_t b = ea >= 0 ? __ldg(a.base_tgt + (ea >> 23) * npb + pb) : -1;
+            sKa[i] = b >= 0 ? ((b + ((ea >> 1) & DZ_LOC_MASK) * nb) << 1) | (ea & 1) : -1;
+        }
+        __syncthreads();
+        const int32_t *repB = a.repB + __ldg(a.locbase_b + pb);
+        for (int64_t w0 = lo + (row & 32); w0 < hi; w0 += 64) {  // the warp's 32 determinants
+            const int64_t d = w0 + (row & 31);
+            const bool live = d < hi;
+            const int32_t lb = live ? (int32_t)(d - x0) : 0;
+            const int64_t off = d - a.a0;
+            const int64_t nt = off >> 6;
+            const int r = (int)(off & 63);
+            const uint4 own = live ? *reinterpret_cast<const uint4 *>(a.masks + nt) : make_uint4(0, 0, 0, 0);
+            const uint32_t all[4] = {__reduce_or_sync(0xFFFFFFFFu, own.x), __reduce_or_sync(0xFFFFFFFFu, own.y),
+                                     __reduce_or_sync(0xFFFFFFFFu, own.z), __reduce_or_sync(0xFFFFFFFFu, own.w)};
+            int turn = 0;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const uint32_t has = w == 0 ? own.x : w == 1 ? own.y : w == 2 ? own.z : own.w;
+#pragma unroll 1
+                for (uint32_t m = all[w]; m; m &= m - 1, turn = (turn + 1) & 3) {
+                    if (turn != quarter) continue;
+                    const int kb = __ffs(m) - 1, k = 32 * w + kb;
+                    const int i0 = 16 * k + 8 * core;
+                    int32_t eb[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int32_t pr = sPair[i0 + e];
+                        eb[e] = live && pr >= 0 ? __ldg(repB + (int64_t)pr * a.nlb + lb) : -1;
+                    }
+                    uint32_t ylo[8], yhi[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int32_t ka = sKa[i0 + e];
+                        const int64_t xa = ka >= 0 ? __ldg(a.Cint + (ka >> 1) + lb) : 0;
+                        const int32_t ob = eb[e] >= 0 ? sOff[eb[e] >> 23] : -1;
+                        const int64_t xb = ob >= 0 ? dg_row[ob + ((eb[e] >> 1) & DZ_LOC_MASK)] : 0;
+                        const int64_t v = ((ka & 1) ? -xa : xa) + ((eb[e] & 1) ? -xb : xb);
+                        const uint64_t y = (uint64_t)v + bias;
+                        ylo[e] = (uint32_t)y;
+                        yhi[e] = (uint32_t)(y >> 32);
+                    }
+                    if (!((has >> kb) & 1u)) continue;
+                    uint8_t *base = a.Dimg + ((size_t)nt * a.n_blk + k) * S * DG_BLK + (r >> 3) * 256 + core * 128 + (r & 7) * 16;
+#pragma unroll
+                    for (int j = 0; j < S; ++j) {
+                        const uint32_t bj = (uint32_t)(j & 3), sel = bj | ((4u + bj) << 8);
+                        uint32_t w4[4];
+#pragma unroll
+                        for (int e = 0; e < 8; e += 2)
+                            w4[e / 2] = j < 4 ? digits_f16x2(ylo[e], ylo[e + 1], sel) : digits_f16x2(yhi[e], yhi[e + 1], sel);
+                        __stcs((uint4 *)(base + j * DG_BLK), make_uint4(w4[0], w4[1], w4[2], w4[3]));
+                    }
+                }
+            }
+        }
+    }
+}
+
+// Shared memory of k_dg_rows; the longest row over the alpha patterns.
+size_t dg_row_smem(const DgSplit &a) { return (size_t)a.row_max * 8 + (size_t)(a.n_pat_b + 48 * a.n_blk) * 4; }
+int64_t dg_row_max(const fci_das_layout &L) {
+    int64_t most = 0;
+    for (int pa = 0; pa < L.n_pat_a; ++pa) {
+        int64_t n = 0;
+        for (int pb = 0; pb < L.n_pat_b; ++pb)
+            if (L.exc_a[pa] + L.exc_b[pb] <= L.max_transfer) n += L.pat_nstr_b[pb];
+        most = std::max(most, n);
+    }
+    return most;
+}
+
+// Digit image and block masks of a piece.  By rows where two CTAs' rows fit an SM (up to
+// about 14,000 target values per alpha string), else determinant by determinant.
+template <int S>
+cudaError_t dg_image_s(const DgSplit &a, cudaStream_t st) {
+    const size_t smem = dg_row_smem(a);
+    if (smem > DG_ROW_SMEM) {
+        k_dg_split<S><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(a.n_nt, 152 * 16)), 256, 0, st>>>(a);
+        return cudaGetLastError();
+    }
+    const cudaError_t e = cudaFuncSetAttribute(k_dg_rows<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_dg_masks<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(a.n_nt, 256), 152 * 8)), 256, 0, st>>>(a);
+    k_dg_rows<S><<<(unsigned)a.nla, DG_ROW_THREADS, smem, st>>>(a);
+    return cudaGetLastError();
+}
+cudaError_t dg_image(const DgSplit &a, int s, cudaStream_t st) {
+    switch (s) {
+        case 4: return dg_image_s<4>(a, st);
+        case 5: return dg_image_s<5>(a, st);
+        case 6: return dg_image_s<6>(a, st);
+        case 7: return dg_image_s<7>(a, st);
+        default: return dg_image_s<8>(a, st);
     }
 }
 
@@ -1329,6 +1510,9 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     sp.perm = L.d_dg_perm;
     sp.cmask = L.d_dg_mask;
     sp.base_tgt = L.d_dz_base;
+    sp.base_int = L.d_dz_base + npab;
+    sp.n_pat_a = L.n_pat_a;
+    sp.row_max = (int)std::min<int64_t>(dg_row_max(L), INT32_MAX);
     sp.nstr_b32 = L.d_dz_base + 2 * npab;
     sp.cat_off = L.d_cat_off;
     sp.locbase_a = L.d_pat_locbase_a;
@@ -1345,16 +1529,8 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
             sp.len = std::min(g.d_cap, elen - d0);
             sp.n_nt = ceil_div(sp.len, OZG_N);
             {
-                phase_scope ps(h, st, FCI_PHASE_GATHER, 1);
-                const unsigned gb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(sp.n_nt, 152 * 16));
-                switch (s) {
-                    case 4: k_dg_split<4><<<gb, 256, 0, st>>>(sp); break;
-                    case 5: k_dg_split<5><<<gb, 256, 0, st>>>(sp); break;
-                    case 6: k_dg_split<6><<<gb, 256, 0, st>>>(sp); break;
-                    case 7: k_dg_split<7><<<gb, 256, 0, st>>>(sp); break;
-                    default: k_dg_split<8><<<gb, 256, 0, st>>>(sp); break;
-                }
-                FCI_CUDA(h, cudaGetLastError());
+                phase_scope ps(h, st, FCI_PHASE_GATHER, 2);
+                FCI_CUDA(h, dg_image(sp, s, st));
             }
             oz_blk_args a;
             a.n_blk = g.n_blk;
