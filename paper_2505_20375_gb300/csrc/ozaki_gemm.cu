@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
         const int qd = warp & 3;
         constexpr int NCOL = OZG_N / (ozg_epi_warps(S) / 4);  // columns per warp: 32 or 16
         const int cw = NCOL * ((warp - 1 - OZG_ISSUERS) >> 2);
-        const int row = 32 * qd + lane;
+        const int row = 32 * qd + (NBUF == 1 ? lane : lane >> 2);  // the first this thread stores
         uint32_t tau = 0;
         for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x, ++tau) {
             const int64_t nt = u / p.n_mt;
@@ -252,11 +252,15 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
             tc_fence_after();
             const uint32_t tl = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * S * OZG_N);
             int64_t *dst = p.E + ((size_t)nt * p.M_pad + (size_t)mt * OZG_M + row) * OZG_N;
-            const bool keep = mt * OZG_M + row < p.M_real;  // rows past the operator's size are never read
-            if (NBUF == 1)
+            if constexpr (NBUF == 1) {
+                const bool keep = mt * OZG_M + row < p.M_real;  // rows past the operator's size are never read
                 ozg_epilogue_grouped<S, W, GH>(tl, cw, dst, keep, [&](int g) { mbar_arrive(smem_u32(&sh->acc_empty[g])); });
-            else
-                ozg_epilogue_whole<S, W>(tl, cw, NCOL, dst, keep, [&]() { mbar_arrive(smem_u32(&sh->acc_empty[buf])); });
+            } else {
+                EpiRows rows;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) rows.p[i] = mt * OZG_M + row + 8 * i < p.M_real ? dst + 8 * i * OZG_N : nullptr;
+                ozg_epilogue_whole<S, W>(tl, cw, NCOL, rows, [&]() { mbar_arrive(smem_u32(&sh->acc_empty[buf])); });
+            }
         }
     }
     tc_fence_before();

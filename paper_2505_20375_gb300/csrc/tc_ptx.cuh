@@ -91,6 +91,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
+// 16 TMEM lanes x 16 columns (two 16x256b tiles) starting at the lane and column of taddr, in
+// the fragment order of that shape: thread T holds, of lane T / 4 and (r[2], r[3]) lane
+// T / 4 + 8, the columns 2 (T % 4) and 2 (T % 4) + 1; r[4 ..] the same of the next 8 columns.
+__device__ __forceinline__ void tmem_ld_16x16(uint32_t taddr, uint32_t *r) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+// 32 lanes x 16 columns of this warp's quadrant: lanes 0-15 in r[0 .. 7], 16-31 in r[8 .. 15].
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[16]) {
+    tmem_ld_16x16(taddr, r);
+    tmem_ld_16x16(taddr + (16u << 16), r + 8);
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Orders every use of r after the preceding tcgen05.wait::ld (the registers of an
