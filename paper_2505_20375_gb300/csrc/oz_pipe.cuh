@@ -114,8 +114,9 @@ __device__ __forceinline__ void epi_store(const EpiRows &rows, int c0, const int
 }
 
 // Single-buffered accumulators (s >= 5): 16 columns from c0 to this lane's row of 64
-// determinants at dst, if keep, read GH levels at a time; each group is handed back (release(g), one lane) as soon as it is in registers, so the next
-// unit's first K step starts on it while the rest is read and combined.
+// determinants at dst, if keep, read GH levels at a time; each group is handed back
+// (release(g), one lane) as soon as it is in registers, so the next unit's first K step
+// starts on it while the rest is read and combined.
 template <int S, int W, int GH, class Release>
 __device__ __forceinline__ void ozg_epilogue_grouped(uint32_t tl, int c0, int64_t *dst, bool keep, Release release) {
     constexpr int L0 = oz_gemm_L0(S, W), NG = (S + GH - 1) / GH, lowshift = W * (L0 - (S - 1));
