@@ -13,6 +13,7 @@
 
 #include <algorithm>
 
+#include "dependent.cuh"
 #include "fci_internal.h"
 
 namespace {
@@ -44,6 +45,8 @@ __global__ void __cluster_dims__(SMALL_BLOCKS, 1, 1) __launch_bounds__(SMALL_THR
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ unsigned long long warp_part[SMALL_THREADS / 32], block_part;
+    await_previous();
+    admit_next();
     const int64_t t0 = (int64_t)blockIdx.x * SMALL_THREADS + threadIdx.x;
     constexpr int64_t step = (int64_t)SMALL_BLOCKS * SMALL_THREADS;
     unsigned long long m = 0;
@@ -71,6 +74,8 @@ __global__ void __cluster_dims__(SMALL_BLOCKS, 1, 1) __launch_bounds__(SMALL_THR
 }
 
 __global__ void k_absmax_bits(const double *__restrict__ x, int64_t n, fci_split_scalars *__restrict__ sc) {
+    await_previous();
+    admit_next();
     unsigned long long m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         m = max(m, abs_bits(x[i]));
@@ -81,6 +86,8 @@ __global__ void k_absmax_bits(const double *__restrict__ x, int64_t n, fci_split
 template <bool PAIRS>
 __global__ void k_to_fixed(const double *__restrict__ C, int64_t n, int top, fci_split_scalars *__restrict__ sc,
                            void *__restrict__ out) {
+    await_previous();
+    admit_next();
     const int sh = shift_of(sc->maxbits, top);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->shC = sh;
@@ -92,16 +99,14 @@ __global__ void k_to_fixed(const double *__restrict__ C, int64_t n, int top, fci
 
 template <bool PAIRS>
 cudaError_t launch(const double *C, int64_t n, int top, fci_split_scalars *sc, void *out, cudaStream_t st) {
-    if (n <= ((int64_t)1 << 14)) {
-        k_fixed_small<PAIRS><<<SMALL_BLOCKS, SMALL_THREADS, 0, st>>>(C, n, top, sc, out);
-        return cudaGetLastError();
-    }
+    if (n <= ((int64_t)1 << 14)) return launch_dependent(true, k_fixed_small<PAIRS>, SMALL_BLOCKS, SMALL_THREADS, 0, st, C, n, top, sc,
+                                out);
     cudaError_t e = cudaMemsetAsync(sc, 0, sizeof *sc, st);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 8);
     k_absmax_bits<<<nb, 256, 0, st>>>(C, n, sc);
-    k_to_fixed<PAIRS><<<nb, 256, 0, st>>>(C, n, top, sc, out);
-    return cudaGetLastError();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_dependent(true, k_to_fixed<PAIRS>, nb, 256, 0, st, C, n, top, sc, out);
 }
 
 }  // namespace

@@ -42,6 +42,7 @@
 
 #include <cuda_fp16.h>
 
+#include "dependent.cuh"
 #include "fci_internal.h"
 #include "oz_gemm.cuh"
 #include "tc_ptx.cuh"
@@ -189,6 +190,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_contract(const __grid_cons
     const int64_t ntiles = (p.N + NT - 1) / NT;
     const int64_t cta = (int64_t)blockIdx.x - cta_lo;
     const int64_t t_begin = ntiles * cta / cta_n, t_end = ntiles * (cta + 1) / cta_n;
+    await_previous();  // C_int; the set-up above reads the operator only
+    // One tile a CTA: the scatter's launch overlaps it.  Larger problems keep the scatter out:
+    // resident beside this CTA's shared memory it would run with the SM's smallest L1.
+    if (t_end - t_begin == 1) admit_next();
 
     if (warp < OZ_PRODUCER_WARPS) {
         // ---------------------------------------------------------------- producers
@@ -420,6 +425,8 @@ __global__ void __launch_bounds__(256) k_scatter_int(uint32_t nsa, uint32_t nsb,
                                                      const double *__restrict__ C, double e_core, int ushift,
                                                      const int *__restrict__ shC, const int *__restrict__ status,
                                                      int *__restrict__ sticky, double *__restrict__ sigma) {
+    await_previous();
+    admit_next();
     const uint32_t ib = blockIdx.x * blockDim.x + threadIdx.x;
     if (ib >= nsb) return;
     const int u = ushift - *shC;
@@ -477,6 +484,8 @@ __global__ void __launch_bounds__(128) k_scatter_int2p(uint32_t nsa, uint32_t ns
                                                        const double *__restrict__ C, double e_core, int ushift,
                                                        const int *__restrict__ shC, const int *__restrict__ status,
                                                        int *__restrict__ sticky, double *__restrict__ sigma) {
+    await_previous();
+    admit_next();
     const uint32_t ib = blockIdx.x * blockDim.x + threadIdx.x;
     if (ib >= nsb) return;
     const int u = ushift - *shC;
@@ -540,6 +549,8 @@ __global__ void __launch_bounds__(256, 6) k_fci_split_rows(uint32_t ndet, uint32
                                                         const int32_t *__restrict__ pairB,
                                                         const int64_t *__restrict__ Cint, uint8_t *__restrict__ Dimg) {
     extern __shared__ int64_t sC[];
+    await_previous();
+    admit_next();
     int32_t *sEa = reinterpret_cast<int32_t *>(sC + nsb);  // [npair_pad]: the row's alpha-move entries
     constexpr uint64_t bias = 0x8080808080808080ull >> (8 * (8 - S));
     constexpr int B_PLANE = OZG_N * KCC * 16;
@@ -698,6 +709,7 @@ int oz_prepare_G(fci_context *h, int s) {
     int rc = fci_dev_alloc(h, &h->d_Gs, img.size() * 2);
     if (rc) return rc;
     FCI_CUDA(h, cudaMemcpy(h->d_Gs, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
+    FCI_CUDA(h, cudaStreamSynchronize(0));  // the copy itself: the contraction reads the image in its prologue
     h->Gs_slices = s;
     h->G_exp = shG;  // stores sh_G
     return FCI_OK;
@@ -767,6 +779,7 @@ static int oz_prepare_Gt(fci_context *h, int s) {
     rc = fci_dev_alloc(h, &h->d_Gt, img.size() * 2);
     if (rc) return rc;
     FCI_CUDA(h, cudaMemcpy(h->d_Gt, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
+    FCI_CUDA(h, cudaStreamSynchronize(0));  // the copy itself: the contraction reads the image in its prologue
     h->Gt_slices = s;
     return FCI_OK;
 }
@@ -837,8 +850,7 @@ static int oz_launch_group(fci_context *h, const OzGroup &grp, int s, int nt, si
     if (!kern) return fci_fail(h, FCI_ERR_UNSUPPORTED, "slice count %d, tile %d", s, nt);
     FCI_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     phase_scope ps(h, st, FCI_PHASE_CONTRACT, 1);
-    kern<<<grp.cta_start[grp.n_jobs], OZ_THREADS, smem, st>>>(grp);
-    FCI_CUDA(h, cudaGetLastError());
+    FCI_CUDA(h, launch_dependent(true, kern, grp.cta_start[grp.n_jobs], OZ_THREADS, smem, st, grp));
     return FCI_OK;
 }
 
@@ -847,11 +859,9 @@ static int oz_finish_job(fci_context *h, const double *C, double *sigma, const O
     phase_scope ps(h, st, FCI_PHASE_SCATTER, 1);
     const int threads = 128;
     dim3 g((unsigned)ceil_div(h->nsb, threads), (unsigned)std::min<int64_t>(h->nsa, 65535));
-    k_scatter_int<<<g, threads, 0, st>>>(h->nsa, h->nsb, h->npair_pad, prm.nt == 32 ? 5 : 6, h->d_pair_a, h->d_pair_b,
-                                       E, prm.npair,
-                                       C, h->e_core,
-                                       8 * prm.L0 - h->G_exp, shC, status, h->d_status, sigma);
-    FCI_CUDA(h, cudaGetLastError());
+    FCI_CUDA(h, launch_dependent(true, k_scatter_int, g, threads, 0, st, h->nsa, h->nsb, h->npair_pad, prm.nt == 32 ? 5 : 6,
+                                 h->d_pair_a, h->d_pair_b, E, prm.npair, C, h->e_core, 8 * prm.L0 - h->G_exp, shC, status,
+                                 h->d_status, sigma));
     return FCI_OK;
 }
 
@@ -894,16 +904,14 @@ static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int
     case S_ * 10 + K_:                                                                                            \
         FCI_CUDA(h, cudaFuncSetAttribute(k_fci_split_rows<S_, K_>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
                                          (int)row_smem));                                                         \
-        k_fci_split_rows<S_, K_><<<gr, 256, row_smem, st>>>((uint32_t)N, (uint32_t)h->nsa, (uint32_t)h->nsb,       \
-                                                            h->npair_pad, n_kc, n_nt, h->d_pair_a, h->d_pair_b,   \
-                                                            Cint, Dimg);                                          \
+        FCI_CUDA(h, launch_dependent(true, k_fci_split_rows<S_, K_>, gr, 256, row_smem, st, N, h->nsa, h->nsb,     \
+                                     h->npair_pad, n_kc, n_nt, h->d_pair_a, h->d_pair_b, Cint, Dimg));            \
         break;
             OZ_SPLIT(2, 2) OZ_SPLIT(3, 2) OZ_SPLIT(4, 2) OZ_SPLIT(5, 2) OZ_SPLIT(6, 2) OZ_SPLIT(7, 2)
             OZ_SPLIT(2, 4) OZ_SPLIT(3, 4) OZ_SPLIT(4, 4) OZ_SPLIT(5, 4) OZ_SPLIT(6, 4) OZ_SPLIT(7, 4)
 #undef OZ_SPLIT
             default: return fci_fail(h, FCI_ERR_UNSUPPORTED, "slice count %d", s);
         }
-        FCI_CUDA(h, cudaGetLastError());
     }
     oz_gemm_args a;
     a.n_mt = 1;

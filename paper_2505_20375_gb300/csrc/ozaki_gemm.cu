@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "dependent.cuh"
 #include "oz_gemm.cuh"
 #include "oz_pipe.cuh"
 #include "tc_ptx.cuh"
@@ -34,6 +35,9 @@ using namespace tc;
 using namespace ozp;
 
 constexpr int OZG_MAX_STAGES = 6;
+// Units up to which the GEMM may start under the digit image's tail (dependent.cuh): gains 2 to 5
+// us at up to 2.9 M determinants (46,000 units); at 11.8 M it lost 20 us of 7,440 (s = 3).
+constexpr int64_t OZG_EARLY_UNITS = 1 << 16;
 constexpr size_t OZG_SMEM_MAX = 232448 - 1024;
 
 struct OzgParams {
@@ -97,16 +101,20 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm(const __grid_cons
     const uint32_t tmem = sh->tmem_base;
     volatile int *abort = &sh->abort;
     const int64_t n_units = p.n_nt * p.n_mt;
+    if (RESA && threadIdx.x == 0) {  // the whole A image, in pieces of at most 32 KB, on its own barrier
+        const uint32_t total = (uint32_t)p.n_kc * STAGE_A, ab = smem_u32(&sh->a_full);
+        mbar_expect_tx(ab, total);
+        for (uint32_t o = 0; o < total; o += 32768u)
+            bulk_g2s(smem_u32(sA + o), p.Gimg + o, total - o < 32768u ? total - o : 32768u, ab);
+    }
+    // The digit image; the set-up above reads the operator only.  No admit_next(): the scatter,
+    // resident early beside this CTA's shared memory, would keep the SM's small L1 (13 orbitals,
+    // s = 6: sigma 2.53 -> 2.75 ms).
+    await_previous();
 
     if (warp == 0) {
         if (lane == 0) {
             // ------------------------------------------------------------ bulk copies
-            if (RESA) {  // the whole A image, in pieces of at most 32 KB, on its own barrier
-                const uint32_t total = (uint32_t)p.n_kc * STAGE_A, ab = smem_u32(&sh->a_full);
-                mbar_expect_tx(ab, total);
-                for (uint32_t o = 0; o < total; o += 32768u)
-                    bulk_g2s(smem_u32(sA + o), p.Gimg + o, total - o < 32768u ? total - o : 32768u, ab);
-            }
             uint32_t q = 0, st = 0, ph = 0;  // stage counter, its ring slot and the slot's use parity
             for (int64_t u = blockIdx.x; u < n_units; u += gridDim.x) {
                 const int64_t nt = u / p.n_mt;
@@ -328,7 +336,7 @@ int oz_gemm_launch(fci_context *h, int s, int w, int kcc, bool resa, const oz_ge
     FCI_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t units = a.n_nt * a.n_mt;
     phase_scope ps(h, st, FCI_PHASE_CONTRACT, 1);
-    kern<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(nsm, units)), ozg_threads(s), smem, st>>>(prm);
-    FCI_CUDA(h, cudaGetLastError());
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nsm, units));
+    FCI_CUDA(h, launch_dependent(units <= OZG_EARLY_UNITS, kern, grid, ozg_threads(s), smem, st, prm));
     return FCI_OK;
 }

@@ -74,3 +74,32 @@ def test_davidson_subspace_sizes(fci_lib, kind, ms):
     r = gpu_fci(p).davidson(max_iter=400, max_subspace=ms, tol_residual=1e-6, tol_energy=1e-12)
     w = np.linalg.eigvalsh(oracle.dense_h(p["hso"], p["gso"], p["dets"]))
     assert r.converged and abs(r.energy - (w[0] + 0.4)) <= max(1e-10, 1e-12 / (w[1] - w[0]))
+
+
+@pytest.mark.parametrize("s", [3, 6])
+@pytest.mark.parametrize("n,na,nb,path", [(6, 3, 3, "fused"), (10, 5, 5, "fused"), (9, 4, 4, "gemm"), (10, 5, 5, "gemm")])
+def test_sigma_calls_back_to_back(fci_lib, monkeypatch, n, na, nb, path, s):
+    """Kernels that start under the one before them: sigma builds queued without a wait, each on
+    the result of the last or on another vector through the same workspace, on two streams in
+    turn, give the bits of builds that are waited for one by one."""
+    monkeypatch.setenv("FCI_OZ_PATH", path)
+    h, g = synth.real_integrals(n, 6, 40 + n)
+    f = gpu_fci(dict(h=h, g=g, e_core=0.2, n=n, na=na, nb=nb))
+    x = [torch.from_numpy(synth.random_vector(f.n_det, seed=k)).cuda() for k in (7, 8)]
+
+    def chain(wait):
+        out, y = [], x[0]
+        for _ in range(12):
+            y = f.sigma(y, precision="oz_bf16", n_slices=s)
+            wait()
+            out += [y, f.sigma(x[1], precision="oz_bf16", n_slices=s)]
+            wait()
+        torch.cuda.synchronize()
+        return out
+
+    ref = chain(torch.cuda.synchronize)
+    f.sync_status()
+    for st in (torch.cuda.current_stream(), torch.cuda.Stream()):
+        with torch.cuda.stream(st):
+            got = chain(lambda: None)
+        assert all(torch.equal(a, b) for a, b in zip(ref, got))
