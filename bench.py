@@ -346,14 +346,15 @@ def run_config(fci, synth, torch, dev, stream, build, precs, dav, peaks, fp64_pe
         ach = work / launches_per_sigma / (cms * 1e-3) / 1e12 if cms > 0 else None
         # FP64, complex and two-pass DAS contractions form the active entries of E only (those a
         # determinant's moves reach): the dense product's rate is then no fraction of a peak
-        active_only = pname == "fp64" or fh.is_complex or das_two_pass
+        active_only = pname == "fp64" or (fh.is_complex and sl > 3) or das_two_pass
         pk = fp64_peak if pname == "fp64" else peaks.get("bf16_tflops", 1891.0)
         rec["roofline"] = {"bound": "alu" if pname == "fp64" else "tensor", "achieved": ach, "peak": pk,
                            "unit": "TFLOP/s", "frac": ach / pk if (ach and pk and not active_only) else None,
                            "kernel": ("k_contract_real / k_contract_spinor (FP64 FMA, active entries)" if pname == "fp64" else
                                       "k_oz_gemm_blk (two-pass DAS, active blocks)" if das_two_pass else
                                       "k_oz_das (fused DAS)" if info["n_categories"] > 0 else
-                                      "k_oz_gemm_blk (complex, real embedding, active blocks)" if fh.is_complex else
+                                      ("k_oz_gemm_blk (complex, real embedding, active blocks)" if active_only else
+                                       "k_oz_gemm (complex, real embedding)") if fh.is_complex else
                                       "alpha/beta split contraction"),
                            "flops_counted": ("dense equivalent: " if active_only else "algorithmic: ") +
                                             "the contraction's multiply-adds over n_pair x n_pair x N_K" +

@@ -84,7 +84,8 @@ struct fci_das_layout {
     // pair of each position of its 16-wide blocks (-1: padding), and per category of the
     // intermediate space the mask of blocks that connect it with the target space
     void *d_dg_G = nullptr;
-    int dg_slices = 0, dg_shG = 0;
+    int dg_slices = 0, dg_shG = 0;  // 100 + s: G in the layout of the dense form
+    mutable double dg_share = -1.0;  // MMA work of the block-sparse form over that of the dense one (-1: not yet known)
     int32_t *d_dg_perm = nullptr;  // [16 n_blk]
     ulonglong2 *d_dg_mask = nullptr;  // [n_cat_int]
     // kernel configuration chosen by the tuner for dz_tuned_slices (0: none)

@@ -195,6 +195,57 @@ __global__ void __launch_bounds__(256) k_cz_split(const CzBlocks bl, int64_t nde
     }
 }
 
+// Dense form, digit image: block (N-tile nt, K-chunk kc) holds S planes of 64 determinants x 32
+// real-embedded K, each in canonical K-major core matrices (8 rows x 16 bytes; core
+// (row / 8, k / 8) at ((row / 8) * 4 + k / 8) * 128).  One CTA of 256 threads fills one
+// block: thread t covers determinant t % 64 and core t / 64 (4 complex pairs = 8 reals).
+template <int S>
+__global__ void __launch_bounds__(256) k_cz_split_dense(int n, int64_t ndet, int n_kc, int64_t n_blocks,
+                                                  const uint64_t *__restrict__ str,
+                                                  const uint64_t *__restrict__ binom,
+                                                  const int64_t *__restrict__ Cint, uint8_t *__restrict__ Dimg) {
+    uint64_t bias = 0;
+#pragma unroll
+    for (int j = 0; j < S; ++j) bias |= (uint64_t)64 << (7 * j);
+    const int row = threadIdx.x & 63, cc = threadIdx.x >> 6;
+    const int n2 = n * n;
+    for (int64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
+        const int64_t nt = blk / n_kc;
+        const int kc = (int)(blk - nt * n_kc);
+        const int64_t K = nt * CZ_N + row;
+        uint64_t y[8];
+        const uint32_t Sm = K < ndet ? (uint32_t)__ldg(str + K) : 0u;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int x = (kc * 32 + cc * 8) / 2 + e;  // complex pair index
+            int64_t vr = 0, vi = 0;
+            if (K < ndet && x < n2) {
+                const int a = x / n, b = x - a * n;
+                if (((Sm >> a) & 1u) && (b == a || !((Sm >> b) & 1u))) {
+                    const uint32_t T = (Sm & ~(1u << a)) | (1u << b);
+                    const int64_t t = cz_rank(T, binom);
+                    const int64_t cr = __ldg(Cint + 2 * t), ci = __ldg(Cint + 2 * t + 1);
+                    const bool neg = cz_sign(Sm, a, b);
+                    vr = neg ? -cr : cr;
+                    vi = neg ? -ci : ci;
+                }
+            }
+            y[2 * e] = (uint64_t)vr + bias;
+            y[2 * e + 1] = (uint64_t)vi + bias;
+        }
+        uint8_t *base = Dimg + (size_t)blk * S * 4096 + ((row >> 3) * 4 + cc) * 128 + (row & 7) * 16;
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+            uint4 w;
+            w.x = digits7_f16x2(y[0], y[1], j);
+            w.y = digits7_f16x2(y[2], y[3], j);
+            w.z = digits7_f16x2(y[4], y[5], j);
+            w.w = digits7_f16x2(y[6], y[7], j);
+            __stcs((uint4 *)(base + j * 4096), w);  // streaming: keep C_int in L2
+        }
+    }
+}
+
 // sigma_I = scale * sum over the replacements of I of sign * E_int[x, T] (complex parts in
 // rows 2x and 2x + 1 of the tile-major E image) + e_core C_I.
 __global__ void __launch_bounds__(128) k_cz_scatter(int n, int64_t ndet, int M_pad, const uint64_t *__restrict__ str,
@@ -242,6 +293,33 @@ uint16_t half_bits_of_small_int(int d) {  // IEEE binary16 of an integer |d| <= 
     return (uint16_t)(sign | ((unsigned)(e + 15) << 10) | mant);
 }
 
+// The dense form: all 2 n^2 rows and columns, M-tiles of 128, K-chunks of 32.
+struct CzGeom {
+    int M_real, n_mt, n_kc;
+};
+CzGeom cz_geom(const fci_context *h) {
+    const int m = 2 * h->n_orb * h->n_orb;
+    return {m, (int)ceil_div(m, OZG_M), (int)ceil_div(m, 32)};
+}
+
+// Which form: the block-sparse GEMM skips half of the MMAs and more, but copies its operator
+// block by block and costs about 3,000 cycles a unit, so it needs many MMAs per unit (slices),
+// many blocks to skip (spinors) and tiles enough to fill the GPU.  us, dense / blocks:
+//   spinors, electrons   s = 3          4              5              6              8
+//   12, 6                108/136        109/140        115/143        119/144        124/152
+//   17, 9                406/538        460/542        529/637        605/644        793/789
+//   19, 9                1,035/1,389    1,296/1,386    1,648/1,752    2,053/1,774    3,012/2,313
+//   20, 10               2,062/2,574    2,710/2,566    3,607/3,331    4,624/3,402    7,031/4,521
+//   22, 5                680/826        825/830        1,011/998      1,224/1,013    1,711/1,272
+//   22, 11               9,664/10,843   13,059/10,780  17,897/14,249  (s = 8 36,463/19,269)
+// 19 spinors with 5 electrons (11,628 determinants) take 473/511 at s = 6.
+// FCI_SPLIT_FORM=dense or blocks overrides it (for tests).
+bool cz_dense(const fci_context *h, int s) {
+    if (!oz_gemm_ring(s, 4, 0)) return false;
+    if (const char *env = getenv("FCI_SPLIT_FORM")) return strcmp(env, "dense") == 0;
+    return s <= 3 || h->n_orb < (s <= 5 ? 20 : 18) || h->ndet < ((int64_t)1 << 14);
+}
+
 }  // namespace
 
 int cz_check(fci_context *h, int s) {
@@ -259,8 +337,11 @@ int cz_check(fci_context *h, int s) {
 // Real-embedded G digit image in the A layout of the block-sparse GEMM, followed by the row
 // map (row of E of each position of a row block).
 static int cz_prepare_G(fci_context *h, int s) {
-    if (h->Gs_slices == s && h->d_Gs) return FCI_OK;
+    const bool dense = cz_dense(h, s);
+    const int key = s + (dense ? 100 : 0);
+    if (h->Gs_slices == key && h->d_Gs) return FCI_OK;
     const CzBlocks bl = cz_blocks(h->n_orb);
+    const CzGeom g = cz_geom(h);
     const int n = h->n_orb, n2 = n * n, np = bl.n_blk * 16;
     std::vector<double> G((size_t)n2 * n2 * 2);
     if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -284,7 +365,9 @@ static int cz_prepare_G(fci_context *h, int s) {
             }
         }
     const size_t map_off = (size_t)bl.n_blk * bl.n_blk * s * 512;
-    std::vector<uint16_t> img(map_off / 2 + (size_t)np * 2, 0);
+    std::vector<uint16_t> img;
+    if (!dense) img.assign(map_off / 2 + (size_t)np * 2, 0);
+    else img.assign((size_t)g.n_mt * g.n_kc * s * 4096, 0);
     for (int pr = 0; pr < np; ++pr)
         for (int pc = 0; pc < np; ++pc) {
             if (row[pr] < 0 || col[pc] < 0) continue;
@@ -292,28 +375,42 @@ static int cz_prepare_G(fci_context *h, int s) {
             const double gr = G[2 * ((size_t)x * n2 + y)], gi = G[2 * ((size_t)x * n2 + y) + 1];
             const int64_t gi64 = llrint(ldexp(u == w ? gr : (u == 0 ? -gi : gi), shG));
             const uint64_t yb = (uint64_t)gi64 + bias;
-            const int r = pr & 15, c = pc & 15;
-            const size_t off = ((size_t)(pr >> 4) * bl.n_blk + (pc >> 4)) * s * 512 + (size_t)(r >> 3) * s * 256 +
-                               (c >> 3) * 128 + (r & 7) * 16 + (c & 7) * 2;
+            size_t off, plane;
+            if (dense) {  // [M-tile][K-chunk][plane][128 x 32]
+                const int m = row[pr], k = col[pc], r = m % OZG_M, c = k % 32;
+                off = ((size_t)(m / OZG_M) * g.n_kc + k / 32) * s * 8192 + ((r >> 3) * 4 + (c >> 3)) * 128 + (r & 7) * 16 +
+                      (c & 7) * 2;
+                plane = 8192;
+            } else {
+                const int r = pr & 15, c = pc & 15;
+                off = ((size_t)(pr >> 4) * bl.n_blk + (pc >> 4)) * s * 512 + (size_t)(r >> 3) * s * 256 + (c >> 3) * 128 +
+                      (r & 7) * 16 + (c & 7) * 2;
+                plane = 256;
+            }
             for (int j = 0; j < s; ++j)
-                img[(off + (size_t)j * 256) / 2] = half_bits_of_small_int((int)((yb >> (7 * j)) & 0x7F) - 64);
+                img[(off + (size_t)j * plane) / 2] = half_bits_of_small_int((int)((yb >> (7 * j)) & 0x7F) - 64);
         }
-    memcpy(reinterpret_cast<char *>(img.data()) + map_off, row.data(), (size_t)np * 4);
+    if (!dense) memcpy(reinterpret_cast<char *>(img.data()) + map_off, row.data(), (size_t)np * 4);
     fci_dev_free(h->d_Gs);
     h->d_Gs = nullptr;
     h->Gs_slices = 0;
     int rc = fci_dev_alloc(h, &h->d_Gs, img.size() * 2);
     if (rc) return rc;
     FCI_CUDA(h, cudaMemcpy(h->d_Gs, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
-    h->Gs_slices = s;
+    h->Gs_slices = key;
     h->G_exp = shG;
     return FCI_OK;
+}
+
+// 2 KB units per slice of a tile's digit image.
+static size_t cz_image_blocks(const fci_context *h, int s) {
+    return cz_dense(h, s) ? 2 * (size_t)cz_geom(h).n_kc : (size_t)cz_blocks(h->n_orb).n_blk;
 }
 
 // C_int, the D digit image, E_int, the block masks, 256 bytes of scalars.
 size_t cz_workspace_bytes(const fci_context *h, int s) {
     const size_t n_nt = (size_t)ceil_div(h->ndet, CZ_N), n2 = (size_t)h->n_orb * h->n_orb;
-    return al256((size_t)h->ndet * 16) + al256(n_nt * cz_blocks(h->n_orb).n_blk * s * 2048) +
+    return al256((size_t)h->ndet * 16) + al256(n_nt * cz_image_blocks(h, s) * s * 2048) +
            al256(n_nt * 2 * n2 * CZ_N * 8) + al256(n_nt * sizeof(ulonglong2)) + 256;
 }
 
@@ -325,11 +422,13 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
     const CzBlocks bl = cz_blocks(h->n_orb);
     const int64_t n_nt = ceil_div(h->ndet, CZ_N);
     const int M_real = 2 * h->n_orb * h->n_orb;
+    const bool dense = cz_dense(h, s);
+    const CzGeom g = cz_geom(h);
     char *p = (char *)ws;
     int64_t *Cint = (int64_t *)p;
     p += al256((size_t)h->ndet * 16);
     uint8_t *Dimg = (uint8_t *)p;
-    p += al256((size_t)n_nt * bl.n_blk * s * 2048);
+    p += al256((size_t)n_nt * cz_image_blocks(h, s) * s * 2048);
     int64_t *E = (int64_t *)p;
     p += al256((size_t)n_nt * M_real * CZ_N * 8);
     ulonglong2 *masks = (ulonglong2 *)p;
@@ -339,14 +438,32 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
     {
         phase_scope ps(h, st, FCI_PHASE_GATHER, 3);
         FCI_CUDA(h, launch_fixed_point(C, 2 * h->ndet, 7 * s - 3, sc, Cint, st));
+        const int64_t n_img = n_nt * g.n_kc;  // dense form
+        const unsigned gb = (unsigned)std::min<int64_t>(n_img, 152 * 16);
         switch (s) {
-#define CZ_SPLIT(S_) case S_: k_cz_split<S_><<<(unsigned)n_nt, 256, 0, st>>>(bl, h->ndet, h->d_str_a, h->d_binom, Cint, Dimg, masks); break;
+#define CZ_SPLIT(S_)                                                                                                  \
+    case S_:                                                                                                          \
+        if (dense) k_cz_split_dense<S_><<<gb, 256, 0, st>>>(h->n_orb, h->ndet, g.n_kc, n_img, h->d_str_a, h->d_binom, Cint, Dimg); \
+        else k_cz_split<S_><<<(unsigned)n_nt, 256, 0, st>>>(bl, h->ndet, h->d_str_a, h->d_binom, Cint, Dimg, masks);   \
+        break;
             CZ_SPLIT(2) CZ_SPLIT(3) CZ_SPLIT(4) CZ_SPLIT(5) CZ_SPLIT(6) CZ_SPLIT(7) CZ_SPLIT(8)
 #undef CZ_SPLIT
         }
         FCI_CUDA(h, cudaGetLastError());
     }
-    {
+    if (dense) {
+        oz_gemm_args a;
+        a.n_mt = g.n_mt;
+        a.n_kc = g.n_kc;
+        a.M_pad = M_real;
+        a.M_real = M_real;
+        a.n_nt = n_nt;
+        a.Gimg = h->d_Gs;
+        a.Dimg = Dimg;
+        a.E = E;
+        a.status = status;
+        if ((rc = oz_gemm_launch(h, s, 7, 4, false, a, st))) return rc;
+    } else {
         oz_blk_args a;
         a.n_blk = bl.n_blk;
         a.M_pad = M_real;

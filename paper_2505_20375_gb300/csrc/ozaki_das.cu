@@ -983,6 +983,11 @@ int dz_num_sms(fci_context *h, int *nsm) {
 namespace {
 
 constexpr int DG_BLK = 2048;  // bytes per slice of one (tile, block): 64 determinants x 16 pairs, f16
+// dense form: all pairs, in chunks of 32
+constexpr int DG_KCC = 4;                      // core matrices (8 pairs) per K-chunk of the GEMM
+constexpr int DG_KW = 8 * DG_KCC;              // 32 pairs per K-chunk
+constexpr int DG_B_PLANE = OZG_N * DG_KW * 2;  // 4 KB: 64 determinants x 32 pairs, f16
+constexpr int DG_A_PLANE = OZG_M * DG_KW * 2;  // 8 KB: 128 pair rows x 32 pairs, f16
 
 // The pairs of the layout in blocks of 16: space pairs (classes) fill whole blocks first,
 // their remainders share blocks (largest first into the first block with room).
@@ -1070,8 +1075,48 @@ void dg_category_masks(const fci_context *h, const DgBlocks &b, std::vector<ulon
     }
 }
 
+// Which form.  share: MMA work of the block-sparse GEMM over that of the dense one, which has
+// the larger tiles (fewer, larger copies; no cost per unit), so the blocks pay where they skip
+// much or the space is large, and sooner with more slices.  us, dense / blocks:
+//   share   intermediate determinants   s = 4          s = 6
+//   0.17    2,832                       35/56          37/59
+//   0.25    82,996                      101/129        127/146
+//   0.05    295,488                     209/179        292/194
+//   0.26    388,080                     276/357        385/414
+//   0.36    684,288                     468/513        661/612
+//   0.43    810,688                     632/857        859/1,058
+//   0.17    2,191,360                   2,714/1,934    4,516/2,429
+//   0.43    3,133,440                   4,450/4,686    7,026/6,304
+//   0.30    4,069,504                   3,169/2,721    4,702/3,265
+//   0.64    8,589,600                   8,312/8,653    11,430/11,160
+// FCI_SPLIT_FORM=dense or blocks overrides it (for tests).
+bool dg_dense(const fci_context *h, const DgBlocks &b, int s) {
+    if (!oz_gemm_ring(s, DG_KCC, 0)) return false;
+    if (const char *env = getenv("FCI_SPLIT_FORM")) return strcmp(env, "dense") == 0;
+    const fci_das_layout &L = h->das;
+    if (L.dg_share < 0.0) {
+        std::vector<ulonglong2> masks;
+        dg_category_masks(h, b, masks);
+        double sum = 0.0;
+        for (int c = 0; c < L.n_cat_int; ++c) {
+            const double len = (double)L.pat_nstr_a[L.cat_pa[c]] * (double)L.pat_nstr_b[L.cat_pb[c]];
+            const int on = __builtin_popcountll(masks[c].x) + __builtin_popcountll(masks[c].y);
+            sum += len * on * on;
+        }
+        const int np = h->npair;
+        L.dg_share = sum / std::max<double>(1.0, (double)L.n_det_int) /
+                     ((double)(8 * ceil_div(np, OZG_M)) * (double)(2 * ceil_div(np, DG_KW)));
+    }
+    const double x = L.dg_share;
+    const int64_t n = L.n_det_int;
+    const bool blocks = s <= 5 ? (x < 0.32 && n >= ((int64_t)1 << 20)) || (x < 0.1 && n >= ((int64_t)1 << 17))
+                               : n >= ((int64_t)1 << 21) || (x < 0.4 && n >= ((int64_t)1 << 19)) ||
+                                     (x < 0.1 && n >= ((int64_t)1 << 16));
+    return !blocks;
+}
+
 struct DgGeom {
-    int n_blk;
+    int n_blk;  // 2 KB units per slice of a tile's digit image
     int64_t e_cap, d_cap;  // determinants per E chunk and per digit-image piece (multiples of 64)
     int n_echunks;
 };
@@ -1099,6 +1144,7 @@ struct DgSplit {
     int64_t a0, len;   // intermediate addresses [a0, a0 + len) of this piece
     int64_t n_nt;      // tiles of 64
     int n_blk, n_cat_int, n_pat_b;
+    int n_kc, npair_pad;  // dense form
     int64_t nla, nlb;
     const int32_t *repA, *repB;
     const int32_t *perm;        // [16 n_blk]: pair of each block position, -1: padding
@@ -1352,6 +1398,78 @@ __global__ void __launch_bounds__(DG_ROW_THREADS, 2) k_dg_rows(const __grid_cons
     }
 }
 
+// Dense form, digit image of one piece: tile nt (64 determinants) holds, per K-chunk of 32
+// pairs, S f16 planes of 64 x 32 in canonical K-major core matrices.  Thread t covers
+// determinant t % 64 of the tile (decoded once: category, patterns, local indices) and
+// pairs 8 (t / 64) .. 8 (t / 64) + 7 of every chunk; D_int of a pair is the alpha move's
+// and the beta move's signed C_int (zero where the move leaves the target space or does
+// not exist; replacement-table rows past n_pair_pad count as absent).  Capped at 64
+// registers for four resident blocks per SM (measured 4% faster than three at C3').
+template <int S>
+__global__ void __launch_bounds__(64 * DG_KCC, 4) k_dg_split_dense(const __grid_constant__ DgSplit a) {
+    constexpr uint64_t bias = 0x8080808080808080ull >> (8 * (8 - S));
+    const int row = threadIdx.x & 63, cc = threadIdx.x >> 6;
+    const int npb = a.n_pat_b;
+    for (int64_t nt = blockIdx.x; nt < a.n_nt; nt += gridDim.x) {
+        const int64_t off = nt * OZG_N + row;
+        const bool live = off < a.len;
+        int32_t pa = 0, pb = 0, la = 0, lb = 0, nb = 1;
+        int64_t ida = 0, idb = 0;
+        if (live) {
+            const int64_t addr = a.a0 + off;
+            const int c = find_cat(a.cat_off, a.n_cat_int, addr);
+            pa = __ldg(a.cat_pa + c);
+            pb = __ldg(a.cat_pb + c);
+            nb = __ldg(a.nstr_b32 + pb);
+            const int32_t rr = (int32_t)(addr - __ldg(a.cat_off + c));
+            la = rr / nb;
+            lb = rr - la * nb;
+            ida = __ldg(a.locbase_a + pa) + la;
+            idb = __ldg(a.locbase_b + pb) + lb;
+        }
+        uint8_t *tile = a.Dimg + (size_t)nt * a.n_kc * S * DG_B_PLANE + ((row >> 3) * DG_KCC + cc) * 128 + (row & 7) * 16;
+#pragma unroll 1
+        for (int kc = 0; kc < a.n_kc; ++kc) {
+            const int rs0 = kc * DG_KW + cc * 8;
+            int32_t ea[8], eb[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const bool ok = live && rs0 + e < a.npair_pad;
+                ea[e] = ok ? __ldg(a.repA + (int64_t)(rs0 + e) * a.nla + ida) : -1;
+                eb[e] = ok ? __ldg(a.repB + (int64_t)(rs0 + e) * a.nlb + idb) : -1;
+            }
+            int32_t Ka[8], Kb[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int32_t ba = ea[e] >= 0 ? __ldg(a.base_tgt + (ea[e] >> 23) * npb + pb) : -1;
+                const int32_t bb = eb[e] >= 0 ? __ldg(a.base_tgt + pa * npb + (eb[e] >> 23)) : -1;
+                Ka[e] = ba >= 0 ? ba + ((ea[e] >> 1) & DZ_LOC_MASK) * nb + lb : -1;
+                Kb[e] = bb >= 0 ? bb + la * __ldg(a.nstr_b32 + (eb[e] >> 23)) + ((eb[e] >> 1) & DZ_LOC_MASK) : -1;
+            }
+            uint32_t ylo[8], yhi[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int64_t xa = Ka[e] >= 0 ? __ldg(a.Cint + Ka[e]) : 0;
+                const int64_t xb = Kb[e] >= 0 ? __ldg(a.Cint + Kb[e]) : 0;
+                const int64_t v = ((ea[e] & 1) ? -xa : xa) + ((eb[e] & 1) ? -xb : xb);
+                const uint64_t y = (uint64_t)v + bias;
+                ylo[e] = (uint32_t)y;
+                yhi[e] = (uint32_t)(y >> 32);
+            }
+            uint8_t *base = tile + (size_t)kc * S * DG_B_PLANE;
+#pragma unroll
+            for (int j = 0; j < S; ++j) {
+                const uint32_t bj = (uint32_t)(j & 3), sel = bj | ((4u + bj) << 8);
+                uint32_t w[4];
+#pragma unroll
+                for (int e = 0; e < 8; e += 2)
+                    w[e / 2] = j < 4 ? digits_f16x2(ylo[e], ylo[e + 1], sel) : digits_f16x2(yhi[e], yhi[e + 1], sel);
+                __stcs((uint4 *)(base + j * DG_B_PLANE), make_uint4(w[0], w[1], w[2], w[3]));
+            }
+        }
+    }
+}
+
 // Shared memory of k_dg_rows; the longest row over the alpha patterns.
 size_t dg_row_smem(const DgSplit &a) { return (size_t)a.row_max * 8 + (size_t)(a.n_pat_b + 48 * a.n_blk) * 4; }
 int64_t dg_row_max(const fci_das_layout &L) {
@@ -1368,7 +1486,11 @@ int64_t dg_row_max(const fci_das_layout &L) {
 // Digit image and block masks of a piece.  By rows where two CTAs' rows fit an SM (up to
 // about 14,000 target values per alpha string), else determinant by determinant.
 template <int S>
-cudaError_t dg_image_s(const DgSplit &a, cudaStream_t st) {
+cudaError_t dg_image_s(const DgSplit &a, bool dense, cudaStream_t st) {
+    if (dense) {
+        k_dg_split_dense<S><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(a.n_nt, 152 * 16)), 64 * DG_KCC, 0, st>>>(a);
+        return cudaGetLastError();
+    }
     const size_t smem = dg_row_smem(a);
     if (smem > DG_ROW_SMEM) {
         k_dg_split<S><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(a.n_nt, 152 * 16)), 256, 0, st>>>(a);
@@ -1380,18 +1502,18 @@ cudaError_t dg_image_s(const DgSplit &a, cudaStream_t st) {
     k_dg_rows<S><<<(unsigned)a.nla, DG_ROW_THREADS, smem, st>>>(a);
     return cudaGetLastError();
 }
-cudaError_t dg_image(const DgSplit &a, int s, cudaStream_t st) {
+cudaError_t dg_image(const DgSplit &a, int s, bool dense, cudaStream_t st) {
     switch (s) {
-        case 4: return dg_image_s<4>(a, st);
-        case 5: return dg_image_s<5>(a, st);
-        case 6: return dg_image_s<6>(a, st);
-        case 7: return dg_image_s<7>(a, st);
-        default: return dg_image_s<8>(a, st);
+        case 4: return dg_image_s<4>(a, dense, st);
+        case 5: return dg_image_s<5>(a, dense, st);
+        case 6: return dg_image_s<6>(a, dense, st);
+        case 7: return dg_image_s<7>(a, dense, st);
+        default: return dg_image_s<8>(a, dense, st);
     }
 }
 
 // The block plan's device tables and the G digit slices in the A layout of the block-sparse GEMM.
-int dg_prepare(fci_context *h, int s, const DgBlocks &b) {
+int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense) {
     fci_das_layout &L = h->das;
     int rc = FCI_OK;
     if (!L.d_dg_mask) {
@@ -1406,7 +1528,8 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b) {
         L.d_dg_mask = dm;
         FCI_CUDA(h, cudaMemcpy(dm, masks.data(), masks.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
     }
-    if (L.dg_slices == s && L.d_dg_G) return FCI_OK;
+    const int key = s + (dense ? 100 : 0);
+    if (L.dg_slices == key && L.d_dg_G) return FCI_OK;
     const int np = h->npair, nb = b.n_blk();
     std::vector<double> G((size_t)np * np);
     if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -1417,17 +1540,27 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b) {
     if (gmax > 0) frexp(gmax, &eG);  // gmax < 2^eG
     const int shG = 8 * s - 2 - eG;
     const uint64_t bias = 0x8080808080808080ull >> (8 * (8 - s));
-    std::vector<uint16_t> img((size_t)nb * nb * s * 256, 0);
+    const int n_kc = (int)ceil_div(np, DG_KW);
+    std::vector<uint16_t> img(dense ? (size_t)ceil_div(np, OZG_M) * n_kc * s * DG_A_PLANE / 2 : (size_t)nb * nb * s * 256, 0);
     for (int pr = 0; pr < 16 * nb; ++pr)
         for (int pc = 0; pc < 16 * nb; ++pc) {
             if (b.perm[pr] < 0 || b.perm[pc] < 0) continue;
             const int64_t gi = llrint(ldexp(G[(size_t)b.perm[pr] * np + b.perm[pc]], shG));
             const uint64_t y = (uint64_t)gi + bias;
-            const int r = pr & 15, c = pc & 15;
-            const size_t off = ((size_t)(pr >> 4) * nb + (pc >> 4)) * s * 512 + (size_t)(r >> 3) * s * 256 + (c >> 3) * 128 +
-                               (r & 7) * 16 + (c & 7) * 2;
+            size_t off, plane;
+            if (dense) {  // [M-tile][K-chunk][plane][128 x 32]
+                const int m = b.perm[pr], k = b.perm[pc], r = m % OZG_M, c = k % DG_KW;
+                off = ((size_t)(m / OZG_M) * n_kc + k / DG_KW) * s * DG_A_PLANE + ((r >> 3) * DG_KCC + (c >> 3)) * 128 +
+                      (r & 7) * 16 + (c & 7) * 2;
+                plane = DG_A_PLANE;
+            } else {
+                const int r = pr & 15, c = pc & 15;
+                off = ((size_t)(pr >> 4) * nb + (pc >> 4)) * s * 512 + (size_t)(r >> 3) * s * 256 + (c >> 3) * 128 +
+                      (r & 7) * 16 + (c & 7) * 2;
+                plane = 256;
+            }
             for (int j = 0; j < s; ++j)
-                img[(off + (size_t)j * 256) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
+                img[(off + (size_t)j * plane) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
         }
     fci_dev_free(L.d_dg_G);
     L.d_dg_G = nullptr;
@@ -1435,7 +1568,7 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b) {
     rc = fci_dev_alloc(h, &L.d_dg_G, img.size() * 2);
     if (rc) return rc;
     FCI_CUDA(h, cudaMemcpy(L.d_dg_G, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
-    L.dg_slices = s;
+    L.dg_slices = key;
     L.dg_shG = shG;
     return FCI_OK;
 }
@@ -1464,7 +1597,9 @@ int das_split_check(fci_context *h, int s) { return s <= 3 ? dz_check(h, s) : dg
 // C_int, the D digit image and block masks of a piece, E_int of a chunk, the partial sums
 // kept across chunks, 256 bytes of scalars.
 size_t dg_workspace_bytes(const fci_context *h, int s) {
-    const DgGeom g = dg_geom(h, std::max(s, 4), dg_blocks(h).n_blk());
+    const DgBlocks blk = dg_blocks(h);
+    const int s4 = std::max(s, 4);
+    const DgGeom g = dg_geom(h, s4, dg_dense(h, blk, s4) ? 2 * (int)ceil_div(h->npair, DG_KW) : blk.n_blk());
     size_t b = al256((size_t)h->das.n_det * 8) + al256((size_t)(g.d_cap / OZG_N) * g.n_blk * std::max(s, 4) * DG_BLK) +
                al256((size_t)(g.d_cap / OZG_N) * sizeof(ulonglong2)) + al256((size_t)g.e_cap * h->npair * 8);
     if (g.n_echunks > 1) b += al256((size_t)h->das.n_det * 8);
@@ -1476,10 +1611,12 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     if (rc) return rc;
     const DgBlocks blk = dg_blocks(h);
     rc = dz_prepare_tables(h, st);
-    if (!rc) rc = dg_prepare(h, s, blk);
+    const bool dense = dg_dense(h, blk, s);
+    const int n_kc = (int)ceil_div(h->npair, DG_KW);
+    if (!rc) rc = dg_prepare(h, s, blk, dense);
     if (rc) return rc;
     const fci_das_layout &L = h->das;
-    const DgGeom g = dg_geom(h, s, blk.n_blk());
+    const DgGeom g = dg_geom(h, s, dense ? 2 * n_kc : blk.n_blk());
     char *p = (char *)ws;
     int64_t *Cint = (int64_t *)p;
     p += al256((size_t)L.n_det * 8);
@@ -1502,7 +1639,9 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     }
     const size_t npab = (size_t)L.n_pat_a * L.n_pat_b;
     DgSplit sp;
-    sp.n_blk = g.n_blk;
+    sp.n_blk = blk.n_blk();
+    sp.n_kc = n_kc;
+    sp.npair_pad = h->npair_pad;
     sp.n_cat_int = L.n_cat_int;
     sp.n_pat_b = L.n_pat_b;
     sp.nla = dz_nloc(L.pat_nstr_a);
@@ -1532,17 +1671,32 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
             sp.n_nt = ceil_div(sp.len, OZG_N);
             {
                 phase_scope ps(h, st, FCI_PHASE_GATHER, 2);
-                FCI_CUDA(h, dg_image(sp, s, st));
+                FCI_CUDA(h, dg_image(sp, s, dense, st));
+            }
+            int64_t *Ep = E + (size_t)(d0 / OZG_N) * h->npair * OZG_N;
+            if (dense) {
+                oz_gemm_args a;
+                a.n_mt = (int)ceil_div(h->npair, OZG_M);
+                a.n_kc = n_kc;
+                a.M_pad = h->npair;
+                a.M_real = h->npair;
+                a.n_nt = sp.n_nt;
+                a.Gimg = L.d_dg_G;
+                a.Dimg = Dimg;
+                a.E = Ep;
+                a.status = status;
+                if ((rc = oz_gemm_launch(h, s, 8, DG_KCC, false, a, st))) return rc;
+                continue;
             }
             oz_blk_args a;
-            a.n_blk = g.n_blk;
+            a.n_blk = blk.n_blk();
             a.M_pad = h->npair;  // E row stride: the n_pair rows of each tile, no padding
             a.n_nt = sp.n_nt;
             a.Gimg = L.d_dg_G;
             a.Dimg = Dimg;
             a.masks = masks;
             a.rowmap = L.d_dg_perm;
-            a.E = E + (size_t)(d0 / OZG_N) * h->npair * OZG_N;
+            a.E = Ep;
             a.status = status;
             if ((rc = oz_blk_launch(h, s, 8, a, st))) return rc;
         }
@@ -1603,6 +1757,7 @@ void dz_free(fci_das_layout &L) {
     L.d_dg_G = nullptr;
     L.dz_slices = 0;
     L.dg_slices = 0;
+    L.dg_share = -1.0;
 }
 
 size_t dz_workspace_bytes(const fci_context *h, int s) {

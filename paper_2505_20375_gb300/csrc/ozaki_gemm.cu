@@ -310,6 +310,7 @@ int oz_gemm_launch(fci_context *h, int s, int w, int kcc, bool resa, const oz_ge
     void (*kern)(const OzgParams) = nullptr;
     if (w == 8 && kcc == 2 && resa) kern = oz_gemm_kernel<8, 2, true>(s);
     if (w == 8 && kcc == 4 && !resa) kern = oz_gemm_kernel<8, 4, false>(s);
+    if (w == 7 && kcc == 4 && !resa) kern = oz_gemm_kernel<7, 4, false>(s);
     if (resa && a.n_mt != 1) kern = nullptr;
     const int ring = oz_gemm_ring(s, kcc, resa ? a.n_kc : 0);
     if (!kern || !ring) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split GEMM: %d slices of %d bits (K-chunk %d, resident %d)", s, w, 8 * kcc, (int)resa);

@@ -103,3 +103,26 @@ def test_sigma_calls_back_to_back(fci_lib, monkeypatch, n, na, nb, path, s):
         with torch.cuda.stream(st):
             got = chain(lambda: None)
         assert all(torch.equal(a, b) for a, b in zip(ref, got))
+
+
+@pytest.mark.parametrize("s", [4, 6, 8])
+@pytest.mark.parametrize("layout", ["spinor", "das one M-tile", "das two M-tiles"])
+def test_dense_and_block_forms_agree(fci_lib, monkeypatch, layout, s):
+    """The two forms of the contraction (every pair, or the blocks a tile uses) give the same
+    bits, each with a workspace of its own size, also when one handle changes between them."""
+    if layout == "spinor":
+        h, g = synth.complex_integrals(11, 6, 71)
+        f = gpu_fci(dict(h=h, g=g, e_core=0.3, n=11, ne=4))
+    else:
+        spaces, ref, nel = ([3, 3, 3], [1, 1, 1], 3) if layout == "das one M-tile" else ([6, 5, 5], [1, 1, 0], 2)
+        h, g = synth.real_integrals(sum(spaces), 6, 72)  # 45 and 136 pairs
+        f = gpu_fci(dict(h=h, g=g, e_core=0.3, n=sum(spaces), na=nel, nb=nel)).build_das(spaces, ref, ref, 1)
+        if s * f.info["n_pair"] > 1023:
+            pytest.skip("more slices than the level sums hold")
+    c = torch.from_numpy(synth.random_vector(f.n_det, seed=7, complex_=f.is_complex)).cuda()
+    out = []
+    for form in ("dense", "blocks", "dense"):
+        monkeypatch.setenv("FCI_SPLIT_FORM", form)
+        out.append(f.sigma(c, precision="oz_bf16", n_slices=s))
+        f.sync_status()
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
