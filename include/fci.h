@@ -430,8 +430,8 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
 /* ------------------------------------------------------- allocation-free sigma */
 
 /* sigma = H C for ONE vector in FP64, like fci_sigma with precision FCI_PREC_FP64, but
- * with its scratch (the D and E intermediates, 2 x n_pair x n_det elements) in a
- * fixed 64 MiB device array inside libfci instead of a caller workspace.  The paper
+ * with its scratch (the E intermediate; the size limit counts 2 x n_pair x n_det elements)
+ * in a fixed 64 MiB device array inside libfci instead of a caller workspace.  The paper
  * has no counterpart; this exists for callers that cannot allocate device memory when
  * they need sigma: a process whose framework already reserved the device memory pool,
  * code running where CUDA allocation calls are not allowed (e.g. a host callback on a
