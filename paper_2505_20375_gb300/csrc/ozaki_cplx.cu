@@ -27,7 +27,9 @@
 // away), and the scatter sums in int64:
 //   sigma_I = 2^{7 L0 - sh_G - sh_C} sum <I|E_x|K> E_int[x, K] + e_core C_I.
 //
-// The GEMM itself is the block-sparse bulk-copy kernel (ozaki_blk.cu) with 7-bit digits.
+// The GEMM itself is the block-sparse bulk-copy kernel (ozaki_blk.cu) with 7-bit digits, or,
+// where that has too little to skip (cz_dense), the dense one (ozaki_gemm.cu) on images of all
+// pairs; sigma has the same bits.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>

@@ -980,6 +980,9 @@ int dz_num_sms(fci_context *h, int *nsm) {
 // that are read are confined to the pairs of those space pairs.  The pairs are permuted into
 // blocks of 16 by space pair, each category has a mask of active blocks, and a tile of 64
 // determinants uses the union of its categories' masks (ozaki_blk.cu).
+// Where most blocks are active or the space is small, the dense form (k_dg_split_dense and
+// k_oz_gemm, all pairs in their own order) is the faster one: dg_dense chooses; sigma has the
+// same bits.
 namespace {
 
 constexpr int DG_BLK = 2048;  // bytes per slice of one (tile, block): 64 determinants x 16 pairs, f16
