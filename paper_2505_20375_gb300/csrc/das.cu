@@ -301,8 +301,7 @@ int das_build(fci_context *h, int S, const int *orbs, const int *ref_a, const in
     auto up = [&](void **dst, const void *src, size_t bytes) -> int {
         int r = fci_dev_alloc(h, dst, bytes);
         if (r) return r;
-        FCI_CUDA(h, cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
-        return FCI_OK;
+        return fci_upload(h, *dst, src, bytes, st);
     };
     std::vector<int32_t> cpa(L.cat_pa.begin(), L.cat_pa.end()), cpb(L.cat_pb.begin(), L.cat_pb.end());
     rc = up((void **)&L.d_cat_of_pair, cat_of.data(), cat_of.size() * 4);
@@ -319,7 +318,6 @@ int das_build(fci_context *h, int S, const int *orbs, const int *ref_a, const in
     if (!rc) rc = up((void **)&L.d_pat_locbase_a, lb_a.data(), lb_a.size() * 8);
     if (!rc) rc = up((void **)&L.d_pat_locbase_b, lb_b.data(), lb_b.size() * 8);
     if (rc) { das_free(h); return rc; }
-    (void)st;
     h->das_active = true;
     h->mode = FCI_MODE_DAS;
     return FCI_OK;

@@ -69,6 +69,12 @@ void fci_dev_free(void *p) {
     if (p) cudaFree(p);
 }
 
+int fci_upload(fci_context *h, void *dst, const void *src, size_t bytes, cudaStream_t s) {
+    FCI_CUDA(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s));
+    FCI_CUDA(h, cudaStreamSynchronize(s));
+    return FCI_OK;
+}
+
 // ------------------------------------------------------------ phase timing
 
 static cudaEvent_t take_event(fci_context *h) {
@@ -107,6 +113,14 @@ static void drain_events(fci_context *h) {
     cudaGetLastError();
     h->ev_pending.clear();
     h->ev_used = 0;
+}
+
+// Waits for the stream, then reads the handle's status word and clears it, in stream order.
+static int take_status(fci_context *h, int *st, cudaStream_t s) {
+    FCI_CUDA(h, cudaMemcpyAsync(st, h->d_status, sizeof *st, cudaMemcpyDeviceToHost, s));
+    FCI_CUDA(h, cudaMemsetAsync(h->d_status, 0, sizeof *st, s));
+    FCI_CUDA(h, cudaStreamSynchronize(s));
+    return FCI_OK;
 }
 
 static int set_dev(fci_context *h) {
@@ -225,11 +239,12 @@ int fci_create(fci_handle *out, int device) {
             bt[p * FCI_BINOM_LD + j] = bt[(p - 1) * FCI_BINOM_LD + j - 1] + (j <= p - 1 ? bt[(p - 1) * FCI_BINOM_LD + j] : 0);
     }
     rc = fci_dev_alloc(h, (void **)&h->d_binom, bt.size() * 8);
-    if (!rc) rc = fci_cuda_check(h, cudaMemcpy(h->d_binom, bt.data(), bt.size() * 8, cudaMemcpyHostToDevice), "binom upload");
+    if (!rc) rc = fci_upload(h, h->d_binom, bt.data(), bt.size() * 8, cudaStreamLegacy);
     h->small_bytes = 1 << 20;
     if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_small, h->small_bytes);
     if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_status, 256);
-    if (!rc) rc = fci_cuda_check(h, cudaMemset(h->d_status, 0, 256), "status word");
+    if (!rc) rc = fci_cuda_check(h, cudaMemsetAsync(h->d_status, 0, 256, cudaStreamLegacy), "status word");
+    if (!rc) rc = fci_cuda_check(h, cudaStreamSynchronize(cudaStreamLegacy), "status word");
     if (rc) {
         g_err = h->err;
         fci_dev_free(h->d_binom);
@@ -266,10 +281,9 @@ int fci_sync_status(fci_handle h, fci_stream stream) {
     int rc = set_dev(h);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    FCI_CUDA(h, cudaStreamSynchronize(s));
     int st = 0;
-    FCI_CUDA(h, cudaMemcpy(&st, h->d_status, sizeof st, cudaMemcpyDeviceToHost));
-    FCI_CUDA(h, cudaMemset(h->d_status, 0, sizeof st));
+    rc = take_status(h, &st, s);
+    if (rc) return rc;
     if (st == FCI_ERR_TIMEOUT) return fci_fail(h, FCI_ERR_TIMEOUT, "a bounded device wait expired; sigma was set to NaN");
     if (st) return fci_fail(h, st, "device status %d", st);
     return FCI_OK;
@@ -410,8 +424,8 @@ static int prepare_operator(fci_context *h, int n_el, cudaStream_t s) {
     }
     int rc = fci_dev_alloc(h, (void **)&h->d_G, G.size() * 8);
     if (rc) return rc;
-    FCI_CUDA(h, cudaMemcpy(h->d_G, G.data(), G.size() * 8, cudaMemcpyHostToDevice));
-    rc = fci_dev_alloc(h, (void **)&h->d_GT, G.size() * 8);
+    rc = fci_upload(h, h->d_G, G.data(), G.size() * 8, s);
+    if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_GT, G.size() * 8);
     if (rc) return rc;
     FCI_CUDA(h, launch_transpose_operator(h->npair, w, h->d_G, h->d_GT, s));
     // diagonal helpers (real parts; exact for Hermitian integrals)
@@ -426,11 +440,10 @@ static int prepare_operator(fci_context *h, int n_el, cudaStream_t s) {
     rc = fci_dev_alloc(h, (void **)&h->d_hd, n * 8);
     if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_J, n2 * 8);
     if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_K, n2 * 8);
-    if (rc) return rc;
-    FCI_CUDA(h, cudaMemcpy(h->d_hd, hd.data(), n * 8, cudaMemcpyHostToDevice));
-    FCI_CUDA(h, cudaMemcpy(h->d_J, J.data(), n2 * 8, cudaMemcpyHostToDevice));
-    FCI_CUDA(h, cudaMemcpy(h->d_K, K.data(), n2 * 8, cudaMemcpyHostToDevice));
-    return FCI_OK;
+    if (!rc) rc = fci_upload(h, h->d_hd, hd.data(), n * 8, s);
+    if (!rc) rc = fci_upload(h, h->d_J, J.data(), n2 * 8, s);
+    if (!rc) rc = fci_upload(h, h->d_K, K.data(), n2 * 8, s);
+    return rc;
 }
 
 int fci_build_strings(fci_handle h, int n_alpha, int n_beta, fci_stream stream) {
@@ -731,7 +744,7 @@ int fci_tune_sigma(fci_handle h, int n_slices, const void *C, void *sigma, void 
         if ((rc = dz_check(h, n_slices))) return rc;
         n = dz_tune_candidates(h, n_slices, a, b, 8);
     } else {
-        if ((rc = oz_prepare_G(h, n_slices))) return rc;
+        if ((rc = oz_prepare_G(h, n_slices, s))) return rc;
         n = oz_tune_candidates(h, n_slices, a, b, 8);
     }
     if (n == 0) return fci_fail(h, FCI_ERR_UNSUPPORTED, "no kernel configuration fits %d slices", n_slices);
@@ -751,11 +764,8 @@ int fci_tune_sigma(fci_handle h, int n_slices, const void *C, void *sigma, void 
         if (!rc) rc = fci_cuda_check(h, cudaEventSynchronize(e1), "sync");
         if (!rc) {
             int st = 0;
-            rc = fci_cuda_check(h, cudaMemcpy(&st, h->d_status, sizeof(int), cudaMemcpyDeviceToHost), "status");
-            if (!rc && st) {
-                cudaMemset(h->d_status, 0, sizeof(int));
-                rc = fci_fail(h, st, "split-precision kernel reported status %d while tuning", st);
-            }
+            rc = take_status(h, &st, s);
+            if (!rc && st) rc = fci_fail(h, st, "split-precision kernel reported status %d while tuning", st);
         }
         float t = 0.f;
         if (!rc) rc = fci_cuda_check(h, cudaEventElapsedTime(&t, e0, e1), "elapsed");

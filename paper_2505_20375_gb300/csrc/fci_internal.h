@@ -174,6 +174,10 @@ int fci_fail(fci_context *h, int code, const char *fmt, ...);
 int fci_cuda_check(fci_context *h, cudaError_t e, const char *what);
 int fci_dev_alloc(fci_context *h, void **p, size_t bytes);
 void fci_dev_free(void *p);
+// Host to device, complete on return.  From pageable memory a plain cudaMemcpy may return
+// while its last part is still on the way to the device, on the default stream, which a
+// non-blocking stream (every stream that PyTorch makes) does not wait for.
+int fci_upload(fci_context *h, void *dst, const void *src, size_t bytes, cudaStream_t s);
 #define FCI_CUDA(h, call)                                            \
     do {                                                             \
         cudaError_t _e = (call);                                     \
@@ -264,7 +268,7 @@ cudaError_t launch_fixed_point_pairs(const double *C, int64_t n, int top, fci_sp
                                      cudaStream_t st);
 
 // ozaki.cu
-int oz_prepare_G(fci_context *h, int n_slices);
+int oz_prepare_G(fci_context *h, int n_slices, cudaStream_t s);
 int oz_tune_candidates(const fci_context *h, int n_slices, int *nt, int *path, int max);  // configurations that fit
 void oz_set_config(fci_context *h, int n_slices, int nt, int path);                     // nt = 0: default
 size_t oz_workspace_bytes(const fci_context *h, int n_slices);

@@ -671,7 +671,7 @@ static uint16_t half_bits_of_small_int(int d) {
     return (uint16_t)(sign | ((unsigned)(e + 15) << 10) | mant);
 }
 
-int oz_prepare_G(fci_context *h, int s) {
+int oz_prepare_G(fci_context *h, int s, cudaStream_t st) {
     if (h->Gs_slices == s && h->d_Gs) return FCI_OK;
     const int np = h->npair, KC = oz_kc(h);
     const int Kp = KC * 8;
@@ -707,9 +707,8 @@ int oz_prepare_G(fci_context *h, int s) {
     fci_dev_free(h->d_Gs);
     h->d_Gs = nullptr;
     int rc = fci_dev_alloc(h, &h->d_Gs, img.size() * 2);
+    if (!rc) rc = fci_upload(h, h->d_Gs, img.data(), img.size() * 2, st);  // the contraction reads it in its prologue
     if (rc) return rc;
-    FCI_CUDA(h, cudaMemcpy(h->d_Gs, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
-    FCI_CUDA(h, cudaStreamSynchronize(0));  // the copy itself: the contraction reads the image in its prologue
     h->Gs_slices = s;
     h->G_exp = shG;  // stores sh_G
     return FCI_OK;
@@ -748,9 +747,9 @@ size_t oz_workspace_bytes(const fci_context *h, int s) {
 }
 
 // G digit image in the A-tile layout of the bulk-copy GEMM ([K-chunk][plane][128 x 32]).
-static int oz_prepare_Gt(fci_context *h, int s) {
+static int oz_prepare_Gt(fci_context *h, int s, cudaStream_t st) {
     if (h->Gt_slices == s && h->d_Gt) return FCI_OK;  // the layout depends on s only
-    int rc = oz_prepare_G(h, s);  // checks, and sh_G
+    int rc = oz_prepare_G(h, s, st);  // checks, and sh_G
     if (rc) return rc;
     const int np = h->npair;
     const OzTwoPass tg = oz_gemm_geom(h, s);
@@ -777,9 +776,8 @@ static int oz_prepare_Gt(fci_context *h, int s) {
     h->d_Gt = nullptr;
     h->Gt_slices = 0;
     rc = fci_dev_alloc(h, &h->d_Gt, img.size() * 2);
+    if (!rc) rc = fci_upload(h, h->d_Gt, img.data(), img.size() * 2, st);  // the GEMM reads it in its prologue
     if (rc) return rc;
-    FCI_CUDA(h, cudaMemcpy(h->d_Gt, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
-    FCI_CUDA(h, cudaStreamSynchronize(0));  // the copy itself: the contraction reads the image in its prologue
     h->Gt_slices = s;
     return FCI_OK;
 }
@@ -789,7 +787,7 @@ static int oz_prepare_job(fci_context *h, const double *C, int s, void *ws, cuda
                           int64_t **E_out, int **shC_out, int **status_out) {
     if (h->mode != FCI_MODE_FCI) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split precision needs alpha/beta strings");
     if (h->ndet >= ((int64_t)1 << 31)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split precision: 2^31 determinants or more");
-    int rc = oz_prepare_G(h, s);
+    int rc = oz_prepare_G(h, s, st);
     if (rc) return rc;
     const int KC = oz_kc(h);
     const int64_t N = h->ndet;
@@ -874,7 +872,7 @@ static int oz_num_sms(fci_context *h, int *nsm) {
 // digits, one M-tile of 128 pair rows), integer scatter.
 static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int s, void *ws, cudaStream_t st) {
     if (h->ndet >= ((int64_t)1 << 31)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split precision: 2^31 determinants or more");
-    int rc = oz_prepare_Gt(h, s);
+    int rc = oz_prepare_Gt(h, s, st);
     if (rc) return rc;
     const OzTwoPass tg = oz_gemm_geom(h, s);
     if (!oz_gemm_ring(s, tg.kcc, tg.resa ? tg.n_kc : 0))

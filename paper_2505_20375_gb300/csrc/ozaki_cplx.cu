@@ -338,7 +338,7 @@ int cz_check(fci_context *h, int s) {
 
 // Real-embedded G digit image in the A layout of the block-sparse GEMM, followed by the row
 // map (row of E of each position of a row block).
-static int cz_prepare_G(fci_context *h, int s) {
+static int cz_prepare_G(fci_context *h, int s, cudaStream_t st) {
     const bool dense = cz_dense(h, s);
     const int key = s + (dense ? 100 : 0);
     if (h->Gs_slices == key && h->d_Gs) return FCI_OK;
@@ -397,8 +397,8 @@ static int cz_prepare_G(fci_context *h, int s) {
     h->d_Gs = nullptr;
     h->Gs_slices = 0;
     int rc = fci_dev_alloc(h, &h->d_Gs, img.size() * 2);
+    if (!rc) rc = fci_upload(h, h->d_Gs, img.data(), img.size() * 2, st);
     if (rc) return rc;
-    FCI_CUDA(h, cudaMemcpy(h->d_Gs, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
     h->Gs_slices = key;
     h->G_exp = shG;
     return FCI_OK;
@@ -419,7 +419,7 @@ size_t cz_workspace_bytes(const fci_context *h, int s) {
 int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, size_t ws_bytes, cudaStream_t st) {
     (void)ws_bytes;
     int rc = cz_check(h, s);
-    if (!rc) rc = cz_prepare_G(h, s);
+    if (!rc) rc = cz_prepare_G(h, s, st);
     if (rc) return rc;
     const CzBlocks bl = cz_blocks(h->n_orb);
     const int64_t n_nt = ceil_div(h->ndet, CZ_N);

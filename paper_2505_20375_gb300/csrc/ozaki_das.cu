@@ -738,7 +738,7 @@ int dz_prepare_tables(fci_context *h, cudaStream_t st) {
             tb[npab + k] = (int32_t)L.cat_off[c];
         }
         for (int b = 0; b < L.n_pat_b; ++b) tb[2 * npab + b] = (int32_t)L.pat_nstr_b[b];
-        FCI_CUDA(h, cudaMemcpy(L.d_dz_base, tb.data(), tb.size() * 4, cudaMemcpyHostToDevice));
+        rc = fci_upload(h, L.d_dz_base, tb.data(), tb.size() * 4, st);  // waits for the two kernels too
     }
     return rc;
 }
@@ -775,8 +775,8 @@ int dz_prepare(fci_context *h, int s, cudaStream_t st) {
         L.d_dz_G = nullptr;
         L.dz_slices = 0;
         rc = fci_dev_alloc(h, &L.d_dz_G, img.size() * 2);
+        if (!rc) rc = fci_upload(h, L.d_dz_G, img.data(), img.size() * 2, st);
         if (rc) return rc;
-        FCI_CUDA(h, cudaMemcpy(L.d_dz_G, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
         L.dz_slices = s;
         L.dz_shG = shG;
     }
@@ -1516,7 +1516,7 @@ cudaError_t dg_image(const DgSplit &a, int s, bool dense, cudaStream_t st) {
 }
 
 // The block plan's device tables and the G digit slices in the A layout of the block-sparse GEMM.
-int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense) {
+int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense, cudaStream_t st) {
     fci_das_layout &L = h->das;
     int rc = FCI_OK;
     if (!L.d_dg_mask) {
@@ -1524,12 +1524,12 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense) {
         dg_category_masks(h, b, masks);
         if (!L.d_dg_perm) {
             if ((rc = fci_dev_alloc(h, (void **)&L.d_dg_perm, b.perm.size() * 4))) return rc;
-            FCI_CUDA(h, cudaMemcpy(L.d_dg_perm, b.perm.data(), b.perm.size() * 4, cudaMemcpyHostToDevice));
+            if ((rc = fci_upload(h, L.d_dg_perm, b.perm.data(), b.perm.size() * 4, st))) return rc;
         }
         ulonglong2 *dm = nullptr;
         if ((rc = fci_dev_alloc(h, (void **)&dm, masks.size() * sizeof(ulonglong2)))) return rc;
         L.d_dg_mask = dm;
-        FCI_CUDA(h, cudaMemcpy(dm, masks.data(), masks.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice));
+        if ((rc = fci_upload(h, dm, masks.data(), masks.size() * sizeof(ulonglong2), st))) return rc;
     }
     const int key = s + (dense ? 100 : 0);
     if (L.dg_slices == key && L.d_dg_G) return FCI_OK;
@@ -1569,8 +1569,8 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense) {
     L.d_dg_G = nullptr;
     L.dg_slices = 0;
     rc = fci_dev_alloc(h, &L.d_dg_G, img.size() * 2);
+    if (!rc) rc = fci_upload(h, L.d_dg_G, img.data(), img.size() * 2, st);
     if (rc) return rc;
-    FCI_CUDA(h, cudaMemcpy(L.d_dg_G, img.data(), img.size() * 2, cudaMemcpyHostToDevice));
     L.dg_slices = key;
     L.dg_shG = shG;
     return FCI_OK;
@@ -1616,7 +1616,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     rc = dz_prepare_tables(h, st);
     const bool dense = dg_dense(h, blk, s);
     const int n_kc = (int)ceil_div(h->npair, DG_KW);
-    if (!rc) rc = dg_prepare(h, s, blk, dense);
+    if (!rc) rc = dg_prepare(h, s, blk, dense, st);
     if (rc) return rc;
     const fci_das_layout &L = h->das;
     const DgGeom g = dg_geom(h, s, dense ? 2 * n_kc : blk.n_blk());
