@@ -134,7 +134,7 @@ struct fci_context {
     int oz_tuned_nt[9] = {0};    // determinants per tile chosen by the tuner, per slice count (0: default)
     int oz_tuned_path[9] = {0};  // 1: two-pass path (D digit image + bulk-copy GEMM) chosen by the tuner
     void *d_Gt = nullptr;        // G digit image in the GEMM's A-tile layout (two-pass path)
-    int Gt_slices = 0;
+    int Gt_slices = 0, Gt_exp = 0;  // and its own shift: d_Gs may be of another slice count by now
 
     fci_das_layout das;
     bool das_active = false;

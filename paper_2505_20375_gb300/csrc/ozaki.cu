@@ -779,6 +779,7 @@ static int oz_prepare_Gt(fci_context *h, int s, cudaStream_t st) {
     if (!rc) rc = fci_upload(h, h->d_Gt, img.data(), img.size() * 2, st);  // the GEMM reads it in its prologue
     if (rc) return rc;
     h->Gt_slices = s;
+    h->Gt_exp = shG;
     return FCI_OK;
 }
 
@@ -925,7 +926,7 @@ static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int
     phase_scope ps(h, st, FCI_PHASE_SCATTER, 1);
     const int threads = 128;
     dim3 g((unsigned)ceil_div(h->nsb, threads), (unsigned)std::min<int64_t>(h->nsa, 65535));
-    const int ush = 8 * oz_gemm_L0(s, 8) - h->G_exp;
+    const int ush = 8 * oz_gemm_L0(s, 8) - h->Gt_exp;
     if ((uint64_t)n_nt * OZG_M * OZG_N < ((uint64_t)1 << 32))
         k_scatter_int2p<true><<<g, threads, 0, st>>>(h->nsa, h->nsb, h->npair_pad, h->d_pair_a, h->d_pair_b, E, C,
                                                      h->e_core, ush, shC, status, h->d_status, sigma);
