@@ -9,6 +9,9 @@
 // one has finished by the time a kernel runs its prologue.  Without a dependent launch on
 // either side both calls do nothing; with early false the launch is an ordinary one.
 //
+// A kernel that lives on L1 is not admitted early beside one that occupies every SM: it runs to
+// its end with the L1 that the SM had then (k_to_fixed in fixed_point.cu, k_oz_gemm).
+//
 // What it is for: a split sigma of a small space is three or four kernels of 5 to 15 us, and
 // their launches and set-up (the operator's digits into shared memory) stood between them.
 // us per sigma of FCI, calls issued back to back, ordinary / dependent launches:

@@ -83,11 +83,16 @@ __global__ void k_absmax_bits(const double *__restrict__ x, int64_t n, fci_split
     if ((threadIdx.x & 31) == 0 && m) atomicMax(&sc->maxbits, m);
 }
 
+// Lets the next kernel in only when its blocks end: the blocks of the FCI digit image that
+// started beside it stayed slow to their end (they live on L1, and an SM that is busy does
+// not change its split between L1 and shared memory), which a grid of one wave never makes
+// up.  us per sigma at s = 3, next kernel let in at the start / at the end: 364 x 3,432
+// strings 1,118 / 874, 220 x 924 208 / 148, 462 x 462 146 / 139, 210 x 210 42 / 42,
+// 924 x 924 443 / 443.
 template <bool PAIRS>
 __global__ void k_to_fixed(const double *__restrict__ C, int64_t n, int top, fci_split_scalars *__restrict__ sc,
                            void *__restrict__ out) {
     await_previous();
-    admit_next();
     const int sh = shift_of(sc->maxbits, top);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->shC = sh;
