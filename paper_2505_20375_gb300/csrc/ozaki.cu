@@ -636,20 +636,35 @@ int oz_ring(int s, int KC, int nt) {
     if (oz_smem_bytes(s, KC, 2, nt) <= OZ_SMEM_MAX) return 2;
     return 0;
 }
-// Tile width of this handle for s slices: the tuner's choice, else FCI_OZ_TILE from the
-// environment (32 or 64), else 64.
 // Contraction path for s slices: 1 = two-pass (digit image of D in HBM, then the
 // bulk-copy GEMM), 0 = fused producer kernel.  The tuner's choice, else FCI_OZ_PATH
-// ("gemm" / "fused") from the environment, else two-pass from 2^13 determinants on (faster
-// there at every slice count: us per sigma, fused / two-pass, 4,900 determinants (8 orbitals)
-// s = 3 32 / 30, s = 6 35 / 32; 15,876 37 / 33, 45 / 38; 63,504 70 / 55, 94 / 71; 853,776
-// 731 / 494, 1028 / 669) and fused below, where both are a chain of launches and small
-// problems share one launch of a group.
-int oz_path(const fci_context *h, int s) {
+// ("gemm" / "fused") from the environment, else two-pass from 2^13 determinants on, fused
+// below, where both are a chain of launches and small problems share one launch of a group.
+// us per sigma, fused / two-pass (strings alpha x beta):
+//            126 x 126    252 x 252    495 x 792    924 x 924
+//   s = 3    30 / 26      62 / 47      351 / 232    717 / 443
+//   s = 6    36 / 32      82 / 66      487 / 338    1,045 / 664
+// Two exceptions:
+//   - few, long rows.  The digit image takes one block per alpha string, whose work grows with
+//     the beta strings, so below 2^20 determinants more than eight beta strings per alpha
+//     string stay fused (any number above 2^20, where the GEMM weighs more):
+//              14 x 3,432   55 x 462   66 x 924   91 x 3,432   45 x 252   220 x 924   364 x 3,432
+//     s = 3    66 / 162     43 / 43    73 / 68    320 / 312    31 / 30    194 / 145   1,192 / 874
+//     s = 6    92 / 246     56 / 59    98 / 99    472 / 470    39 / 38    264 / 206   1,738 / 1,347
+//   - groups (jobs: the split FCI problems of one slice count in the call).  The two-pass jobs
+//     of a group run one after another, the fused ones share a launch, so from four jobs on
+//     the line is at 2^15.  us per group:
+//              16 x 10,584   4 x 15,876   16 x 15,876   16 x 44,100
+//     s = 3    341 / 430     101 / 103    425 / 463     811 / 671
+//     s = 6    384 / 507     121 / 126    506 / 561     1,010 / 901
+int oz_path(const fci_context *h, int s, int jobs = 1) {
     if (s >= 2 && s <= 8 && h->oz_tuned_nt[s]) return h->oz_tuned_path[s];
     if (const char *env = getenv("FCI_OZ_PATH")) return strcmp(env, "gemm") == 0 ? 1 : 0;
-    return (h->ndet >= ((int64_t)1 << 13) && s <= 7) ? 1 : 0;
+    if (s > 7 || h->ndet < ((int64_t)1 << (jobs >= 4 ? 15 : 13))) return 0;
+    return h->ndet >= ((int64_t)1 << 20) || h->nsb <= 8 * h->nsa;
 }
+// Tile width of this handle for s slices: the tuner's choice, else FCI_OZ_TILE from the
+// environment (32 or 64), else 64.
 int oz_nt(const fci_context *h, int s) {
     if (s >= 2 && s <= 8 && h->oz_tuned_nt[s]) return h->oz_tuned_nt[s];
     if (const char *env = getenv("FCI_OZ_TILE")) {
@@ -1009,7 +1024,7 @@ static int oz_sigma_group_nt(fci_context *const *hs, const double *const *Cs, do
 int oz_sigma_group(fci_context *const *hs, const double *const *Cs, double *const *sigmas, void *const *wss, int n,
                    int s, cudaStream_t st) {
     for (int i = 0; i < n; ++i)
-        if (oz_path(hs[i], s) == 1) {
+        if (oz_path(hs[i], s, n) == 1) {
             const int rc = oz_sigma_fci_gemm(hs[i], Cs[i], sigmas[i], s, wss[i], st);
             if (rc) return rc;
         }
@@ -1019,7 +1034,7 @@ int oz_sigma_group(fci_context *const *hs, const double *const *Cs, double *cons
         std::vector<double *> s2;
         std::vector<void *> w2;
         for (int i = 0; i < n; ++i)
-            if (oz_path(hs[i], s) == 0 && oz_nt(hs[i], s) == nt) {
+            if (oz_path(hs[i], s, n) == 0 && oz_nt(hs[i], s) == nt) {
                 h2.push_back(hs[i]);
                 c2.push_back(Cs[i]);
                 s2.push_back(sigmas[i]);
