@@ -272,8 +272,10 @@ int davidson_solve(fci_handle h, const fci_davidson_opts *opts, void *C_io, doub
 /* fci_sigma for one vector, replayed from a CUDA graph: the first call with a given
  * (C, sigma, precision, n_slices, workspace, stream) runs the sigma once, then captures
  * its kernel sequence into a graph kept in the handle (at most 64 graphs; the oldest is
- * dropped); later calls with the same arguments launch the graph.  Must not be called
- * while `stream` is itself being captured.  Results equal fci_sigma's. */
+ * dropped); later calls with the same arguments launch the graph.  Rebuilding the handle's
+ * integrals, strings or layout drops its graphs; sigma builds and solves with other slice
+ * counts leave them valid (the operator images of every slice count in use are kept).  Must
+ * not be called while `stream` is itself being captured.  Results equal fci_sigma's. */
 int fci_sigma_graph(fci_handle h, const void *C, void *sigma, int precision, int n_slices, void *workspace,
                     size_t workspace_bytes, fci_stream stream);
 /* Drop the handle's cached sigma graphs (e.g. before freeing the buffers they name). */
@@ -329,7 +331,7 @@ int fci_sigma_grouped(const fci_sigma_job *jobs, int n_jobs, fci_stream stream);
  * field of every job equal, same stream) runs it once, then captures its launches into a
  * graph kept in a process-wide cache (at most 16 lists; the oldest is dropped); later
  * calls with the same list launch the graph.  Destroying a handle, or rebuilding its
- * strings or integrals, drops the graphs that name it.  `stream` must not be the legacy
+ * integrals, strings or layout, drops the graphs that name it.  `stream` must not be the legacy
  * default stream (the list is then run without a graph) nor itself be capturing.  Results
  * equal fci_sigma_grouped's.  This is how the serving loop replays the batched sigma
  * builds of its active solves while the set of solves does not change. */

@@ -75,6 +75,27 @@ int fci_upload(fci_context *h, void *dst, const void *src, size_t bytes, cudaStr
     return FCI_OK;
 }
 
+int fci_image_build(fci_context *h, fci_image &img, const void *src, size_t bytes, int sh, cudaStream_t s) {
+    void *d = nullptr;
+    int rc = fci_dev_alloc(h, &d, bytes);
+    if (!rc) rc = fci_upload(h, d, src, bytes, s);
+    if (rc) {
+        fci_dev_free(d);
+        return rc;
+    }
+    img.d = d;
+    img.sh = sh;
+    return FCI_OK;
+}
+
+void fci_images_free(fci_image (&img)[2][FCI_IMAGE_SLICES]) {
+    for (auto &form : img)
+        for (fci_image &i : form) {
+            fci_dev_free(i.d);
+            i = fci_image();
+        }
+}
+
 // ------------------------------------------------------------ phase timing
 
 static cudaEvent_t take_event(fci_context *h) {
@@ -179,18 +200,13 @@ static void free_strings(fci_context *h) {
     fci_dev_free(h->d_pair_a_t); fci_dev_free(h->d_pair_b_t);
     fci_dev_free(h->d_dstr);
     fci_dev_free(h->d_G); fci_dev_free(h->d_GT); fci_dev_free(h->d_hd); fci_dev_free(h->d_J); fci_dev_free(h->d_K);
-    fci_dev_free(h->d_Gs);
-    fci_dev_free(h->d_Gt);
+    fci_images_free(h->img);
     h->d_str_a = h->d_str_b = nullptr;
     h->d_rep_a = h->d_rep_b = nullptr;
     h->d_pair_a = h->d_pair_b = nullptr;
     h->d_pair_a_t = h->d_pair_b_t = nullptr;
     h->d_dstr = nullptr;
     h->d_G = h->d_GT = h->d_hd = h->d_J = h->d_K = nullptr;
-    h->d_Gs = nullptr;
-    h->Gs_slices = 0;
-    h->d_Gt = nullptr;
-    h->Gt_slices = 0;
     das_free(h);
     h->mode = FCI_MODE_NONE;
     h->nsa = h->nsb = h->ndet = 0;
@@ -511,6 +527,7 @@ int das_build_categories(fci_handle h, int n_spaces, const int *orbs_per_space, 
     if (!orbs_per_space || !ref_alpha || !ref_beta) return fci_fail(h, FCI_ERR_ARG, "NULL DAS argument");
     int rc = set_dev(h);
     if (rc) return rc;
+    drop_graphs(h);  // the tables of the layout before are freed
     return das_build(h, n_spaces, orbs_per_space, ref_alpha, ref_beta, max_transfer, (cudaStream_t)stream);
 }
 

@@ -46,6 +46,15 @@ __host__ __device__ inline int pair_index(int a, int b) {
     return hi * (hi + 1) / 2 + lo;
 }
 
+// A digit image of the operator, G_int = round(G 2^sh), in the layout of one kernel.  Images
+// are built on first use, one per slice count and form, and stay until the strings or the
+// layout are rebuilt: captured graphs name them.
+struct fci_image {
+    void *d = nullptr;
+    int sh = 0;
+};
+constexpr int FCI_IMAGE_SLICES = 9;  // indexed by the slice count, 2 .. 8
+
 struct fci_das_layout {
     int n_spaces = 0;
     int space_orbs[8] = {0};
@@ -74,17 +83,15 @@ struct fci_das_layout {
     int32_t *d_str_of_loc_b = nullptr;
     int64_t *d_pat_locbase_a = nullptr, *d_pat_locbase_b = nullptr;  // offsets into str_of_loc
     // split-precision operands (built on first use): replacement tables that pack the
-    // target string's pattern and local index, block offsets per pattern pair, and the
-    // G digit slices in the layout of the MMA's B operand
+    // target string's pattern and local index, and block offsets per pattern pair
     int32_t *d_dz_rep_a = nullptr, *d_dz_rep_b = nullptr;  // [n_pair_pad][n_str]
     int32_t *d_dz_base = nullptr;  // [target | intermediate block offset per pattern pair (-1: none) | n_str_b]
-    void *d_dz_G = nullptr;
-    int dz_slices = 0, dz_shG = 0;
-    // the two-pass form (s >= 4): G digit slices in the A layout of the block-sparse GEMM, the
-    // pair of each position of its 16-wide blocks (-1: padding), and per category of the
-    // intermediate space the mask of blocks that connect it with the target space
-    void *d_dg_G = nullptr;
-    int dg_slices = 0, dg_shG = 0;  // 100 + s: G in the layout of the dense form
+    // operator images: [0] the B operand of the fused form (s <= 3), the A layout of the
+    // block-sparse GEMM (s >= 4); [1] the dense form's (s >= 4)
+    fci_image img[2][FCI_IMAGE_SLICES];
+    // the two-pass form (s >= 4): the pair of each position of its 16-wide blocks (-1: padding),
+    // and per category of the intermediate space the mask of blocks that connect it with the
+    // target space
     mutable double dg_share = -1.0;  // MMA work of the block-sparse form over that of the dense one (-1: not yet known)
     int32_t *d_dg_perm = nullptr;  // [16 n_blk]
     ulonglong2 *d_dg_mask = nullptr;  // [n_cat_int]
@@ -126,15 +133,11 @@ struct fci_context {
     // own one- and two-electron diagonal energy, then sum_{q in string} J_pq for every p;
     // filled by launch_diag_strings before each use of the diagonal (alpha/beta modes)
     double *d_dstr = nullptr;
-    // Ozaki split of G (bf16 digit slices, canonical UMMA layout) and its scale
-    void *d_Gs = nullptr;
-    int Gs_slices = 0;
-    double G_scale = 0.0;  // |G| <= 2^G_exp
-    int G_exp = 0;
+    // operator images (Ozaki split of G): alpha/beta strings [0] fused kernel, [1] two-pass GEMM;
+    // spinor strings [0] block-sparse GEMM, [1] dense GEMM
+    fci_image img[2][FCI_IMAGE_SLICES];
     int oz_tuned_nt[9] = {0};    // determinants per tile chosen by the tuner, per slice count (0: default)
     int oz_tuned_path[9] = {0};  // 1: two-pass path (D digit image + bulk-copy GEMM) chosen by the tuner
-    void *d_Gt = nullptr;        // G digit image in the GEMM's A-tile layout (two-pass path)
-    int Gt_slices = 0, Gt_exp = 0;  // and its own shift: d_Gs may be of another slice count by now
 
     fci_das_layout das;
     bool das_active = false;
@@ -178,6 +181,9 @@ void fci_dev_free(void *p);
 // while its last part is still on the way to the device, on the default stream, which a
 // non-blocking stream (every stream that PyTorch makes) does not wait for.
 int fci_upload(fci_context *h, void *dst, const void *src, size_t bytes, cudaStream_t s);
+// The image, allocated and filled from the host; left empty on failure.
+int fci_image_build(fci_context *h, fci_image &img, const void *src, size_t bytes, int sh, cudaStream_t s);
+void fci_images_free(fci_image (&img)[2][FCI_IMAGE_SLICES]);
 #define FCI_CUDA(h, call)                                            \
     do {                                                             \
         cudaError_t _e = (call);                                     \

@@ -687,7 +687,7 @@ static uint16_t half_bits_of_small_int(int d) {
 }
 
 int oz_prepare_G(fci_context *h, int s, cudaStream_t st) {
-    if (h->Gs_slices == s && h->d_Gs) return FCI_OK;
+    if (s >= 2 && s <= OZ_MAXS && h->img[0][s].d) return FCI_OK;
     const int np = h->npair, KC = oz_kc(h);
     const int Kp = KC * 8;
     if (np > 128) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split precision needs <= 128 orbital pairs (n <= 15)");
@@ -719,14 +719,7 @@ int oz_prepare_G(fci_context *h, int s, cudaStream_t st) {
             }
         }
     }
-    fci_dev_free(h->d_Gs);
-    h->d_Gs = nullptr;
-    int rc = fci_dev_alloc(h, &h->d_Gs, img.size() * 2);
-    if (!rc) rc = fci_upload(h, h->d_Gs, img.data(), img.size() * 2, st);  // the contraction reads it in its prologue
-    if (rc) return rc;
-    h->Gs_slices = s;
-    h->G_exp = shG;  // stores sh_G
-    return FCI_OK;
+    return fci_image_build(h, h->img[0][s], img.data(), img.size() * 2, shG, st);
 }
 
 // Two-pass path geometry: one M-tile of 128 pair rows.  K-chunks of 16 (kcc = 2) with the G
@@ -763,16 +756,17 @@ size_t oz_workspace_bytes(const fci_context *h, int s) {
 
 // G digit image in the A-tile layout of the bulk-copy GEMM ([K-chunk][plane][128 x 32]).
 static int oz_prepare_Gt(fci_context *h, int s, cudaStream_t st) {
-    if (h->Gt_slices == s && h->d_Gt) return FCI_OK;  // the layout depends on s only
     int rc = oz_prepare_G(h, s, st);  // checks, and sh_G
     if (rc) return rc;
+    fci_image &image = h->img[1][s];
+    if (image.d) return FCI_OK;  // the layout depends on s only
     const int np = h->npair;
     const OzTwoPass tg = oz_gemm_geom(h, s);
     const int n_kc = tg.n_kc, kw = 8 * tg.kcc;  // K per chunk
     std::vector<double> G((size_t)np * np);
     if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
         return fci_cuda_check(h, cudaGetLastError(), "G download");
-    const int shG = h->G_exp;
+    const int shG = h->img[0][s].sh;
     uint64_t bias = 0;
     for (int j = 0; j < s; ++j) bias |= (uint64_t)0x80 << (8 * j);
     const size_t a_plane = (size_t)OZG_M * kw * 2, stageA = (size_t)s * a_plane;
@@ -787,15 +781,7 @@ static int oz_prepare_Gt(fci_context *h, int s, cudaStream_t st) {
             for (int j = 0; j < s; ++j)
                 img[(off + (size_t)j * a_plane) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
         }
-    fci_dev_free(h->d_Gt);
-    h->d_Gt = nullptr;
-    h->Gt_slices = 0;
-    rc = fci_dev_alloc(h, &h->d_Gt, img.size() * 2);
-    if (!rc) rc = fci_upload(h, h->d_Gt, img.data(), img.size() * 2, st);  // the GEMM reads it in its prologue
-    if (rc) return rc;
-    h->Gt_slices = s;
-    h->Gt_exp = shG;
-    return FCI_OK;
+    return fci_image_build(h, image, img.data(), img.size() * 2, shG, st);
 }
 
 // Fixed-point conversion of C and the job's kernel parameters (first half of a split sigma).
@@ -829,7 +815,7 @@ static int oz_prepare_job(fci_context *h, const double *C, int s, void *ws, cuda
     prm.pairA = h->d_pair_a;
     prm.pairB = h->d_pair_b;
     prm.Cint = Cint;
-    prm.Gimg = (const uint4 *)h->d_Gs;
+    prm.Gimg = (const uint4 *)h->img[0][s].d;
     prm.E = E;
     prm.ldE = 0;
     prm.status = status;
@@ -874,7 +860,7 @@ static int oz_finish_job(fci_context *h, const double *C, double *sigma, const O
     const int threads = 128;
     dim3 g((unsigned)ceil_div(h->nsb, threads), (unsigned)std::min<int64_t>(h->nsa, 65535));
     FCI_CUDA(h, launch_dependent(true, k_scatter_int, g, threads, 0, st, h->nsa, h->nsb, h->npair_pad, prm.nt == 32 ? 5 : 6,
-                                 h->d_pair_a, h->d_pair_b, E, prm.npair, C, h->e_core, 8 * prm.L0 - h->G_exp, shC, status,
+                                 h->d_pair_a, h->d_pair_b, E, prm.npair, C, h->e_core, 8 * prm.L0 - h->img[0][prm.s].sh, shC, status,
                                  h->d_status, sigma));
     return FCI_OK;
 }
@@ -933,7 +919,7 @@ static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int
     a.M_pad = OZG_M;
     a.M_real = h->npair;
     a.n_nt = n_nt;
-    a.Gimg = h->d_Gt;
+    a.Gimg = h->img[1][s].d;
     a.Dimg = Dimg;
     a.E = E;
     a.status = status;
@@ -941,7 +927,7 @@ static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int
     phase_scope ps(h, st, FCI_PHASE_SCATTER, 1);
     const int threads = 128;
     dim3 g((unsigned)ceil_div(h->nsb, threads), (unsigned)std::min<int64_t>(h->nsa, 65535));
-    const int ush = 8 * oz_gemm_L0(s, 8) - h->Gt_exp;
+    const int ush = 8 * oz_gemm_L0(s, 8) - h->img[1][s].sh;
     if ((uint64_t)n_nt * OZG_M * OZG_N < ((uint64_t)1 << 32))
         k_scatter_int2p<true><<<g, threads, 0, st>>>(h->nsa, h->nsb, h->npair_pad, h->d_pair_a, h->d_pair_b, E, C,
                                                      h->e_core, ush, shC, status, h->d_status, sigma);

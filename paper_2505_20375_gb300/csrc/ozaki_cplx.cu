@@ -340,8 +340,8 @@ int cz_check(fci_context *h, int s) {
 // map (row of E of each position of a row block).
 static int cz_prepare_G(fci_context *h, int s, cudaStream_t st) {
     const bool dense = cz_dense(h, s);
-    const int key = s + (dense ? 100 : 0);
-    if (h->Gs_slices == key && h->d_Gs) return FCI_OK;
+    fci_image &image = h->img[dense][s];
+    if (image.d) return FCI_OK;
     const CzBlocks bl = cz_blocks(h->n_orb);
     const CzGeom g = cz_geom(h);
     const int n = h->n_orb, n2 = n * n, np = bl.n_blk * 16;
@@ -393,15 +393,7 @@ static int cz_prepare_G(fci_context *h, int s, cudaStream_t st) {
                 img[(off + (size_t)j * plane) / 2] = half_bits_of_small_int((int)((yb >> (7 * j)) & 0x7F) - 64);
         }
     if (!dense) memcpy(reinterpret_cast<char *>(img.data()) + map_off, row.data(), (size_t)np * 4);
-    fci_dev_free(h->d_Gs);
-    h->d_Gs = nullptr;
-    h->Gs_slices = 0;
-    int rc = fci_dev_alloc(h, &h->d_Gs, img.size() * 2);
-    if (!rc) rc = fci_upload(h, h->d_Gs, img.data(), img.size() * 2, st);
-    if (rc) return rc;
-    h->Gs_slices = key;
-    h->G_exp = shG;
-    return FCI_OK;
+    return fci_image_build(h, image, img.data(), img.size() * 2, shG, st);
 }
 
 // 2 KB units per slice of a tile's digit image.
@@ -425,6 +417,7 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
     const int64_t n_nt = ceil_div(h->ndet, CZ_N);
     const int M_real = 2 * h->n_orb * h->n_orb;
     const bool dense = cz_dense(h, s);
+    const fci_image &image = h->img[dense][s];
     const CzGeom g = cz_geom(h);
     char *p = (char *)ws;
     int64_t *Cint = (int64_t *)p;
@@ -460,7 +453,7 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
         a.M_pad = M_real;
         a.M_real = M_real;
         a.n_nt = n_nt;
-        a.Gimg = h->d_Gs;
+        a.Gimg = image.d;
         a.Dimg = Dimg;
         a.E = E;
         a.status = status;
@@ -470,10 +463,10 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
         a.n_blk = bl.n_blk;
         a.M_pad = M_real;
         a.n_nt = n_nt;
-        a.Gimg = h->d_Gs;
+        a.Gimg = image.d;
         a.Dimg = Dimg;
         a.masks = masks;
-        a.rowmap = (const int32_t *)((const char *)h->d_Gs + (size_t)bl.n_blk * bl.n_blk * s * 512);
+        a.rowmap = (const int32_t *)((const char *)image.d + (size_t)bl.n_blk * bl.n_blk * s * 512);
         a.E = E;
         a.status = status;
         if ((rc = oz_blk_launch(h, s, 7, a, st))) return rc;
@@ -483,7 +476,7 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
         const int L0 = oz_gemm_L0(s, 7);
         k_cz_scatter<<<(unsigned)ceil_div(h->ndet, 128), 128, 0, st>>>(h->n_orb, h->ndet, M_real, h->d_str_a,
                                                                         h->d_binom, E, C, h->e_core,
-                                                                        7 * L0 - h->G_exp, shC, status, h->d_status,
+                                                                        7 * L0 - image.sh, shC, status, h->d_status,
                                                                         sigma);
         FCI_CUDA(h, cudaGetLastError());
     }

@@ -750,7 +750,8 @@ int dz_prepare(fci_context *h, int s, cudaStream_t st) {
     int rc = dz_check(h, s);
     if (!rc) rc = dz_prepare_tables(h, st);
     if (rc) return rc;
-    if (L.dz_slices != s || !L.d_dz_G) {
+    fci_image &image = L.img[0][s];
+    if (!image.d) {
         const int np = h->npair, Np = h->npair_pad, KC = Np / 8;
         std::vector<double> G((size_t)np * np);
         if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -771,16 +772,9 @@ int dz_prepare(fci_context *h, int s, cudaStream_t st) {
                 const size_t off = ((size_t)(pq >> 3) * KC + (rs >> 3)) * 128 + (pq & 7) * 16 + (rs & 7) * 2;
                 for (int j = 0; j < s; ++j) img[(j * slice + off) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
             }
-        fci_dev_free(L.d_dz_G);
-        L.d_dz_G = nullptr;
-        L.dz_slices = 0;
-        rc = fci_dev_alloc(h, &L.d_dz_G, img.size() * 2);
-        if (!rc) rc = fci_upload(h, L.d_dz_G, img.data(), img.size() * 2, st);
-        if (rc) return rc;
-        L.dz_slices = s;
-        L.dz_shG = shG;
+        rc = fci_image_build(h, image, img.data(), img.size() * 2, shG, st);
     }
-    return FCI_OK;
+    return rc;
 }
 
 // Intermediate-space chunk: whole categories whose E fits the cap (a single category
@@ -875,7 +869,7 @@ void dz_params(const DzJob &j, int s, const DzGeom &g, int chunk, DzParams &prm)
     prm.locbase_a = L.d_pat_locbase_a;
     prm.locbase_b = L.d_pat_locbase_b;
     prm.Cint = j.Cint;
-    prm.Gimg = (const uint4 *)L.d_dz_G;
+    prm.Gimg = (const uint4 *)L.img[0][s].d;
     prm.E = j.E;
     prm.status = j.status;
     const char *to = getenv("FCI_WAIT_TIMEOUT_MS");
@@ -932,7 +926,7 @@ int dz_scatter(const DzJob &j, int s, int chunk, cudaStream_t st) {
     a.E = j.E;
     a.C = j.C;
     a.e_core = h->e_core;
-    a.ushift = 8 * (s - 1) - L.dz_shG;
+    a.ushift = 8 * (s - 1) - L.img[0][s].sh;
     a.shC = j.shC;
     a.status = j.status;
     a.sticky = h->d_status;
@@ -1531,8 +1525,8 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense, cudaStream_
         L.d_dg_mask = dm;
         if ((rc = fci_upload(h, dm, masks.data(), masks.size() * sizeof(ulonglong2), st))) return rc;
     }
-    const int key = s + (dense ? 100 : 0);
-    if (L.dg_slices == key && L.d_dg_G) return FCI_OK;
+    fci_image &image = L.img[dense][s];
+    if (image.d) return FCI_OK;
     const int np = h->npair, nb = b.n_blk();
     std::vector<double> G((size_t)np * np);
     if (cudaMemcpy(G.data(), h->d_G, G.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -1565,15 +1559,7 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense, cudaStream_
             for (int j = 0; j < s; ++j)
                 img[(off + (size_t)j * plane) / 2] = half_bits_of_small_int((int)((y >> (8 * j)) & 0xFF) - 128);
         }
-    fci_dev_free(L.d_dg_G);
-    L.d_dg_G = nullptr;
-    L.dg_slices = 0;
-    rc = fci_dev_alloc(h, &L.d_dg_G, img.size() * 2);
-    if (!rc) rc = fci_upload(h, L.d_dg_G, img.data(), img.size() * 2, st);
-    if (rc) return rc;
-    L.dg_slices = key;
-    L.dg_shG = shG;
-    return FCI_OK;
+    return fci_image_build(h, image, img.data(), img.size() * 2, shG, st);
 }
 
 }  // namespace
@@ -1619,6 +1605,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     if (!rc) rc = dg_prepare(h, s, blk, dense, st);
     if (rc) return rc;
     const fci_das_layout &L = h->das;
+    const fci_image &image = L.img[dense][s];
     const DgGeom g = dg_geom(h, s, dense ? 2 * n_kc : blk.n_blk());
     char *p = (char *)ws;
     int64_t *Cint = (int64_t *)p;
@@ -1684,7 +1671,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
                 a.M_pad = h->npair;
                 a.M_real = h->npair;
                 a.n_nt = sp.n_nt;
-                a.Gimg = L.d_dg_G;
+                a.Gimg = image.d;
                 a.Dimg = Dimg;
                 a.E = Ep;
                 a.status = status;
@@ -1695,7 +1682,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
             a.n_blk = blk.n_blk();
             a.M_pad = h->npair;  // E row stride: the n_pair rows of each tile, no padding
             a.n_nt = sp.n_nt;
-            a.Gimg = L.d_dg_G;
+            a.Gimg = image.d;
             a.Dimg = Dimg;
             a.masks = masks;
             a.rowmap = L.d_dg_perm;
@@ -1725,7 +1712,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
         sc.E = E;
         sc.C = C;
         sc.e_core = h->e_core;
-        sc.ushift = 8 * oz_gemm_L0(s, 8) - L.dg_shG;
+        sc.ushift = 8 * oz_gemm_L0(s, 8) - image.sh;
         sc.shC = shC;
         sc.status = status;
         sc.sticky = h->d_status;
@@ -1748,18 +1735,13 @@ void dz_free(fci_das_layout &L) {
     fci_dev_free(L.d_dz_rep_a);
     fci_dev_free(L.d_dz_rep_b);
     fci_dev_free(L.d_dz_base);
-    fci_dev_free(L.d_dz_G);
-    fci_dev_free(L.d_dg_G);
+    fci_images_free(L.img);
     fci_dev_free(L.d_dg_perm);
     fci_dev_free(L.d_dg_mask);
     L.d_dg_perm = nullptr;
     L.d_dg_mask = nullptr;
     L.d_dz_rep_a = L.d_dz_rep_b = nullptr;
     L.d_dz_base = nullptr;
-    L.d_dz_G = nullptr;
-    L.d_dg_G = nullptr;
-    L.dz_slices = 0;
-    L.dg_slices = 0;
     L.dg_share = -1.0;
 }
 

@@ -2,7 +2,7 @@
 import pytest
 import torch
 
-from paper_2505_20375_gb300 import synth
+from paper_2505_20375_gb300 import fci, synth
 
 from helpers import ENERGY_TOL, gpu_fci
 
@@ -34,3 +34,70 @@ def test_mixed_davidson_after_tuning_the_final_slice_count(fci_lib, monkeypatch)
                    final_precision="oz_bf16", final_slices=6)
     r64 = f.davidson(tol_residual=1e-6, tol_energy=1e-10)
     assert r.converged and abs(r.energy - r64.energy) < ENERGY_TOL
+
+
+def _problem(kind):
+    if kind == "spinor":
+        h, g = synth.complex_integrals(10, 6, 46)
+        f = gpu_fci(dict(h=h, g=g, e_core=0.2, n=10, ne=4))
+    else:
+        h, g = synth.real_integrals(9, 6, 46)
+        f = gpu_fci(dict(h=h, g=g, e_core=0.2, n=9, na=3, nb=3))
+        if kind == "das":
+            f.build_das([3, 3, 3], [1, 1, 1], [1, 1, 1], 1)
+    return f, torch.from_numpy(synth.random_vector(f.n_det, seed=7, complex_=f.is_complex)).cuda()
+
+
+def _workspace(f, counts):
+    nb = max(f.sigma_workspace_bytes("oz_bf16", s) for s in counts)
+    buf = torch.empty(nb + 256, dtype=torch.uint8, device="cuda")
+    return buf, (buf.data_ptr() + 255) & ~255, nb
+
+
+# (3, 2): the two images of one form; (3, 6): on the DAS layout the two forms; (6, 4): the
+# one of the two-pass form
+@pytest.mark.parametrize("counts", [(3, 2), (3, 6), (6, 4)])
+@pytest.mark.parametrize("kind", ["fci", "das", "spinor"])
+def test_graphs_of_two_slice_counts_replay_in_turn(fci_lib, kind, counts):
+    """A captured sigma names the operator image of its slice count, which stays through
+    builds with other counts, also for the grouped graph."""
+    f, c = _problem(kind)
+    want = {s: f.sigma(c, precision="oz_bf16", n_slices=s) for s in counts}
+    buf, ws, nb = _workspace(f, counts)
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    outs = {(how, s): torch.empty_like(c) for how in ("single", "grouped") for s in counts}
+    with torch.cuda.stream(st):
+        for _ in range(3):
+            for (how, s), o in outs.items():
+                o.fill_(float("nan"))
+                if how == "single":
+                    f.sigma_graph_into(c.data_ptr(), o.data_ptr(), "oz_bf16", s, ws, nb, stream=st)
+                else:
+                    fci.sigma_grouped([(f, c, o, "oz_bf16", s, ws, nb)], stream=st, graph=True)
+                assert torch.equal(o, want[s])
+    f.sync_status(st)
+    f.clear_graphs()
+    fci.clear_grouped_graphs()
+
+
+def test_rebuilding_the_layout_drops_the_graphs(fci_lib):
+    """das_build_categories frees the tables of the layout before; a graph of that layout with
+    the same arguments must not replay."""
+    f, c = _problem("das")
+    buf, ws, nb = _workspace(f, (3,))
+    big = torch.empty(8 * nb + 256, dtype=torch.uint8, device="cuda")
+    ws, nb = (big.data_ptr() + 255) & ~255, 8 * nb
+    out = torch.empty(4 * f.n_det, dtype=torch.float64, device="cuda")
+    st = torch.cuda.Stream()
+    x = torch.from_numpy(synth.random_vector(4 * f.n_det, seed=8)).cuda()
+    torch.cuda.synchronize()
+    for ref in ([1, 1, 1], [2, 1, 0], [1, 1, 1]):
+        f.build_das([3, 3, 3], ref, ref, 1)
+        n = f.n_det
+        assert n <= x.numel() and f.sigma_workspace_bytes("oz_bf16", 3) <= nb
+        for _ in range(2):
+            f.sigma_graph_into(x.data_ptr(), out.data_ptr(), "oz_bf16", 3, ws, nb, stream=st)
+            f.sync_status(st)
+            assert torch.equal(out[:n], f.sigma(x[:n].contiguous(), precision="oz_bf16", n_slices=3))
+            torch.cuda.synchronize()
