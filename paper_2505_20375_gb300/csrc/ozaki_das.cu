@@ -713,17 +713,23 @@ int dz_check(fci_context *h, int s) {
 
 namespace {
 
-// The packed replacement tables and the block-offset table (both split forms).
+// The packed replacement tables and the block-offset table (both split forms), all three or
+// none: a call that runs out of memory half-way leaves nothing behind for the next one.
 int dz_prepare_tables(fci_context *h, cudaStream_t st) {
     fci_das_layout &L = h->das;
     int rc = FCI_OK;
-    if (!L.d_dz_rep_a) {
+    if (!L.d_dz_base) {
         const int Np = h->npair_pad;
         const int64_t nla = dz_nloc(L.pat_nstr_a), nlb = dz_nloc(L.pat_nstr_b);
         rc = fci_dev_alloc(h, (void **)&L.d_dz_rep_a, (size_t)Np * nla * 4);
         if (!rc) rc = fci_dev_alloc(h, (void **)&L.d_dz_rep_b, (size_t)Np * nlb * 4);
         if (!rc) rc = fci_dev_alloc(h, (void **)&L.d_dz_base, (size_t)(2 * L.n_pat_a * L.n_pat_b + L.n_pat_b) * 4);
-        if (rc) return rc;
+        if (rc) {
+            fci_dev_free(L.d_dz_rep_a);
+            fci_dev_free(L.d_dz_rep_b);
+            L.d_dz_rep_a = L.d_dz_rep_b = nullptr;
+            return rc;
+        }
         k_dz_rep<<<152 * 8, 256, 0, st>>>(h->d_pair_a, h->nsa, Np, L.d_str_of_loc_a, nla, L.d_pat_of_a, L.d_loc_a,
                                           L.d_dz_rep_a);
         k_dz_rep<<<152 * 8, 256, 0, st>>>(h->d_pair_b, h->nsb, Np, L.d_str_of_loc_b, nlb, L.d_pat_of_b, L.d_loc_b,
