@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_lincomb(const double *__restric
                 }
                 out[2 * j] = re;
                 out[2 * j + 1] = im;
-                            } else {
+            } else {
                 double acc = accumulate ? out[j] : 0.0;
 #pragma unroll 4
                 for (int i = 0; i < k; ++i) acc = fma(sy[2 * i], V[i * ldv + j], acc);
@@ -442,6 +442,7 @@ __global__ void __cluster_dims__(JAC_CLUSTER, 1, 1) __launch_bounds__(JAC_THREAD
     const int rank = (int)cluster.block_rank();
     double *Ab = jac_smem, *Qb = jac_smem + 2 * m * ld;
     const int t = threadIdx.x, nt = blockDim.x;
+    if (t == 0) best = 0;  // stays if NaN leaves no entry with the wanted rank (the host sees lam)
     for (int i = t; i < m * m; i += nt) {
         const int r = i / m, c = i % m;
         double v;
