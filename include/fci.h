@@ -319,12 +319,14 @@ typedef struct {
 } fci_sigma_job;
 
 /* sigma builds of several problems (different handles, sizes and integrals) in one pass
- * on `stream`: jobs that use FCI_PREC_OZ_BF16 with the same slice count share ONE
- * persistent launch of the tcgen05 contraction kernel (the uneven tile ranges of all jobs
- * in one grid, CTAs split in proportion to each job's tiles; alpha/beta-string jobs and
- * DAS jobs form separate launches); the other jobs run one after another.  All handles must be on the same device; a handle may
- * appear in at most one job.  Asynchronous.  This is the batching the serving loop uses
- * for the sigma builds of concurrent Davidson solves (not a step of the paper's method). */
+ * on `stream`: jobs that use the fused split kernels (FCI_PREC_OZ_BF16; small alpha/beta
+ * problems, DAS with 2 or 3 slices) with the same slice count share ONE persistent launch
+ * of the tcgen05 contraction kernel (the uneven tile ranges of all jobs in one grid, CTAs
+ * split in proportion to each job's tiles; alpha/beta-string jobs and DAS jobs form
+ * separate launches); the other jobs run one after another.  All handles must be on the
+ * same device; a handle may appear in at most one job.  Asynchronous.  This is the batching
+ * the serving loop uses for the sigma builds of concurrent Davidson solves (not a step of
+ * the paper's method). */
 int fci_sigma_grouped(const fci_sigma_job *jobs, int n_jobs, fci_stream stream);
 
 /* fci_sigma_grouped replayed from a CUDA graph: the first call with a given job list (every
@@ -390,11 +392,15 @@ enum { FCI_PHASE_GATHER = 0, FCI_PHASE_CONTRACT = 1, FCI_PHASE_SCATTER = 2, FCI_
 
 /* Enable (1) or disable (0) CUDA-event timing of the sigma phases (gather of D, the
  * contraction E = g' D, the scatter into sigma, other kernels).  Events are recorded on
- * the stream each kernel is launched on.  Adds no synchronisation to fci_sigma. */
+ * the stream each kernel is launched on.  Adds no synchronisation to fci_sigma.  A form
+ * that gathers D inside its contraction kernel (FP64, the fused split kernels) reports no
+ * gather phase; the fixed-point conversion of C counts as gather where a digit image of D
+ * follows it for alpha/beta or spinor strings, else as other. */
 int fci_set_phase_timing(fci_handle h, int enable);
 /* Synchronise with the recorded events and return, per phase, the summed kernel time
- * in milliseconds (ms[FCI_N_PHASES]) and the number of kernel launches
- * (launches[FCI_N_PHASES]); either pointer may be NULL.  reset != 0 clears the sums. */
+ * in milliseconds (ms[FCI_N_PHASES]) and the number of kernels launched
+ * (launches[FCI_N_PHASES]; copies and clears do not count); either pointer may be NULL.
+ * reset != 0 clears the sums. */
 int fci_get_phase_times(fci_handle h, double *ms, int64_t *launches, int reset);
 
 /* ------------------------------------------------ categorically compressed sigma */

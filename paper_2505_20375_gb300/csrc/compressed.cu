@@ -845,7 +845,7 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     unsigned long long cnt[3] = {0, 0, 0};
     // 1. the intermediate determinants one move from a nonzero coefficient, and D on them
     {
-        phase_scope ps(h, s, FCI_PHASE_GATHER, 4);
+        phase_scope ps(h, s, FCI_PHASE_GATHER, 10);
         FCI_CUDA(h, cudaMemsetAsync(a.hj, 0xFF, z.capj * 8, s));
         FCI_CUDA(h, cudaMemsetAsync(a.counts, 0, 256, s));
         const int64_t moves = nnz_c * (a.nent_a + a.nent_b);
@@ -879,7 +879,7 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     }
     // 3. the support of sigma, distinct and sorted
     {
-        phase_scope ps(h, s, FCI_PHASE_OTHER, 3);
+        phase_scope ps(h, s, FCI_PHASE_OTHER, 2);
         FCI_CUDA(h, cudaMemsetAsync(a.hl, 0xFF, z.capl * 8, s));
         k_cs_support<<<grid_of(n1 * (a.nent_a + a.nent_b)), 256, 0, s>>>(a, n1);
         k_cs_compact<<<grid_of((int64_t)z.capl / 8), 256, 0, s>>>(a.hl, nullptr, z.capl, a.l_addr, a.counts + 1);
@@ -893,9 +893,9 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
         return fci_fail(h, FCI_ERR_ARG, "output capacity %lld < %lld support entries", (long long)capacity, (long long)n2);
     uint64_t *src = (uint64_t *)a.l_addr, *dst = (uint64_t *)(w + z.off_tmp);
     {
-        phase_scope ps(h, s, FCI_PHASE_OTHER, 1);
         int bits = 1;
         while (bits < 63 && ((uint64_t)1 << bits) < (uint64_t)h->das.n_det) ++bits;
+        phase_scope ps(h, s, FCI_PHASE_OTHER, 3 * (int)ceil_div(bits, 8));
         const int64_t nt = ceil_div(n2, RS_TILE);
         unsigned long long *hist = (unsigned long long *)(w + z.off_hist);
         const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nt, 152 * 8));

@@ -268,6 +268,7 @@ struct fci_split_scalars {
     int shC, pad;
     int status, pad2;
 };
+int fixed_point_launches(int64_t n);  // kernels of one conversion of n values
 cudaError_t launch_fixed_point(const double *C, int64_t n, int top, fci_split_scalars *sc, int64_t *Cint,
                                cudaStream_t st);
 cudaError_t launch_fixed_point_pairs(const double *C, int64_t n, int top, fci_split_scalars *sc, int32_t *Cint,

@@ -38,6 +38,7 @@ __device__ __forceinline__ void store(void *out, int64_t i, double c, int sh) {
 }
 
 constexpr int SMALL_BLOCKS = 8, SMALL_THREADS = 512;
+constexpr int64_t SMALL_VALUES = (int64_t)1 << 14;  // the line above
 template <bool PAIRS>
 __global__ void __cluster_dims__(SMALL_BLOCKS, 1, 1) __launch_bounds__(SMALL_THREADS)
     k_fixed_small(const double *__restrict__ C, int64_t n, int top, fci_split_scalars *__restrict__ sc,
@@ -104,8 +105,8 @@ __global__ void k_to_fixed(const double *__restrict__ C, int64_t n, int top, fci
 
 template <bool PAIRS>
 cudaError_t launch(const double *C, int64_t n, int top, fci_split_scalars *sc, void *out, cudaStream_t st) {
-    if (n <= ((int64_t)1 << 14)) return launch_dependent(true, k_fixed_small<PAIRS>, SMALL_BLOCKS, SMALL_THREADS, 0, st, C, n, top, sc,
-                                out);
+    if (n <= SMALL_VALUES)
+        return launch_dependent(true, k_fixed_small<PAIRS>, SMALL_BLOCKS, SMALL_THREADS, 0, st, C, n, top, sc, out);
     cudaError_t e = cudaMemsetAsync(sc, 0, sizeof *sc, st);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 8);
@@ -115,6 +116,8 @@ cudaError_t launch(const double *C, int64_t n, int top, fci_split_scalars *sc, v
 }
 
 }  // namespace
+
+int fixed_point_launches(int64_t n) { return n <= SMALL_VALUES ? 1 : 2; }
 
 cudaError_t launch_fixed_point(const double *C, int64_t n, int top, fci_split_scalars *sc, int64_t *Cint,
                                cudaStream_t st) {

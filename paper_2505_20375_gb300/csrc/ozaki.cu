@@ -801,7 +801,7 @@ static int oz_prepare_job(fci_context *h, const double *C, int s, void *ws, cuda
     fci_split_scalars *sc = (fci_split_scalars *)p;
     int *shC = &sc->shC, *status = &sc->status;
     {
-        phase_scope ps(h, st, FCI_PHASE_OTHER, 2);
+        phase_scope ps(h, st, FCI_PHASE_OTHER, fixed_point_launches(N));
         FCI_CUDA(h, launch_fixed_point(C, N, 8 * s - 3, sc, Cint, st));
     }
     prm.N = N;
@@ -894,7 +894,7 @@ static int oz_sigma_fci_gemm(fci_context *h, const double *C, double *sigma, int
     fci_split_scalars *sc = (fci_split_scalars *)misc;
     int *shC = &sc->shC, *status = &sc->status;
     {
-        phase_scope ps(h, st, FCI_PHASE_GATHER, 3);
+        phase_scope ps(h, st, FCI_PHASE_GATHER, fixed_point_launches(N) + 1);
         FCI_CUDA(h, launch_fixed_point(C, N, 8 * s - 3, sc, Cint, st));
         const size_t row_smem = (size_t)h->nsb * 8 + (size_t)h->npair_pad * 4;  // one C row + its alpha entries
         if (row_smem > OZ_SMEM_MAX) return fci_fail(h, FCI_ERR_UNSUPPORTED, "split precision: %lld beta strings", (long long)h->nsb);

@@ -431,7 +431,7 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
     fci_split_scalars *sc = (fci_split_scalars *)p;
     int *shC = &sc->shC, *status = &sc->status;
     {
-        phase_scope ps(h, st, FCI_PHASE_GATHER, 3);
+        phase_scope ps(h, st, FCI_PHASE_GATHER, fixed_point_launches(2 * h->ndet) + 1);
         FCI_CUDA(h, launch_fixed_point(C, 2 * h->ndet, 7 * s - 3, sc, Cint, st));
         const int64_t n_img = n_nt * g.n_kc;  // dense form
         const unsigned gb = (unsigned)std::min<int64_t>(n_img, 152 * 16);

@@ -841,7 +841,7 @@ int dz_prepare_job(fci_context *h, const double *C, double *sigma, int s, void *
     fci_split_scalars *sc = (fci_split_scalars *)p;
     j.shC = &sc->shC;
     j.status = &sc->status;
-    phase_scope ps(h, st, FCI_PHASE_OTHER, 2);
+    phase_scope ps(h, st, FCI_PHASE_OTHER, fixed_point_launches(L.n_det));
     FCI_CUDA(h, launch_fixed_point_pairs(C, L.n_det, 8 * s - 3, sc, j.Cint, st));
     return FCI_OK;
 }
@@ -1486,6 +1486,8 @@ int64_t dg_row_max(const fci_das_layout &L) {
     return most;
 }
 
+int dg_image_launches(const DgSplit &a, bool dense) { return !dense && dg_row_smem(a) <= DG_ROW_SMEM ? 2 : 1; }
+
 // Digit image and block masks of a piece.  By rows where two CTAs' rows fit an SM (up to
 // about 14,000 target values per alpha string), else determinant by determinant.
 template <int S>
@@ -1630,7 +1632,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     fci_split_scalars *scal = (fci_split_scalars *)p;
     int *shC = &scal->shC, *status = &scal->status;
     {
-        phase_scope ps(h, st, FCI_PHASE_OTHER, 2);
+        phase_scope ps(h, st, FCI_PHASE_OTHER, fixed_point_launches(L.n_det));
         FCI_CUDA(h, launch_fixed_point(C, L.n_det, 8 * s - 3, scal, Cint, st));
     }
     const size_t npab = (size_t)L.n_pat_a * L.n_pat_b;
@@ -1666,7 +1668,7 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
             sp.len = std::min(g.d_cap, elen - d0);
             sp.n_nt = ceil_div(sp.len, OZG_N);
             {
-                phase_scope ps(h, st, FCI_PHASE_GATHER, 2);
+                phase_scope ps(h, st, FCI_PHASE_GATHER, dg_image_launches(sp, dense));
                 FCI_CUDA(h, dg_image(sp, s, dense, st));
             }
             int64_t *Ep = E + (size_t)(d0 / OZG_N) * h->npair * OZG_N;
