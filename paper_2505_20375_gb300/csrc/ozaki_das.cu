@@ -1486,7 +1486,13 @@ int64_t dg_row_max(const fci_das_layout &L) {
     return most;
 }
 
-int dg_image_launches(const DgSplit &a, bool dense) { return !dense && dg_row_smem(a) <= DG_ROW_SMEM ? 2 : 1; }
+// Whether the rows fit; FCI_DAS_ROW_BYTES lowers the limit (for tests of the other form).
+bool dg_by_rows(const DgSplit &a) {
+    size_t limit = DG_ROW_SMEM;
+    if (const char *env = getenv("FCI_DAS_ROW_BYTES")) limit = std::min<size_t>(limit, (size_t)std::max(0ll, atoll(env)));
+    return dg_row_smem(a) <= limit;
+}
+int dg_image_launches(const DgSplit &a, bool dense) { return !dense && dg_by_rows(a) ? 2 : 1; }
 
 // Digit image and block masks of a piece.  By rows where two CTAs' rows fit an SM (up to
 // about 14,000 target values per alpha string), else determinant by determinant.
@@ -1496,11 +1502,11 @@ cudaError_t dg_image_s(const DgSplit &a, bool dense, cudaStream_t st) {
         k_dg_split_dense<S><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(a.n_nt, 152 * 16)), 64 * DG_KCC, 0, st>>>(a);
         return cudaGetLastError();
     }
-    const size_t smem = dg_row_smem(a);
-    if (smem > DG_ROW_SMEM) {
+    if (!dg_by_rows(a)) {
         k_dg_split<S><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(a.n_nt, 152 * 16)), 256, 0, st>>>(a);
         return cudaGetLastError();
     }
+    const size_t smem = dg_row_smem(a);
     const cudaError_t e = cudaFuncSetAttribute(k_dg_rows<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_dg_masks<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(a.n_nt, 256), 152 * 8)), 256, 0, st>>>(a);
