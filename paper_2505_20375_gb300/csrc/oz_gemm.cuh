@@ -52,7 +52,7 @@ int oz_gemm_launch(fci_context *h, int s, int w, int kcc, bool resa, const oz_ge
 //   Dimg: [tile][K block][plane][row group of 8][K core][8 x 16 bytes] (inactive blocks unread)
 //   rowmap: [16 n_blk] row of E of each position, -1 for padding
 //   E: [tile][M_pad][64], written for the rows of active blocks
-// Digit widths w: 7 (s = 2 .. 8) and 8 (s = 4 .. 8).
+// Digit widths w: 7 and 8, s = 4 .. 8.
 constexpr int OZG_MAX_BLK = 128;
 struct oz_blk_args {
     int n_blk, M_pad;

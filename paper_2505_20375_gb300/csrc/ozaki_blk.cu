@@ -322,9 +322,7 @@ __global__ void __launch_bounds__(ozg_threads(S), 1) k_oz_gemm_blk(const __grid_
 
 template <int W>
 void (*blk_kernel(int s))(const BlkParams) {
-    switch (s) {
-        case 2: return k_oz_gemm_blk<2, W>;
-        case 3: return k_oz_gemm_blk<3, W>;
+    switch (s) {  // 2 and 3 slices take the dense form or the fused DAS kernel
         case 4: return k_oz_gemm_blk<4, W>;
         case 5: return k_oz_gemm_blk<5, W>;
         case 6: return k_oz_gemm_blk<6, W>;
@@ -339,13 +337,13 @@ size_t blk_fixed() { return 1024 + sizeof(BlkShared) + 64; }
 }  // namespace
 
 int oz_blk_ring(int s) {
-    if (s < 2 || s > OZG_MAXS) return 0;
+    if (s < 4 || s > OZG_MAXS) return 0;
     const size_t r = (BLK_SMEM_MAX - blk_fixed()) / blk_stage(s);
     return r < 2 ? 0 : (int)std::min<size_t>(BLK_MAX_STAGES, r);
 }
 
 int oz_blk_launch(fci_context *h, int s, int w, const oz_blk_args &a, cudaStream_t st) {
-    void (*kern)(const BlkParams) = w == 7 ? blk_kernel<7>(s) : w == 8 && s >= 4 ? blk_kernel<8>(s) : nullptr;
+    void (*kern)(const BlkParams) = w == 7 ? blk_kernel<7>(s) : w == 8 ? blk_kernel<8>(s) : nullptr;
     const int ring = oz_blk_ring(s);
     if (!kern || !ring || a.n_blk > OZG_MAX_BLK)
         return fci_fail(h, FCI_ERR_UNSUPPORTED, "block-sparse split GEMM: %d slices of %d bits, %d blocks", s, w, a.n_blk);

@@ -315,11 +315,13 @@ CzGeom cz_geom(const fci_context *h) {
 //   22, 5                680/826        825/830        1,011/998      1,224/1,013    1,711/1,272
 //   22, 11               9,664/10,843   13,059/10,780  17,897/14,249  (s = 8 36,463/19,269)
 // 19 spinors with 5 electrons (11,628 determinants) take 473/511 at s = 6.
-// FCI_SPLIT_FORM=dense or blocks overrides it (for tests).
+// Up to 3 slices always take the dense form; above, FCI_SPLIT_FORM=dense or blocks overrides
+// the rule (for tests).
 bool cz_dense(const fci_context *h, int s) {
+    if (s <= 3) return true;
     if (!oz_gemm_ring(s, 4, 0)) return false;
     if (const char *env = getenv("FCI_SPLIT_FORM")) return strcmp(env, "dense") == 0;
-    return s <= 3 || h->n_orb < (s <= 5 ? 20 : 18) || h->ndet < ((int64_t)1 << 14);
+    return h->n_orb < (s <= 5 ? 20 : 18) || h->ndet < ((int64_t)1 << 14);
 }
 
 }  // namespace
@@ -332,7 +334,8 @@ int cz_check(fci_context *h, int s) {
     if ((int64_t)s * nnz * 4096 >= ((int64_t)1 << 24))
         return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices x %lld nonzero terms could exceed 2^24 in a level sum", s,
                         (long long)nnz);
-    if (!oz_blk_ring(s)) return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices do not fit two pipeline stages", s);
+    if (!(cz_dense(h, s) ? oz_gemm_ring(s, 4, 0) : oz_blk_ring(s)))
+        return fci_fail(h, FCI_ERR_UNSUPPORTED, "%d slices do not fit two pipeline stages", s);
     return FCI_OK;
 }
 
@@ -435,14 +438,13 @@ int cz_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, si
         FCI_CUDA(h, launch_fixed_point(C, 2 * h->ndet, 7 * s - 3, sc, Cint, st));
         const int64_t n_img = n_nt * g.n_kc;  // dense form
         const unsigned gb = (unsigned)std::min<int64_t>(n_img, 152 * 16);
-        switch (s) {
-#define CZ_SPLIT(S_)                                                                                                  \
-    case S_:                                                                                                          \
-        if (dense) k_cz_split_dense<S_><<<gb, 256, 0, st>>>(h->n_orb, h->ndet, g.n_kc, n_img, h->d_str_a, h->d_binom, Cint, Dimg); \
-        else k_cz_split<S_><<<(unsigned)n_nt, 256, 0, st>>>(bl, h->ndet, h->d_str_a, h->d_binom, Cint, Dimg, masks);   \
-        break;
-            CZ_SPLIT(2) CZ_SPLIT(3) CZ_SPLIT(4) CZ_SPLIT(5) CZ_SPLIT(6) CZ_SPLIT(7) CZ_SPLIT(8)
-#undef CZ_SPLIT
+        switch (dense ? s : 10 + s) {
+#define CZ_DENSE(S_) case S_: k_cz_split_dense<S_><<<gb, 256, 0, st>>>(h->n_orb, h->ndet, g.n_kc, n_img, h->d_str_a, h->d_binom, Cint, Dimg); break;
+#define CZ_BLOCKS(S_) case 10 + S_: k_cz_split<S_><<<(unsigned)n_nt, 256, 0, st>>>(bl, h->ndet, h->d_str_a, h->d_binom, Cint, Dimg, masks); break;
+            CZ_DENSE(2) CZ_DENSE(3) CZ_DENSE(4) CZ_DENSE(5) CZ_DENSE(6) CZ_DENSE(7) CZ_DENSE(8)
+            CZ_BLOCKS(4) CZ_BLOCKS(5) CZ_BLOCKS(6) CZ_BLOCKS(7) CZ_BLOCKS(8)
+#undef CZ_DENSE
+#undef CZ_BLOCKS
         }
         FCI_CUDA(h, cudaGetLastError());
     }
