@@ -1,14 +1,18 @@
-// Correctly rounded FP64 quotient, reciprocal and square root in few instructions, for a warp
-// that works through a chain of them.  On GB300 a warp gets one FP64 instruction through
+// FP64 quotient, reciprocal and square root as the operators round them, in few instructions,
+// for a warp that works through a chain of them.  On GB300 a warp gets one FP64 instruction through
 // every 64 cycles, dependent or not; a division takes 564 cycles and a square root 686.  The
 // forms below take a 22-bit start from the FP32 unit, two Newton terms at once, and one
 // residual correction by fused multiply-adds, which rounds correctly when the value it
-// corrects is within one unit in the last place (Markstein, "Computation of elementary
-// functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990): 7 instructions
-// for a quotient, 5 for the reciprocal, 9 for a root, 2 for the reciprocal of a root just
-// taken.  Equal to the operators on 1.6e9 random pairs.  Operands outside a wide middle range
-// of exponents (where a start or a residual could over- or underflow) take the plain
-// operators, as do zeros, infinities and NaN.
+// corrects is within one unit in the last place and the reciprocal that it uses is correctly
+// rounded (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990): 7 instructions for a quotient, 5 for the
+// reciprocal, 9 for a root, 2 for the reciprocal of a root just taken.  The reciprocals here
+// are within 2^-66 of the true value before their rounding, not proven rounded; the results
+// have the operators' bits on the random, special and near-midpoint operands of
+// tests/test_gpu_fp64_fast.py.  One class is left out: the reciprocal of a value with every
+// mantissa bit set may miss the last bit.  Operands outside a wide middle range of exponents
+// (where a start or a residual could over- or underflow) take the plain operators, as do
+// zeros, infinities and NaN.
 #pragma once
 
 #include <stdint.h>
@@ -43,8 +47,9 @@ __device__ __forceinline__ double rcp_start(double d) { return widen(__frcp_rn(m
 __device__ __forceinline__ double divide(double n, double d) {
     if (!middle(d) || !middle(n)) return n / d;
     const double r0 = copysign(rcp_start(d), d);
-    const double e = fma(-d, r0, 1.0), r = fma(r0, e, r0);
-    const double q0 = n * r0, q1 = fma(q0, fma(e, e, e), q0);  // 1 / (1 - e) = 1 + e + e^2 + O(2^-66)
+    const double e = fma(-d, r0, 1.0), t = fma(e, e, e);  // 1 / (1 - e) = 1 + e + e^2 + O(2^-66)
+    const double r = fma(r0, t, r0);
+    const double q0 = n * r0, q1 = fma(q0, t, q0);
     return fma(fma(-d, q1, n), r, q1);
 }
 
@@ -75,8 +80,7 @@ __device__ __forceinline__ double root(double x, double &y) {
     return fma(fma(-s1, s1, x), halve(y), s1);
 }
 
-// 1 / s, where y is 1 / s to about one unit in the last place (s with every mantissa bit set
-// excepted: the correction may then miss the last bit).
+// 1 / s, where y is 1 / s to about one unit in the last place.
 __device__ __forceinline__ double reciprocal_near(double s, double y) {
     if (!middle(s)) return 1.0 / s;
     return fma(fma(-s, y, 1.0), y, y);
