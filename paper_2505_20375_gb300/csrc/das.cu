@@ -317,6 +317,7 @@ int das_build(fci_context *h, int S, const int *orbs, const int *ref_a, const in
     if (!rc) rc = up((void **)&L.d_str_of_loc_b, sol_b.data(), std::max<size_t>(1, sol_b.size()) * 4);
     if (!rc) rc = up((void **)&L.d_pat_locbase_a, lb_a.data(), lb_a.size() * 8);
     if (!rc) rc = up((void **)&L.d_pat_locbase_b, lb_b.data(), lb_b.size() * 8);
+    if (!rc) rc = fci_wait(h, st);
     if (rc) { das_free(h); return rc; }
     h->das_active = true;
     h->mode = FCI_MODE_DAS;

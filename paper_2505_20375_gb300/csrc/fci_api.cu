@@ -71,6 +71,10 @@ void fci_dev_free(void *p) {
 
 int fci_upload(fci_context *h, void *dst, const void *src, size_t bytes, cudaStream_t s) {
     FCI_CUDA(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s));
+    return FCI_OK;
+}
+
+int fci_wait(fci_context *h, cudaStream_t s) {
     FCI_CUDA(h, cudaStreamSynchronize(s));
     return FCI_OK;
 }
@@ -79,6 +83,7 @@ int fci_image_build(fci_context *h, fci_image &img, const void *src, size_t byte
     void *d = nullptr;
     int rc = fci_dev_alloc(h, &d, bytes);
     if (!rc) rc = fci_upload(h, d, src, bytes, s);
+    if (!rc) rc = fci_wait(h, s);
     if (rc) {
         fci_dev_free(d);
         return rc;
@@ -260,7 +265,7 @@ int fci_create(fci_handle *out, int device) {
     if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_small, h->small_bytes);
     if (!rc) rc = fci_dev_alloc(h, (void **)&h->d_status, 256);
     if (!rc) rc = fci_cuda_check(h, cudaMemsetAsync(h->d_status, 0, 256, cudaStreamLegacy), "status word");
-    if (!rc) rc = fci_cuda_check(h, cudaStreamSynchronize(cudaStreamLegacy), "status word");
+    if (!rc) rc = fci_wait(h, cudaStreamLegacy);
     if (rc) {
         g_err = h->err;
         fci_dev_free(h->d_binom);
@@ -459,6 +464,7 @@ static int prepare_operator(fci_context *h, int n_el, cudaStream_t s) {
     if (!rc) rc = fci_upload(h, h->d_hd, hd.data(), n * 8, s);
     if (!rc) rc = fci_upload(h, h->d_J, J.data(), n2 * 8, s);
     if (!rc) rc = fci_upload(h, h->d_K, K.data(), n2 * 8, s);
+    if (!rc) rc = fci_wait(h, s);
     return rc;
 }
 

@@ -177,10 +177,13 @@ int fci_fail(fci_context *h, int code, const char *fmt, ...);
 int fci_cuda_check(fci_context *h, cudaError_t e, const char *what);
 int fci_dev_alloc(fci_context *h, void **p, size_t bytes);
 void fci_dev_free(void *p);
-// Host to device, complete on return.  From pageable memory a plain cudaMemcpy may return
-// while its last part is still on the way to the device, on the default stream, which a
-// non-blocking stream (every stream that PyTorch makes) does not wait for.
+// Host to device in the order of the stream.  From pageable memory a plain cudaMemcpy may
+// return while its last part is still on the way to the device, on the default stream, which
+// a non-blocking stream (every stream that PyTorch makes) does not wait for.  Every call that
+// uploads a table waits for the stream once before it returns (fci_wait), with the source
+// still alive: later calls may use the table on other streams.
 int fci_upload(fci_context *h, void *dst, const void *src, size_t bytes, cudaStream_t s);
+int fci_wait(fci_context *h, cudaStream_t s);
 // The image, allocated and filled from the host; left empty on failure.
 int fci_image_build(fci_context *h, fci_image &img, const void *src, size_t bytes, int sh, cudaStream_t s);
 void fci_images_free(fci_image (&img)[2][FCI_IMAGE_SLICES]);

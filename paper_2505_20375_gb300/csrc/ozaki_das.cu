@@ -744,7 +744,8 @@ int dz_prepare_tables(fci_context *h, cudaStream_t st) {
             tb[npab + k] = (int32_t)L.cat_off[c];
         }
         for (int b = 0; b < L.n_pat_b; ++b) tb[2 * npab + b] = (int32_t)L.pat_nstr_b[b];
-        rc = fci_upload(h, L.d_dz_base, tb.data(), tb.size() * 4, st);  // waits for the two kernels too
+        rc = fci_upload(h, L.d_dz_base, tb.data(), tb.size() * 4, st);
+        if (!rc) rc = fci_wait(h, st);
     }
     return rc;
 }
@@ -1538,6 +1539,7 @@ int dg_prepare(fci_context *h, int s, const DgBlocks &b, bool dense, cudaStream_
         if ((rc = fci_dev_alloc(h, (void **)&dm, masks.size() * sizeof(ulonglong2)))) return rc;
         L.d_dg_mask = dm;
         if ((rc = fci_upload(h, dm, masks.data(), masks.size() * sizeof(ulonglong2), st))) return rc;
+        if ((rc = fci_wait(h, st))) return rc;
     }
     fci_image &image = L.img[dense][s];
     if (image.d) return FCI_OK;
