@@ -25,17 +25,19 @@
 //      order (alpha then beta; absent J have E = 0): the arithmetic and its order are those
 //      of the dense FP64 DAS path, so the result equals the dense sigma on the support and
 //      the dense sigma is zero elsewhere.  The columns J that L reaches share its beta
-//      string (an alpha move) or its alpha string (a beta move), so they are found on the
-//      lists of columns per string.  Entries with short lists (most: the alpha-beta doubles
-//      of a nonzero determinant) take one thread each, those with long lists (its same-spin
-//      doubles and singles) one warp each; only where the lists are longer than a walk of
-//      L's replacements is that walk made, each J looked up in the first table.
+//      string (an alpha move) or its alpha string (a beta move).  For a sparse vector
+//      (cs_by_lists) they are found on lists of the columns per string: entries with short
+//      lists (most: the alpha-beta doubles of a nonzero determinant) take one thread each,
+//      those with long lists (its same-spin doubles and singles) one warp each.  Where the
+//      columns crowd, and for entries with very long lists or many terms, a walk of L's
+//      replacements looks each J up in the first table.
 // The pair tables are read string-major (one string's row contiguous; copies built on the
 // first call and kept by the handle).  Hash tables use open addressing with linear
 // probing over a power-of-two capacity of at least twice the largest number of keys, so no
 // probe sequence runs past a free slot; every probe loop is bounded by the capacity all
 // the same and reports an overflow instead.
 #include <stdint.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <cooperative_groups.h>
@@ -104,17 +106,18 @@ struct CsArgs {
     int64_t *j_addr;                 // [n1]: the J of each column
     uint32_t *bm_a, *bm_b;           // bit A (B) set: some column has alpha (beta) string A (B)
     const uint64_t *str_a, *str_b;   // string masks
-    // columns per string: entries off[S] .. off[S + 1] of list_a (list_b) hold the columns with
+    // columns per string: entries off_a[S] .. off_a[S + 1] (off_b) of list hold the columns with
     // alpha (beta) string S, as (column, mask of its other string)
-    uint32_t *off_a, *off_b;         // [n_str + 1]
-    int2 *list_a, *list_b;           // [n1]
-    int64_t *work;                   // support entries left to the warp form
+    uint32_t *off_a, *off_b;         // [n_str + 1] each, one after the other
+    int2 *list;                      // [2 n1]: alpha, then beta
+    bool by_lists;                   // the lists are built
+    int64_t *work, *walk;            // support entries left to the warp form, and to the walk
     double *D, *E;                   // [n_pair][ldd]
     int64_t ldd;
     unsigned long long *hl;          // target determinants L of the support
     uint64_t hl_mask;
     int64_t *l_addr;                 // [n2]
-    unsigned long long *counts;      // [0]: columns n1, [1]: support n2, [2]: overflow flag, [3]: entries in work
+    unsigned long long *counts;      // [0]: columns n1, [1]: support n2, [2]: overflow flag, [3]: entries in work, [4]: in walk
     double e_core;
 };
 
@@ -184,7 +187,9 @@ __device__ __forceinline__ bool cs_coef(const CsArgs &a, int64_t K, double &v) {
 // D[pair, column] for every column J and pair: the alpha source and the beta source of J
 // under the pair, each looked up among the nonzero coefficients (Algorithm 1's
 // intersection of J's excitation list with the compressed vector).  One warp per column, so
-// that J is decoded once.
+// that J is decoded once; its first lane marks J's strings in the bitmaps (a walk of the
+// replacements looks a candidate column up only if both of its strings occur in some column)
+// and counts the columns per string.
 __global__ void __launch_bounds__(256) k_cs_gather(const __grid_constant__ CsArgs a, int64_t n1) {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -192,6 +197,14 @@ __global__ void __launch_bounds__(256) k_cs_gather(const __grid_constant__ CsArg
         int32_t A, B;
         int pb;
         das_strings(a.d, a.n_cat_int, a.j_addr[j], A, B, pb);
+        if (lane == 0) {
+            atomicOr(a.bm_a + (A >> 5), 1u << (A & 31));
+            atomicOr(a.bm_b + (B >> 5), 1u << (B & 31));
+            if (a.by_lists) {
+                atomicAdd(a.off_a + A, 1u);
+                atomicAdd(a.off_b + B, 1u);
+            }
+        }
         for (int pp = lane; pp < a.npair; pp += 32) {
             double d = 0.0, v;
             const int32_t ea = __ldg(a.pair_a + (int64_t)A * a.ldp + pp);
@@ -258,26 +271,16 @@ __global__ void k_cs_transpose(const int32_t *__restrict__ src, int64_t R, int64
     }
 }
 
-// The alpha and beta strings of every column, as bitmaps (a walk of the replacements looks a
-// candidate column up only if both of its strings occur in some column), and the lists of
-// columns per string: FILL = false counts them (into off[S]), FILL = true, after the scan,
-// writes them backwards from the end of each string's range, which leaves off[S] at its start
-// (the order inside a list is free: the terms found on it are sorted).
-template <bool FILL>
-__global__ void k_cs_mark(const __grid_constant__ CsArgs a, int64_t n1) {
+// The lists of columns per string, after the gather has counted them (into off[S]) and the
+// scan: written backwards from the end of each string's range, which leaves off[S] at its
+// start (the order inside a list is free: the terms found on it are sorted).
+__global__ void k_cs_lists(const __grid_constant__ CsArgs a, int64_t n1) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n1; j += (int64_t)gridDim.x * blockDim.x) {
         int32_t A, B;
         int pb;
         das_strings(a.d, a.n_cat_int, a.j_addr[j], A, B, pb);
-        if (FILL) {
-            a.list_a[atomicSub(a.off_a + A, 1u) - 1u] = make_int2((int)j, (int)(uint32_t)a.str_b[B]);
-            a.list_b[atomicSub(a.off_b + B, 1u) - 1u] = make_int2((int)j, (int)(uint32_t)a.str_a[A]);
-        } else {
-            atomicOr(a.bm_a + (A >> 5), 1u << (A & 31));
-            atomicOr(a.bm_b + (B >> 5), 1u << (B & 31));
-            atomicAdd(a.off_a + A, 1u);
-            atomicAdd(a.off_b + B, 1u);
-        }
+        a.list[atomicSub(a.off_a + A, 1u) - 1u] = make_int2((int)j, (int)(uint32_t)a.str_b[B]);
+        a.list[atomicSub(a.off_b + B, 1u) - 1u] = make_int2((int)j, (int)(uint32_t)a.str_a[A]);
     }
 }
 
@@ -420,9 +423,18 @@ __device__ __forceinline__ double cs_value(const CsArgs &a, int64_t L, double ac
     return fma(a.e_core, cl, acc);  // as the dense FP64 scatter
 }
 
+// Appends o to a list, one addition to its count for the threads of a warp that come together.
+__device__ __forceinline__ void cs_append(int64_t *list, unsigned long long *count, int64_t o) {
+    const cooperative_groups::coalesced_group g = cooperative_groups::coalesced_threads();
+    unsigned long long at = 0;
+    if (g.thread_rank() == 0) at = atomicAdd(count, (unsigned long long)g.size());
+    list[g.shfl(at, 0) + g.thread_rank()] = o;
+}
+
 // Thread form: entries whose two lists hold at most CS_SHORT columns, none of them L itself.
-// The (at most CS_SHORT) terms go into ascending keys.  The others are appended to `work`.
-constexpr int CS_SHORT = 8;
+// The (at most CS_SHORT) terms go into ascending keys.  The others are left to the warp form,
+// above CS_LIST columns to the walk.
+constexpr int CS_SHORT = 8, CS_LIST = 400, CS_LONG = 64;
 __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
                                                   int64_t n2, double *__restrict__ out_val) {
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n2; o += (int64_t)gridDim.x * blockDim.x) {
@@ -432,6 +444,7 @@ __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs
         das_strings(a.d, a.d.n_cat, L, A, B, pb);
         const uint32_t b0 = __ldg(a.off_b + B), nb = __ldg(a.off_b + B + 1) - b0;
         const uint32_t a0 = __ldg(a.off_a + A), na = __ldg(a.off_a + A + 1) - a0;
+        const bool walk = na + nb > CS_LIST;
         bool ok = na + nb <= CS_SHORT;
         uint32_t key[CS_SHORT];
         int32_t col[CS_SHORT];
@@ -444,7 +457,7 @@ __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs
             const uint32_t SA = (uint32_t)__ldg(a.str_a + A), SB = (uint32_t)__ldg(a.str_b + B);
             for (uint32_t c = 0; c < na + nb; ++c) {
                 const bool alpha = c < nb;  // the columns with L's beta string are its alpha moves
-                const int2 nd = __ldg(alpha ? a.list_b + b0 + c : a.list_a + a0 + (c - nb));
+                const int2 nd = __ldg(a.list + (alpha ? b0 + c : a0 + (c - nb)));
                 const uint32_t S = alpha ? SA : SB, x = S ^ (uint32_t)nd.y;
                 const int d = __popc(x);
                 if (d == 0) ok = false;
@@ -465,10 +478,8 @@ __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs
             }
         }
         if (!ok) {
-            const cooperative_groups::coalesced_group g = cooperative_groups::coalesced_threads();
-            unsigned long long at = 0;
-            if (g.thread_rank() == 0) at = atomicAdd(a.counts + 3, (unsigned long long)g.size());
-            a.work[g.shfl(at, 0) + g.thread_rank()] = o;
+            if (walk) cs_append(a.walk, a.counts + 4, o);
+            else cs_append(a.work, a.counts + 3, o);
             continue;
         }
         double e[CS_SHORT], acc = 0.0;
@@ -482,12 +493,97 @@ __global__ void __launch_bounds__(256) k_cs_sigma(const __grid_constant__ CsArgs
     }
 }
 
+// Walk over the pairs of L's replacements, looking each J up in the first table: 32 pairs at a
+// time by a warp while the entries are few, by a thread each once there are many.
+constexpr int CS_WALK_WARPS = 1 << 14;  // entries up to which a warp takes one
+__device__ __forceinline__ bool cs_look(const CsArgs &a, const uint32_t *__restrict__ bm, int32_t e, int32_t other, bool alpha,
+                                        const double *__restrict__ Ep, double &v) {
+    if (e < 0 || !bit(bm, e >> 1)) return false;
+    const int64_t J = alpha ? das_addr(a.d, e >> 1, other) : das_addr(a.d, other, e >> 1);
+    const int64_t c = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+    if (c < 0) return false;
+    v = (e & 1) ? -Ep[c] : Ep[c];
+    return true;
+}
+template <bool WARP>
+__device__ __forceinline__ void cs_walk(const CsArgs &a, int64_t L, double *__restrict__ out) {
+    int32_t A, B;
+    int pb;
+    das_strings(a.d, a.d.n_cat, L, A, B, pb);
+    const int32_t *ra = a.pair_a + (int64_t)A * a.ldp, *rb = a.pair_b + (int64_t)B * a.ldp;
+    // an alpha move keeps B and a beta move keeps A: no column has them, no lookup
+    const bool try_a = bit(a.bm_b, B), try_b = bit(a.bm_a, A);
+    double acc = 0.0;
+    if (WARP) {
+        for (int p0 = 0; p0 < a.npair && (try_a || try_b); p0 += 32) {
+            const int pp = p0 + (threadIdx.x & 31);
+            const bool in = pp < a.npair;
+            const double *Ep = a.E + (int64_t)pp * a.ldd;
+            double va = 0.0, vb = 0.0;
+            const bool fa = cs_look(a, a.bm_a, try_a && in ? __ldg(ra + pp) : -1, B, true, Ep, va);
+            const bool fb = cs_look(a, a.bm_b, try_b && in ? __ldg(rb + pp) : -1, A, false, Ep, vb);
+            const unsigned ma = __ballot_sync(0xFFFFFFFFu, fa), mb = __ballot_sync(0xFFFFFFFFu, fb);
+            for (unsigned m = ma | mb; m; m &= m - 1) {  // the terms in pair order
+                const int src = __ffs(m) - 1;
+                const double ta = __shfl_sync(0xFFFFFFFFu, va, src), tb = __shfl_sync(0xFFFFFFFFu, vb, src);
+                if ((ma >> src) & 1u) acc += ta;
+                if ((mb >> src) & 1u) acc += tb;
+            }
+        }
+        if ((threadIdx.x & 31) == 0) *out = cs_value(a, L, acc);
+    } else {
+        const int4 none = make_int4(-1, -1, -1, -1);
+        for (int p4 = 0; p4 < a.npair && (try_a || try_b); p4 += 4) {  // rows past n_pair hold -1
+            const int4 ia = try_a ? __ldg(reinterpret_cast<const int4 *>(ra + p4)) : none;
+            const int4 ib = try_b ? __ldg(reinterpret_cast<const int4 *>(rb + p4)) : none;
+            const int32_t ea[4] = {ia.x, ia.y, ia.z, ia.w}, eb[4] = {ib.x, ib.y, ib.z, ib.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double *Ep = a.E + (int64_t)(p4 + k) * a.ldd;
+                const int32_t xa = ea[k];
+                if (xa >= 0 && bit(a.bm_a, xa >> 1)) {
+                    const int64_t J = das_addr(a.d, xa >> 1, B);
+                    const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+                    if (col >= 0) {
+                        const double e = Ep[col];
+                        acc += (xa & 1) ? -e : e;
+                    }
+                }
+                const int32_t xb = eb[k];
+                if (xb >= 0 && bit(a.bm_b, xb >> 1)) {
+                    const int64_t J = das_addr(a.d, A, xb >> 1);
+                    const int64_t col = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
+                    if (col >= 0) {
+                        const double e = Ep[col];
+                        acc += (xb & 1) ? -e : e;
+                    }
+                }
+            }
+        }
+        *out = cs_value(a, L, acc);
+    }
+}
+// Every entry.
+template <bool WARP>
+__global__ void __launch_bounds__(256) k_cs_sigma_all(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
+                                                      int64_t n2, double *__restrict__ out_val) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t o = WARP ? t >> 5 : t; o < n2; o += WARP ? nt >> 5 : nt) cs_walk<WARP>(a, l_sorted[o], out_val + o);
+}
+// The entries that the list forms have left.
+__global__ void __launch_bounds__(256) k_cs_sigma_rest(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
+                                                       double *__restrict__ out_val) {
+    const int64_t n = (int64_t)a.counts[4], t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    if (n <= CS_WALK_WARPS)
+        for (int64_t it = t >> 5; it < n; it += nt >> 5) cs_walk<true>(a, l_sorted[a.walk[it]], out_val + a.walk[it]);
+    else
+        for (int64_t it = t; it < n; it += nt) cs_walk<false>(a, l_sorted[a.walk[it]], out_val + a.walk[it]);
+}
+
 // Warp form.  The lanes check 32 columns of a list at a time; the terms (at most CS_LONG,
 // the diagonal ones included if L itself is a column) are ranked by key in shared memory
-// and added in that order.  Entries with longer lists or more terms walk their
-// replacements, 32 pairs at a time, each lane looking up its pair's two columns; the terms
-// of the lanes are added in pair order.
-constexpr int CS_LONG = 128;
+// and added in that order.  Entries with more terms are left to the walk: a warp adds one
+// term at a time, a walk by threads 32.
 __global__ void __launch_bounds__(256) k_cs_sigma_warp(const __grid_constant__ CsArgs a, const int64_t *__restrict__ l_sorted,
                                                        double *__restrict__ out_val) {
     __shared__ uint32_t s_key[8][CS_LONG];
@@ -504,13 +600,13 @@ __global__ void __launch_bounds__(256) k_cs_sigma_warp(const __grid_constant__ C
         double acc = 0.0;
         int terms = 0;
         bool itself = false;
-        bool ok = na + nb <= (uint32_t)a.npair;
-        if (ok) {
+        bool ok = true;
+        {
             const uint32_t SA = (uint32_t)__ldg(a.str_a + A), SB = (uint32_t)__ldg(a.str_b + B);
             for (uint32_t c0 = 0; c0 < na + nb && ok; c0 += 32) {
                 const uint32_t c = c0 + lane;
                 const bool alpha = c < nb, live = c < na + nb;
-                const int2 nd = live ? __ldg(alpha ? a.list_b + b0 + c : a.list_a + a0 + (c - nb)) : make_int2(0, 0);
+                const int2 nd = live ? __ldg(a.list + (alpha ? b0 + c : a0 + (c - nb))) : make_int2(0, 0);
                 const uint32_t S = alpha ? SA : SB, x = live ? S ^ (uint32_t)nd.y : ~0u;
                 const bool hit = __popc(x) == 2;
                 const unsigned hits = __ballot_sync(0xFFFFFFFFu, hit);
@@ -560,43 +656,10 @@ __global__ void __launch_bounds__(256) k_cs_sigma_warp(const __grid_constant__ C
             }
         }
         if (!ok) {
-            acc = 0.0;
-            // an alpha move keeps B and a beta move keeps A: no column has them, no lookup
-            const bool try_a = bit(a.bm_b, B), try_b = bit(a.bm_a, A);
-            const int32_t *ra = a.pair_a + (int64_t)A * a.ldp, *rb = a.pair_b + (int64_t)B * a.ldp;
-            for (int p0 = 0; p0 < a.npair && (try_a || try_b); p0 += 32) {
-                const int pp = p0 + lane;
-                const int32_t ea = try_a && pp < a.npair ? __ldg(ra + pp) : -1, eb = try_b && pp < a.npair ? __ldg(rb + pp) : -1;
-                double va = 0.0, vb = 0.0;
-                bool fa = false, fb = false;
-                if (ea >= 0 && bit(a.bm_a, ea >> 1)) {
-                    const int64_t J = das_addr(a.d, ea >> 1, B);
-                    const int64_t c = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
-                    if (c >= 0) {
-                        fa = true;
-                        va = a.E[(int64_t)pp * a.ldd + c];
-                        if (ea & 1) va = -va;
-                    }
-                }
-                if (eb >= 0 && bit(a.bm_b, eb >> 1)) {
-                    const int64_t J = das_addr(a.d, A, eb >> 1);
-                    const int64_t c = J >= 0 ? ht_find(a.hj, a.hj_col, a.hj_mask, (uint64_t)J) : -1;
-                    if (c >= 0) {
-                        fb = true;
-                        vb = a.E[(int64_t)pp * a.ldd + c];
-                        if (eb & 1) vb = -vb;
-                    }
-                }
-                const unsigned ma = __ballot_sync(0xFFFFFFFFu, fa), mb = __ballot_sync(0xFFFFFFFFu, fb);
-                for (unsigned m = ma | mb; m; m &= m - 1) {
-                    const int src = __ffs(m) - 1;
-                    const double ta = __shfl_sync(0xFFFFFFFFu, va, src), tb = __shfl_sync(0xFFFFFFFFu, vb, src);
-                    if ((ma >> src) & 1u) acc += ta;
-                    if ((mb >> src) & 1u) acc += tb;
-                }
-            }
+            if (lane == 0) a.walk[atomicAdd(a.counts + 4, 1ull)] = o;
+            continue;
         }
-        if (lane == 0) out_val[o] = !ok || itself ? cs_value(a, L, acc) : fma(a.e_core, 0.0, acc);
+        if (lane == 0) out_val[o] = itself ? cs_value(a, L, acc) : fma(a.e_core, 0.0, acc);
     }
 }
 
@@ -723,6 +786,27 @@ struct CsSizes {
     int64_t n_sums;  // scan blocks over the strings of both spins
 };
 
+// Whether sigma is found on the lists of columns per string, or by walking the replacements of
+// every support entry.  Lists pay while they are short: for a sparse vector whose
+// coefficients reach columns of their own.  The columns of neighbouring coefficients
+// coincide (n1 below nnz times the moves of a determinant, the diagonal ones as one), and the
+// lists of a nearly full space hold about as many as a walk's n_pair; then a walk by
+// threads, whose neighbours look up the same columns, is the faster one.  us per sigma,
+// lists / walk:
+//                                                       columns / moves   lists    walk
+//   24 orbitals, 400 coefficients at random             1.00              6,596    20,652
+//   24 orbitals, the first 200                          0.72              3,128    3,100
+//   24 orbitals, the first 1,000                        0.66              16,786   11,486
+//   16 orbitals, the first 4,000                        0.52              7,973    5,704
+//   15 orbitals, 4,000 at random (lists of 0.6 n_pair)  0.99              18,378   24,140
+//   12 orbitals, 1,000 at random (1.0 n_pair)           0.96              1,548    1,306
+// FCI_CS_FORM=lists or walk overrides the rule (for tests).
+bool cs_by_lists(const fci_context *h, int64_t nnz_c, int64_t n1) {
+    if (const char *env = getenv("FCI_CS_FORM")) return strcmp(env, "lists") == 0;
+    const int64_t moves = 1 + (h->nent_a - h->na) + (h->nent_b - h->nb);
+    return 10 * n1 >= 7 * nnz_c * moves && 5 * n1 < 4 * h->npair * std::min(h->nsa, h->nsb);
+}
+
 CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
     CsSizes z;
     const int64_t nm = h->nent_a + h->nent_b;
@@ -745,7 +829,7 @@ CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
     z.bm_bytes = (size_t)((h->nsa + 31) / 32 + (h->nsb + 31) / 32) * 4;
     z.off_bm = o; o += al(z.bm_bytes);
     z.str_bytes = (size_t)(h->nsa + 1 + h->nsb + 1) * 4;
-    z.n_sums = ceil_div(h->nsa + 1, SCAN_TILE) + ceil_div(h->nsb + 1, SCAN_TILE);
+    z.n_sums = ceil_div(h->nsa + 1 + h->nsb + 1, SCAN_TILE);
     z.off_str = o; o += al(z.str_bytes + (size_t)z.n_sums * 4);
     z.off_list = o; o += al((size_t)z.n1max * 2 * sizeof(int2));
     z.off_work = z.off_hl;  // the support's hash table is done with by then (8 bytes per slot, two slots per entry)
@@ -827,9 +911,9 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     a.off_a = (uint32_t *)(w + z.off_str);
     a.off_b = a.off_a + h->nsa + 1;
     uint32_t *sums = a.off_b + h->nsb + 1;
-    a.list_a = (int2 *)(w + z.off_list);
-    a.list_b = a.list_a + z.n1max;
+    a.list = (int2 *)(w + z.off_list);
     a.work = (int64_t *)(w + z.off_work);
+    a.walk = a.work + z.n2max;
     a.hj = (unsigned long long *)(w + z.off_hj);
     a.hj_col = (int32_t *)(w + z.off_hjc);
     a.hj_mask = z.capj - 1;
@@ -845,7 +929,7 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     unsigned long long cnt[3] = {0, 0, 0};
     // 1. the intermediate determinants one move from a nonzero coefficient, and D on them
     {
-        phase_scope ps(h, s, FCI_PHASE_GATHER, 10);
+        phase_scope ps(h, s, FCI_PHASE_GATHER, 4);
         FCI_CUDA(h, cudaMemsetAsync(a.hj, 0xFF, z.capj * 8, s));
         FCI_CUDA(h, cudaMemsetAsync(a.counts, 0, 256, s));
         const int64_t moves = nnz_c * (a.nent_a + a.nent_b);
@@ -855,18 +939,16 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
         FCI_CUDA(h, cudaMemcpyAsync(cnt, a.counts, sizeof cnt, cudaMemcpyDeviceToHost, s));
         FCI_CUDA(h, cudaStreamSynchronize(s));
         if (cnt[2]) return fci_fail(h, FCI_ERR_CUDA, "compressed sigma: hash table overflow");
+        a.by_lists = cs_by_lists(h, nnz_c, (int64_t)cnt[0]);
+        FCI_CUDA(h, cudaMemsetAsync(a.bm_a, 0, (size_t)((char *)sums - (char *)a.bm_a), s));  // and the counts
         k_cs_gather<<<grid_of((int64_t)cnt[0] * 32), 256, 0, s>>>(a, (int64_t)cnt[0]);
-        FCI_CUDA(h, cudaMemsetAsync(a.bm_a, 0, z.bm_bytes, s));
-        FCI_CUDA(h, cudaMemsetAsync(a.off_a, 0, z.str_bytes, s));
-        k_cs_mark<false><<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
-        auto scan = [&](uint32_t *c, int64_t m, uint32_t *block_sums) {
-            const unsigned nb = (unsigned)ceil_div(m, SCAN_TILE);
-            k_cs_scan_sums<<<nb, 256, 0, s>>>(c, m, block_sums);
-            k_cs_scan<<<nb, 256, 0, s>>>(c, m, block_sums);
-        };
-        scan(a.off_a, h->nsa + 1, sums);
-        scan(a.off_b, h->nsb + 1, sums + ceil_div(h->nsa + 1, SCAN_TILE));
-        k_cs_mark<true><<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
+        if (a.by_lists) {
+            const int64_t m = h->nsa + 1 + h->nsb + 1;
+            k_cs_scan_sums<<<(unsigned)z.n_sums, 256, 0, s>>>(a.off_a, m, sums);
+            k_cs_scan<<<(unsigned)z.n_sums, 256, 0, s>>>(a.off_a, m, sums);
+            k_cs_lists<<<grid_of((int64_t)cnt[0]), 256, 0, s>>>(a, (int64_t)cnt[0]);
+            ps.launches += 3;
+        }
         FCI_CUDA(h, cudaGetLastError());
     }
     const int64_t n1 = (int64_t)cnt[0];
@@ -910,9 +992,16 @@ int fci_sigma_compressed(fci_handle h, const int64_t *c_addr, const double *c_va
     }
     // 4. sigma on the support
     {
-        phase_scope ps(h, s, FCI_PHASE_SCATTER, 2);
-        k_cs_sigma<<<grid_of(n2), 256, 0, s>>>(a, out_addr, n2, out_val);
-        k_cs_sigma_warp<<<152 * 8, 256, 0, s>>>(a, out_addr, out_val);
+        phase_scope ps(h, s, FCI_PHASE_SCATTER, a.by_lists ? 3 : 1);
+        if (a.by_lists) {
+            k_cs_sigma<<<grid_of(n2), 256, 0, s>>>(a, out_addr, n2, out_val);
+            k_cs_sigma_warp<<<152 * 8, 256, 0, s>>>(a, out_addr, out_val);
+            k_cs_sigma_rest<<<152 * 8, 256, 0, s>>>(a, out_addr, out_val);
+        } else if (n2 <= CS_WALK_WARPS) {
+            k_cs_sigma_all<true><<<grid_of(32 * n2), 256, 0, s>>>(a, out_addr, n2, out_val);
+        } else {
+            k_cs_sigma_all<false><<<grid_of(n2), 256, 0, s>>>(a, out_addr, n2, out_val);
+        }
         FCI_CUDA(h, cudaGetLastError());
     }
     FCI_CUDA(h, cudaStreamSynchronize(s));

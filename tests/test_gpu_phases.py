@@ -50,13 +50,15 @@ def test_kernels_of_a_sigma_by_phase(fci_lib, monkeypatch, make, s, form, want):
     assert tuple(t[k]["launches"] for k in ("gather", "contract", "scatter", "other")) == want
 
 
-def test_kernels_of_a_compressed_sigma_by_phase(fci_lib):
-    """Columns: expansion, category ranges, compaction, gather, two passes over the columns and
-    two scans of two kernels; support: emission, compaction and three kernels per 8 bits of the
-    largest address; the two forms of the sum."""
+@pytest.mark.parametrize("form,gather,scatter", [("lists", 7, 3), ("walk", 4, 1)])
+def test_kernels_of_a_compressed_sigma_by_phase(fci_lib, monkeypatch, form, gather, scatter):
+    """Columns: expansion, category ranges, compaction, gather and, with lists, a scan of two kernels
+    and the lists per string; support: emission, compaction and three kernels per 8 bits of the
+    largest address; the sum in three forms or one."""
+    monkeypatch.setenv("FCI_CS_FORM", form)
     f = _das()
     f.set_phase_timing(True)
     f.sigma_compressed(torch.arange(20, device="cuda"), torch.ones(20, dtype=torch.float64, device="cuda"))
     t = f.phase_times()
     bits = (f.n_det - 1).bit_length()
-    assert tuple(t[k]["launches"] for k in ("gather", "contract", "scatter", "other")) == (10, 1, 2, 2 + 3 * -(-bits // 8))
+    assert tuple(t[k]["launches"] for k in ("gather", "contract", "scatter", "other")) == (gather, 1, scatter, 2 + 3 * -(-bits // 8))
