@@ -213,6 +213,7 @@ static void free_strings(fci_context *h) {
     h->d_dstr = nullptr;
     h->d_G = h->d_GT = h->d_hd = h->d_J = h->d_K = nullptr;
     das_free(h);
+    h->cz_share = -1.0;
     h->mode = FCI_MODE_NONE;
     h->nsa = h->nsb = h->ndet = 0;
 }

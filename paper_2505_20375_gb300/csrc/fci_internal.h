@@ -136,6 +136,7 @@ struct fci_context {
     // operator images (Ozaki split of G): alpha/beta strings [0] fused kernel, [1] two-pass GEMM;
     // spinor strings [0] block-sparse GEMM, [1] dense GEMM
     fci_image img[2][FCI_IMAGE_SLICES];
+    mutable double cz_share = -1.0;  // spinor strings: block-sparse work over dense work (-1: not yet known)
     int oz_tuned_nt[9] = {0};    // determinants per tile chosen by the tuner, per slice count (0: default)
     int oz_tuned_path[9] = {0};  // 1: two-pass path (D digit image + bulk-copy GEMM) chosen by the tuner
 

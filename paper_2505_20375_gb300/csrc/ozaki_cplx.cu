@@ -304,24 +304,67 @@ CzGeom cz_geom(const fci_context *h) {
     return {m, (int)ceil_div(m, OZG_M), (int)ceil_div(m, 32)};
 }
 
+// Work of the block-sparse GEMM over that of the dense one: the mean over sampled tiles of
+// (units x active blocks), against M-tiles x K-chunks.  The masks are those of k_cz_split.
+double cz_share(const fci_context *h) {
+    if (h->cz_share >= 0.0) return h->cz_share;
+    const CzBlocks c = cz_blocks(h->n_orb);
+    const CzGeom g = cz_geom(h);
+    const int64_t tiles = ceil_div(h->ndet, CZ_N), samples = std::min<int64_t>(tiles, 24);
+    auto choose = [](int n, int k) {
+        double r = 1.0;
+        for (int i = 1; i <= k; ++i) r = r * (n - k + i) / i;
+        return k > n ? 0.0 : r;  // below 2^53: exact
+    };
+    double sum = 0.0;
+    for (int64_t i = 0; i < samples; ++i) {
+        const int64_t first = (2 * i + 1) * tiles / (2 * samples) * CZ_N, last = std::min(first + CZ_N, h->ndet);
+        uint64_t S = 0;  // the string of rank `first`: strings ascend by value
+        double r = (double)first;
+        for (int p = h->n_orb - 1, k = h->na; k > 0; --p)
+            if (choose(p, k) <= r) {
+                r -= choose(p, k--);
+                S |= (uint64_t)1 << p;
+            }
+        uint64_t occ = 0, full = ~(uint64_t)0;
+        for (int64_t t = first; t < last; ++t) {
+            occ |= S;
+            full &= S;
+            const uint64_t low = S & (~S + 1), up = S + low;  // the next string with as many bits
+            if (low) S = (((up ^ S) >> 2) / low) | up;
+        }
+        int on = c.L;
+        for (int a = c.L; a < c.n; ++a) {
+            if ((occ >> a) & 1)
+                for (int b = 0; b < c.ubk; ++b)
+                    on += ((~full | ((uint64_t)1 << a)) & ((uint64_t)0xFF << (c.L + 8 * b))) != 0;
+            on += ((occ >> a) & 1) + !((full >> a) & 1);
+        }
+        sum += (double)ceil_div(on, 8) * on;
+    }
+    return h->cz_share = sum / (double)samples / ((double)g.n_mt * g.n_kc);
+}
+
 // Which form: the block-sparse GEMM skips half of the MMAs and more, but copies its operator
 // block by block and costs about 3,000 cycles a unit, so it needs many MMAs per unit (slices),
-// many blocks to skip (spinors) and tiles enough to fill the GPU.  us, dense / blocks:
-//   spinors, electrons   s = 3          4              5              6              8
-//   12, 6                108/136        109/140        115/143        119/144        124/152
-//   17, 9                406/538        460/542        529/637        605/644        793/789
-//   19, 9                1,035/1,389    1,296/1,386    1,648/1,752    2,053/1,774    3,012/2,313
-//   20, 10               2,062/2,574    2,710/2,566    3,607/3,331    4,624/3,402    7,031/4,521
-//   22, 5                680/826        825/830        1,011/998      1,224/1,013    1,711/1,272
-//   22, 11               9,664/10,843   13,059/10,780  17,897/14,249  (s = 8 36,463/19,269)
-// 19 spinors with 5 electrons (11,628 determinants) take 473/511 at s = 6.
+// blocks to skip (cz_share; crowded or padded strings skip few) and tiles enough to fill the
+// GPU.  us, dense / blocks:
+//   spinors, electrons, share   s = 4           5               6               8
+//   12, 6                       109/140         115/143         119/144         124/152
+//   21, 5    1.09               598/648         710/767         845/784         1,164/972
+//   19, 10   1.10               1,321/1,440     1,677/1,809     2,079/1,847     3,038/2,405
+//   20, 10   1.08               2,710/2,566     3,607/3,331     4,624/3,402     7,031/4,521
+//   22, 11   0.93               13,059/10,780   17,897/14,249   (s = 8 36,463/19,269)
+//   22, 16   1.20               1,953/2,157     2,451/2,665     3,079/2,698     4,430/3,499
+//   25, 20   1.37               2,448/3,279     3,010/4,063     3,677/4,095     5,254/5,388
 // Up to 3 slices always take the dense form; above, FCI_SPLIT_FORM=dense or blocks overrides
 // the rule (for tests).
 bool cz_dense(const fci_context *h, int s) {
     if (s <= 3) return true;
     if (!oz_gemm_ring(s, 4, 0)) return false;
     if (const char *env = getenv("FCI_SPLIT_FORM")) return strcmp(env, "dense") == 0;
-    return h->n_orb < (s <= 5 ? 20 : 18) || h->ndet < ((int64_t)1 << 14);
+    if (h->n_orb < (s <= 5 ? 20 : 18) || h->ndet < ((int64_t)1 << (s <= 5 ? 16 : 14))) return true;
+    return cz_share(h) > (s <= 5 ? 1.1 : s == 6 ? 1.26 : 1.36);
 }
 
 }  // namespace

@@ -1159,6 +1159,7 @@ struct DgSplit {
     const int32_t *cat_pa, *cat_pb;
     const int32_t *base_int;  // the same for blocks of the intermediate space
     int n_pat_a, row_max;     // longest row: target values that share an alpha string
+    bool long_rows;           // the categories' rows are long on average (dg_by_rows)
     const int64_t *Cint;
     uint8_t *Dimg;
     ulonglong2 *masks;  // [n_nt]
@@ -1281,8 +1282,9 @@ __global__ void k_dg_masks(const __grid_constant__ DgSplit a) {
 // warp load and bound the kernel).  Alpha moves lead from a category to runs of consecutive
 // values: their targets are resolved once per category.  Thread (determinant of 64, core,
 // quarter): the quarters take the active blocks in turn.  The image
-// of 16 orbitals, 12 electrons, one transfer at s = 6: 5.1 ms a determinant at a time, 4.5 by
-// rows.
+// of 16 orbitals, 12 electrons, one transfer at s = 6: 5.1 ms a determinant at a time, 4.4 by
+// rows.  Every category costs the CTA two barriers and a pass over the pairs, so short blocks
+// make it the slower form (dg_by_rows).
 constexpr int DG_ROW_THREADS = 512;
 constexpr size_t DG_ROW_SMEM = 113 * 1024;
 template <int S>
@@ -1487,16 +1489,22 @@ int64_t dg_row_max(const fci_das_layout &L) {
     return most;
 }
 
-// Whether the rows fit; FCI_DAS_ROW_BYTES lowers the limit (for tests of the other form).
+// Whether the image is formed by rows: they fit, and an alpha string has 192 determinants per
+// category on average.  us per image at s = 4, by rows / by determinants, and that average:
+//   16 orbitals, 12 electrons (4 x 4)   284   3,767 / 4,232    (3 x 5 + 2) 5 spaces   48   193 / 70
+//   15 orbitals (4, 7, 4)               209   351 / 350        (2, 2, 6, 6)           23   132 / 23
+//   14 orbitals (4, 6, 4)               165   268 / 198        (6, 1, 4, 2, 2)        10   264 / 25
+// FCI_DAS_ROW_BYTES, if set, is the limit of shared memory instead, for any length (for tests
+// of both forms).
 bool dg_by_rows(const DgSplit &a) {
-    size_t limit = DG_ROW_SMEM;
-    if (const char *env = getenv("FCI_DAS_ROW_BYTES")) limit = std::min<size_t>(limit, (size_t)std::max(0ll, atoll(env)));
-    return dg_row_smem(a) <= limit;
+    if (const char *env = getenv("FCI_DAS_ROW_BYTES"))
+        return dg_row_smem(a) <= std::min<size_t>(DG_ROW_SMEM, (size_t)std::max(0ll, atoll(env)));
+    return a.long_rows && dg_row_smem(a) <= DG_ROW_SMEM;
 }
 int dg_image_launches(const DgSplit &a, bool dense) { return !dense && dg_by_rows(a) ? 2 : 1; }
 
-// Digit image and block masks of a piece.  By rows where two CTAs' rows fit an SM (up to
-// about 14,000 target values per alpha string), else determinant by determinant.
+// Digit image and block masks of a piece, by rows (two CTAs' rows fit an SM up to about 14,000
+// target values per alpha string) or determinant by determinant.
 template <int S>
 cudaError_t dg_image_s(const DgSplit &a, bool dense, cudaStream_t st) {
     if (dense) {
@@ -1660,6 +1668,9 @@ int dg_sigma(fci_context *h, const double *C, double *sigma, int s, void *ws, cu
     sp.base_int = L.d_dz_base + npab;
     sp.n_pat_a = L.n_pat_a;
     sp.row_max = (int)std::min<int64_t>(dg_row_max(L), INT32_MAX);
+    int64_t rows = 0;  // (alpha string, category)
+    for (int c = 0; c < L.n_cat_int; ++c) rows += L.pat_nstr_a[L.cat_pa[c]];
+    sp.long_rows = L.n_det_int >= 192 * rows;
     sp.nstr_b32 = L.d_dz_base + 2 * npab;
     sp.cat_off = L.d_cat_off;
     sp.locbase_a = L.d_pat_locbase_a;

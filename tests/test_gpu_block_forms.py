@@ -59,8 +59,7 @@ def test_das_blocks(fci_lib, monkeypatch, spaces, ref, nel, T, s, image):
     """Both digit images of the block form: the bits of the dense form, and up to 7 slices the
     exact integer model (to the rounding of its inputs, as for the dense form)."""
     monkeypatch.setenv("FCI_SPLIT_FORM", "blocks")
-    if image == "determinants":
-        monkeypatch.setenv("FCI_DAS_ROW_BYTES", "0")
+    monkeypatch.setenv("FCI_DAS_ROW_BYTES", "1000000" if image == "rows" else "0")
     h, g, f, c = _das(spaces, ref, nel, T)
     got = _sigma(f, c, s)
     if s <= 7 and image == "rows":
@@ -80,8 +79,7 @@ def test_das_blocks_in_chunks_and_pieces(fci_lib, monkeypatch, spaces, ref, nel,
     monkeypatch.setenv("FCI_SPLIT_FORM", "dense")
     want = _sigma(f, c, s)
     monkeypatch.setenv("FCI_SPLIT_FORM", "blocks")
-    if image == "determinants":
-        monkeypatch.setenv("FCI_DAS_ROW_BYTES", "0")
+    monkeypatch.setenv("FCI_DAS_ROW_BYTES", "1000000" if image == "rows" else "0")
     monkeypatch.setenv("FCI_DAS_IMAGE_DETS", "150")
     assert torch.equal(want, _sigma(f, c, s))
     monkeypatch.setenv("FCI_DAS_CHUNK_DETS", "700")
@@ -116,14 +114,15 @@ def test_bounded_wait_of_the_block_form(fci_lib, monkeypatch, kind, s):
 
 @pytest.mark.parametrize("kind,s", [("spinor", 6), ("spinor", 4), ("das", 6)])
 def test_default_rule_takes_the_blocks(fci_lib, monkeypatch, kind, s):
-    """20 spinors, and 16 orbitals in four spaces with 2.2 M intermediate determinants: the block
-    form (its workspace; its two kernels for the digit image), the bits of the dense one."""
+    """20 spinors, and 14 orbitals in three spaces with 2.5 M intermediate determinants in rows
+    of more than 192: the block form (its workspace; its two kernels for the digit image), the bits
+    of the dense one."""
     if kind == "spinor":
         h, g = synth.complex_integrals(20, 4, 71)
-        f = gpu_fci(dict(h=h, g=g, e_core=0.3, n=20, ne=6))
+        f = gpu_fci(dict(h=h, g=g, e_core=0.3, n=20, ne=8))
         c = torch.from_numpy(synth.random_vector(f.n_det, seed=7, complex_=True)).cuda()
     else:
-        f, c = _das([4, 4, 4, 4], [1, 1, 1, 1], 4, 1)[2:]
+        f, c = _das([6, 6, 2], [4, 3, 1], 8, 0)[2:]
     f.set_phase_timing(True)
 
     def run():

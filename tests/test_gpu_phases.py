@@ -33,7 +33,8 @@ def _spinor(n, ne):
     (_das, 0, "dense", (0, 1, 1, 0)),
     (_das, 3, "dense", (0, 1, 1, 1)),
     (_das, 6, "dense", (1, 1, 1, 1)),
-    (_das, 6, "blocks", (2, 1, 1, 1)),                   # block masks, digit image by rows
+    (_das, 6, "blocks", (1, 1, 1, 1)),                   # short rows: image by determinants
+    (lambda: _fci(11, 4, 4).build_das([11], [4], [4], 0), 6, "blocks", (2, 1, 1, 2)),  # masks, image by rows
     (lambda: _spinor(10, 4), 0, "dense", (0, 1, 1, 0)),
     (lambda: _spinor(10, 4), 6, "blocks", (2, 1, 1, 0)),
     (lambda: _spinor(16, 6), 3, "dense", (2, 1, 1, 0)),  # 8,008 complex determinants: 16,016 values
