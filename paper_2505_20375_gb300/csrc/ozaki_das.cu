@@ -1081,18 +1081,21 @@ void dg_category_masks(const fci_context *h, const DgBlocks &b, std::vector<ulon
 
 // Which form.  share: MMA work of the block-sparse GEMM over that of the dense one, which has
 // the larger tiles (fewer, larger copies; no cost per unit), so the blocks pay where they skip
-// much or the space is large, and sooner with more slices.  us, dense / blocks:
+// enough, and sooner with more slices.  Spaces below 2^16 determinants (5 waves of tiles and
+// fewer) stay dense.  us, dense / blocks:
 //   share   intermediate determinants   s = 4          s = 6
-//   0.17    2,832                       35/56          37/59
-//   0.25    82,996                      101/129        127/146
-//   0.05    295,488                     209/179        292/194
-//   0.26    388,080                     276/357        385/414
-//   0.36    684,288                     468/513        661/612
-//   0.43    810,688                     632/857        859/1,058
-//   0.17    2,191,360                   2,714/1,934    4,516/2,429
-//   0.43    3,133,440                   4,450/4,686    7,026/6,304
-//   0.30    4,069,504                   3,169/2,721    4,702/3,265
-//   0.64    8,589,600                   8,312/8,653    11,430/11,160
+//   0.02    58,048                      126/88         171/93
+//   0.17    80,929                      110/97         146/108
+//   0.05    460,492                     637/359        1,019/406
+//   0.11    1,056,240                   795/590        1,191/646
+//   0.21    1,724,356                   1,305/1,004    1,952/1,224
+//   0.19    5,309,136                   6,435/4,378    10,783/5,870
+//   0.32    683,165                     501/508        692/613
+//   0.31    3,257,232                   2,640/2,190    3,857/2,767
+//   0.40    560,400                     440/471        598/582
+//   0.58    147,875                     209/213        272/261
+//   0.60    53,190                      95/106         125/127
+//   0.46    10,711,870                  8,679/8,057    12,722/10,485
 // FCI_SPLIT_FORM=dense or blocks overrides it (for tests).
 bool dg_dense(const fci_context *h, const DgBlocks &b, int s) {
     if (!oz_gemm_ring(s, DG_KCC, 0)) return false;
@@ -1113,10 +1116,8 @@ bool dg_dense(const fci_context *h, const DgBlocks &b, int s) {
     }
     const double x = L.dg_share;
     const int64_t n = L.n_det_int;
-    const bool blocks = s <= 5 ? (x < 0.32 && n >= ((int64_t)1 << 20)) || (x < 0.1 && n >= ((int64_t)1 << 17))
-                               : n >= ((int64_t)1 << 21) || (x < 0.4 && n >= ((int64_t)1 << 19)) ||
-                                     (x < 0.1 && n >= ((int64_t)1 << 16));
-    return !blocks;
+    const bool blocks = s <= 5 ? x < 0.32 : x < 0.45 || n >= ((int64_t)1 << 21);
+    return !blocks || n < ((int64_t)1 << 16);
 }
 
 struct DgGeom {
