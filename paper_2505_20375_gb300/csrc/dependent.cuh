@@ -10,7 +10,7 @@
 // either side both calls do nothing; with early false the launch is an ordinary one.
 //
 // A kernel that lives on L1 is not admitted early beside one that occupies every SM: it runs to
-// its end with the L1 that the SM had then (k_to_fixed in fixed_point.cu, k_oz_gemm).
+// its end with the L1 that the SM had then (k_to_fixed in fixed_point.cu, k_oz_contract, k_oz_gemm).
 //
 // What it is for: a split sigma of a small space is three or four kernels of 5 to 15 us, and
 // their launches and set-up (the operator's digits into shared memory) stood between them.
