@@ -790,7 +790,7 @@ struct CsSizes {
 // every support entry.  Lists pay while they are short: for a sparse vector whose
 // coefficients reach columns of their own.  The columns of neighbouring coefficients
 // coincide (n1 below nnz times the moves of a determinant, the diagonal ones as one), and the
-// lists of a nearly full space hold about as many as a walk's n_pair; then a walk by
+// lists of a nearly full space hold about as many as a walk has pairs; then a walk by
 // threads, whose neighbours look up the same columns, is the faster one.  us per sigma,
 // lists / walk:
 //                                                       columns / moves   lists    walk
@@ -804,7 +804,14 @@ struct CsSizes {
 bool cs_by_lists(const fci_context *h, int64_t nnz_c, int64_t n1) {
     if (const char *env = getenv("FCI_CS_FORM")) return strcmp(env, "lists") == 0;
     const int64_t moves = 1 + (h->nent_a - h->na) + (h->nent_b - h->nb);
-    return 10 * n1 >= 7 * nnz_c * moves && 5 * n1 < 4 * h->npair * std::min(h->nsa, h->nsb);
+    // half of the columns keep the alpha string of their coefficient, half the beta string: the
+    // mean lists of a target determinant's two strings, at least
+    const fci_das_layout &L = h->das;
+    int64_t na = 0, nb = 0;  // strings of target determinants
+    for (int p = 0; p < L.n_pat_a; ++p) na += L.exc_a[p] <= L.max_transfer ? L.pat_nstr_a[p] : 0;
+    for (int p = 0; p < L.n_pat_b; ++p) nb += L.exc_b[p] <= L.max_transfer ? L.pat_nstr_b[p] : 0;
+    const double lists = 0.5 * (double)n1 * (1.0 / (double)na + 1.0 / (double)nb);
+    return 10 * n1 >= 7 * nnz_c * moves && lists < 0.8 * h->npair;
 }
 
 CsSizes cs_sizes(const fci_context *h, int64_t nnz_c) {
