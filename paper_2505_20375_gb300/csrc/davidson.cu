@@ -4,8 +4,8 @@
 // Every vector operation runs here in FP64 (complex vectors as interleaved pairs):
 // subspace projections V^H w, Ritz combinations, the residual, the preconditioner with
 // its 1e-12 guard and eps * ||s|| threshold, two rounds of classical Gram-Schmidt and
-// the projected eigenproblem (one thread block; complex Hermitian matrices through their
-// real symmetric embedding [[A, -B], [B, A]]).  The host reads back a handful of scalars per
+// the projected eigenproblem (a cluster of eight thread blocks; complex Hermitian matrices
+// through their real symmetric embedding [[A, -B], [B, A]]).  The host reads back a handful of scalars per
 // iteration to decide convergence.  On small spaces the vector work is a chain of short
 // launches, so every reduction ends inside its own kernel: the last block to finish adds
 // the block partials in a fixed order and applies what follows (a sign, the new column of

@@ -16,8 +16,8 @@
 // their launches and set-up (the operator's digits into shared memory) stood between them.
 // us per sigma of FCI, calls issued back to back, ordinary / dependent launches:
 //   determinants      4,900       14,400      63,504      853,776     2,944,656
-//   s = 3             28.7/21.0   32.8/26.7   52.5/48.0   450/442     1,631/1,624
-//   s = 6             32.8/23.2   39.0/32.8   71.0/68.6   671/662     2,534/2,523
+//   s = 3             28.7/20.7   32.8/26.7   52.5/46.6   450/442     1,631/1,627
+//   s = 6             32.8/23.6   39.0/32.9   71.0/65.2   671/663     2,534/2,530
 #pragma once
 
 #include <cuda_runtime.h>
